@@ -1,20 +1,30 @@
-// mpipe_linear_fwd: C[M, N] = epilogue(A[M, K] * W[N, K]^T), the dense projections of the packed encoder layer
-// (QKV, attention output, MLP) on the token matrix [T, hidden].  bf16 operands, fp32 accumulation in TMEM.
-// mpipe_linear_dgrad: dX[M, K] = epilogue(dY[M, N] * W[N, K]) -- the same kernel with the second operand read as
-// [contraction][output] (an MN-major B: four 64-column atoms per stage, loaded as four TMA boxes).
-// mpipe_linear_wgrad: dW[N, K] += dY[M, N]^T * X[M, K] in fp32 -- both operands MN-major (the token index is the
-// contraction), the token range split over CTAs, partial tiles added with TMA reduce-add.
+// The dense projections of the packed encoder layer (QKV, attention output, MLP) and their gradients on the token matrix
+// [T, hidden]; bf16 operands, fp32 accumulation in TMEM.
+//   mpipe_linear_fwd    C[M, N]  = epilogue(A[M, K] W[N, K]^T)      both operands K-major
+//   mpipe_linear_dgrad  dX[M, K] = epilogue(dY[M, N] W[N, K])       second operand [contraction][output], MN-major
+//   mpipe_linear_wgrad  dW[N, K] += dY[M, N]^T X[M, K] in fp32      both operands MN-major (the token index is the contraction);
+//                       the token range is split over CTA pairs, partial tiles are added with TMA reduce-add
 //
-// Persistent kernel, one CTA per SM, static round-robin over 128 x 256 output tiles (n fastest, so that the
-// CTAs of a wave share the few weight tiles in L2 and walk down the token rows together).
-//   warp 0      TMA producer: A box [128 rows][64 k], W box [256 rows][64 k] per stage, 128-byte swizzle, 4 stages
-//   warp 1      tcgen05 issuer: 4 x (M 128, N 256, K 16) smem x smem MMAs per stage into one of TWO 256-column
-//               TMEM accumulators, so the epilogue of tile i overlaps the main loop of tile i + 1
+// One kernel, a CTA PAIR (cta_group::2) per 256 x BN output tile: each CTA holds 128 rows of A, half of the BN columns of B and
+// 128 x BN of the fp32 result in its TMEM.  What bounds a projection of a full-size microbatch is the tensor pipe, and next to
+// it the operand traffic from L2: a 128 x 256 tile on one CTA asks 96 bytes per clock and SM while the pipe runs at its peak, the
+// pair 64.  Persistent: pair i takes tiles i, i + pairs, ... (n fastest, so that a wave shares the weight tiles in L2 and walks
+// down the token rows together).  Warp roles of each CTA (384 threads):
+//   warps 0, 3  TMA producers of the CTA's half, A box [128 rows][64 k] and B box [BN / 2 rows][64 k] (MN-major: boxes of 64
+//               columns) per stage, 128-byte swizzle, 5 to 8 stages; the bytes of both CTAs are counted on the even CTA's barrier
+//   warp 1      (even CTA) tcgen05 issuer: 4 x (M 256, N BN, K 16) per stage into one of TWO accumulators of up to 256 columns, so
+//               that the epilogue of tile i overlaps the main loop of tile i + 1
 //   warp 2      TMEM allocation
-//   warps 4-11  epilogue: thread = output row = TMEM lane; warpgroup 0 takes columns 0..127, warpgroup 1
-//               columns 128..255; 32 columns per TMEM round trip; + bias, GELU, + residual in fp32, bf16 into a
-//               64-byte-swizzled [128 rows][32 columns] staging box (two per warpgroup), one TMA store per box --
-//               row-per-thread global stores cost 32 L1 wavefronts per instruction and bound the K = 1024 cases
+//   warps 4-11  epilogue: thread = output row = TMEM lane; the two warpgroups take alternate 64-column chunks.  Every warp owns two
+//               [32 rows][64 columns] staging boxes (128-byte swizzle): a side operand (residual, or the pre-activation the
+//               gradient of GELU needs) arrives in the box by TMA before the accumulator is ready, the result replaces it in
+//               place, and one TMA store takes it out.  No barrier between warps: with one staging box per warpgroup and two
+//               named barriers per 32 columns the epilogue of the GELU projections was longer than their main loop.
+// Small problems (fewer tiles than pairs): a cluster of `splits` pairs shares a tile, each taking a part of the contraction; the
+// partial results meet in shared memory (every pair finishes the chunks it owns from the others' fp32 partials).
+// Measured against the one-CTA 128 x 256 kernel with warpgroup-wide staging that this replaces (us, M = 50 439): fc1 + GELU
+// 1024 -> 4096 398 -> 328, its gradient with GELU' 480 -> 383, attention output + residual 115 -> 90, QKV 241 -> 225 (1410
+// TFLOP/s), weight gradient 1024 x 4096 348 -> 292; M = 777: fc2 27.9 -> 14.7 (split), weight gradient 1024 x 4096 34 -> 14.
 // Every mbarrier wait is bounded (status MPIPE_ERR_TIMEOUT), as in the attention kernels.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -27,43 +37,50 @@
 
 namespace mpipe {
 
-constexpr int kGemmBM = 128, kGemmBN = 256, kGemmBK = 64, kGemmStages = 4;
+constexpr int kGemmBM = 128, kGemmBK = 64;                    // rows per CTA (256 per pair), contraction per stage
+constexpr int kGemmMaxBN = 256;
 constexpr int kGemmThreads = 384;
-constexpr int kGemmABytes = kGemmBM * kGemmBK * 2;   // 16 KB
-constexpr int kGemmBBytes = kGemmBN * kGemmBK * 2;   // 32 KB
-constexpr int kGemmStageBytes = kGemmABytes + kGemmBBytes;
-constexpr int kGemmOutBox = kGemmBM * 64;            // [128 rows][32 bf16] staging box
-constexpr int kGemmSmemOut = kGemmStages * kGemmStageBytes;   // 2 warpgroups x 2 boxes
-constexpr int kGemmSmem = kGemmSmemOut + 4 * kGemmOutBox + 1024;
+constexpr int kGemmABytes = kGemmBM * kGemmBK * 2;            // 16 KB
+constexpr int kGemmRing = 160 * 1024, kGemmMaxStages = 8;     // 5 stages at BN 256 and 192, 6 at 128, 8 at 64
+constexpr int kGemmBox = 32 * 128;                            // [32 rows][128 bytes] staging box of one warp
+constexpr int kGemmSmemOut = kGemmRing;                       // 8 warps x 2 boxes
+constexpr int kGemmSmem = kGemmSmemOut + 8 * 2 * kGemmBox + 1024;
+constexpr int kGemmMaxSplits = 2;   // four pairs per tile never beat two (measured)
+// a tile's fp32 partials from the other splits: (splits - 1) senders x (BN / 64 / splits) chunks of [16 column groups][128 rows][16 B]
+constexpr int kGemmPartChunk = 16 * 128 * 16;
 static_assert(kGemmSmem <= 227 * 1024, "shared memory budget");
+static_assert((kGemmMaxSplits - 1) * 2 * kGemmPartChunk <= kGemmSmemOut, "partials reuse the stages");
+
+enum { kEpiPlain = 0, kEpiGelu = 1, kEpiGeluGrad = 2 };
 
 struct GemmParams {
     int32_t M, N, K;
+    int32_t bn;                      // columns of a tile: 64, 128, 192 or 256
+    int32_t stages;                  // of kGemmABytes + 64 bn bytes each in the ring
     int32_t tiles_m, tiles_n;
+    int32_t splits;                  // pairs that share a tile's contraction (weight gradient: parts of the token range)
     const __nv_bfloat16* bias;       // [N] or null
-    const __nv_bfloat16* residual;   // [M, ldr] or null
-    const __nv_bfloat16* aux;        // [M, ldx] or null: pre-activation u; the result is multiplied by GELU'(u)
-    int64_t ldx;
-    __nv_bfloat16* C;                // [M, ldc]
-    int64_t ldr, ldc;
-    int32_t gelu;
-    int32_t store_pre;               // with gelu: also store the pre-activation (bf16) through map_u
-    int32_t splits;                  // weight gradient: parts the contraction (token) range is cut into
+    const __nv_bfloat16* direct_res; // [M, ldr] or null: residual read by the epilogue threads (when the boxes carry something else)
+    int64_t ldr;
+    int32_t side;                    // the side operand of map_s: residual (plain, GELU) or pre-activation (GELU gradient)
+    int32_t store_pre;               // GELU only: also store the pre-activation (bf16) through map_u
     int32_t* status_buf;
 };
 
 struct GemmBarriers {
-    uint64_t full[kGemmStages], empty[kGemmStages], acc_full[2], acc_empty[2];
+    uint64_t full[kGemmMaxStages], empty[kGemmMaxStages], acc_full[2], acc_empty[2], side_full[8][2];
 };
 
-// kBMode 0: W tile [256 output rows][64 k], K-major (forward).  kBMode 1: W tile [64 contraction rows][256 output
-// columns], MN-major: four [64][64] atoms 8 KB apart (input gradient).  kBMode 2 (weight gradient): as 1, and the first
-// operand too is [64 contraction rows][128 output columns], MN-major, two atoms; work items are (tile, split) pairs and
-// the fp32 result is added to the output with TMA reductions instead of being stored as bf16.
-template <int kBMode>
+__device__ __forceinline__ float2 bf16x2_to_f2(uint32_t w) {
+    return make_float2(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
+}
+
+// kMode 0: forward, 1: input gradient, 2: weight gradient (see above)
+template <int kMode, int kEpi>
 __global__ void __launch_bounds__(kGemmThreads, 1)
 linear_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_w,
-                  const __grid_constant__ CUtensorMap map_c, const __grid_constant__ CUtensorMap map_u, const GemmParams p) {
+              const __grid_constant__ CUtensorMap map_c, const __grid_constant__ CUtensorMap map_s,
+              const __grid_constant__ CUtensorMap map_u, const GemmParams p) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     __shared__ GemmBarriers bars;
@@ -71,319 +88,465 @@ linear_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
     __shared__ int abort_flag;
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const uint32_t crank = cluster_ctarank();
+    const int half = int(crank & 1);                          // which 128 rows of A / half of B this CTA holds
+    const uint32_t lead = crank & ~1u;                        // the pair's issuing CTA
     if (tid == 0) {
         abort_flag = 0;
-        for (int s = 0; s < kGemmStages; ++s) {
+        for (int s = 0; s < kGemmMaxStages; ++s) {
             mbar_init(&bars.full[s], 1);
             mbar_init(&bars.empty[s], 1);
         }
         for (int a = 0; a < 2; ++a) {
             mbar_init(&bars.acc_full[a], 1);
-            mbar_init(&bars.acc_empty[a], 8);
+            mbar_init(&bars.acc_empty[a], 16);                // the epilogue warps of both CTAs
         }
+        for (int w = 0; w < 8; ++w)
+            for (int b = 0; b < 2; ++b) mbar_init(&bars.side_full[w][b], 1);
         fence_mbar_init();
     }
     if (warp == 2) {
-        tmem_alloc(&tmem_base_slot, 512);
-        tmem_relinquish();
+        tmem_alloc_pair(&tmem_base_slot, 512);
+        tmem_relinquish_pair();
     }
+    if (lane == 0) {   // descriptors first: an epilogue that meets a cold one waits a microsecond for it
+        if (warp == 0) prefetch_tmap(&map_a);
+        if (warp == 3) prefetch_tmap(&map_w);
+        if (warp == 4) prefetch_tmap(&map_c);
+        if (warp == 5) prefetch_tmap(&map_s);
+        if (warp == 6) prefetch_tmap(&map_u);
+    }
+    __syncwarp();
     tc_fence_before();
-    __syncthreads();
+    cluster_sync_all();                                       // the peer's barriers exist before anything arrives on them
     tc_fence_after();
     const uint32_t tmem = tmem_base_slot;
     const int nk = (p.K + kGemmBK - 1) / kGemmBK;
-    const int n_tiles = p.tiles_m * p.tiles_n * (kBMode == 2 ? p.splits : 1);   // work items
-    // work item -> output tile and range of contraction blocks
-    // (weight gradient: the split index is the slow one, so that the CTAs of a wave work on the same token range and
-    //  share its dY and X rows through L2)
     const int n_out_tiles = p.tiles_m * p.tiles_n;
-    auto tile_of = [&](int t) { return kBMode == 2 ? t % n_out_tiles : t; };
-    auto kb_lo_of = [&](int t) { return kBMode == 2 ? int((long long)(t / n_out_tiles) * nk / p.splits) : 0; };
-    auto kb_hi_of = [&](int t) { return kBMode == 2 ? int((long long)(t / n_out_tiles + 1) * nk / p.splits) : nk; };
+    const int n_items = n_out_tiles * (kMode == 2 ? p.splits : 1);
+    const int ksplit = kMode == 2 ? 1 : p.splits;             // pairs per cluster
+    const int cid = int(blockIdx.x) / (2 * ksplit), n_clusters = int(gridDim.x) / (2 * ksplit);
+    const int my_split = int(crank >> 1);
+    // work item -> output tile and range of contraction blocks (weight gradient: the split index is the slow one, so that the
+    // pairs of a wave work on the same token range and share its dY and X rows through L2)
+    auto tile_of = [&](int t) { return kMode == 2 ? t % n_out_tiles : t; };
+    auto kb_lo_of = [&](int t) { return int((long long)(kMode == 2 ? t / n_out_tiles : my_split) * nk / p.splits); };
+    auto kb_hi_of = [&](int t) { return int((long long)(kMode == 2 ? t / n_out_tiles + 1 : my_split + 1) * nk / p.splits); };
+    const int bn = p.bn, bn_half = bn >> 1;
+    const int stage_bytes = kGemmABytes + bn_half * kGemmBK * 2, n_stages = p.stages;
 
-    if (warp == 0) {
+    if (warp == 0 || warp == 3) {
+        // Two producers, one per operand: a thread gets a TMA instruction out every ~90 clocks and a barrier test through in
+        // ~110, so one thread issuing both operands' boxes was the slowest role below BN 256 (455 clocks per stage whatever BN)
+        // and in the weight gradient, whose stages are four boxes (660).
         if (lane == 0) {
-            prefetch_tmap(&map_a);
-            prefetch_tmap(&map_w);
-            uint32_t it = 0;
+            const bool is_a = warp == 0;
+            const uint32_t tx = 2u * uint32_t(stage_bytes);   // both CTAs' boxes; out-of-range elements are zero-filled and still counted
+            const uint32_t bar0 = mapa_u32(smem_u32(&bars.full[0]), lead);
+            uint32_t s = 0, ph = 1;                           // ring position; parity of the "empty" phase awaited
             bool ok = true;
-            for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x) {
-                const int m0 = (tile_of(t) / p.tiles_n) * kGemmBM, n0 = (tile_of(t) % p.tiles_n) * kGemmBN;
-                for (int kb = kb_lo_of(t); kb < kb_hi_of(t); ++kb, ++it) {
-                    const int s = it % kGemmStages;
-                    ok = mbar_wait<100>(&bars.empty[s], ((it / kGemmStages) & 1) ^ 1, &abort_flag);
+            for (int t = cid; t < n_items && ok; t += n_clusters) {
+                const int m0 = (tile_of(t) / p.tiles_n) * 2 * kGemmBM + half * kGemmBM;
+                const int n0 = (tile_of(t) % p.tiles_n) * bn + half * bn_half;
+                const int kb_hi = kb_hi_of(t);
+                for (int kb = kb_lo_of(t); kb < kb_hi; ++kb) {
+                    ok = mbar_wait(&bars.empty[s], ph, &abort_flag);
                     if (!ok) break;
-                    uint8_t* st = smem + s * kGemmStageBytes;
-                    mbar_expect_tx(&bars.full[s], kGemmStageBytes);   // out-of-range rows / columns are zero-filled, still counted
-                    if (kBMode == 2) {
+                    uint8_t* st = smem + s * stage_bytes;
+                    const uint32_t bar = bar0 + s * 8;
+                    if (is_a) {
+                        if (half == 0) mbar_expect_tx(&bars.full[s], tx);
+                        if (kMode == 2) {
 #pragma unroll
-                        for (int i = 0; i < kGemmBM / 64; ++i)
-                            tma_load_3d(st + i * (kGemmBK * 128), &map_a, &bars.full[s], m0 + 64 * i, 0, kb * kGemmBK);
+                            for (int i = 0; i < kGemmBM / 64; ++i)
+                                tma_load_3d_pair(st + i * (kGemmBK * 128), &map_a, bar, m0 + 64 * i, 0, kb * kGemmBK);
+                        } else {
+                            tma_load_3d_pair(st, &map_a, bar, kb * kGemmBK, 0, m0);
+                        }
+                    } else if (kMode == 0) {
+                        tma_load_3d_pair(st + kGemmABytes, &map_w, bar, kb * kGemmBK, 0, n0);
                     } else {
-                        tma_load_3d(st, &map_a, &bars.full[s], kb * kGemmBK, 0, m0);
+                        for (int i = 0; i < bn_half / 64; ++i)
+                            tma_load_3d_pair(st + kGemmABytes + i * (kGemmBK * 128), &map_w, bar, n0 + 64 * i, 0, kb * kGemmBK);
                     }
-                    if (kBMode == 0) {
-                        tma_load_3d(st + kGemmABytes, &map_w, &bars.full[s], kb * kGemmBK, 0, n0);
-                    } else {
-#pragma unroll
-                        for (int i = 0; i < kGemmBN / 64; ++i)
-                            tma_load_3d(st + kGemmABytes + i * (kGemmBK * 128), &map_w, &bars.full[s], n0 + 64 * i, 0, kb * kGemmBK);
-                    }
+                    if (++s == uint32_t(n_stages)) { s = 0; ph ^= 1; }
                 }
             }
         }
         __syncwarp();
-    } else if (warp == 1) {
+    } else if (warp == 1 && half == 0) {
         const bool leader = elect_one();
         const uint32_t sbase = smem_u32(smem);
         constexpr uint32_t hi128 = umma_desc_hi(1024, kSwizzle128);
-        constexpr uint32_t idesc = umma_idesc_bf16(kGemmBM, kGemmBN, kBMode == 2 ? 1 : 0, kBMode != 0 ? 1 : 0);
-        uint32_t it = 0, tile_it = 0;
+        const uint32_t idesc = umma_idesc_bf16(2 * kGemmBM, bn, kMode == 2 ? 1 : 0, kMode != 0 ? 1 : 0);
+        const uint16_t pair_mask = uint16_t(3u << lead);
+        uint32_t s = 0, ph = 0, tile_it = 0;
         bool ok = true;
-        for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x, ++tile_it) {
-            if (kb_lo_of(t) >= kb_hi_of(t)) { --tile_it; continue; }   // an empty split: no role touches it
+        for (int t = cid; t < n_items && ok; t += n_clusters, ++tile_it) {
+            const int lo = kb_lo_of(t), hi = kb_hi_of(t);
+            if (lo >= hi) { --tile_it; continue; }   // an empty split: no role touches it
             const uint32_t acc = tile_it & 1;
             ok = mbar_wait(&bars.acc_empty[acc], ((tile_it >> 1) & 1) ^ 1, &abort_flag);
             if (!ok) break;
             tc_fence_after();
-            for (int kb = kb_lo_of(t); kb < kb_hi_of(t); ++kb, ++it) {
-                const int s = it % kGemmStages;
-                ok = mbar_wait(&bars.full[s], (it / kGemmStages) & 1, &abort_flag);
+            for (int kb = lo; kb < hi; ++kb) {
+                ok = mbar_wait(&bars.full[s], ph, &abort_flag);
                 if (!ok) break;
                 tc_fence_after();
-                const uint32_t a_lo = umma_desc_lo(sbase + s * kGemmStageBytes, kBMode == 2 ? kGemmBK * 128 : 0);
-                constexpr uint32_t a_step = kBMode == 2 ? 128 : 2;
-                const uint32_t b_lo = umma_desc_lo(sbase + s * kGemmStageBytes + kGemmABytes, kBMode == 0 ? 0 : kGemmBK * 128);
-                constexpr uint32_t b_step = kBMode == 0 ? 2 : 128;   // one K-step: 32 bytes along a row, or 16 rows of 128 bytes
+                const uint32_t a_lo = umma_desc_lo(sbase + s * stage_bytes, kMode == 2 ? kGemmBK * 128 : 0);
+                constexpr uint32_t a_step = kMode == 2 ? 128 : 2;
+                const uint32_t b_lo = umma_desc_lo(sbase + s * stage_bytes + kGemmABytes, kMode == 0 ? 0 : kGemmBK * 128);
+                constexpr uint32_t b_step = kMode == 0 ? 2 : 128;   // one K-step: 32 bytes along a row, or 16 rows of 128 bytes
                 if (leader) {
 #pragma unroll
                     for (int ks = 0; ks < kGemmBK / 16; ++ks)
-                        umma_ss(tmem + acc * kGemmBN, umma_desc(a_lo + ks * a_step, hi128), umma_desc(b_lo + ks * b_step, hi128), idesc,
-                                (kb > kb_lo_of(t) || ks > 0) ? 1u : 0u);
-                    umma_commit(&bars.empty[s]);
+                        umma_ss_pair(tmem + acc * kGemmMaxBN, umma_desc(a_lo + ks * a_step, hi128), umma_desc(b_lo + ks * b_step, hi128),
+                                     idesc, (kb > lo || ks > 0) ? 1u : 0u);
+                    umma_commit_pair(&bars.empty[s], pair_mask);
                 }
+                if (++s == uint32_t(n_stages)) { s = 0; ph ^= 1; }
             }
             if (!ok) break;
-            if (leader) umma_commit(&bars.acc_full[acc]);
+            if (leader) umma_commit_pair(&bars.acc_full[acc], pair_mask);
         }
         __syncwarp();
     } else if (warp >= 4) {
-        const int wg = (warp - 4) >> 2;                 // column half of the tile
-        const int r = ((warp & 3) << 5) | lane;         // output row inside the tile = TMEM lane
-        const uint32_t lane_base = uint32_t((warp & 3) * 32) << 16;
-        const int wt = tid - (4 + 4 * wg) * 32;         // thread index inside the warpgroup
-        uint8_t* boxes = smem + kGemmSmemOut + wg * 2 * kGemmOutBox;
-        uint32_t tile_it = 0, box_it = 0;
+        const int ew = warp - 4, wg = ew >> 2, quarter = warp & 3;
+        const uint32_t lane_base = uint32_t(quarter * 32) << 16;
+        uint8_t* boxes = smem + kGemmSmemOut + ew * 2 * kGemmBox;
+        uint32_t acc_empty_addr[2] = {mapa_u32(smem_u32(&bars.acc_empty[0]), lead), mapa_u32(smem_u32(&bars.acc_empty[1]), lead)};
+        const int n_chunks = bn >> 6;
+        uint32_t tile_it = 0, bc = 0;   // bc: boxes used so far by this warp; box = bc & 1
         bool ok = true;
-        for (int t = blockIdx.x; t < n_tiles; t += gridDim.x, ++tile_it) {
-            // no early exit: the warpgroup meets at named barriers, so after a time-out it keeps walking empty tiles
+        for (int t = cid; t < n_items; t += n_clusters, ++tile_it) {
             if (kb_lo_of(t) >= kb_hi_of(t)) { --tile_it; continue; }
             const uint32_t acc = tile_it & 1;
-            const int m0 = (tile_of(t) / p.tiles_n) * kGemmBM;
-            const int m = m0 + r;
-            const int n_base = (tile_of(t) % p.tiles_n) * kGemmBN + wg * (kGemmBN / 2);
-            const bool row_ok = m < p.M;
-            const __nv_bfloat16* rrow = (p.residual != nullptr && row_ok) ? p.residual + int64_t(m) * p.ldr : nullptr;
-            // the residual row is fetched one 32-column chunk ahead (each thread reads its own row: latency, not bandwidth)
-            uint4 res[4];
-            auto load_res = [&](int c0) {
-#pragma unroll
-                for (int g8 = 0; g8 < 4; ++g8) {
-                    const int n = n_base + c0 + 8 * g8;
-                    res[g8] = (rrow != nullptr && n < p.N) ? __ldg(reinterpret_cast<const uint4*>(rrow + n)) : make_uint4(0u, 0u, 0u, 0u);
+            const uint32_t tacc = tmem + lane_base + acc * kGemmMaxBN;
+            const int m0 = (tile_of(t) / p.tiles_n) * 2 * kGemmBM + half * kGemmBM + quarter * 32;   // first row of this warp
+            const int n0 = (tile_of(t) % p.tiles_n) * bn;
+            const bool rows_in = m0 < p.M;
+            // the chunks this warp finishes: wg, wg + 2, ... of the tile; with a split contraction, those its pair owns
+            const int own = n_chunks / ksplit;                                // chunks per pair
+            auto chunk_of = [&](int i) { return ksplit == 1 ? i : my_split * own + i; };
+            auto active = [&](int i) { return rows_in && n0 + 64 * chunk_of(i) < p.N; };
+            if (kMode != 2 && p.side && ok) {   // the side operand of both chunks, before the accumulator is ready
+                uint32_t b = bc;
+                for (int i = wg; i < own; i += 2) {
+                    if (!active(i)) continue;
+                    if (lane == 0) {
+                        if (i == wg) bulk_wait_group_read<1>();   // the store that used this box two boxes ago has read it
+                        else bulk_wait_group_read<0>();
+                        mbar_expect_tx(&bars.side_full[ew][b & 1], kGemmBox);
+                        tma_load_3d(boxes + (b & 1) * kGemmBox, &map_s, &bars.side_full[ew][b & 1], n0 + 64 * chunk_of(i), 0, m0);
+                    }
+                    ++b;
                 }
-            };
-            const __nv_bfloat16* xrow = (p.aux != nullptr && row_ok) ? p.aux + int64_t(m) * p.ldx : nullptr;
-            uint4 aux[4];
-            auto load_aux = [&](int c0) {
-#pragma unroll
-                for (int g8 = 0; g8 < 4; ++g8) {
-                    const int n = n_base + c0 + 8 * g8;
-                    aux[g8] = (xrow != nullptr && n < p.N) ? __ldg(reinterpret_cast<const uint4*>(xrow + n)) : make_uint4(0u, 0u, 0u, 0u);
-                }
-            };
-            if (p.residual != nullptr) load_res(0);
-            if (p.aux != nullptr) load_aux(0);
+            }
             if (ok) ok = mbar_wait(&bars.acc_full[acc], (tile_it >> 1) & 1, &abort_flag);
             tc_fence_after();
+            if (kMode != 2 && ksplit > 1) {
+                // every pair of the cluster is past its main loop: the stages of all of them can take partials
+                __syncwarp();
+                cluster_sync_all();
+                for (int c = wg; c < n_chunks; c += 2) {
+                    const int owner = c / own;
+                    if (owner == my_split) continue;
+                    const int slot = (my_split < owner ? my_split : my_split - 1) * own + (c - owner * own);
+                    const uint32_t dst = mapa_u32(smem_u32(smem + slot * kGemmPartChunk + (quarter * 32 + lane) * 16), uint32_t(2 * owner + half));
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        uint32_t v[32];
+                        tmem_ld32(tacc + c * 64 + h * 32, v);
+                        tmem_wait_ld();
+#pragma unroll
+                        for (int g = 0; g < 8; ++g)
+                            st_cluster_v4(dst + (h * 8 + g) * 2048, v[4 * g], v[4 * g + 1], v[4 * g + 2], v[4 * g + 3]);
+                    }
+                }
+                __syncwarp();
+                cluster_sync_all();
+            }
+            bool released = false;
+            auto release = [&]() {   // this warp has read its part of the accumulator
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive_cluster(acc_empty_addr[acc]);
+                released = true;
+            };
 #pragma unroll 1
-            for (int c0 = 0; c0 < kGemmBN / 2; c0 += 32, ++box_it) {
-                uint32_t v[32];
-                uint32_t out[16];
-                uint32_t pre[16];   // pre-activation of the same 32 columns (only with store_pre)
-                uint4 rcur[4];
-                uint4 xcur[4];
-                if (p.residual != nullptr) {
+            for (int i = wg; i < own; i += 2) {
+                const int c = chunk_of(i);
+                const bool last = i + 2 >= own;
+                if (!active(i) || !ok) continue;
+                const int n = n0 + 64 * c;
+                uint32_t v[64];
+                tmem_ld32(tacc + c * 64, *reinterpret_cast<uint32_t(*)[32]>(&v[0]));
+                tmem_ld32(tacc + c * 64 + 32, *reinterpret_cast<uint32_t(*)[32]>(&v[32]));
+                tmem_wait_ld();
+                if (last) release();
+                if (kMode == 2) {   // fp32 partial tile, added to the output: two [32 rows][32 fp32] boxes
 #pragma unroll
-                    for (int g8 = 0; g8 < 4; ++g8) rcur[g8] = res[g8];
-                    if (c0 + 32 < kGemmBN / 2) load_res(c0 + 32);
-                }
-                if (p.aux != nullptr) {
-#pragma unroll
-                    for (int g8 = 0; g8 < 4; ++g8) xcur[g8] = aux[g8];
-                    if (c0 + 32 < kGemmBN / 2) load_aux(c0 + 32);
-                }
-                if (ok) {
-                    tmem_ld32(tmem + lane_base + acc * kGemmBN + wg * (kGemmBN / 2) + c0, v);
-                    tmem_wait_ld();
-                    if (c0 + 32 == kGemmBN / 2) {   // this thread's part of the accumulator is in registers
-                        tc_fence_before();
+                    for (int h = 0; h < 2; ++h, ++bc) {
+                        uint8_t* box = boxes + (bc & 1) * kGemmBox;
+                        if (lane == 0) bulk_wait_group_read<1>();
                         __syncwarp();
-                        if (lane == 0) mbar_arrive(&bars.acc_empty[acc]);
-                    }
 #pragma unroll
-                    for (int g8 = 0; g8 < 4; ++g8) {   // 8 columns = 16 bytes of output
-                        const int n = n_base + c0 + 8 * g8;
-                        const bool col_ok = n < p.N;     // N is a multiple of 8; the store clips what lies outside
-                        float f[8];
-#pragma unroll
-                        for (int i = 0; i < 8; ++i) f[i] = __uint_as_float(v[8 * g8 + i]);
-                        if (p.bias != nullptr && col_ok) {
-                            const uint4 b4 = __ldg(reinterpret_cast<const uint4*>(p.bias + n));
-                            const uint32_t bw[4] = {b4.x, b4.y, b4.z, b4.w};
-#pragma unroll
-                            for (int i = 0; i < 4; ++i) {
-                                f[2 * i] += __uint_as_float(bw[i] << 16);
-                                f[2 * i + 1] += __uint_as_float(bw[i] & 0xffff0000u);
-                            }
+                        for (int g = 0; g < 8; ++g)
+                            *reinterpret_cast<uint4*>(box + lane * 128 + ((g ^ (lane & 7)) << 4)) =
+                                make_uint4(v[32 * h + 4 * g], v[32 * h + 4 * g + 1], v[32 * h + 4 * g + 2], v[32 * h + 4 * g + 3]);
+                        fence_async_smem();
+                        __syncwarp();
+                        if (lane == 0) {
+                            if (n + 32 * h < p.N) tma_reduce_add_3d(&map_c, box, n + 32 * h, 0, m0);
+                            bulk_commit_group();
                         }
-                        if (p.gelu) {
-                            if (p.store_pre) {
-#pragma unroll
-                                for (int i = 0; i < 4; ++i) pre[4 * g8 + i] = pack_bf16(f[2 * i], f[2 * i + 1]);
-                            }
-#pragma unroll
-                            for (int i = 0; i < 8; ++i) f[i] = gelu_erf(f[i]);   // of the fp32 value, in both modes
-                        }
-                        if (p.aux != nullptr) {
-                            const uint32_t xw[4] = {xcur[g8].x, xcur[g8].y, xcur[g8].z, xcur[g8].w};
-#pragma unroll
-                            for (int i = 0; i < 4; ++i) {
-                                f[2 * i] *= gelu_erf_grad(__uint_as_float(xw[i] << 16));
-                                f[2 * i + 1] *= gelu_erf_grad(__uint_as_float(xw[i] & 0xffff0000u));
-                            }
-                        }
-                        if (p.residual != nullptr) {
-                            const uint32_t rw[4] = {rcur[g8].x, rcur[g8].y, rcur[g8].z, rcur[g8].w};
-#pragma unroll
-                            for (int i = 0; i < 4; ++i) {
-                                f[2 * i] += __uint_as_float(rw[i] << 16);
-                                f[2 * i + 1] += __uint_as_float(rw[i] & 0xffff0000u);
-                            }
-                        }
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) out[4 * g8 + i] = pack_bf16(f[2 * i], f[2 * i + 1]);
-                    }
-                }
-                if (kBMode == 2) {   // fp32 partial tile: one [128 rows][32 fp32] box (128-byte swizzle), added to the output
-                    if (wt == 0) bulk_wait_group_read<0>();
-                    named_barrier_sync(1 + wg, 128);
-                    if (ok) {
-#pragma unroll
-                        for (int ch = 0; ch < 8; ++ch)
-                            *reinterpret_cast<uint4*>(boxes + r * 128 + ((ch ^ (r & 7)) << 4)) =
-                                make_uint4(v[4 * ch], v[4 * ch + 1], v[4 * ch + 2], v[4 * ch + 3]);
-                    }
-                    fence_async_smem();
-                    named_barrier_sync(1 + wg, 128);
-                    if (ok && wt == 0) {
-                        tma_reduce_add_3d(&map_c, boxes, n_base + c0, 0, m0);
-                        bulk_commit_group();
                     }
                     continue;
                 }
-                // one [128 rows][32 bf16] box per output: the result, and before it the pre-activation if asked for
-                auto emit = [&](const CUtensorMap* map, const uint32_t (&w)[16]) {
-                    uint8_t* box = boxes + (box_it & 1) * kGemmOutBox;
-                    if (wt == 0) bulk_wait_group_read<1>();   // the store issued two boxes ago has read this box
-                    named_barrier_sync(1 + wg, 128);
-                    if (ok) {
+                if (ksplit > 1) {   // the other pairs' partials of this chunk
+                    for (int s = 0; s < ksplit - 1; ++s) {
+                        const uint4* part = reinterpret_cast<const uint4*>(smem + (s * own + i) * kGemmPartChunk) + quarter * 32 + lane;
 #pragma unroll
-                        for (int g8 = 0; g8 < 4; ++g8)
-                            *reinterpret_cast<uint4*>(box + r * 64 + ((g8 ^ ((r >> 1) & 3)) << 4)) =
-                                make_uint4(w[4 * g8], w[4 * g8 + 1], w[4 * g8 + 2], w[4 * g8 + 3]);
+                        for (int g = 0; g < 16; ++g) {
+                            const uint4 q = part[g * 128];
+                            v[4 * g] = __float_as_uint(__uint_as_float(v[4 * g]) + __uint_as_float(q.x));
+                            v[4 * g + 1] = __float_as_uint(__uint_as_float(v[4 * g + 1]) + __uint_as_float(q.y));
+                            v[4 * g + 2] = __float_as_uint(__uint_as_float(v[4 * g + 2]) + __uint_as_float(q.z));
+                            v[4 * g + 3] = __float_as_uint(__uint_as_float(v[4 * g + 3]) + __uint_as_float(q.w));
+                        }
                     }
-                    fence_async_smem();
-                    named_barrier_sync(1 + wg, 128);
-                    if (ok && wt == 0) {
-                        tma_store_3d(map, box, n_base + c0, 0, m0);
-                        bulk_commit_group();
-                    }
-                };
-                if (p.gelu && p.store_pre) {
-                    emit(&map_u, pre);
-                    ++box_it;
                 }
-                emit(&map_c, out);
+                uint8_t* box = boxes + (bc & 1) * kGemmBox;          // result (and side operand, in place)
+                uint8_t* pre_box = boxes + ((bc & 1) ^ 1) * kGemmBox; // pre-activation, when it is stored too
+                if (p.side) {
+                    ok = mbar_wait(&bars.side_full[ew][bc & 1], (bc >> 1) & 1, &abort_flag);
+                    if (!ok) continue;
+                } else {
+                    if (lane == 0) {   // the box's (both boxes') last store has been read
+                        if (kEpi == kEpiGelu && p.store_pre) bulk_wait_group_read<0>();
+                        else bulk_wait_group_read<1>();
+                    }
+                    __syncwarp();
+                }
+                const __nv_bfloat16* rrow = nullptr;
+                if (p.direct_res != nullptr && m0 + lane < p.M) rrow = p.direct_res + int64_t(m0 + lane) * p.ldr + n;
+#pragma unroll
+                for (int g = 0; g < 8; ++g) {   // 8 columns = 16 bytes of output
+                    const bool col_ok = n + 8 * g < p.N;   // N is a multiple of 8; the store clips what lies outside
+                    uint4* slot = reinterpret_cast<uint4*>(box + lane * 128 + ((g ^ (lane & 7)) << 4));
+                    float2 f[4];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) f[j] = make_float2(__uint_as_float(v[8 * g + 2 * j]), __uint_as_float(v[8 * g + 2 * j + 1]));
+                    if (kMode == 0 && p.bias != nullptr && col_ok) {
+                        const uint4 b4 = __ldg(reinterpret_cast<const uint4*>(p.bias + n + 8 * g));
+                        const uint32_t bw[4] = {b4.x, b4.y, b4.z, b4.w};
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) f[j] = add2(f[j], bf16x2_to_f2(bw[j]));
+                    }
+                    if (kEpi == kEpiGelu) {
+                        if (p.store_pre)
+                            *reinterpret_cast<uint4*>(pre_box + lane * 128 + ((g ^ (lane & 7)) << 4)) =
+                                make_uint4(pack_bf16(f[0].x, f[0].y), pack_bf16(f[1].x, f[1].y), pack_bf16(f[2].x, f[2].y), pack_bf16(f[3].x, f[3].y));
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) f[j] = gelu_erf2(f[j]);   // of the fp32 value, whether or not u is stored
+                    }
+                    if (p.side) {
+                        const uint4 s4 = *slot;
+                        const uint32_t sw[4] = {s4.x, s4.y, s4.z, s4.w};
+#pragma unroll
+                        for (int j = 0; j < 4; ++j)
+                            f[j] = kEpi == kEpiGeluGrad ? mul2(f[j], gelu_erf_grad2(bf16x2_to_f2(sw[j]))) : add2(f[j], bf16x2_to_f2(sw[j]));
+                    }
+                    if (kEpi == kEpiGeluGrad && rrow != nullptr && col_ok) {
+                        const uint4 r4 = __ldg(reinterpret_cast<const uint4*>(rrow + 8 * g));
+                        const uint32_t rw[4] = {r4.x, r4.y, r4.z, r4.w};
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) f[j] = add2(f[j], bf16x2_to_f2(rw[j]));
+                    }
+                    *slot = make_uint4(pack_bf16(f[0].x, f[0].y), pack_bf16(f[1].x, f[1].y), pack_bf16(f[2].x, f[2].y), pack_bf16(f[3].x, f[3].y));
+                }
+                fence_async_smem();
+                __syncwarp();
+                if (lane == 0) {
+                    if (kEpi == kEpiGelu && p.store_pre) tma_store_3d(&map_u, pre_box, n, 0, m0);
+                    tma_store_3d(&map_c, box, n, 0, m0);
+                    bulk_commit_group();
+                }
+                ++bc;
             }
+            if (!released) release();
         }
-        if (wt == 0) bulk_wait_group<0>();   // shared memory must outlive the copy engine's reads
+        if (lane == 0) bulk_wait_group_read<0>();   // shared memory must outlive the copy engine's reads
+        __syncwarp();
+    }
+    if (kMode != 2 && ksplit > 1 && warp < 4) {   // the two meetings of the split contraction
+        __syncwarp();
+        cluster_sync_all();
+        cluster_sync_all();
     }
 
+    __syncwarp();
     tc_fence_before();
-    __syncthreads();
-    if (warp == 2) tmem_dealloc(tmem, 512);
+    cluster_sync_all();   // neither CTA frees TMEM or leaves while the pair's MMAs or the cluster's stores may still touch it
+    if (warp == 2) tmem_dealloc_pair(tmem, 512);
     if (tid == 0 && abort_flag) report_status(p.status_buf, MPIPE_ERR_TIMEOUT, int32_t(blockIdx.x));
 }
 
-}  // namespace mpipe
-
-namespace mpipe {
-
-// Shared host side of the two entry points.  n_out / n_contract are the output columns and the contraction length.
-// `pre` (optional, forward with GELU only): bf16 [M, ldp] that receives the pre-activation a W^T + bias as well.
-static int32_t launch_linear(int b_mode, const void* a, const void* w, const void* bias, const void* residual, const void* aux,
-                             void* c, int32_t M, int32_t n_out, int32_t n_contract, int64_t lda, int64_t ldw, int64_t ldr,
-                             int64_t ldx, int64_t ldc, int32_t gelu, int32_t* status_buf, void* stream,
-                             void* pre = nullptr, int64_t ldp = 0) {
-    if (M < 0 || n_out <= 0 || n_contract <= 0) return MPIPE_ERR_INVALID_ARG;
-    if (M == 0) return MPIPE_OK;
-    if (a == nullptr || w == nullptr || c == nullptr) return MPIPE_ERR_INVALID_ARG;
-    if ((n_out % 8) != 0 || (n_contract % 8) != 0) return MPIPE_ERR_UNSUPPORTED;
-    const int64_t w_cols = b_mode == 0 ? n_contract : n_out;
-    if (lda < n_contract || ldw < w_cols || ldc < n_out || (residual != nullptr && ldr < n_out) || (aux != nullptr && ldx < n_out))
-        return MPIPE_ERR_INVALID_ARG;
-    if ((lda % 8) != 0 || (ldw % 8) != 0 || (ldc % 8) != 0 || (residual != nullptr && (ldr % 8) != 0) || (aux != nullptr && (ldx % 8) != 0))
-        return MPIPE_ERR_UNSUPPORTED;
-    if (!aligned16(a) || !aligned16(w) || !aligned16(c) || !aligned16(bias) || !aligned16(residual) || !aligned16(aux))
-        return MPIPE_ERR_UNSUPPORTED;
-    if (pre != nullptr && (b_mode != 0 || !gelu || ldp < n_out || (ldp % 8) != 0 || !aligned16(pre))) return MPIPE_ERR_INVALID_ARG;
-    cudaStream_t st = static_cast<cudaStream_t>(stream);
-    CUtensorMap map_a, map_w, map_c, map_u;
-    bool ok = make_tensor_map_thd(&map_a, a, M, 1, n_contract, lda, lda, kGemmBK, kGemmBM, 128) &&
-              make_tensor_map_thd(&map_c, c, M, 1, n_out, ldc, ldc, 32, kGemmBM, 64);
-    map_u = map_c;
-    if (pre != nullptr) ok = ok && make_tensor_map_thd(&map_u, pre, M, 1, n_out, ldp, ldp, 32, kGemmBM, 64);
-    if (b_mode == 0)   // W[n_out rows, n_contract columns]: boxes of 256 rows x 64 k
-        ok = ok && make_tensor_map_thd(&map_w, w, n_out, 1, n_contract, ldw, ldw, kGemmBK, kGemmBN, 128);
-    else               // W[n_contract rows, n_out columns]: boxes of 64 contraction rows x 64 output columns
-        ok = ok && make_tensor_map_thd(&map_w, w, n_contract, 1, n_out, ldw, ldw, 64, kGemmBK, 128);
-    if (!ok) return MPIPE_ERR_CUDA;
-    GemmParams p;
-    p.M = M; p.N = n_out; p.K = n_contract;
-    p.tiles_m = cdiv(M, kGemmBM);
-    p.tiles_n = cdiv(n_out, kGemmBN);
-    p.bias = static_cast<const __nv_bfloat16*>(bias);
-    p.residual = static_cast<const __nv_bfloat16*>(residual);
-    p.aux = static_cast<const __nv_bfloat16*>(aux);
-    p.C = static_cast<__nv_bfloat16*>(c);
-    p.ldr = ldr; p.ldx = ldx; p.ldc = ldc;
-    p.gelu = gelu;
-    p.store_pre = pre != nullptr ? 1 : 0;
-    p.splits = 1;
-    p.status_buf = status_buf;
-    const long long tiles = (long long)p.tiles_m * p.tiles_n;
-    const int grid = int(tiles < sm_count() ? tiles : sm_count());
-    profile_start(kProfileLinear, st);
-    if (b_mode == 0) {
-        if (!ensure_dynamic_smem<linear_kernel<0>>(kGemmSmem)) return MPIPE_ERR_CUDA;
-        linear_kernel<0><<<grid, kGemmThreads, kGemmSmem, st>>>(map_a, map_w, map_c, map_u, p);
-    } else {
-        if (!ensure_dynamic_smem<linear_kernel<1>>(kGemmSmem)) return MPIPE_ERR_CUDA;
-        linear_kernel<1><<<grid, kGemmThreads, kGemmSmem, st>>>(map_a, map_w, map_c, map_u, p);
+// ---- choice of tile width and contraction split, in SM clocks; the constants are fitted to graph-replayed sweeps of every width
+// and split over M 86..12000 and hidden 320..1280 (the pick is within 5 % of the best measured in all but a few of them).
+struct GemmShape {
+    int bn, splits;
+};
+// One stage (64 of the contraction) of a 256 x bn tile with all SMs at work: 2 bn clocks of tensor pipe at bn 256 and 192 plus
+// what the operand traffic of the other SMs adds, the issuing thread's ~450 below.
+static double gemm_stage_clk(int bn) { return bn == 256 ? 640.0 : bn == 192 ? 510.0 : 470.0; }
+// Launch, first loads, and the epilogue of the last tile (two 64-column chunks per warp above bn 128; GELU ~3000 a chunk).
+static double gemm_fixed_clk(int bn, bool gelu) {
+    const int chunks = bn > 128 ? 2 : 1;
+    return 8500.0 + (bn == 64 ? 2800.0 : 3600.0 * chunks) + (gelu ? 3000.0 * chunks : 0.0);
+}
+static int gemm_stages(int bn) {
+    const int n = kGemmRing / (kGemmABytes + 64 * bn);
+    return n < kGemmMaxStages ? n : kGemmMaxStages;
+}
+// Clusters of `ctas` CTAs that fit on the current device at once (the GPCs' SM counts limit clusters of more than two).
+template <auto kernel>
+static int max_clusters(int ctas) {
+    static int cached[64][2 * kGemmMaxSplits + 1] = {};
+    int dev = -1;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+    if (cached[dev][ctas] == 0) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(unsigned(ctas));
+        cfg.blockDim = dim3(kGemmThreads);
+        cfg.dynamicSmemBytes = kGemmSmem;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = unsigned(ctas);
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        int n = 0;
+        if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
+            (void)cudaGetLastError();
+            n = 0;
+        }
+        cached[dev][ctas] = n > 0 ? n : -1;
     }
+    return cached[dev][ctas] > 0 ? cached[dev][ctas] : 0;
+}
+template <auto kernel>
+static GemmShape choose_shape(int b_mode, bool gelu, int M, int N, int K) {
+    const int nk = cdiv(K, kGemmBK), tiles_m = cdiv(M, 2 * kGemmBM);
+    const int pairs = max_clusters<kernel>(2) > 0 ? max_clusters<kernel>(2) : 1;
+    GemmShape best = {kGemmMaxBN, 1};
+    double best_clk = 1e30;
+    for (int bn = kGemmMaxBN; bn >= 64; bn -= 64) {
+        if (b_mode == 1 && (bn % 128) != 0) continue;      // MN-major B: each CTA holds whole 64-column atoms
+        const long long tiles = (long long)tiles_m * cdiv(N, bn);
+        for (int sp = 1; sp <= kGemmMaxSplits; ++sp) {
+            if (sp > 1 && ((bn / 64) % sp != 0 || nk < 4 * sp || tiles > max_clusters<kernel>(2 * sp))) continue;
+            const long long waves = sp > 1 ? 1 : (tiles + pairs - 1) / pairs;
+            const double clk = waves * cdiv(nk, sp) * gemm_stage_clk(bn) + gemm_fixed_clk(bn, gelu) + (sp > 1 ? 1800.0 : 0.0);
+            if (clk < best_clk) {
+                best_clk = clk;
+                best = {bn, sp};
+            }
+        }
+    }
+    return best;
+}
+
+template <auto kernel>
+static int32_t launch_gemm(int cluster_ctas, int grid, const CUtensorMap& map_a, const CUtensorMap& map_w, const CUtensorMap& map_c,
+                           const CUtensorMap& map_s, const CUtensorMap& map_u, const GemmParams& p, cudaStream_t st) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(unsigned(grid));
+    cfg.blockDim = dim3(kGemmThreads);
+    cfg.dynamicSmemBytes = kGemmSmem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = unsigned(cluster_ctas);
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    profile_start(kProfileLinear, st);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, map_a, map_w, map_c, map_s, map_u, p);
     profile_stop(kProfileLinear, st);
-    return cudaGetLastError() == cudaSuccess ? MPIPE_OK : MPIPE_ERR_CUDA;
+    return e == cudaSuccess && cudaGetLastError() == cudaSuccess ? MPIPE_OK : MPIPE_ERR_CUDA;
+}
+
+struct LinearCall {   // one forward projection or input gradient
+    const void *a, *w, *bias, *residual, *aux;
+    void *c, *pre;
+    int32_t M, n_out, n_contract;
+    int64_t lda, ldw, ldr, ldx, ldc, ldp;
+    int32_t gelu;
+    int32_t* status_buf;
+};
+
+template <int kMode, int kEpi>
+static int32_t launch_linear_as(const LinearCall& x, cudaStream_t st) {
+    if (!ensure_dynamic_smem<linear_kernel<kMode, kEpi>>(kGemmSmem)) return MPIPE_ERR_CUDA;
+    const GemmShape shape = choose_shape<linear_kernel<kMode, kEpi>>(kMode, kEpi != kEpiPlain, x.M, x.n_out, x.n_contract);
+    GemmParams p = {};
+    p.M = x.M; p.N = x.n_out; p.K = x.n_contract;
+    p.bn = shape.bn;
+    p.stages = gemm_stages(p.bn);
+    p.splits = shape.splits;
+    p.tiles_m = cdiv(x.M, 2 * kGemmBM);
+    p.tiles_n = cdiv(x.n_out, p.bn);
+    p.bias = static_cast<const __nv_bfloat16*>(x.bias);
+    // the boxes bring one side operand; the gradient of GELU takes them for u and reads a residual directly
+    const void* side = kEpi == kEpiGeluGrad ? x.aux : x.residual;
+    const int64_t ld_side = kEpi == kEpiGeluGrad ? x.ldx : x.ldr;
+    if (kEpi == kEpiGeluGrad) p.direct_res = static_cast<const __nv_bfloat16*>(x.residual);
+    p.ldr = x.ldr;
+    p.side = side != nullptr ? 1 : 0;
+    p.store_pre = x.pre != nullptr ? 1 : 0;
+    p.status_buf = x.status_buf;
+    CUtensorMap map_a, map_w, map_c;
+    bool ok = make_tensor_map_thd(&map_a, x.a, x.M, 1, x.n_contract, x.lda, x.lda, kGemmBK, kGemmBM, 128) &&
+              make_tensor_map_thd(&map_c, x.c, x.M, 1, x.n_out, x.ldc, x.ldc, 64, 32, 128);
+    CUtensorMap map_s = map_c, map_u = map_c;
+    if (side != nullptr) ok = ok && make_tensor_map_thd(&map_s, side, x.M, 1, x.n_out, ld_side, ld_side, 64, 32, 128);
+    if (x.pre != nullptr) ok = ok && make_tensor_map_thd(&map_u, x.pre, x.M, 1, x.n_out, x.ldp, x.ldp, 64, 32, 128);
+    if (kMode == 0)   // W[n_out rows, n_contract columns]: boxes of bn / 2 rows x 64 k
+        ok = ok && make_tensor_map_thd(&map_w, x.w, x.n_out, 1, x.n_contract, x.ldw, x.ldw, kGemmBK, p.bn / 2, 128);
+    else              // W[n_contract rows, n_out columns]: boxes of 64 contraction rows x 64 output columns
+        ok = ok && make_tensor_map_thd(&map_w, x.w, x.n_contract, 1, x.n_out, x.ldw, x.ldw, 64, kGemmBK, 128);
+    if (!ok) return MPIPE_ERR_CUDA;
+    const long long tiles = (long long)p.tiles_m * p.tiles_n;
+    const int cap = max_clusters<linear_kernel<kMode, kEpi>>(2 * p.splits);
+    if (cap <= 0) return MPIPE_ERR_CUDA;
+    if (tiles > 0x7fffffffLL / (2 * kGemmMaxSplits)) return MPIPE_ERR_UNSUPPORTED;
+    // a split contraction takes one cluster per tile (its CTAs meet once at a cluster barrier), everything else is persistent
+    const int clusters = int(p.splits > 1 || tiles < cap ? tiles : cap);
+    return launch_gemm<linear_kernel<kMode, kEpi>>(2 * p.splits, clusters * 2 * p.splits, map_a, map_w, map_c, map_s, map_u, p, st);
+}
+
+// Shared host side of the two entry points: checks, then the instantiation the epilogue needs.
+static int32_t launch_linear(int b_mode, const LinearCall& x, void* stream) {
+    if (x.M < 0 || x.n_out <= 0 || x.n_contract <= 0) return MPIPE_ERR_INVALID_ARG;
+    if (x.M == 0) return MPIPE_OK;
+    if (x.a == nullptr || x.w == nullptr || x.c == nullptr) return MPIPE_ERR_INVALID_ARG;
+    if ((x.n_out % 8) != 0 || (x.n_contract % 8) != 0) return MPIPE_ERR_UNSUPPORTED;
+    const int64_t w_cols = b_mode == 0 ? x.n_contract : x.n_out;
+    if (x.lda < x.n_contract || x.ldw < w_cols || x.ldc < x.n_out || (x.residual != nullptr && x.ldr < x.n_out) ||
+        (x.aux != nullptr && x.ldx < x.n_out))
+        return MPIPE_ERR_INVALID_ARG;
+    if ((x.lda % 8) != 0 || (x.ldw % 8) != 0 || (x.ldc % 8) != 0 || (x.residual != nullptr && (x.ldr % 8) != 0) ||
+        (x.aux != nullptr && (x.ldx % 8) != 0))
+        return MPIPE_ERR_UNSUPPORTED;
+    if (!aligned16(x.a) || !aligned16(x.w) || !aligned16(x.c) || !aligned16(x.bias) || !aligned16(x.residual) || !aligned16(x.aux))
+        return MPIPE_ERR_UNSUPPORTED;
+    // the two outputs of a kept pre-activation take both staging boxes: no residual beside it
+    if (x.pre != nullptr && (b_mode != 0 || !x.gelu || x.residual != nullptr || x.ldp < x.n_out || (x.ldp % 8) != 0 || !aligned16(x.pre)))
+        return MPIPE_ERR_INVALID_ARG;
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    if (b_mode == 0) return x.gelu ? launch_linear_as<0, kEpiGelu>(x, st) : launch_linear_as<0, kEpiPlain>(x, st);
+    return x.aux != nullptr ? launch_linear_as<1, kEpiGeluGrad>(x, st) : launch_linear_as<1, kEpiPlain>(x, st);
 }
 
 // dW[n_rows, n_cols] (fp32) += dY[tokens, n_rows]^T X[tokens, n_cols]
@@ -398,35 +561,42 @@ static int32_t launch_wgrad(const void* dy, const void* x, float* dw, int32_t to
     CUtensorMap map_a, map_w, map_c;
     if (!make_tensor_map_thd(&map_a, dy, tokens, 1, n_rows, lddy, lddy, 64, kGemmBK, 128) ||
         !make_tensor_map_thd(&map_w, x, tokens, 1, n_cols, ldx, ldx, 64, kGemmBK, 128) ||
-        !make_tensor_map_thd(&map_c, dw, n_rows, 1, n_cols, lddw, lddw, 32, kGemmBM, 128, 4))
+        !make_tensor_map_thd(&map_c, dw, n_rows, 1, n_cols, lddw, lddw, 32, 32, 128, 4))
         return MPIPE_ERR_CUDA;
-    GemmParams p;
-    p.M = n_rows; p.N = n_cols; p.K = tokens;
-    p.tiles_m = cdiv(n_rows, kGemmBM);
-    p.tiles_n = cdiv(n_cols, kGemmBN);
-    p.bias = nullptr; p.residual = nullptr; p.aux = nullptr; p.C = nullptr;
-    p.ldr = p.ldx = p.ldc = 0;
-    p.gelu = 0;
-    p.store_pre = 0;
-    p.status_buf = status_buf;
-    // split the token range so that (tiles x splits) fills whole waves of the SMs; more splits mean more reduction traffic
-    const int sms = sm_count(), tiles = p.tiles_m * p.tiles_n, nk = cdiv(tokens, kGemmBK);
-    int best = 1;
-    double best_score = -1.0;
-    for (int sp = 1; sp <= 32 && sp <= nk; ++sp) {
-        const long long items = (long long)tiles * sp;
-        const double eff = double(items) / double(((items + sms - 1) / sms) * sms);
-        const double score = eff - 0.004 * sp;
-        if (score > best_score) { best_score = score; best = sp; }
+    if (!ensure_dynamic_smem<linear_kernel<2, kEpiPlain>>(kGemmSmem)) return MPIPE_ERR_CUDA;
+    const int pairs = max_clusters<linear_kernel<2, kEpiPlain>>(2);
+    if (pairs <= 0) return MPIPE_ERR_CUDA;
+    // Tile width and split of the token range, in SM clocks (fitted like choose_shape's constants).  A pair's fp32 tile leaves at
+    // about 12 bytes per clock and SM (the L2's rate of fp32 reductions with every SM adding) beside the next item's main loop.
+    // A long token range runs into the power limit, where the sum of the work counts and not its spread over the pairs: no
+    // estimate goes below the work at 68 % of the tensor peak, and among equals the fewest splits (least reduction traffic) win
+    // (1024 x 4096 over 50 439 tokens: 322 us unsplit on 64 of the 74 pairs, 355 to 415 us for any split).
+    GemmParams p = {};
+    const int nk = cdiv(tokens, kGemmBK);
+    double best_clk = 1e30;
+    for (int bn = kGemmMaxBN; bn >= 128; bn -= 128) {
+        const long long tiles = (long long)cdiv(n_rows, 2 * kGemmBM) * cdiv(n_cols, bn);
+        const double red = bn == 256 ? 11000.0 : 6500.0, stage = bn == 256 ? 600.0 : 450.0, fixed = bn == 256 ? 16200.0 : 12500.0;
+        const double power = double(tiles) * nk * 2 * bn / (0.68 * pairs);
+        for (int sp = 1; sp <= 64 && sp <= nk; ++sp) {
+            const long long waves = (tiles * sp + pairs - 1) / pairs;
+            const double loop = cdiv(nk, sp) * stage, run = waves * ((loop > red ? loop : red) + 1000.0);
+            const double clk = (run > power ? run : power) + fixed;
+            if (clk < best_clk * 0.999) {
+                best_clk = clk;
+                p.bn = bn;
+                p.splits = sp;
+            }
+        }
     }
-    p.splits = best;
-    const long long items = (long long)tiles * p.splits;
-    const int grid = int(items < sms ? items : sms);
-    if (!ensure_dynamic_smem<linear_kernel<2>>(kGemmSmem)) return MPIPE_ERR_CUDA;
-    profile_start(kProfileLinear, st);
-    linear_kernel<2><<<grid, kGemmThreads, kGemmSmem, st>>>(map_a, map_w, map_c, map_c, p);
-    profile_stop(kProfileLinear, st);
-    return cudaGetLastError() == cudaSuccess ? MPIPE_OK : MPIPE_ERR_CUDA;
+    p.stages = gemm_stages(p.bn);
+    p.M = n_rows; p.N = n_cols; p.K = tokens;
+    p.tiles_m = cdiv(n_rows, 2 * kGemmBM);
+    p.tiles_n = cdiv(n_cols, p.bn);
+    p.status_buf = status_buf;
+    const long long items = (long long)p.tiles_m * p.tiles_n * p.splits;
+    const int clusters = int(items < pairs ? items : pairs);
+    return launch_gemm<linear_kernel<2, kEpiPlain>>(2, 2 * clusters, map_a, map_w, map_c, map_c, map_c, p, st);
 }
 
 // fc1 of a TRAINED layer forward: act = GELU(a W^T + bias) and pre = a W^T + bias from ONE accumulator, so that the
@@ -434,7 +604,8 @@ static int32_t launch_wgrad(const void* dy, const void* x, float* dw, int32_t to
 int32_t linear_fwd_gelu_keep_preact(const void* a, const void* w, const void* bias, void* act, void* pre, int32_t M, int32_t N,
                                     int32_t K, int64_t lda, int64_t ldw, int64_t ldact, int64_t ldpre, int32_t* status_buf,
                                     void* stream) {
-    return launch_linear(0, a, w, bias, nullptr, nullptr, act, M, N, K, lda, ldw, 0, 0, ldact, 1, status_buf, stream, pre, ldpre);
+    const LinearCall x = {a, w, bias, nullptr, nullptr, act, pre, M, N, K, lda, ldw, 0, 0, ldact, ldpre, 1, status_buf};
+    return launch_linear(0, x, stream);
 }
 
 }  // namespace mpipe
@@ -450,15 +621,16 @@ int32_t mpipe_linear_fwd(const void* a, const void* w, const void* bias, const v
                          int32_t N, int32_t K, int64_t lda, int64_t ldw, int64_t ldr, int64_t ldc, int32_t flags,
                          int32_t* status_buf, void* stream) {
     if ((flags & ~(MPIPE_LINEAR_GELU)) != 0) return MPIPE_ERR_INVALID_ARG;
-    return mpipe::launch_linear(0, a, w, bias, residual, nullptr, c, M, N, K, lda, ldw, ldr, 0, ldc,
-                                (flags & MPIPE_LINEAR_GELU) ? 1 : 0, status_buf, stream);
+    const mpipe::LinearCall x = {a, w, bias, residual, nullptr, c, nullptr, M, N, K, lda, ldw, ldr, 0, ldc, 0,
+                                 (flags & MPIPE_LINEAR_GELU) ? 1 : 0, status_buf};
+    return mpipe::launch_linear(0, x, stream);
 }
 
 int32_t mpipe_linear_dgrad(const void* dy, const void* w, const void* gelu_input, const void* residual, void* dx, int32_t M,
                            int32_t N, int32_t K, int64_t lddy, int64_t ldw, int64_t ldu, int64_t ldr, int64_t lddx,
                            int32_t* status_buf, void* stream) {
-    return mpipe::launch_linear(1, dy, w, nullptr, residual, gelu_input, dx, M, K, N, lddy, ldw, ldr, ldu, lddx, 0, status_buf,
-                                stream);
+    const mpipe::LinearCall x = {dy, w, nullptr, residual, gelu_input, dx, nullptr, M, K, N, lddy, ldw, ldr, ldu, lddx, 0, 0, status_buf};
+    return mpipe::launch_linear(1, x, stream);
 }
 
 }  // extern "C"
