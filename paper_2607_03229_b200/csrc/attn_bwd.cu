@@ -179,7 +179,10 @@ attn_bwd_kernel(const __grid_constant__ BwdMaps maps, const BwdParams p) {
     // The plan comes from device memory: it is checked as a whole before any role starts (see plan_ok_cta); a
     // rejected plan leaves every role with nothing to do.
     __shared__ int plan_flag;
+    // (the kernel before this one is always the prepass, which does not write the plan and has waited for what did)
     const int n_units = plan_ok_cta(p.items, p.n_items, kBT, p.total_tokens, p.status_buf, &plan_flag) ? p.n_items * p.n_heads : 0;
+    pdl_wait();
+    pdl_launch();
     // Units are sorted by decreasing cost; CTAs walk them in boustrophedon order (0..G-1, then G-1..0, ...) so
     // that the CTA that got the most expensive unit of one round gets the cheapest of the next.
     auto unit_of = [&](int round) {
@@ -664,6 +667,8 @@ bwd_prepass_kernel(const __nv_bfloat16* __restrict__ dout, const __nv_bfloat16* 
                    float* __restrict__ dq_acc) {
     constexpr int kLanes = (D == 64) ? 8 : 16;   // lanes per row (D = 80 uses 10 of 16)
     constexpr int kRowsPerBlock = 256 / kLanes;
+    pdl_wait();
+    pdl_launch();
     const int64_t n_rows = int64_t(total_tokens) * n_heads;
     const int sub = threadIdx.x % kLanes;
     for (int64_t row0 = int64_t(blockIdx.x) * kRowsPerBlock; row0 < n_rows; row0 += int64_t(gridDim.x) * kRowsPerBlock) {
@@ -699,6 +704,8 @@ bwd_prepass_kernel(const __nv_bfloat16* __restrict__ dout, const __nv_bfloat16* 
 __global__ void __launch_bounds__(256)
 bwd_dq_convert_kernel(const float* __restrict__ acc, __nv_bfloat16* __restrict__ dq, int64_t tok_stride_g,
                       int64_t head_stride_g, int32_t total_tokens, int32_t n_heads, int32_t head_dim, float scale) {
+    pdl_wait();
+    pdl_launch();
     const int chunks = head_dim / 8;
     const int64_t idx = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
     if (idx >= int64_t(total_tokens) * n_heads * chunks) return;
@@ -734,19 +741,20 @@ static int32_t launch_bwd(const void* dout, const void* q, const void* k, const 
     const int64_t rows = int64_t(total_tokens) * n_heads;
     const int64_t prepass_blocks = (rows + (D == 64 ? 32 : 16) - 1) / (D == 64 ? 32 : 16);
     const int64_t prepass_cap = int64_t(sm_count()) * 64;
-    bwd_prepass_kernel<D><<<unsigned(prepass_blocks < prepass_cap ? prepass_blocks : prepass_cap), 256, 0, stream>>>(
-        static_cast<const __nv_bfloat16*>(dout), static_cast<const __nv_bfloat16*>(o), ts_o, hs_o, total_tokens, n_heads,
-        delta, dq_acc);
+    cudaError_t e = launch_kernel(bwd_prepass_kernel<D>, unsigned(prepass_blocks < prepass_cap ? prepass_blocks : prepass_cap), 256, 0, stream, 1,
+                                  static_cast<const __nv_bfloat16*>(dout), static_cast<const __nv_bfloat16*>(o), ts_o, hs_o, total_tokens,
+                                  n_heads, delta, dq_acc);
+    if (e != cudaSuccess) return MPIPE_ERR_CUDA;
     const int n_units = prm.n_items * prm.n_heads;
     const int grid = n_units < sm_count() ? n_units : sm_count();
     profile_start(kProfileBwdMain, stream);
-    attn_bwd_kernel<D><<<grid, kBwdThreads, Cfg::kSmemAlloc, stream>>>(m, prm);
+    e = launch_kernel(attn_bwd_kernel<D>, unsigned(grid), kBwdThreads, Cfg::kSmemAlloc, stream, 1, m, prm);
     profile_stop(kProfileBwdMain, stream);
+    if (e != cudaSuccess) return MPIPE_ERR_CUDA;
     const int64_t chunks = rows * (D / 8);
-    bwd_dq_convert_kernel<<<unsigned((chunks + 255) / 256), 256, 0, stream>>>(
-        dq_acc, static_cast<__nv_bfloat16*>(dq), prm.tok_stride_g, prm.head_stride_g, total_tokens, n_heads, D,
-        prm.scale);
-    return cudaGetLastError() == cudaSuccess ? MPIPE_OK : MPIPE_ERR_CUDA;
+    e = launch_kernel(bwd_dq_convert_kernel, unsigned((chunks + 255) / 256), 256, 0, stream, 1, static_cast<const float*>(dq_acc),
+                      static_cast<__nv_bfloat16*>(dq), prm.tok_stride_g, prm.head_stride_g, total_tokens, n_heads, D, prm.scale);
+    return e == cudaSuccess && cudaGetLastError() == cudaSuccess ? MPIPE_OK : MPIPE_ERR_CUDA;
 }
 
 static size_t round256(size_t x) { return (x + 255) & ~size_t(255); }

@@ -66,6 +66,7 @@ struct FwdParams {
     int64_t tok_stride_o, head_stride_o;
     int32_t total_tokens;
     float scale_log2;  // softmax_scale * log2(e)
+    int32_t settled;   // the items were complete before the previous kernel of the stream started
     int32_t* status_buf;
 };
 
@@ -126,9 +127,13 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
     const uint32_t tmem = tmem_base_slot;
     // TMEM columns: S_0 [0,128), S_1 [128,256), O_0 [256,256+D), O_1 [384,384+D); P_w overlays S_w.
     // The plan comes from device memory: it is checked as a whole before any role starts (see plan_ok_cta); a
-    // rejected plan leaves every role with nothing to do.
+    // rejected plan leaves every role with nothing to do.  Inside a layer (`settled`) the plan is older than the kernel
+    // before this one and is checked while that kernel still runs.
     __shared__ int plan_flag;
+    if (!p.settled) pdl_wait();
     const int n_units = plan_ok_cta(p.items, p.n_items, 2 * kTileM, p.total_tokens, p.status_buf, &plan_flag) ? p.n_items * p.n_heads : 0;
+    if (p.settled) pdl_wait();
+    pdl_launch();
     // Units are sorted by decreasing cost; CTAs walk them in boustrophedon order (0..G-1, then G-1..0, ...) so
     // that the CTA that got the most expensive unit of one round gets the cheapest of the next.
     auto unit_of = [&](int round) {
@@ -522,24 +527,17 @@ static int32_t launch_fwd(const void* q, const void* k, const void* v, int64_t t
     const int n_units = prm.n_items * prm.n_heads;
     const int grid = n_units < sm_count() ? n_units : sm_count();
     profile_start(kProfileFwd, stream);
-    attn_fwd_kernel<D><<<grid, kFwdThreads, Cfg::kSmemAlloc, stream>>>(mq, mk, mv, mqt, mkt, prm);
+    const cudaError_t e = launch_kernel(attn_fwd_kernel<D>, unsigned(grid), kFwdThreads, Cfg::kSmemAlloc, stream, 1, mq, mk, mv, mqt, mkt, prm);
     profile_stop(kProfileFwd, stream);
-    return cudaGetLastError() == cudaSuccess ? MPIPE_OK : MPIPE_ERR_CUDA;
+    return e == cudaSuccess && cudaGetLastError() == cudaSuccess ? MPIPE_OK : MPIPE_ERR_CUDA;
 }
 
-}  // namespace mpipe
-
-extern "C" {
-
-int32_t mpipe_fwd_tile_rows(void) { return 2 * mpipe::kTileM; }
-
-int32_t mpipe_varlen_attn_fwd(const void* q, const void* k, const void* v, void* o, float* lse,
+int32_t varlen_attn_fwd(const void* q, const void* k, const void* v, void* o, float* lse,
                               int64_t tok_stride_qkv, int64_t head_stride_qkv, int64_t tok_stride_o,
                               int64_t head_stride_o, const int32_t* cu_seqlens_dev, int32_t n_seg,
                               int32_t total_tokens, int32_t max_seqlen, const mpipe_work_item_t* fwd_items_dev,
                               int32_t n_fwd_items, int32_t n_heads, int32_t head_dim, float softmax_scale,
-                              int32_t mode, int32_t* status_buf, void* stream) {
-    using namespace mpipe;
+                              int32_t mode, int32_t* status_buf, void* stream, bool settled) {
     if (mode != MPIPE_ENC_FROZEN && mode != MPIPE_ENC_TRAINED) return MPIPE_ERR_INVALID_ARG;
     if (n_seg < 0 || total_tokens < 0 || max_seqlen < 0 || n_fwd_items < 0 || n_heads <= 0) return MPIPE_ERR_INVALID_ARG;
     if (head_dim != 64 && head_dim != 80) return MPIPE_ERR_UNSUPPORTED;
@@ -566,11 +564,29 @@ int32_t mpipe_varlen_attn_fwd(const void* q, const void* k, const void* v, void*
     prm.head_stride_o = head_stride_o;
     prm.total_tokens = total_tokens;
     prm.scale_log2 = softmax_scale * 1.4426950408889634f;
+    prm.settled = settled ? 1 : 0;
     prm.status_buf = status_buf;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if (head_dim == 64)
         return launch_fwd<64>(q, k, v, tok_stride_qkv, head_stride_qkv, total_tokens, n_heads, prm, st);
     return launch_fwd<80>(q, k, v, tok_stride_qkv, head_stride_qkv, total_tokens, n_heads, prm, st);
+}
+
+}  // namespace mpipe
+
+extern "C" {
+
+int32_t mpipe_fwd_tile_rows(void) { return 2 * mpipe::kTileM; }
+
+int32_t mpipe_varlen_attn_fwd(const void* q, const void* k, const void* v, void* o, float* lse,
+                              int64_t tok_stride_qkv, int64_t head_stride_qkv, int64_t tok_stride_o,
+                              int64_t head_stride_o, const int32_t* cu_seqlens_dev, int32_t n_seg,
+                              int32_t total_tokens, int32_t max_seqlen, const mpipe_work_item_t* fwd_items_dev,
+                              int32_t n_fwd_items, int32_t n_heads, int32_t head_dim, float softmax_scale,
+                              int32_t mode, int32_t* status_buf, void* stream) {
+    return mpipe::varlen_attn_fwd(q, k, v, o, lse, tok_stride_qkv, head_stride_qkv, tok_stride_o, head_stride_o, cu_seqlens_dev,
+                                  n_seg, total_tokens, max_seqlen, fwd_items_dev, n_fwd_items, n_heads, head_dim, softmax_scale,
+                                  mode, status_buf, stream, false);
 }
 
 }  // extern "C"

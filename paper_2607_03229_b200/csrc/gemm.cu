@@ -121,6 +121,8 @@ linear_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
     cluster_sync_all();                                       // the peer's barriers exist before anything arrives on them
     tc_fence_after();
     const uint32_t tmem = tmem_base_slot;
+    pdl_wait();
+    pdl_launch();
     const int nk = (p.K + kGemmBK - 1) / kGemmBK;
     const int n_out_tiles = p.tiles_m * p.tiles_n;
     const int n_items = n_out_tiles * (kMode == 2 ? p.splits : 1);
@@ -460,19 +462,9 @@ static GemmShape choose_shape(int b_mode, bool gelu, int M, int N, int K) {
 template <auto kernel>
 static int32_t launch_gemm(int cluster_ctas, int grid, const CUtensorMap& map_a, const CUtensorMap& map_w, const CUtensorMap& map_c,
                            const CUtensorMap& map_s, const CUtensorMap& map_u, const GemmParams& p, cudaStream_t st) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(unsigned(grid));
-    cfg.blockDim = dim3(kGemmThreads);
-    cfg.dynamicSmemBytes = kGemmSmem;
-    cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = unsigned(cluster_ctas);
-    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
     profile_start(kProfileLinear, st);
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, map_a, map_w, map_c, map_s, map_u, p);
+    const cudaError_t e = launch_kernel(kernel, unsigned(grid), kGemmThreads, kGemmSmem, st, unsigned(cluster_ctas), map_a, map_w, map_c,
+                                        map_s, map_u, p);
     profile_stop(kProfileLinear, st);
     return e == cudaSuccess && cudaGetLastError() == cudaSuccess ? MPIPE_OK : MPIPE_ERR_CUDA;
 }

@@ -10,7 +10,6 @@
 #include <algorithm>
 
 #include "common.h"
-#include "gelu.cuh"
 
 namespace mpipe {
 
@@ -22,6 +21,8 @@ template <int kChunks>
 __global__ void __launch_bounds__(256) layernorm_kernel(const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __restrict__ gamma,
                                                         const __nv_bfloat16* __restrict__ beta, __nv_bfloat16* __restrict__ y,
                                                         int32_t T, int32_t hidden, int64_t ldx, int64_t ldy, float eps) {
+    pdl_wait();
+    pdl_launch();
     const int row = blockIdx.x * 8 + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
     if (row >= T) return;
@@ -89,6 +90,8 @@ __global__ void __launch_bounds__(256) layernorm_kernel(const __nv_bfloat16* __r
 __global__ void __launch_bounds__(256) rope_kernel(__nv_bfloat16* __restrict__ qk, int64_t tok_stride, int64_t k_offset,
                                                    const float* __restrict__ cos_t, const float* __restrict__ sin_t, int32_t T,
                                                    int32_t n_heads, int32_t head_dim, float sin_sign) {
+    pdl_wait();
+    pdl_launch();
     const int half = head_dim >> 1, chunks = half >> 3;
     const int64_t idx = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
     const int64_t total = int64_t(T) * 2 * n_heads * chunks;
@@ -141,6 +144,8 @@ __global__ void __launch_bounds__(128) layernorm_bwd_kernel(const __nv_bfloat16*
     float* my_b = my_g + kCols;
     for (int i = threadIdx.x; i < 4 * 2 * kCols; i += 128) red[i] = 0.f;
     __syncthreads();
+    pdl_wait();
+    pdl_launch();
     const uint4* g4 = reinterpret_cast<const uint4*>(gamma);
     for (int row = blockIdx.x * 4 + warp; row < T; row += gridDim.x * 4) {
         const uint4* xr = reinterpret_cast<const uint4*>(x + int64_t(row) * ldx);
@@ -254,6 +259,8 @@ __global__ void __launch_bounds__(128) layernorm_bwd_kernel(const __nv_bfloat16*
 __global__ void __launch_bounds__(256) colsum_kernel(const __nv_bfloat16* __restrict__ a, float* __restrict__ out, int32_t T, int32_t N,
                                                      int64_t lda, int32_t n_groups, int32_t n_slices) {
     __shared__ float red[8][256];
+    pdl_wait();
+    pdl_launch();
     const int cl = threadIdx.x & 31, rl = threadIdx.x >> 5;
     const int group = blockIdx.x % n_groups, slice = blockIdx.x / n_groups;
     const int chunk = group * 32 + cl;
@@ -312,7 +319,8 @@ int32_t mpipe_layernorm_fwd(const void* x, const void* gamma, const void* beta, 
     auto* yp = static_cast<__nv_bfloat16*>(y);
     profile_start(kProfileLayerNorm, st);
     const int chunks = cdiv(hidden, 256);   // 16-byte chunks per lane: instantiate what the row length needs, not the maximum
-#define MPIPE_LN_LAUNCH(C) layernorm_kernel<C><<<grid, 256, 0, st>>>(xp, gp, bp, yp, n_tokens, hidden, ldx, ldy, eps)
+    cudaError_t e;
+#define MPIPE_LN_LAUNCH(C) e = launch_kernel(layernorm_kernel<C>, unsigned(grid), 256, 0, st, 1, xp, gp, bp, yp, n_tokens, hidden, ldx, ldy, eps)
     if (chunks <= 1) MPIPE_LN_LAUNCH(1);
     else if (chunks <= 2) MPIPE_LN_LAUNCH(2);
     else if (chunks <= 3) MPIPE_LN_LAUNCH(3);
@@ -322,7 +330,7 @@ int32_t mpipe_layernorm_fwd(const void* x, const void* gamma, const void* beta, 
     else MPIPE_LN_LAUNCH(kLnMaxChunks);
 #undef MPIPE_LN_LAUNCH
     profile_stop(kProfileLayerNorm, st);
-    return cudaGetLastError() == cudaSuccess ? MPIPE_OK : MPIPE_ERR_CUDA;
+    return e == cudaSuccess && cudaGetLastError() == cudaSuccess ? MPIPE_OK : MPIPE_ERR_CUDA;
 }
 
 int32_t mpipe_rope_apply(void* qk, int64_t tok_stride, int64_t k_offset, const float* cos_table, const float* sin_table,
@@ -336,9 +344,10 @@ int32_t mpipe_rope_apply(void* qk, int64_t tok_stride, int64_t k_offset, const f
     const int64_t total = int64_t(n_tokens) * 2 * n_heads * (head_dim / 16);
     const int64_t blocks = (total + 255) / 256;
     if (blocks > 0x7fffffffLL) return MPIPE_ERR_UNSUPPORTED;
-    rope_kernel<<<int(blocks), 256, 0, static_cast<cudaStream_t>(stream)>>>(static_cast<__nv_bfloat16*>(qk), tok_stride, k_offset, cos_table,
-                                                                           sin_table, n_tokens, n_heads, head_dim, 1.0f);
-    return cudaGetLastError() == cudaSuccess ? MPIPE_OK : MPIPE_ERR_CUDA;
+    const cudaError_t e = launch_kernel(rope_kernel, unsigned(blocks), 256, 0, static_cast<cudaStream_t>(stream), 1,
+                                        static_cast<__nv_bfloat16*>(qk), tok_stride, k_offset, cos_table, sin_table, n_tokens, n_heads,
+                                        head_dim, 1.0f);
+    return e == cudaSuccess && cudaGetLastError() == cudaSuccess ? MPIPE_OK : MPIPE_ERR_CUDA;
 }
 
 int32_t mpipe_rope_apply_bwd(void* dqk, int64_t tok_stride, int64_t k_offset, const float* cos_table, const float* sin_table,
@@ -352,9 +361,10 @@ int32_t mpipe_rope_apply_bwd(void* dqk, int64_t tok_stride, int64_t k_offset, co
     const int64_t total = int64_t(n_tokens) * 2 * n_heads * (head_dim / 16);
     const int64_t blocks = (total + 255) / 256;
     if (blocks > 0x7fffffffLL) return MPIPE_ERR_UNSUPPORTED;
-    rope_kernel<<<int(blocks), 256, 0, static_cast<cudaStream_t>(stream)>>>(static_cast<__nv_bfloat16*>(dqk), tok_stride, k_offset, cos_table,
-                                                                           sin_table, n_tokens, n_heads, head_dim, -1.0f);
-    return cudaGetLastError() == cudaSuccess ? MPIPE_OK : MPIPE_ERR_CUDA;
+    const cudaError_t e = launch_kernel(rope_kernel, unsigned(blocks), 256, 0, static_cast<cudaStream_t>(stream), 1,
+                                        static_cast<__nv_bfloat16*>(dqk), tok_stride, k_offset, cos_table, sin_table, n_tokens, n_heads,
+                                        head_dim, -1.0f);
+    return e == cudaSuccess && cudaGetLastError() == cudaSuccess ? MPIPE_OK : MPIPE_ERR_CUDA;
 }
 
 int32_t mpipe_layernorm_bwd(const void* x, const void* dy, const void* gamma, const void* dres, void* dx, float* dgamma, float* dbeta,
@@ -372,13 +382,14 @@ int32_t mpipe_layernorm_bwd(const void* x, const void* dy, const void* gamma, co
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const int grid = std::min(cdiv(n_tokens, 4), sm_count() * 6);
     const int chunks = cdiv(hidden, 256);
+    cudaError_t e;
 #define MPIPE_LNB_LAUNCH(C)                                                                                                    \
     do {                                                                                                                       \
         cudaFuncSetAttribute(layernorm_bwd_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, 4 * 2 * (C) * 256 * 4);      \
-        layernorm_bwd_kernel<C><<<grid, 128, 4 * 2 * (C) * 256 * 4, st>>>(                                                      \
-            static_cast<const __nv_bfloat16*>(x), static_cast<const __nv_bfloat16*>(dy), static_cast<const __nv_bfloat16*>(gamma), \
-            static_cast<const __nv_bfloat16*>(dres), static_cast<__nv_bfloat16*>(dx), dgamma, dbeta, n_tokens, hidden, ldx, lddy, \
-            ldr, lddx, eps);                                                                                                   \
+        e = launch_kernel(layernorm_bwd_kernel<C>, unsigned(grid), 128, 4 * 2 * (C) * 256 * 4, st, 1,                           \
+                          static_cast<const __nv_bfloat16*>(x), static_cast<const __nv_bfloat16*>(dy),                          \
+                          static_cast<const __nv_bfloat16*>(gamma), static_cast<const __nv_bfloat16*>(dres),                    \
+                          static_cast<__nv_bfloat16*>(dx), dgamma, dbeta, n_tokens, hidden, ldx, lddy, ldr, lddx, eps);         \
     } while (0)
     if (chunks <= 1) MPIPE_LNB_LAUNCH(1);
     else if (chunks <= 2) MPIPE_LNB_LAUNCH(2);
@@ -386,7 +397,7 @@ int32_t mpipe_layernorm_bwd(const void* x, const void* dy, const void* gamma, co
     else if (chunks <= 5) MPIPE_LNB_LAUNCH(5);
     else MPIPE_LNB_LAUNCH(kLnMaxChunks);
 #undef MPIPE_LNB_LAUNCH
-    return cudaGetLastError() == cudaSuccess ? MPIPE_OK : MPIPE_ERR_CUDA;
+    return e == cudaSuccess && cudaGetLastError() == cudaSuccess ? MPIPE_OK : MPIPE_ERR_CUDA;
 }
 
 int32_t mpipe_colsum_accumulate(const void* a, float* out, int32_t n_tokens, int32_t n_cols, int64_t lda, void* stream) {
@@ -397,9 +408,9 @@ int32_t mpipe_colsum_accumulate(const void* a, float* out, int32_t n_tokens, int
     if ((n_cols % 8) != 0 || (lda % 8) != 0 || !aligned16(a)) return MPIPE_ERR_UNSUPPORTED;
     const int n_groups = cdiv(n_cols, 256);
     const int n_slices = std::max(1, std::min(cdiv(n_tokens, 8), (sm_count() * 6) / n_groups));
-    colsum_kernel<<<n_groups * n_slices, 256, 0, static_cast<cudaStream_t>(stream)>>>(static_cast<const __nv_bfloat16*>(a), out, n_tokens,
-                                                                                      n_cols, lda, n_groups, n_slices);
-    return cudaGetLastError() == cudaSuccess ? MPIPE_OK : MPIPE_ERR_CUDA;
+    const cudaError_t e = launch_kernel(colsum_kernel, unsigned(n_groups * n_slices), 256, 0, static_cast<cudaStream_t>(stream), 1,
+                                        static_cast<const __nv_bfloat16*>(a), out, n_tokens, n_cols, lda, n_groups, n_slices);
+    return e == cudaSuccess && cudaGetLastError() == cudaSuccess ? MPIPE_OK : MPIPE_ERR_CUDA;
 }
 
 size_t mpipe_encoder_layer_workspace_bytes(int32_t n_tokens, int32_t hidden, int32_t ffn) {
@@ -444,9 +455,9 @@ int32_t mpipe_encoder_layer_fwd(const void* x, void* y, const mpipe_layer_weight
     const uint8_t* q = qkv;
     const uint8_t* k = qkv + size_t(hidden) * 2;
     const uint8_t* v = qkv + size_t(hidden) * 4;
-    if ((rc = mpipe_varlen_attn_fwd(q, k, v, attn, lse, 3 * int64_t(hidden), head_dim, hidden, head_dim, cu_seqlens_dev, n_seg,
-                                    n_tokens, max_seqlen, fwd_items_dev, n_fwd_items, n_heads, head_dim, softmax_scale, mode,
-                                    status_buf, stream)) != MPIPE_OK) return rc;
+    if ((rc = varlen_attn_fwd(q, k, v, attn, lse, 3 * int64_t(hidden), head_dim, hidden, head_dim, cu_seqlens_dev, n_seg,
+                              n_tokens, max_seqlen, fwd_items_dev, n_fwd_items, n_heads, head_dim, softmax_scale, mode,
+                              status_buf, stream, true)) != MPIPE_OK) return rc;
     if ((rc = mpipe_linear_fwd(attn, w->w_o, w->b_o, x, x1, n_tokens, hidden, hidden, hidden, hidden, hidden, hidden, 0,
                                status_buf, stream)) != MPIPE_OK) return rc;
     if ((rc = mpipe_layernorm_fwd(x1, w->ln2_gamma, w->ln2_beta, norm, n_tokens, hidden, hidden, hidden, ln_eps, stream)) != MPIPE_OK) return rc;

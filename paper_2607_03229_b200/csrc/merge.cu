@@ -27,6 +27,8 @@ __global__ void __launch_bounds__(kMergeThreads)
 merge_rows_kernel(const uint4* __restrict__ src, int64_t src_row_stride16, uint4* __restrict__ dst,
                   int64_t dst_row_stride16, const int32_t* __restrict__ positions, int32_t n_rows,
                   int32_t n_indexed_rows, int32_t chunks_per_row, int32_t* status_buf) {
+    pdl_wait();
+    pdl_launch();
     const int64_t total = int64_t(n_rows) * chunks_per_row;
     const int64_t step = int64_t(gridDim.x) * kMergeThreads * kMergeUnroll;
     for (int64_t base = int64_t(blockIdx.x) * kMergeThreads * kMergeUnroll + threadIdx.x; base < total; base += step) {
@@ -73,16 +75,11 @@ static int32_t merge_launch(bool scatter, const void* src, int64_t src_stride, v
     const int grid = int(want < cap ? want : cap);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     profile_start(kProfileMerge, st);
-    if (scatter)
-        merge_rows_kernel<true><<<grid, kMergeThreads, 0, st>>>(
-            static_cast<const uint4*>(src), src_stride / 8, static_cast<uint4*>(dst), dst_stride / 8, positions_dev,
-            n_enc_tokens, n_llm_tokens, chunks, status_buf);
-    else
-        merge_rows_kernel<false><<<grid, kMergeThreads, 0, st>>>(
-            static_cast<const uint4*>(src), src_stride / 8, static_cast<uint4*>(dst), dst_stride / 8, positions_dev,
-            n_enc_tokens, n_llm_tokens, chunks, status_buf);
+    const cudaError_t e = launch_kernel(scatter ? merge_rows_kernel<true> : merge_rows_kernel<false>, unsigned(grid), kMergeThreads, 0, st, 1,
+                                        static_cast<const uint4*>(src), src_stride / 8, static_cast<uint4*>(dst), dst_stride / 8,
+                                        positions_dev, n_enc_tokens, n_llm_tokens, chunks, status_buf);
     profile_stop(kProfileMerge, st);
-    return cudaGetLastError() == cudaSuccess ? MPIPE_OK : MPIPE_ERR_CUDA;
+    return e == cudaSuccess && cudaGetLastError() == cudaSuccess ? MPIPE_OK : MPIPE_ERR_CUDA;
 }
 
 }  // namespace mpipe
