@@ -324,10 +324,10 @@ int32_t mpipe_colsum_accumulate(const void* a, float* out, int32_t n_tokens, int
  * dx = dL/dx (bf16 [n_tokens, hidden]) and ADDS the parameter gradients, in fp32, to the twelve buffers of `grads`
  * (same shapes as the weights; the caller zeroes them at the start of a step, every microbatch accumulates).
  * fwd_workspace is the workspace of the matching mpipe_encoder_layer_fwd call (TRAINED mode, same x, weights, plan and
- * rope tables), untouched since: it holds the rotated q | k | v, the attention output, x1, GELU(u) and (TRAINED forward
- * only) the MLP pre-activation u; its LN slot is overwritten here.  lse is that call's LSE.  The two LayerNorm outputs
- * are recomputed instead of being stored by the forward.  workspace: device, 256-byte aligned,
- * >= mpipe_encoder_layer_bwd_workspace_bytes.  About twenty launches on `stream`, nothing allocated.  bwd_items_dev /
+ * rope tables), untouched since: it holds the LN2 output, the rotated q | k | v, the attention output, x1, GELU(u) and
+ * (TRAINED forward only) the MLP pre-activation u; nothing in it is changed here.  lse is that call's LSE.  The LN1 output
+ * is recomputed instead of being stored by the forward.  workspace: device, 256-byte aligned,
+ * >= mpipe_encoder_layer_bwd_workspace_bytes.  Fifteen launches on `stream`, nothing allocated.  bwd_items_dev /
  * n_bwd_items are the plan's backward list.  Sums over tokens use fp32 atomics and TMA reductions: parameter gradients
  * are reproducible to rounding order only.
  */

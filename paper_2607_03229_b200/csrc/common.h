@@ -62,6 +62,19 @@ int32_t linear_fwd_gelu_keep_preact(const void* a, const void* w, const void* bi
                                     int32_t K, int64_t lda, int64_t ldw, int64_t ldact, int64_t ldpre, int32_t* status_buf,
                                     void* stream);
 
+// Defined in gemm.cu, used by the layer backward: mpipe_linear_wgrad that also adds the column sums of dy to db (fp32 [N]).
+int32_t linear_wgrad_bias(const void* dy, const void* x, float* dw, float* db, int32_t n_tokens, int32_t N, int32_t K, int64_t lddy,
+                          int64_t ldx, int64_t lddw, int32_t* status_buf, void* stream);
+
+// Defined in attn_bwd.cu, used by the layer backward: mpipe_varlen_attn_bwd whose dQ and dK leave turned back by the rotary tables
+// (both NULL: as they are).
+int32_t varlen_attn_bwd_rope(const void* dout, const void* q, const void* k, const void* v, const void* o, const float* lse, void* dq,
+                             void* dk, void* dv, int64_t tok_stride_qkv, int64_t head_stride_qkv, int64_t tok_stride_o,
+                             int64_t head_stride_o, int64_t tok_stride_grad, int64_t head_stride_grad, const int32_t* cu_seqlens_dev,
+                             int32_t n_seg, int32_t total_tokens, int32_t max_seqlen, const mpipe_work_item_t* bwd_items_dev,
+                             int32_t n_bwd_items, int32_t n_heads, int32_t head_dim, float softmax_scale, const float* rope_cos,
+                             const float* rope_sin, void* workspace, size_t workspace_bytes, int32_t* status_buf, void* stream);
+
 // Defined in attn_fwd.cu, used by the layer forward: mpipe_varlen_attn_fwd; `settled` says that the device copy of the plan was
 // complete before the previous kernel of the stream started (true behind any other kernel of the layer).
 int32_t varlen_attn_fwd(const void* q, const void* k, const void* v, void* o, float* lse, int64_t tok_stride_qkv,

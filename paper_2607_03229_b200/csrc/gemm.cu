@@ -39,7 +39,8 @@ namespace mpipe {
 
 constexpr int kGemmBM = 128, kGemmBK = 64;                    // rows per CTA (256 per pair), contraction per stage
 constexpr int kGemmMaxBN = 256;
-constexpr int kGemmThreads = 384;
+// the weight gradient has four more warps, which add up the columns of its first operand (the bias gradient) from the stages
+__host__ __device__ constexpr int gemm_threads(int mode) { return mode == 2 ? 512 : 384; }
 constexpr int kGemmABytes = kGemmBM * kGemmBK * 2;            // 16 KB
 constexpr int kGemmRing = 160 * 1024, kGemmMaxStages = 8;     // 5 stages at BN 256 and 192, 6 at 128, 8 at 64
 constexpr int kGemmBox = 32 * 128;                            // [32 rows][128 bytes] staging box of one warp
@@ -64,11 +65,12 @@ struct GemmParams {
     int64_t ldr;
     int32_t side;                    // the side operand of map_s: residual (plain, GELU) or pre-activation (GELU gradient)
     int32_t store_pre;               // GELU only: also store the pre-activation (bf16) through map_u
+    float* colsum;                   // weight gradient: [M] or null, the column sums of the first operand are added to it
     int32_t* status_buf;
 };
 
 struct GemmBarriers {
-    uint64_t full[kGemmMaxStages], empty[kGemmMaxStages], acc_full[2], acc_empty[2], side_full[8][2];
+    uint64_t full[kGemmMaxStages], empty[kGemmMaxStages], done[kGemmMaxStages], acc_full[2], acc_empty[2], side_full[8][2];
 };
 
 __device__ __forceinline__ float2 bf16x2_to_f2(uint32_t w) {
@@ -77,7 +79,7 @@ __device__ __forceinline__ float2 bf16x2_to_f2(uint32_t w) {
 
 // kMode 0: forward, 1: input gradient, 2: weight gradient (see above)
 template <int kMode, int kEpi>
-__global__ void __launch_bounds__(kGemmThreads, 1)
+__global__ void __launch_bounds__(gemm_threads(kMode), 1)
 linear_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_w,
               const __grid_constant__ CUtensorMap map_c, const __grid_constant__ CUtensorMap map_s,
               const __grid_constant__ CUtensorMap map_u, const GemmParams p) {
@@ -96,6 +98,7 @@ linear_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
         for (int s = 0; s < kGemmMaxStages; ++s) {
             mbar_init(&bars.full[s], 1);
             mbar_init(&bars.empty[s], 1);
+            mbar_init(&bars.done[s], 1);
         }
         for (int a = 0; a < 2; ++a) {
             mbar_init(&bars.acc_full[a], 1);
@@ -134,6 +137,8 @@ linear_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
     auto tile_of = [&](int t) { return kMode == 2 ? t % n_out_tiles : t; };
     auto kb_lo_of = [&](int t) { return int((long long)(kMode == 2 ? t / n_out_tiles : my_split) * nk / p.splits); };
     auto kb_hi_of = [&](int t) { return int((long long)(kMode == 2 ? t / n_out_tiles + 1 : my_split + 1) * nk / p.splits); };
+    // weight gradient: the items whose first operand is also summed (each of its blocks meets one of them once)
+    auto sums = [&](int t) { return kMode == 2 && p.colsum != nullptr && tile_of(t) % p.tiles_n == 0; };
     const int bn = p.bn, bn_half = bn >> 1;
     const int stage_bytes = kGemmABytes + bn_half * kGemmBK * 2, n_stages = p.stages;
 
@@ -204,7 +209,7 @@ linear_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
                     for (int ks = 0; ks < kGemmBK / 16; ++ks)
                         umma_ss_pair(tmem + acc * kGemmMaxBN, umma_desc(a_lo + ks * a_step, hi128), umma_desc(b_lo + ks * b_step, hi128),
                                      idesc, (kb > lo || ks > 0) ? 1u : 0u);
-                    umma_commit_pair(&bars.empty[s], pair_mask);
+                    umma_commit_pair(sums(t) ? &bars.done[s] : &bars.empty[s], pair_mask);   // (then the summing warps free the stage)
                 }
                 if (++s == uint32_t(n_stages)) { s = 0; ph ^= 1; }
             }
@@ -212,6 +217,57 @@ linear_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
             if (leader) umma_commit_pair(&bars.acc_full[acc], pair_mask);
         }
         __syncwarp();
+    } else if (kMode == 2 && warp >= 12) {
+        // Column sums of the first operand: a stage's [64 tokens][128 columns] read once more from shared memory after the MMAs
+        // have read it.  A separate pass over dY is 20 to 85 us per projection of a 50 439-token microbatch, this hides beside
+        // the main loop (8 x 16 bytes per thread and stage).  No early exit: the four warps meet at a named barrier.
+        const int hw = warp - 12, lc = lane & 7;
+        uint32_t s = 0, phases = 0;
+        bool ok = true;
+        for (int t = cid; t < n_items; t += n_clusters) {
+            const bool mine = sums(t);
+            float2 acc[2][4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) acc[0][j] = acc[1][j] = make_float2(0.f, 0.f);
+            const int kb_hi = kb_hi_of(t);
+            for (int kb = kb_lo_of(t); kb < kb_hi; ++kb) {
+                if (mine) {
+                    if (ok) ok = mbar_wait(&bars.done[s], (phases >> s) & 1, &abort_flag);
+                    phases ^= 1u << s;
+                    if (ok) {
+#pragma unroll
+                        for (int a = 0; a < 2; ++a)
+#pragma unroll
+                            for (int i = 0; i < 4; ++i) {
+                                const int r = 16 * hw + 4 * i + (lane >> 3);
+                                const uint4 q = *reinterpret_cast<const uint4*>(smem + s * stage_bytes + a * (kGemmBK * 128) + r * 128 + ((lc ^ (r & 7)) << 4));
+                                acc[a][0] = add2(acc[a][0], bf16x2_to_f2(q.x));
+                                acc[a][1] = add2(acc[a][1], bf16x2_to_f2(q.y));
+                                acc[a][2] = add2(acc[a][2], bf16x2_to_f2(q.z));
+                                acc[a][3] = add2(acc[a][3], bf16x2_to_f2(q.w));
+                            }
+                    }
+                    named_barrier_sync(1, 128);
+                    if (hw == 0 && lane == 0) mbar_arrive(&bars.empty[s]);
+                }
+                if (++s == uint32_t(n_stages)) s = 0;
+            }
+            if (!mine || !ok) continue;
+            const int m0 = (tile_of(t) / p.tiles_n) * 2 * kGemmBM + half * kGemmBM;
+#pragma unroll
+            for (int a = 0; a < 2; ++a)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {   // over the four row lanes of a column chunk; lane group g then adds pair j = g
+                    float2 v = acc[a][j];
+                    v = add2(v, make_float2(__shfl_xor_sync(0xffffffffu, v.x, 8), __shfl_xor_sync(0xffffffffu, v.y, 8)));
+                    v = add2(v, make_float2(__shfl_xor_sync(0xffffffffu, v.x, 16), __shfl_xor_sync(0xffffffffu, v.y, 16)));
+                    const int m = m0 + 64 * a + lc * 8 + 2 * j;
+                    if ((lane >> 3) == j && m < p.M) {   // M is a multiple of 8
+                        atomicAdd(p.colsum + m, v.x);
+                        atomicAdd(p.colsum + m + 1, v.y);
+                    }
+                }
+        }
     } else if (warp >= 4) {
         const int ew = warp - 4, wg = ew >> 2, quarter = warp & 3;
         const uint32_t lane_base = uint32_t(quarter * 32) << 16;
@@ -413,14 +469,14 @@ static int gemm_stages(int bn) {
 }
 // Clusters of `ctas` CTAs that fit on the current device at once (the GPCs' SM counts limit clusters of more than two).
 template <auto kernel>
-static int max_clusters(int ctas) {
+static int max_clusters(int ctas, int threads = gemm_threads(0)) {
     static int cached[64][2 * kGemmMaxSplits + 1] = {};
     int dev = -1;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
     if (cached[dev][ctas] == 0) {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(unsigned(ctas));
-        cfg.blockDim = dim3(kGemmThreads);
+        cfg.blockDim = dim3(unsigned(threads));
         cfg.dynamicSmemBytes = kGemmSmem;
         cudaLaunchAttribute at[1];
         at[0].id = cudaLaunchAttributeClusterDimension;
@@ -460,10 +516,10 @@ static GemmShape choose_shape(int b_mode, bool gelu, int M, int N, int K) {
 }
 
 template <auto kernel>
-static int32_t launch_gemm(int cluster_ctas, int grid, const CUtensorMap& map_a, const CUtensorMap& map_w, const CUtensorMap& map_c,
+static int32_t launch_gemm(int threads, int cluster_ctas, int grid, const CUtensorMap& map_a, const CUtensorMap& map_w, const CUtensorMap& map_c,
                            const CUtensorMap& map_s, const CUtensorMap& map_u, const GemmParams& p, cudaStream_t st) {
     profile_start(kProfileLinear, st);
-    const cudaError_t e = launch_kernel(kernel, unsigned(grid), kGemmThreads, kGemmSmem, st, unsigned(cluster_ctas), map_a, map_w, map_c,
+    const cudaError_t e = launch_kernel(kernel, unsigned(grid), unsigned(threads), kGemmSmem, st, unsigned(cluster_ctas), map_a, map_w, map_c,
                                         map_s, map_u, p);
     profile_stop(kProfileLinear, st);
     return e == cudaSuccess && cudaGetLastError() == cudaSuccess ? MPIPE_OK : MPIPE_ERR_CUDA;
@@ -515,7 +571,7 @@ static int32_t launch_linear_as(const LinearCall& x, cudaStream_t st) {
     if (tiles > 0x7fffffffLL / (2 * kGemmMaxSplits)) return MPIPE_ERR_UNSUPPORTED;
     // a split contraction takes one cluster per tile (its CTAs meet once at a cluster barrier), everything else is persistent
     const int clusters = int(p.splits > 1 || tiles < cap ? tiles : cap);
-    return launch_gemm<linear_kernel<kMode, kEpi>>(2 * p.splits, clusters * 2 * p.splits, map_a, map_w, map_c, map_s, map_u, p, st);
+    return launch_gemm<linear_kernel<kMode, kEpi>>(gemm_threads(kMode), 2 * p.splits, clusters * 2 * p.splits, map_a, map_w, map_c, map_s, map_u, p, st);
 }
 
 // Shared host side of the two entry points: checks, then the instantiation the epilogue needs.
@@ -541,8 +597,8 @@ static int32_t launch_linear(int b_mode, const LinearCall& x, void* stream) {
     return x.aux != nullptr ? launch_linear_as<1, kEpiGeluGrad>(x, st) : launch_linear_as<1, kEpiPlain>(x, st);
 }
 
-// dW[n_rows, n_cols] (fp32) += dY[tokens, n_rows]^T X[tokens, n_cols]
-static int32_t launch_wgrad(const void* dy, const void* x, float* dw, int32_t tokens, int32_t n_rows, int32_t n_cols, int64_t lddy,
+// dW[n_rows, n_cols] (fp32) += dY[tokens, n_rows]^T X[tokens, n_cols]; with db also db[n_rows] += column sums of dY
+static int32_t launch_wgrad(const void* dy, const void* x, float* dw, float* db, int32_t tokens, int32_t n_rows, int32_t n_cols, int64_t lddy,
                             int64_t ldx, int64_t lddw, int32_t* status_buf, void* stream) {
     if (tokens < 0 || n_rows <= 0 || n_cols <= 0) return MPIPE_ERR_INVALID_ARG;
     if (tokens == 0) return MPIPE_OK;
@@ -556,7 +612,7 @@ static int32_t launch_wgrad(const void* dy, const void* x, float* dw, int32_t to
         !make_tensor_map_thd(&map_c, dw, n_rows, 1, n_cols, lddw, lddw, 32, 32, 128, 4))
         return MPIPE_ERR_CUDA;
     if (!ensure_dynamic_smem<linear_kernel<2, kEpiPlain>>(kGemmSmem)) return MPIPE_ERR_CUDA;
-    const int pairs = max_clusters<linear_kernel<2, kEpiPlain>>(2);
+    const int pairs = max_clusters<linear_kernel<2, kEpiPlain>>(2, gemm_threads(2));
     if (pairs <= 0) return MPIPE_ERR_CUDA;
     // Tile width and split of the token range, in SM clocks (fitted like choose_shape's constants).  A pair's fp32 tile leaves at
     // about 12 bytes per clock and SM (the L2's rate of fp32 reductions with every SM adding) beside the next item's main loop.
@@ -585,10 +641,17 @@ static int32_t launch_wgrad(const void* dy, const void* x, float* dw, int32_t to
     p.M = n_rows; p.N = n_cols; p.K = tokens;
     p.tiles_m = cdiv(n_rows, 2 * kGemmBM);
     p.tiles_n = cdiv(n_cols, p.bn);
+    p.colsum = db;
     p.status_buf = status_buf;
     const long long items = (long long)p.tiles_m * p.tiles_n * p.splits;
     const int clusters = int(items < pairs ? items : pairs);
-    return launch_gemm<linear_kernel<2, kEpiPlain>>(2, 2 * clusters, map_a, map_w, map_c, map_c, map_c, p, st);
+    return launch_gemm<linear_kernel<2, kEpiPlain>>(gemm_threads(2), 2, 2 * clusters, map_a, map_w, map_c, map_c, map_c, p, st);
+}
+
+// Weight and bias gradient of a projection in one launch.
+int32_t linear_wgrad_bias(const void* dy, const void* x, float* dw, float* db, int32_t n_tokens, int32_t N, int32_t K, int64_t lddy,
+                          int64_t ldx, int64_t lddw, int32_t* status_buf, void* stream) {
+    return launch_wgrad(dy, x, dw, db, n_tokens, N, K, lddy, ldx, lddw, status_buf, stream);
 }
 
 // fc1 of a TRAINED layer forward: act = GELU(a W^T + bias) and pre = a W^T + bias from ONE accumulator, so that the
@@ -606,7 +669,7 @@ extern "C" {
 
 int32_t mpipe_linear_wgrad(const void* dy, const void* x, float* dw, int32_t n_tokens, int32_t N, int32_t K, int64_t lddy,
                            int64_t ldx, int64_t lddw, int32_t* status_buf, void* stream) {
-    return mpipe::launch_wgrad(dy, x, dw, n_tokens, N, K, lddy, ldx, lddw, status_buf, stream);
+    return mpipe::launch_wgrad(dy, x, dw, nullptr, n_tokens, N, K, lddy, ldx, lddw, status_buf, stream);
 }
 
 int32_t mpipe_linear_fwd(const void* a, const void* w, const void* bias, const void* residual, void* c, int32_t M,

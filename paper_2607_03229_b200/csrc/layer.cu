@@ -10,6 +10,7 @@
 #include <algorithm>
 
 #include "common.h"
+#include "sm100_ptx.cuh"
 
 namespace mpipe {
 
@@ -125,131 +126,156 @@ __global__ void __launch_bounds__(256) rope_kernel(__nv_bfloat16* __restrict__ q
 }
 
 // LayerNorm backward.  With xhat = (x - mean) rstd and g = dy gamma:  dx = rstd (g - mean(g) - xhat mean(g xhat)) + dres,
-// dgamma += sum_t dy xhat, dbeta += sum_t dy.  One warp per row as in the forward; a block of four warps walks rows
-// blockIdx.x * 4 + warp, + gridDim.x * 4, ...  Each warp keeps its own column sums in shared memory (plain
-// read-modify-write: a lane owns its columns, a warp handles one row at a time), so registers hold one row only and
-// several blocks fit an SM; at the end the four copies are added and each column costs one global atomic per block
-// (same-address atomics serialise in L2, so the grid is kept to a few blocks per SM).
+// dgamma += sum_t dy xhat, dbeta += sum_t dy.  HBM-bound: 8 bytes per element.  One warp per row as in the forward, a block of
+// four warps walks rows blockIdx.x * 4 + warp, + gridDim.x * 4, ...; a lane's column sums stay in registers for the whole walk (in
+// shared memory they were four read-modify-writes per element), and the next row is copied into shared memory (cp.async, each
+// lane its own 16-byte chunks, so nobody waits for anybody) while the current one is worked on: eight warps keep 48 to 60 KB
+// in flight per SM.  At the end the four warps' sums are added in shared memory and each column costs one global atomic
+// per block.  50 439 x 1024: 103 -> 72 us (5.7 TB/s), 65 536 x 1280: 131 -> 115, 3489 x 1024: 12.6 -> 7.8.  A spilled column
+// sum costs more than more warps gain: 16 warps of 128 registers took 100 us.
 template <int kChunks>
-__global__ void __launch_bounds__(128) layernorm_bwd_kernel(const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __restrict__ dy,
-                                                            const __nv_bfloat16* __restrict__ gamma, const __nv_bfloat16* __restrict__ dres,
-                                                            __nv_bfloat16* __restrict__ dx, float* __restrict__ dgamma,
-                                                            float* __restrict__ dbeta, int32_t T, int32_t hidden, int64_t ldx,
-                                                            int64_t lddy, int64_t ldr, int64_t lddx, float eps) {
-    extern __shared__ float red[];   // [4 warps][2][kChunks * 256]
-    constexpr int kCols = kChunks * 256;
+struct LnbCfg {
+    static constexpr int kBlocks = kChunks <= 2 ? 4 : kChunks <= 3 ? 3 : 2;   // per SM: as many as leave the column sums in registers
+    static constexpr int kRowBytes = 3 * kChunks * 512;                       // x, dy, dres of one row
+    static constexpr int kSmem = 4 * 2 * kRowBytes;                           // four warps, two rows each
+};
+template <int kChunks>
+__global__ void __launch_bounds__(128, LnbCfg<kChunks>::kBlocks)
+layernorm_bwd_kernel(const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __restrict__ dy, const __nv_bfloat16* __restrict__ gamma,
+                     const __nv_bfloat16* __restrict__ dres, __nv_bfloat16* __restrict__ dx, float* __restrict__ dgamma,
+                     float* __restrict__ dbeta, int32_t T, int32_t hidden, int64_t ldx, int64_t lddy, int64_t ldr, int64_t lddx,
+                     float eps) {
+    extern __shared__ __align__(16) uint8_t rows_smem[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int n_chunks = hidden >> 3;
-    float* my_g = red + warp * 2 * kCols;
-    float* my_b = my_g + kCols;
-    for (int i = threadIdx.x; i < 4 * 2 * kCols; i += 128) red[i] = 0.f;
-    __syncthreads();
+    const float inv_h = 1.0f / float(hidden);
+    constexpr int kRoll = kChunks > 6 ? 2 : kChunks;   // loops that do not index the sums: rolled where registers are short
+    uint8_t* mine = rows_smem + warp * 2 * LnbCfg<kChunks>::kRowBytes + lane * 16;   // + stage, + (array * kChunks + chunk) * 512
+    for (int i = 0; i < 2 * 3 * kChunks; ++i) *reinterpret_cast<uint4*>(mine + i * 512) = make_uint4(0u, 0u, 0u, 0u);   // chunks past the row
     pdl_wait();
     pdl_launch();
-    const uint4* g4 = reinterpret_cast<const uint4*>(gamma);
-    for (int row = blockIdx.x * 4 + warp; row < T; row += gridDim.x * 4) {
-        const uint4* xr = reinterpret_cast<const uint4*>(x + int64_t(row) * ldx);
-        const uint4* dr = reinterpret_cast<const uint4*>(dy + int64_t(row) * lddy);
-        const uint4* rr = dres != nullptr ? reinterpret_cast<const uint4*>(dres + int64_t(row) * ldr) : nullptr;
-        uint4 xq[kChunks], dq[kChunks], rq[kChunks];
-#pragma unroll
-        for (int i = 0; i < kChunks; ++i) {   // every load of the row is issued before the first use
-            const int c = lane + 32 * i;
-            const bool in = c < n_chunks;
-            xq[i] = in ? xr[c] : make_uint4(0u, 0u, 0u, 0u);
-            dq[i] = in ? dr[c] : make_uint4(0u, 0u, 0u, 0u);
-            rq[i] = (in && rr != nullptr) ? rr[c] : make_uint4(0u, 0u, 0u, 0u);
-        }
-        float xv[kChunks][8];
-        float sum = 0.f;
-#pragma unroll
-        for (int i = 0; i < kChunks; ++i) {
-            const uint32_t w[4] = {xq[i].x, xq[i].y, xq[i].z, xq[i].w};
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                xv[i][2 * j] = __uint_as_float(w[j] << 16);
-                xv[i][2 * j + 1] = __uint_as_float(w[j] & 0xffff0000u);
-                sum += xv[i][2 * j] + xv[i][2 * j + 1];   // chunks past the row hold zeros
-            }
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-        const float mean = sum / float(hidden);
-        float sq = 0.f;
-#pragma unroll
-        for (int i = 0; i < kChunks; ++i)
-            if (lane + 32 * i < n_chunks)
-#pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    const float d = xv[i][j] - mean;
-                    sq = fmaf(d, d, sq);
-                }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
-        const float rstd = rsqrtf(sq / float(hidden) + eps);
-        float gv[kChunks][8];
-        float s1 = 0.f, s2 = 0.f;   // sum g, sum g xhat
+    auto unpack = [](uint32_t w) { return make_float2(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u)); };
+    auto fetch = [&](int64_t row, int stage) {
+        uint8_t* dst = mine + stage * LnbCfg<kChunks>::kRowBytes;
 #pragma unroll
         for (int i = 0; i < kChunks; ++i) {
             const int c = lane + 32 * i;
             if (c < n_chunks) {
-                const uint4 gq = __ldg(g4 + c);
-                const uint32_t w[4] = {dq[i].x, dq[i].y, dq[i].z, dq[i].w}, gw[4] = {gq.x, gq.y, gq.z, gq.w};
-                float4* pg = reinterpret_cast<float4*>(my_g + c * 8);
-                float4* pb = reinterpret_cast<float4*>(my_b + c * 8);
-                float4 ag[2] = {pg[0], pg[1]}, ab[2] = {pb[0], pb[1]};
-                float* fg = reinterpret_cast<float*>(ag);
-                float* fb = reinterpret_cast<float*>(ab);
-#pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    const float d = (j & 1) ? __uint_as_float(w[j >> 1] & 0xffff0000u) : __uint_as_float(w[j >> 1] << 16);
-                    const float gm = (j & 1) ? __uint_as_float(gw[j >> 1] & 0xffff0000u) : __uint_as_float(gw[j >> 1] << 16);
-                    const float xh = (xv[i][j] - mean) * rstd;
-                    xv[i][j] = xh;
-                    gv[i][j] = d * gm;
-                    s1 += gv[i][j];
-                    s2 = fmaf(gv[i][j], xh, s2);
-                    fg[j] = fmaf(d, xh, fg[j]);
-                    fb[j] += d;
-                }
-                pg[0] = ag[0]; pg[1] = ag[1];
-                pb[0] = ab[0]; pb[1] = ab[1];
+                cp_async16(dst + i * 512, x + row * ldx + c * 8);
+                cp_async16(dst + (kChunks + i) * 512, dy + row * lddy + c * 8);
+                if (dres != nullptr) cp_async16(dst + (2 * kChunks + i) * 512, dres + row * ldr + c * 8);
             }
         }
+    };
+    float2 sg[kChunks][4], sb[kChunks][4];
+#pragma unroll
+    for (int i = 0; i < kChunks; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) sg[i][j] = sb[i][j] = make_float2(0.f, 0.f);
+    const int64_t stride = int64_t(gridDim.x) * 4;
+    int64_t row = int64_t(blockIdx.x) * 4 + warp;
+    int stage = 0;
+    if (row < T) fetch(row, 0);
+    cp_async_commit();
+    for (; row < T; row += stride, stage ^= 1) {
+        if (row + stride < T) fetch(row + stride, stage ^ 1);
+        cp_async_commit();
+        cp_async_wait<1>();
+        const uint8_t* src = mine + stage * LnbCfg<kChunks>::kRowBytes;
+        auto x_of = [&](int i) { return *reinterpret_cast<const uint4*>(src + i * 512); };
+        float2 a = make_float2(0.f, 0.f), b = make_float2(0.f, 0.f);
+#pragma unroll kRoll
+        for (int i = 0; i < kChunks; ++i) {
+            const uint4 q = x_of(i);
+            a = add2(a, add2(unpack(q.x), unpack(q.y)));
+            b = add2(b, add2(unpack(q.z), unpack(q.w)));
+        }
+        a = add2(a, b);
+        float sum = a.x + a.y;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        const float mean = sum * inv_h;
+        const float2 nm = make_float2(-mean, -mean);
+        a = b = make_float2(0.f, 0.f);
+#pragma unroll kRoll
+        for (int i = 0; i < kChunks; ++i)
+            if (lane + 32 * i < n_chunks) {
+                const uint4 xq = x_of(i);
+                const uint32_t xw[4] = {xq.x, xq.y, xq.z, xq.w};
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const float2 d = add2(unpack(xw[j]), nm);
+                    if (j & 1) a = fma2(d, d, a);
+                    else b = fma2(d, d, b);
+                }
+            }
+        a = add2(a, b);
+        float sq = a.x + a.y;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+        const float rstd = rsqrtf(sq * inv_h + eps);
+        const float2 rs = make_float2(rstd, rstd);
+        float2 a1 = make_float2(0.f, 0.f), a2 = make_float2(0.f, 0.f);   // sum g, sum g xhat
+#pragma unroll
+        for (int i = 0; i < kChunks; ++i) {
+            const int c = lane + 32 * i;
+            const uint4 gq = c < n_chunks ? __ldg(reinterpret_cast<const uint4*>(gamma) + c) : make_uint4(0u, 0u, 0u, 0u);
+            const uint4 xq = x_of(i), dq = *reinterpret_cast<const uint4*>(src + (kChunks + i) * 512);
+            const uint32_t xw[4] = {xq.x, xq.y, xq.z, xq.w}, gw[4] = {gq.x, gq.y, gq.z, gq.w}, dw[4] = {dq.x, dq.y, dq.z, dq.w};
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const float2 xh = mul2(add2(unpack(xw[j]), nm), rs), d = unpack(dw[j]), g = mul2(d, unpack(gw[j]));
+                a1 = add2(a1, g);
+                a2 = fma2(g, xh, a2);
+                sg[i][j] = fma2(d, xh, sg[i][j]);   // chunks past the row hold d = 0
+                sb[i][j] = add2(sb[i][j], d);
+            }
+        }
+        float s1 = a1.x + a1.y, s2 = a2.x + a2.y;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
             s1 += __shfl_xor_sync(0xffffffffu, s1, o);
             s2 += __shfl_xor_sync(0xffffffffu, s2, o);
         }
-        const float m1 = s1 / float(hidden), m2 = s2 / float(hidden);
-        uint4* outr = reinterpret_cast<uint4*>(dx + int64_t(row) * lddx);
-#pragma unroll
+        const float2 m1 = make_float2(-s1 * inv_h, -s1 * inv_h), m2 = make_float2(-s2 * inv_h, -s2 * inv_h);
+        uint4* outr = reinterpret_cast<uint4*>(dx + row * lddx);
+#pragma unroll kRoll
         for (int i = 0; i < kChunks; ++i) {
             const int c = lane + 32 * i;
-            if (c < n_chunks) {
-                const uint32_t rw[4] = {rq[i].x, rq[i].y, rq[i].z, rq[i].w};
-                uint32_t o[4];
+            if (c >= n_chunks) continue;
+            const uint4 gq = __ldg(reinterpret_cast<const uint4*>(gamma) + c);
+            const uint4 xq = x_of(i), dq = *reinterpret_cast<const uint4*>(src + (kChunks + i) * 512);
+            const uint4 rq = *reinterpret_cast<const uint4*>(src + (2 * kChunks + i) * 512);
+            const uint32_t xw[4] = {xq.x, xq.y, xq.z, xq.w}, gw[4] = {gq.x, gq.y, gq.z, gq.w}, dw[4] = {dq.x, dq.y, dq.z, dq.w},
+                           rw[4] = {rq.x, rq.y, rq.z, rq.w};
+            uint32_t o[4];
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const float lo = rstd * (gv[i][2 * j] - m1 - xv[i][2 * j] * m2) + __uint_as_float(rw[j] << 16);
-                    const float hi = rstd * (gv[i][2 * j + 1] - m1 - xv[i][2 * j + 1] * m2) + __uint_as_float(rw[j] & 0xffff0000u);
-                    const __nv_bfloat162 pk = __floats2bfloat162_rn(lo, hi);
-                    o[j] = *reinterpret_cast<const uint32_t*>(&pk);
-                }
-                outr[c] = make_uint4(o[0], o[1], o[2], o[3]);
+            for (int j = 0; j < 4; ++j) {
+                const float2 xh = mul2(add2(unpack(xw[j]), nm), rs), g = mul2(unpack(dw[j]), unpack(gw[j]));
+                const float2 v = fma2(rs, fma2(xh, m2, add2(g, m1)), unpack(rw[j]));
+                o[j] = pack_bf16(v.x, v.y);
             }
+            outr[c] = make_uint4(o[0], o[1], o[2], o[3]);
         }
     }
-    __syncthreads();
-    for (int col = threadIdx.x; col < hidden; col += 128) {
-        float sg = 0.f, sb = 0.f;
+    cp_async_wait<0>();
+    float* red = reinterpret_cast<float*>(rows_smem);   // [4 warps][kChunks * 256], over the rows
+    static_assert(LnbCfg<kChunks>::kSmem >= 4 * kChunks * 256 * 4, "the sums fit where the rows were");
 #pragma unroll
-        for (int w = 0; w < 4; ++w) {
-            sg += red[w * 2 * kCols + col];
-            sb += red[w * 2 * kCols + kCols + col];
+    for (int which = 0; which < 2; ++which) {
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < kChunks; ++i) {
+            const float2 (&v)[4] = which == 0 ? sg[i] : sb[i];
+            float4* dst = reinterpret_cast<float4*>(red + (warp * kChunks * 32 + lane + 32 * i) * 8);
+            dst[0] = make_float4(v[0].x, v[0].y, v[1].x, v[1].y);
+            dst[1] = make_float4(v[2].x, v[2].y, v[3].x, v[3].y);
         }
-        atomicAdd(dgamma + col, sg);
-        atomicAdd(dbeta + col, sb);
+        __syncthreads();
+        float* out = which == 0 ? dgamma : dbeta;
+        constexpr int kCols = kChunks * 256;
+        for (int col = threadIdx.x; col < hidden; col += 128)
+            atomicAdd(out + col, (red[col] + red[kCols + col]) + (red[2 * kCols + col] + red[3 * kCols + col]));
     }
 }
 
@@ -380,21 +406,22 @@ int32_t mpipe_layernorm_bwd(const void* x, const void* dy, const void* gamma, co
         return MPIPE_ERR_UNSUPPORTED;
     if (!aligned16(x) || !aligned16(dy) || !aligned16(gamma) || !aligned16(dres) || !aligned16(dx)) return MPIPE_ERR_UNSUPPORTED;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    const int grid = std::min(cdiv(n_tokens, 4), sm_count() * 6);
     const int chunks = cdiv(hidden, 256);
     cudaError_t e;
-#define MPIPE_LNB_LAUNCH(C)                                                                                                    \
-    do {                                                                                                                       \
-        cudaFuncSetAttribute(layernorm_bwd_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, 4 * 2 * (C) * 256 * 4);      \
-        e = launch_kernel(layernorm_bwd_kernel<C>, unsigned(grid), 128, 4 * 2 * (C) * 256 * 4, st, 1,                           \
-                          static_cast<const __nv_bfloat16*>(x), static_cast<const __nv_bfloat16*>(dy),                          \
-                          static_cast<const __nv_bfloat16*>(gamma), static_cast<const __nv_bfloat16*>(dres),                    \
-                          static_cast<__nv_bfloat16*>(dx), dgamma, dbeta, n_tokens, hidden, ldx, lddy, ldr, lddx, eps);         \
+#define MPIPE_LNB_LAUNCH(C)                                                                                                       \
+    do {                                                                                                                          \
+        if (!ensure_dynamic_smem<layernorm_bwd_kernel<C>>(LnbCfg<C>::kSmem)) return MPIPE_ERR_CUDA;                               \
+        e = launch_kernel(layernorm_bwd_kernel<C>, unsigned(std::min(cdiv(n_tokens, 4), sm_count() * LnbCfg<C>::kBlocks)), 128,   \
+                          LnbCfg<C>::kSmem, st, 1, static_cast<const __nv_bfloat16*>(x), static_cast<const __nv_bfloat16*>(dy),   \
+                          static_cast<const __nv_bfloat16*>(gamma), static_cast<const __nv_bfloat16*>(dres),                      \
+                          static_cast<__nv_bfloat16*>(dx), dgamma, dbeta, n_tokens, hidden, ldx, lddy, ldr, lddx, eps);           \
     } while (0)
     if (chunks <= 1) MPIPE_LNB_LAUNCH(1);
     else if (chunks <= 2) MPIPE_LNB_LAUNCH(2);
+    else if (chunks <= 3) MPIPE_LNB_LAUNCH(3);
     else if (chunks <= 4) MPIPE_LNB_LAUNCH(4);
     else if (chunks <= 5) MPIPE_LNB_LAUNCH(5);
+    else if (chunks <= 6) MPIPE_LNB_LAUNCH(6);
     else MPIPE_LNB_LAUNCH(kLnMaxChunks);
 #undef MPIPE_LNB_LAUNCH
     return e == cudaSuccess && cudaGetLastError() == cudaSuccess ? MPIPE_OK : MPIPE_ERR_CUDA;
@@ -500,7 +527,7 @@ int32_t mpipe_encoder_layer_bwd(const void* dy, const void* x, void* dx, const m
     const int32_t head_dim = hidden / n_heads;
     const size_t t = size_t(n_tokens);
     const int64_t h = hidden, h3 = 3 * int64_t(hidden), f = ffn;
-    // what the forward left in its workspace: LN output (stale), packed q|k|v (q, k rotated), attention output, x1, GELU(u), u
+    // what the forward left in its workspace: m = LN2(x1), packed q|k|v (q, k rotated), attention output, x1, GELU(u), u
     uint8_t* fw = static_cast<uint8_t*>(fwd_workspace);
     uint8_t* norm = fw;               fw += align256(t * hidden * 2);
     uint8_t* qkv = fw;                fw += align256(t * 3 * hidden * 2);
@@ -517,28 +544,21 @@ int32_t mpipe_encoder_layer_bwd(const void* dy, const void* x, void* dx, const m
     const size_t attn_ws_bytes = mpipe_attn_workspace_bytes(n_tokens, n_heads, head_dim, MPIPE_ENC_TRAINED);
     int32_t rc;
 #define MPIPE_TRY(call) do { if ((rc = (call)) != MPIPE_OK) return rc; } while (0)
-    // ---- MLP branch: y = x1 + GELU(m W1^T + b1) W2^T + b2, m = LN2(x1)
-    MPIPE_TRY(mpipe_layernorm_fwd(x1, w->ln2_gamma, w->ln2_beta, norm, n_tokens, hidden, h, h, ln_eps, stream));                 // m
-    MPIPE_TRY(mpipe_linear_wgrad(dy, act, g->w_fc2, n_tokens, hidden, ffn, h, f, f, status_buf, stream));                          // dW2 += dy^T GELU(u)
-    MPIPE_TRY(mpipe_colsum_accumulate(dy, g->b_fc2, n_tokens, hidden, h, stream));
+    // ---- MLP branch: y = x1 + GELU(m W1^T + b1) W2^T + b2, m = LN2(x1) (still in the forward's LN slot)
+    MPIPE_TRY(linear_wgrad_bias(dy, act, g->w_fc2, g->b_fc2, n_tokens, hidden, ffn, h, f, f, status_buf, stream));                 // dW2 += dy^T GELU(u), db2
     MPIPE_TRY(mpipe_linear_dgrad(dy, w->w_fc2, ubuf, nullptr, dubuf, n_tokens, hidden, ffn, h, f, f, 0, f, status_buf, stream));    // du = (dy W2) o GELU'(u)
-    MPIPE_TRY(mpipe_linear_wgrad(dubuf, norm, g->w_fc1, n_tokens, ffn, hidden, f, h, h, status_buf, stream));                     // dW1 += du^T m
-    MPIPE_TRY(mpipe_colsum_accumulate(dubuf, g->b_fc1, n_tokens, ffn, f, stream));
+    MPIPE_TRY(linear_wgrad_bias(dubuf, norm, g->w_fc1, g->b_fc1, n_tokens, ffn, hidden, f, h, h, status_buf, stream));            // dW1 += du^T m, db1
     MPIPE_TRY(mpipe_linear_dgrad(dubuf, w->w_fc1, nullptr, nullptr, tmp, n_tokens, ffn, hidden, f, h, 0, 0, h, status_buf, stream)); // dm = du W1
     MPIPE_TRY(mpipe_layernorm_bwd(x1, tmp, w->ln2_gamma, dy, dx1, g->ln2_gamma, g->ln2_beta, n_tokens, hidden, h, h, h, h, ln_eps, stream)); // dx1 = dy + LN2'(dm)
     // ---- attention branch: x1 = x + o Wo^T + bo, o = attention(rope(a Wqkv^T + bqkv)), a = LN1(x)
-    MPIPE_TRY(mpipe_linear_wgrad(dx1, attn, g->w_o, n_tokens, hidden, hidden, h, h, h, status_buf, stream));                       // dWo += dx1^T o
-    MPIPE_TRY(mpipe_colsum_accumulate(dx1, g->b_o, n_tokens, hidden, h, stream));
+    MPIPE_TRY(linear_wgrad_bias(dx1, attn, g->w_o, g->b_o, n_tokens, hidden, hidden, h, h, h, status_buf, stream));                // dWo += dx1^T o, dbo
     MPIPE_TRY(mpipe_linear_dgrad(dx1, w->w_o, nullptr, nullptr, tmp, n_tokens, hidden, hidden, h, h, 0, 0, h, status_buf, stream)); // do = dx1 Wo
-    MPIPE_TRY(mpipe_varlen_attn_bwd(tmp, qkv, qkv + size_t(hidden) * 2, qkv + size_t(hidden) * 4, attn, lse, dqkv, dqkv + size_t(hidden) * 2,
-                                    dqkv + size_t(hidden) * 4, h3, head_dim, h, head_dim, h3, head_dim, cu_seqlens_dev, n_seg, n_tokens,
-                                    max_seqlen, bwd_items_dev, n_bwd_items, n_heads, head_dim, softmax_scale, MPIPE_ENC_TRAINED, attn_ws,
-                                    attn_ws_bytes, status_buf, stream));
-    if (rope_cos != nullptr)
-        MPIPE_TRY(mpipe_rope_apply_bwd(dqkv, h3, hidden, rope_cos, rope_sin, n_tokens, n_heads, head_dim, stream));
-    MPIPE_TRY(mpipe_layernorm_fwd(x, w->ln1_gamma, w->ln1_beta, norm, n_tokens, hidden, h, h, ln_eps, stream));                    // a (recomputed)
-    MPIPE_TRY(mpipe_linear_wgrad(dqkv, norm, g->w_qkv, n_tokens, 3 * hidden, hidden, h3, h, h, status_buf, stream));               // dWqkv += dqkv^T a
-    MPIPE_TRY(mpipe_colsum_accumulate(dqkv, g->b_qkv, n_tokens, 3 * hidden, h3, stream));
+    MPIPE_TRY(varlen_attn_bwd_rope(tmp, qkv, qkv + size_t(hidden) * 2, qkv + size_t(hidden) * 4, attn, lse, dqkv, dqkv + size_t(hidden) * 2,
+                                   dqkv + size_t(hidden) * 4, h3, head_dim, h, head_dim, h3, head_dim, cu_seqlens_dev, n_seg, n_tokens,
+                                   max_seqlen, bwd_items_dev, n_bwd_items, n_heads, head_dim, softmax_scale, rope_cos, rope_sin, attn_ws,
+                                   attn_ws_bytes, status_buf, stream));
+    MPIPE_TRY(mpipe_layernorm_fwd(x, w->ln1_gamma, w->ln1_beta, tmp, n_tokens, hidden, h, h, ln_eps, stream));                     // a (recomputed)
+    MPIPE_TRY(linear_wgrad_bias(dqkv, tmp, g->w_qkv, g->b_qkv, n_tokens, 3 * hidden, hidden, h3, h, h, status_buf, stream));       // dWqkv += dqkv^T a, dbqkv
     MPIPE_TRY(mpipe_linear_dgrad(dqkv, w->w_qkv, nullptr, nullptr, tmp, n_tokens, 3 * hidden, hidden, h3, h, 0, 0, h, status_buf, stream)); // da = dqkv Wqkv
     MPIPE_TRY(mpipe_layernorm_bwd(x, tmp, w->ln1_gamma, dx1, dx, g->ln1_gamma, g->ln1_beta, n_tokens, hidden, h, h, h, h, ln_eps, stream)); // dx = dx1 + LN1'(da)
 #undef MPIPE_TRY
