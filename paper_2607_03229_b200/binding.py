@@ -1,4 +1,5 @@
-"""ctypes binding of libmpipe_enc.so: argument marshalling only.
+"""Binding of libmpipe_enc.so: argument marshalling only (ctypes; the calls of the per-microbatch path -- plan, upload, attention,
+merge -- natively in ``_hostpath.so``, which a small microbatch is bound by).
 
 Every function has the name of the C entry point without the ``mpipe_`` prefix and forwards
 to it; all arithmetic of the hot path runs in the CUDA kernels behind the C ABI
@@ -8,6 +9,7 @@ CPU fallback: if the shared library is missing the import of this module's funct
 from __future__ import annotations
 
 import ctypes
+import importlib.util
 import os
 from dataclasses import dataclass
 from typing import List, Optional
@@ -21,7 +23,10 @@ LIB_PATH = os.path.join(_HERE, "libmpipe_enc.so")
 OK, ERR_INVALID_ARG, ERR_UNSUPPORTED, ERR_WORKSPACE, ERR_CUDA, ERR_TIMEOUT, ERR_INDEX = range(7)
 FROZEN, TRAINED = 0, 1
 
+HOSTPATH = os.path.join(_HERE, "_hostpath.so")
 _lib = None
+_host = None            # the native marshalling module
+_tile_rows = (0, 0)     # the library's native tile heights
 
 
 class WorkItem(ctypes.Structure):
@@ -91,18 +96,29 @@ EXPORTED_SYMBOLS = tuple(_SIGNATURES)
 
 def load() -> ctypes.CDLL:
     """Load the shared library (built in-tree by ``build.py``); raises if it is not there."""
-    global _lib
+    global _lib, _host, _tile_rows
     if _lib is None:
-        if not os.path.exists(LIB_PATH):
-            raise RuntimeError(
-                f"{LIB_PATH} is missing: build it with `python -m paper_2607_03229_b200.build` "
-                "(there is no fallback path)")
+        for path in (LIB_PATH, HOSTPATH):
+            if not os.path.exists(path):
+                raise RuntimeError(f"{path} is missing: build it with `python -m paper_2607_03229_b200.build` "
+                                   "(there is no fallback path)")
         lib = ctypes.CDLL(LIB_PATH)
         for name, (res, args) in _SIGNATURES.items():
             fn = getattr(lib, name)
             fn.restype, fn.argtypes = res, args
-        _lib = lib
+        spec = importlib.util.spec_from_file_location("_hostpath", HOSTPATH)
+        host = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(host)
+        host.bind(*(ctypes.cast(getattr(lib, "mpipe_" + f), ctypes.c_void_p).value for f in
+                    ("seg_plan", "varlen_attn_fwd", "varlen_attn_bwd", "merge_tokens", "merge_tokens_bwd")))
+        _host, _tile_rows, _lib = host, (lib.mpipe_fwd_tile_rows(), lib.mpipe_bwd_tile_rows()), lib
     return _lib
+
+
+def _native():
+    if _lib is None:
+        load()
+    return _host
 
 
 class MpipeError(RuntimeError):
@@ -161,6 +177,7 @@ class SegPlan:
     fwd_items_dev: Optional[torch.Tensor] = None
     bwd_items_dev: Optional[torch.Tensor] = None
     _host_staging: Optional[torch.Tensor] = None
+    _packed: Optional[tuple] = None   # (bytearray, forward offset, backward offset, the three arrays as views of it)
 
     @property
     def n_seg(self) -> int:
@@ -169,6 +186,13 @@ class SegPlan:
     def to_device(self, device="cuda") -> "SegPlan":
         """Upload cu_seqlens and both item lists with ONE asynchronous copy from a pinned staging buffer
         (stream-ordered on the current stream; the host does not wait for the device)."""
+        if self._packed is not None:
+            buf, off_f, off_b, cu, fwd, bwd = self._packed
+            dev = torch.device(device)
+            if dev.type == "cuda" and self.cu_seqlens is cu and self.fwd_items is fwd and self.bwd_items is bwd:
+                self._host_staging, self.cu_seqlens_dev, self.fwd_items_dev, self.bwd_items_dev = _native().upload(
+                    buf, cu.size, off_f, fwd.size, off_b, bwd.size, -1 if dev.index is None else dev.index)
+                return self
         parts = [np.ascontiguousarray(self.cu_seqlens).view(np.int32).reshape(-1),
                  np.ascontiguousarray(self.fwd_items).view(np.int32).reshape(-1),
                  np.ascontiguousarray(self.bwd_items).view(np.int32).reshape(-1)]
@@ -190,21 +214,21 @@ class SegPlan:
 
 
 def seg_plan(patch_counts, mode: int, fwd_rows: Optional[int] = None, bwd_rows: Optional[int] = None) -> SegPlan:
-    """mpipe_seg_plan with the two-call pattern (count, then fill).  Host only."""
-    lib = load()
-    counts = np.ascontiguousarray(np.asarray(patch_counts, dtype=np.int32).reshape(-1))
-    n_seg = counts.size
-    fwd_rows = fwd_tile_rows() if fwd_rows is None else fwd_rows
-    bwd_rows = bwd_tile_rows() if bwd_rows is None else bwd_rows
-    cu = np.zeros(n_seg + 1, dtype=np.int32)
-    total, mx, nf, nb = (ctypes.c_int32() for _ in range(4))
-    args = (_ptr(counts), n_seg, fwd_rows, bwd_rows, mode, _ptr(cu), ctypes.addressof(total), ctypes.addressof(mx))
-    _check(lib.mpipe_seg_plan(*args, None, ctypes.addressof(nf), None, ctypes.addressof(nb)), "mpipe_seg_plan")
-    fwd = np.zeros(nf.value, dtype=ITEM_DTYPE)
-    bwd = np.zeros(nb.value, dtype=ITEM_DTYPE)
-    _check(lib.mpipe_seg_plan(*args, _ptr(fwd), ctypes.addressof(nf), _ptr(bwd), ctypes.addressof(nb)),
-           "mpipe_seg_plan")
-    return SegPlan(mode, cu, total.value, mx.value, fwd, bwd)
+    """mpipe_seg_plan.  Host only."""
+    host = _native()
+    fwd_rows = _tile_rows[0] if fwd_rows is None else fwd_rows
+    bwd_rows = _tile_rows[1] if bwd_rows is None else bwd_rows
+    counts = patch_counts
+    got = host.seg_plan(counts, mode, fwd_rows, bwd_rows) if type(counts) is list else None
+    if got is None:   # not a list of plain integers: numpy's conversion rules
+        counts = np.asarray(patch_counts, dtype=np.int32).reshape(-1).tolist()
+        got = host.seg_plan(counts, mode, fwd_rows, bwd_rows)
+    status, buf, off_f, n_f, off_b, n_b, total, mx = got
+    _check(status, "mpipe_seg_plan")
+    words = np.frombuffer(buf, dtype=np.int32)
+    cu = words[:len(counts) + 1]
+    fwd, bwd = (words[o:o + 6 * n].view(ITEM_DTYPE) for o, n in ((off_f, n_f), (off_b, n_b)))
+    return SegPlan(mode, cu, total, mx, fwd, bwd, _packed=(buf, off_f, off_b, cu, fwd, bwd))
 
 
 def attn_workspace_bytes(total_tokens: int, n_heads: int, head_dim: int, mode: int) -> int:
@@ -227,24 +251,14 @@ def _check_plan(plan: SegPlan, T: int, items_dev, n_items: int, what: str) -> No
 
 def varlen_attn_fwd(q, k, v, o, lse, plan: SegPlan, softmax_scale: float, status_buf=None, stream=None) -> None:
     """mpipe_varlen_attn_fwd.  q,k,v,o: bf16 CUDA tensors [T,H,D]; lse: fp32 [H,T] or None (frozen)."""
-    T, H, D = q.shape
-    assert k.shape == q.shape and v.shape == q.shape and o.shape == q.shape
-    assert q.dtype == k.dtype == v.dtype == o.dtype == torch.bfloat16
-    _check_plan(plan, T, plan.fwd_items_dev, int(plan.fwd_items.size), "varlen_attn_fwd")
-    ts, hs = _thd_strides(q)
-    assert _thd_strides(k) == (ts, hs) and _thd_strides(v) == (ts, hs), "q, k, v must share strides"
-    tso, hso = _thd_strides(o)
-    if lse is not None:
-        assert lse.dtype == torch.float32 and lse.is_contiguous() and tuple(lse.shape) == (H, T)
-    st = load().mpipe_varlen_attn_fwd(
-        _ptr(q), _ptr(k), _ptr(v), _ptr(o), _ptr(lse), ts, hs, tso, hso, _ptr(plan.cu_seqlens_dev), plan.n_seg,
-        plan.total_tokens, plan.max_seqlen, _ptr(plan.fwd_items_dev), int(plan.fwd_items.size), H, D,
-        softmax_scale, plan.mode, _ptr(status_buf), _stream(stream))
-    _check(st, "mpipe_varlen_attn_fwd")
+    st = _native().attn_fwd(q, k, v, o, lse, plan.mode, plan.n_seg, plan.total_tokens, plan.max_seqlen, plan.cu_seqlens_dev,
+                            plan.fwd_items_dev, plan.fwd_items.size, softmax_scale, status_buf, stream)
+    if st:
+        _check(st, "mpipe_varlen_attn_fwd")
 
 
 def _bwd_args(what, dout, q, k, v, o, lse, dq, dk, dv, plan: SegPlan, softmax_scale: float):
-    """Shape / dtype / stride checks and argument marshalling shared by the two backward entry points."""
+    """Shape / dtype / stride checks and argument marshalling of the backward with built-in scratch."""
     T, H, D = q.shape
     ts, hs = _thd_strides(q)
     tso, hso = _thd_strides(o)
@@ -267,10 +281,10 @@ def _bwd_args(what, dout, q, k, v, o, lse, dq, dk, dv, plan: SegPlan, softmax_sc
 def varlen_attn_bwd(dout, q, k, v, o, lse, dq, dk, dv, plan: SegPlan, softmax_scale: float, workspace,
                     status_buf=None, stream=None) -> None:
     """mpipe_varlen_attn_bwd.  A frozen plan returns at once (nothing is launched)."""
-    args = _bwd_args("varlen_attn_bwd", dout, q, k, v, o, lse, dq, dk, dv, plan, softmax_scale)
-    ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    st = load().mpipe_varlen_attn_bwd(*args, _ptr(workspace), ws_bytes, _ptr(status_buf), _stream(stream))
-    _check(st, "mpipe_varlen_attn_bwd")
+    st = _native().attn_bwd(dout, q, k, v, o, lse, dq, dk, dv, plan.mode, plan.n_seg, plan.total_tokens, plan.max_seqlen,
+                            plan.cu_seqlens_dev, plan.bwd_items_dev, plan.bwd_items.size, softmax_scale, workspace, status_buf, stream)
+    if st:
+        _check(st, "mpipe_varlen_attn_bwd")
 
 
 LINEAR_GELU = 1
@@ -489,26 +503,16 @@ def varlen_attn_bwd_static(dout, q, k, v, o, lse, dq, dk, dv, plan: SegPlan, sof
 
 def merge_tokens(enc_tokens, llm_embeds, positions_dev, mode: int = TRAINED, status_buf=None, stream=None) -> None:
     """mpipe_merge_tokens: llm_embeds[positions[i], :] = enc_tokens[i, :], in place."""
-    n_enc = int(positions_dev.numel())
-    n_llm, hidden = llm_embeds.shape
-    assert enc_tokens.dtype == llm_embeds.dtype == torch.bfloat16 and positions_dev.dtype == torch.int32
-    assert enc_tokens.shape[0] == n_enc and (n_enc == 0 or enc_tokens.shape[1] == hidden)
-    assert llm_embeds.stride(1) == 1 and (n_enc == 0 or enc_tokens.stride(1) == 1)
-    st = load().mpipe_merge_tokens(_ptr(enc_tokens), enc_tokens.stride(0) if n_enc else hidden, _ptr(llm_embeds),
-                                   llm_embeds.stride(0), _ptr(positions_dev), n_enc, n_llm, hidden, mode,
-                                   _ptr(status_buf), _stream(stream))
-    _check(st, "mpipe_merge_tokens")
+    st = _native().merge(enc_tokens, llm_embeds, positions_dev, mode, status_buf, stream, 0)
+    if st:
+        _check(st, "mpipe_merge_tokens")
 
 
 def merge_tokens_bwd(d_llm_embeds, d_enc, positions_dev, mode: int, status_buf=None, stream=None) -> None:
     """mpipe_merge_tokens_bwd: d_enc[i, :] = d_llm_embeds[positions[i], :]; no-op when frozen."""
-    n_enc = int(positions_dev.numel())
-    n_llm, hidden = d_llm_embeds.shape
-    assert d_llm_embeds.dtype == torch.bfloat16 and positions_dev.dtype == torch.int32
-    st = load().mpipe_merge_tokens_bwd(_ptr(d_llm_embeds), d_llm_embeds.stride(0), _ptr(d_enc),
-                                       d_enc.stride(0) if n_enc else hidden, _ptr(positions_dev), n_enc, n_llm,
-                                       hidden, mode, _ptr(status_buf), _stream(stream))
-    _check(st, "mpipe_merge_tokens_bwd")
+    st = _native().merge(d_enc, d_llm_embeds, positions_dev, mode, status_buf, stream, 1)
+    if st:
+        _check(st, "mpipe_merge_tokens_bwd")
 
 
 class PeerRows:

@@ -5,10 +5,13 @@ import glob
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libmpipe_enc.so")
+HOST_SRC = os.path.join(CSRC, "hostpath.cpp")
+HOST_LIB = os.path.join(HERE, "_hostpath.so")
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-std=c++17", "-lineinfo",
@@ -21,19 +24,30 @@ def sources():
 
 
 def _deps():
-    return sources() + glob.glob(os.path.join(CSRC, "*.h")) + glob.glob(os.path.join(CSRC, "*.cuh")) + \
+    return sources() + [HOST_SRC] + glob.glob(os.path.join(CSRC, "*.h")) + glob.glob(os.path.join(CSRC, "*.cuh")) + \
         [os.path.join(HERE, "..", "include", "mpipe_enc.h")]
 
 
 def is_stale() -> bool:
-    if not os.path.exists(LIB):
+    if not os.path.exists(LIB) or not os.path.exists(HOST_LIB):
         return True
-    t = os.path.getmtime(LIB)
+    t = min(os.path.getmtime(LIB), os.path.getmtime(HOST_LIB))
     return any(os.path.getmtime(f) > t for f in _deps())
 
 
+def host_command(out: str):
+    """The Python marshalling module: plain C++ against Python's and torch's headers."""
+    import torch
+    tdir = os.path.dirname(torch.__file__)
+    inc = [sysconfig.get_paths()["include"], os.path.join(tdir, "include"), os.path.join(tdir, "include", "torch", "csrc", "api", "include"),
+           "/usr/local/cuda/include"]
+    return ([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
+             f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}"] + ["-I" + d for d in inc] +
+            [HOST_SRC, "-o", out, "-L" + os.path.join(tdir, "lib"), "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch", "-ltorch_python"])
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
-    """Compile every .cu under csrc/ into one shared library.  Returns its path."""
+    """Compile every .cu under csrc/ into one shared library, and the Python marshalling module.  Returns the library's path."""
     if not force and not is_stale():
         return LIB
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
@@ -47,6 +61,8 @@ def build(force: bool = False, verbose: bool = False) -> str:
             cmd.insert(1, "-Xptxas=-v")
         procs.append((src, subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)))
         objs.append(obj)
+    host_tmp = HOST_LIB + f".{os.getpid()}.tmp"
+    procs.append((HOST_SRC, subprocess.Popen(host_command(host_tmp), stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)))
     failed = False
     for src, p in procs:
         out, _ = p.communicate()
@@ -57,6 +73,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
         raise RuntimeError("nvcc failed")
     tmp = LIB + f".{os.getpid()}.tmp"
     subprocess.run([nvcc] + NVCC_FLAGS + objs + ["-o", tmp], check=True)
+    os.replace(host_tmp, HOST_LIB)
     os.replace(tmp, LIB)
     return LIB
 

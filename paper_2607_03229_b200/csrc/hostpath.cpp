@@ -1,0 +1,341 @@
+// Python -> C ABI marshalling of the calls a training step makes for every microbatch: the segment plan and its upload, attention
+// forward and backward, the merge.  The same checks and the same C entry points as the ctypes route, but read natively from the
+// tensors: a step of a small microbatch is bound by the host (four images, 229 tokens: 125 us of Python around 20 us of kernels,
+// of which reading shapes, strides, types and pointers attribute by attribute, and torch's Python-level current stream, were the
+// larger part).  No state is kept but the addresses of the C functions, which load() hands over once.
+#include <Python.h>
+
+#include <ATen/ATen.h>
+#include <c10/cuda/CUDAStream.h>
+#include <torch/csrc/autograd/python_variable.h>
+
+#include <cstring>
+#include <vector>
+
+#include "../../include/mpipe_enc.h"
+
+namespace {
+
+decltype(&mpipe_seg_plan) f_seg_plan = nullptr;
+decltype(&mpipe_varlen_attn_fwd) f_attn_fwd = nullptr;
+decltype(&mpipe_varlen_attn_bwd) f_attn_bwd = nullptr;
+decltype(&mpipe_merge_tokens) f_merge = nullptr;
+decltype(&mpipe_merge_tokens_bwd) f_merge_bwd = nullptr;
+
+struct Failed {};   // a Python exception is set
+struct WithoutGil {   // around calls that may block in the driver: other Python threads go on, as under ctypes
+    PyThreadState* state = PyEval_SaveThread();
+    ~WithoutGil() { PyEval_RestoreThread(state); }
+};
+
+#define REQUIRE(cond, ...)                              \
+    do {                                                \
+        if (!(cond)) {                                  \
+            PyErr_Format(PyExc_AssertionError, __VA_ARGS__); \
+            throw Failed();                             \
+        }                                               \
+    } while (0)
+
+const at::Tensor& tensor(PyObject* o, const char* what) {
+    REQUIRE(THPVariable_Check(o), "%s must be a tensor", what);
+    return THPVariable_Unpack(o);
+}
+void* data(const at::Tensor& t) { return t.numel() != 0 ? t.data_ptr() : nullptr; }
+// What a pointer argument may be: None, a tensor, an integer address, an object with a `ctypes.data` address (numpy).
+void* pointer(PyObject* o) {
+    if (o == Py_None) return nullptr;
+    if (THPVariable_Check(o)) return data(THPVariable_Unpack(o));
+    PyObject* num = nullptr;
+    if (PyObject* ct = PyObject_HasAttrString(o, "ctypes") ? PyObject_GetAttrString(o, "ctypes") : nullptr) {
+        num = PyObject_GetAttrString(ct, "data");
+        Py_DECREF(ct);
+    } else {
+        num = PyNumber_Long(o);
+    }
+    if (num == nullptr) throw Failed();
+    void* p = PyLong_AsVoidPtr(num);
+    Py_DECREF(num);
+    if (p == nullptr && PyErr_Occurred()) throw Failed();
+    return p;
+}
+void* stream_of(PyObject* o) {
+    if (o == Py_None) return c10::cuda::getCurrentCUDAStream().stream();
+    if (PyObject_HasAttrString(o, "cuda_stream")) {
+        PyObject* s = PyObject_GetAttrString(o, "cuda_stream");
+        if (s == nullptr) throw Failed();
+        void* p = PyLong_AsVoidPtr(s);
+        Py_DECREF(s);
+        if (p == nullptr && PyErr_Occurred()) throw Failed();
+        return p;
+    }
+    return pointer(o);
+}
+long integer(PyObject* o) {
+    const long v = PyLong_AsLong(o);
+    if (v == -1 && PyErr_Occurred()) throw Failed();
+    return v;
+}
+float real(PyObject* o) {
+    const double v = PyFloat_AsDouble(o);
+    if (v == -1.0 && PyErr_Occurred()) throw Failed();
+    return float(v);
+}
+bool is_bf16(const at::Tensor& t) { return t.scalar_type() == at::kBFloat16; }
+bool same_strides(const at::Tensor& a, const at::Tensor& b) { return a.stride(0) == b.stride(0) && a.stride(1) == b.stride(1); }
+void check_thd(const at::Tensor& t) {
+    REQUIRE(t.dim() == 3 && t.stride(2) == 1, "expected [tokens, heads, head_dim] with contiguous head_dim");
+}
+
+// The plan as the wrappers pass it: mode, n_seg, total_tokens, max_seqlen, cu_seqlens_dev, items_dev, n_items.
+struct Plan {
+    int32_t mode, n_seg, total, max_len, n_items;
+    const int32_t* cu = nullptr;
+    const mpipe_work_item_t* items = nullptr;
+};
+Plan plan_of(PyObject* const* a, int64_t T, const char* what, bool used) {
+    Plan p;
+    p.mode = int32_t(integer(a[0]));
+    p.n_seg = int32_t(integer(a[1]));
+    p.total = int32_t(integer(a[2]));
+    p.max_len = int32_t(integer(a[3]));
+    p.n_items = int32_t(integer(a[6]));
+    if (used) {
+        REQUIRE(p.total == T, "%s: plan was made for %d tokens, tensors hold %lld", what, p.total, (long long)T);
+        if (T > 0 && p.n_items > 0) {
+            REQUIRE(a[4] != Py_None && a[5] != Py_None, "%s: plan.to_device() first", what);
+            const at::Tensor& items = tensor(a[5], "items");
+            REQUIRE(items.numel() == 6 * int64_t(p.n_items) && items.scalar_type() == at::kInt, "%s: items do not match the plan", what);
+        }
+    }
+    p.cu = static_cast<const int32_t*>(pointer(a[4]));
+    p.items = static_cast<const mpipe_work_item_t*>(pointer(a[5]));
+    return p;
+}
+
+template <typename F>
+PyObject* guarded(F&& f) {
+    try {
+        return f();
+    } catch (const Failed&) {
+    } catch (const std::exception& e) {
+        PyErr_SetString(PyExc_RuntimeError, e.what());
+    }
+    return nullptr;
+}
+bool count_is(Py_ssize_t n, Py_ssize_t want) {
+    if (n == want) return true;
+    PyErr_Format(PyExc_TypeError, "%zd arguments expected, got %zd", want, n);
+    return false;
+}
+
+PyObject* bind(PyObject*, PyObject* const* a, Py_ssize_t n) {
+    if (!count_is(n, 5)) return nullptr;
+    return guarded([&]() -> PyObject* {
+        f_seg_plan = reinterpret_cast<decltype(f_seg_plan)>(pointer(a[0]));
+        f_attn_fwd = reinterpret_cast<decltype(f_attn_fwd)>(pointer(a[1]));
+        f_attn_bwd = reinterpret_cast<decltype(f_attn_bwd)>(pointer(a[2]));
+        f_merge = reinterpret_cast<decltype(f_merge)>(pointer(a[3]));
+        f_merge_bwd = reinterpret_cast<decltype(f_merge_bwd)>(pointer(a[4]));
+        Py_RETURN_NONE;
+    });
+}
+
+// seg_plan(counts: list of int, mode, fwd_rows, bwd_rows) -> (status, buffer, fwd offset, n_fwd, bwd offset, n_bwd, total, max), offsets in
+// int32 words of the bytearray [cu_seqlens | forward items | backward items], every section on 16 bytes; None when a count is
+// not a plain int of 32 bits.
+PyObject* seg_plan(PyObject*, PyObject* const* a, Py_ssize_t n) {
+    if (!count_is(n, 4)) return nullptr;
+    return guarded([&]() -> PyObject* {
+        REQUIRE(PyList_CheckExact(a[0]), "counts must be a list");
+        const Py_ssize_t n_seg = PyList_GET_SIZE(a[0]);
+        const int32_t mode = int32_t(integer(a[1])), fr = int32_t(integer(a[2])), br = int32_t(integer(a[3]));
+        std::vector<int32_t> counts(static_cast<size_t>(n_seg) + 1);
+        int64_t want_f = 0, want_b = 0;
+        for (Py_ssize_t i = 0; i < n_seg; ++i) {
+            PyObject* o = PyList_GET_ITEM(a[0], i);
+            int overflow = 0;
+            const long v = PyLong_CheckExact(o) ? PyLong_AsLongAndOverflow(o, &overflow) : 0;
+            if (!PyLong_CheckExact(o) || overflow != 0 || v != long(int32_t(v))) Py_RETURN_NONE;
+            counts[size_t(i)] = int32_t(v);
+            if (v > 0 && fr > 0 && br > 0) {
+                want_f += (v + fr - 1) / fr;
+                want_b += (v + br - 1) / br;
+            }
+        }
+        if (mode != MPIPE_ENC_TRAINED) want_b = 0;
+        auto up4 = [](int64_t w) { return (w + 3) / 4 * 4; };
+        const int64_t off_f = up4(n_seg + 1), off_b = off_f + up4(6 * want_f), words = off_b + up4(6 * want_b);
+        if (want_f > 0x7fffffff / 6 || want_b > 0x7fffffff / 6) Py_RETURN_NONE;
+        PyObject* buf = PyByteArray_FromStringAndSize(nullptr, Py_ssize_t(words * 4));
+        if (buf == nullptr) throw Failed();
+        int32_t* w = reinterpret_cast<int32_t*>(PyByteArray_AS_STRING(buf));
+        std::memset(w, 0, size_t(words) * 4);
+        int32_t total = 0, mx = 0, nf = 0, nb = 0;
+        mpipe_work_item_t none;   // a non-null list pointer for empty lists
+        const int32_t st = f_seg_plan(counts.data(), int32_t(n_seg), fr, br, mode, w, &total, &mx,
+                                      want_f > 0 ? reinterpret_cast<mpipe_work_item_t*>(w + off_f) : &none, &nf,
+                                      want_b > 0 ? reinterpret_cast<mpipe_work_item_t*>(w + off_b) : &none, &nb);
+        PyObject* r = Py_BuildValue("(iNLiLiii)", int(st), buf, (long long)off_f, int(nf), (long long)off_b, int(nb), int(total), int(mx));
+        if (r == nullptr) throw Failed();
+        return r;
+    });
+}
+
+// upload(buffer, n_seg + 1, fwd offset, n_fwd, bwd offset, n_bwd, device index or -1) -> (pinned staging, cu, fwd items, bwd items): one
+// asynchronous copy on the current stream.
+PyObject* upload(PyObject*, PyObject* const* a, Py_ssize_t n) {
+    if (!count_is(n, 7)) return nullptr;
+    return guarded([&]() -> PyObject* {
+        REQUIRE(PyByteArray_Check(a[0]), "buffer must be a bytearray");
+        const int64_t words = PyByteArray_GET_SIZE(a[0]) / 4;
+        const int64_t n_cu = integer(a[1]), off_f = integer(a[2]), nf = integer(a[3]), off_b = integer(a[4]), nb = integer(a[5]);
+        REQUIRE(n_cu <= words && off_f + 6 * nf <= words && off_b + 6 * nb <= words, "sections outside the buffer");
+        const long dev = integer(a[6]);
+        const at::TensorOptions ints = at::TensorOptions().dtype(at::kInt);
+        const at::Tensor host = at::empty({words}, ints.pinned_memory(true));
+        std::memcpy(host.data_ptr(), PyByteArray_AS_STRING(a[0]), size_t(words) * 4);
+        at::Tensor d = at::empty({words}, ints.device(at::Device(at::kCUDA, c10::DeviceIndex(dev))));
+        {
+            WithoutGil off;
+            d.copy_(host, /*non_blocking=*/true);
+        }
+        PyObject* r = PyTuple_New(4);
+        if (r == nullptr) throw Failed();
+        PyTuple_SET_ITEM(r, 0, THPVariable_Wrap(host));
+        PyTuple_SET_ITEM(r, 1, THPVariable_Wrap(d.as_strided({n_cu}, {1}, 0)));
+        PyTuple_SET_ITEM(r, 2, THPVariable_Wrap(d.as_strided({nf, 6}, {6, 1}, off_f)));
+        PyTuple_SET_ITEM(r, 3, THPVariable_Wrap(d.as_strided({nb, 6}, {6, 1}, off_b)));
+        return r;
+    });
+}
+
+// attn_fwd(q, k, v, o, lse, <plan: 7>, scale, status, stream) -> status
+PyObject* attn_fwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
+    if (!count_is(n, 15)) return nullptr;
+    return guarded([&]() -> PyObject* {
+        const at::Tensor &q = tensor(a[0], "q"), &k = tensor(a[1], "k"), &v = tensor(a[2], "v"), &o = tensor(a[3], "o");
+        check_thd(q);
+        check_thd(k);
+        check_thd(v);
+        check_thd(o);
+        const int64_t T = q.size(0), H = q.size(1), D = q.size(2);
+        REQUIRE(k.sizes() == q.sizes() && v.sizes() == q.sizes() && o.sizes() == q.sizes(), "q, k, v, o must have one shape");
+        REQUIRE(is_bf16(q) && is_bf16(k) && is_bf16(v) && is_bf16(o), "q, k, v, o must be bf16");
+        REQUIRE(same_strides(q, k) && same_strides(q, v), "q, k, v must share strides");
+        const Plan p = plan_of(a + 5, T, "varlen_attn_fwd", true);
+        float* lse = nullptr;
+        if (a[4] != Py_None) {
+            const at::Tensor& l = tensor(a[4], "lse");
+            REQUIRE(l.scalar_type() == at::kFloat && l.is_contiguous() && l.dim() == 2 && l.size(0) == H && l.size(1) == T,
+                    "lse must be a contiguous fp32 [heads, tokens]");
+            lse = static_cast<float*>(data(l));
+        }
+        const float scale = real(a[12]);
+        int32_t* status = static_cast<int32_t*>(pointer(a[13]));
+        void* stream = stream_of(a[14]);
+        int32_t st;
+        {
+            WithoutGil off;
+            st = f_attn_fwd(data(q), data(k), data(v), data(o), lse, q.stride(0), q.stride(1), o.stride(0), o.stride(1), p.cu, p.n_seg, p.total,
+                            p.max_len, p.items, p.n_items, int32_t(H), int32_t(D), scale, p.mode, status, stream);
+        }
+        return PyLong_FromLong(st);
+    });
+}
+
+// attn_bwd(dout, q, k, v, o, lse, dq, dk, dv, <plan: 7>, scale, workspace, status, stream) -> status
+PyObject* attn_bwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
+    if (!count_is(n, 20)) return nullptr;
+    return guarded([&]() -> PyObject* {
+        static const char* const names[9] = {"dout", "q", "k", "v", "o", "lse", "dq", "dk", "dv"};
+        const at::Tensor& q = tensor(a[1], "q");
+        const at::Tensor& o = tensor(a[4], "o");
+        check_thd(q);
+        check_thd(o);
+        const int64_t T = q.size(0), H = q.size(1), D = q.size(2);
+        const bool trained = integer(a[9]) == MPIPE_ENC_TRAINED;
+        int64_t tsg = q.stride(0), hsg = q.stride(1);
+        if (trained) {
+            for (int i : {0, 2, 3, 4, 6, 7, 8}) {
+                const at::Tensor& t = tensor(a[i], names[i]);
+                REQUIRE(t.sizes() == q.sizes() && is_bf16(t), "varlen_attn_bwd: %s must be bf16 of q's shape", names[i]);
+                check_thd(t);
+            }
+            const at::Tensor& l = tensor(a[5], "lse");
+            REQUIRE(l.scalar_type() == at::kFloat && l.is_contiguous() && l.dim() == 2 && l.size(0) == H && l.size(1) == T,
+                    "lse must be a contiguous fp32 [heads, tokens]");
+            const at::Tensor& dq = tensor(a[6], "dq");
+            REQUIRE(same_strides(q, tensor(a[2], "k")) && same_strides(q, tensor(a[3], "v")), "q, k, v must share strides");
+            REQUIRE(same_strides(o, tensor(a[0], "dout")), "dout must share o's strides");
+            REQUIRE(same_strides(dq, tensor(a[7], "dk")) && same_strides(dq, tensor(a[8], "dv")), "dq, dk, dv must share strides");
+            tsg = dq.stride(0);
+            hsg = dq.stride(1);
+        }
+        const Plan p = plan_of(a + 9, T, "varlen_attn_bwd", trained);
+        size_t ws_bytes = 0;
+        if (a[17] != Py_None) {
+            const at::Tensor& w = tensor(a[17], "workspace");
+            ws_bytes = size_t(w.numel()) * w.element_size();
+        }
+        void* const ptr[9] = {pointer(a[0]), data(q), pointer(a[2]), pointer(a[3]), data(o), pointer(a[5]), pointer(a[6]), pointer(a[7]), pointer(a[8])};
+        const float scale = real(a[16]);
+        void* ws = pointer(a[17]);
+        int32_t* status = static_cast<int32_t*>(pointer(a[18]));
+        void* stream = stream_of(a[19]);
+        int32_t st;
+        {
+            WithoutGil off;
+            st = f_attn_bwd(ptr[0], ptr[1], ptr[2], ptr[3], ptr[4], static_cast<const float*>(ptr[5]), ptr[6], ptr[7], ptr[8], q.stride(0),
+                            q.stride(1), o.stride(0), o.stride(1), tsg, hsg, p.cu, p.n_seg, p.total, p.max_len, p.items, p.n_items, int32_t(H),
+                            int32_t(D), scale, p.mode, ws, ws_bytes, status, stream);
+        }
+        return PyLong_FromLong(st);
+    });
+}
+
+// merge(enc, llm, positions, mode, status, stream, backward) -> status
+PyObject* merge(PyObject*, PyObject* const* a, Py_ssize_t n) {
+    if (!count_is(n, 7)) return nullptr;
+    return guarded([&]() -> PyObject* {
+        const at::Tensor& pos = tensor(a[2], "positions");
+        const at::Tensor& llm = tensor(a[1], "llm_embeds");
+        const int64_t n_enc = pos.numel();
+        const bool backward = integer(a[6]) != 0;
+        REQUIRE(llm.dim() == 2 && is_bf16(llm) && pos.scalar_type() == at::kInt, "llm_embeds must be a bf16 matrix, positions int32");
+        const int64_t hidden = llm.size(1);
+        const bool has_enc = a[0] != Py_None;   // (the frozen backward touches nothing and needs no output)
+        REQUIRE(has_enc || n_enc == 0 || backward, "encoder rows missing");
+        int64_t ld = hidden;
+        if (has_enc) {
+            const at::Tensor& enc = tensor(a[0], "enc_tokens");
+            if (!backward) {
+                REQUIRE(is_bf16(enc) && enc.dim() >= 1 && enc.size(0) == n_enc && (n_enc == 0 || (enc.dim() == 2 && enc.size(1) == hidden)),
+                        "enc_tokens must be bf16 with a row of llm_embeds' width for every position");
+                REQUIRE(llm.stride(1) == 1 && (n_enc == 0 || enc.stride(1) == 1), "rows must be contiguous");
+            }
+            if (n_enc != 0) ld = enc.stride(0);
+        }
+        void* enc_ptr = pointer(a[0]);
+        const int32_t mode = int32_t(integer(a[3]));
+        int32_t* status = static_cast<int32_t*>(pointer(a[4]));
+        void* stream = stream_of(a[5]);
+        const int32_t* positions = static_cast<const int32_t*>(data(pos));
+        int32_t st;
+        {
+            WithoutGil off;
+            st = backward ? f_merge_bwd(data(llm), llm.stride(0), enc_ptr, ld, positions, int32_t(n_enc), int32_t(llm.size(0)), int32_t(hidden),
+                                        mode, status, stream)
+                          : f_merge(enc_ptr, ld, data(llm), llm.stride(0), positions, int32_t(n_enc), int32_t(llm.size(0)), int32_t(hidden), mode,
+                                    status, stream);
+        }
+        return PyLong_FromLong(st);
+    });
+}
+
+#define FAST(name) {#name, reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(name)), METH_FASTCALL, nullptr}
+PyMethodDef methods[] = {FAST(bind), FAST(seg_plan), FAST(upload), FAST(attn_fwd), FAST(attn_bwd), FAST(merge), {nullptr, nullptr, 0, nullptr}};
+PyModuleDef module = {PyModuleDef_HEAD_INIT, "_hostpath", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
+
+}  // namespace
+
+PyMODINIT_FUNC PyInit__hostpath(void) { return PyModule_Create(&module); }

@@ -1,0 +1,49 @@
+"""The native marshalling of the per-microbatch calls: every accepted form of the patch counts gives the same plan, and what does
+not fit together is refused before anything is called."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2607_03229_b200 import binding as B
+from paper_2607_03229_b200 import build as build_mod
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    build_mod.build()
+
+
+@pytest.mark.parametrize("counts", [[], [0], [1], [300, 0, 17, 256]])
+@pytest.mark.parametrize("mode", [B.FROZEN, B.TRAINED])
+def test_every_form_of_counts_gives_one_plan(counts, mode):
+    plans = [B.seg_plan(c, mode) for c in (counts, tuple(counts), np.array(counts, dtype=np.int64), [np.int32(c) for c in counts])]
+    for p in plans:
+        assert p.cu_seqlens.dtype == np.int32 and p.fwd_items.dtype == B.ITEM_DTYPE and p.n_seg == len(counts)
+        for name in ("cu_seqlens", "fwd_items", "bwd_items"):
+            assert np.array_equal(getattr(p, name), getattr(plans[0], name)) and getattr(p, name).flags.writeable
+    p = plans[0].to_device("cpu")
+    assert p.cu_seqlens_dev.tolist() == plans[1].cu_seqlens.tolist() and p.fwd_items_dev.shape == (plans[1].fwd_items.size, 6)
+
+
+def test_counts_beyond_32_bits_are_refused():
+    with pytest.raises(OverflowError):
+        B.seg_plan([1 << 40], B.TRAINED)
+    with pytest.raises(B.MpipeError):
+        B.seg_plan([(1 << 31) - 1, 1], B.TRAINED)
+
+
+def test_mismatched_tensors_are_refused():
+    T, H, D = 40, 2, 64
+    t = lambda *s, dt=torch.bfloat16: torch.zeros(s, dtype=dt)
+    plan = B.seg_plan([T], B.TRAINED)
+    ok = dict(q=t(T, H, D), k=t(T, H, D), v=t(T, H, D), o=t(T, H, D), lse=t(H, T, dt=torch.float32))
+    for name, bad in (("k", t(T, H, D + 16)), ("v", t(T, H, D, dt=torch.float16)), ("o", t(T + 1, H, D)), ("lse", t(T, H, dt=torch.float32)),
+                      ("k", t(H, T, D).transpose(0, 1))):
+        with pytest.raises(AssertionError):
+            B.varlen_attn_fwd(plan=plan, softmax_scale=0.125, **dict(ok, **{name: bad}))
+    with pytest.raises(AssertionError):      # the plan has not been uploaded
+        B.varlen_attn_fwd(plan=plan, softmax_scale=0.125, **ok)
+    with pytest.raises(AssertionError):      # the plan is for other tensors
+        B.varlen_attn_fwd(plan=B.seg_plan([T + 1], B.TRAINED), softmax_scale=0.125, **ok)
+    with pytest.raises(AssertionError):
+        B.merge_tokens(t(T, 64), t(100, 128), torch.zeros(T, dtype=torch.int32))
