@@ -473,7 +473,7 @@ int32_t mpipe_encoder_layer_fwd(const void* x, void* y, const mpipe_layer_weight
     uint8_t* ubuf = ws;
     int32_t rc;
     if ((rc = mpipe_layernorm_fwd(x, w->ln1_gamma, w->ln1_beta, norm, n_tokens, hidden, hidden, hidden, ln_eps, stream)) != MPIPE_OK) return rc;
-    if ((rc = mpipe_linear_fwd(norm, w->w_qkv, w->b_qkv, nullptr, qkv, n_tokens, 3 * hidden, hidden, hidden, hidden, 0,
+    if ((rc = linear_fwd_in_layer(norm, w->w_qkv, w->b_qkv, nullptr, qkv, n_tokens, 3 * hidden, hidden, hidden, hidden, 0,
                                3 * int64_t(hidden), 0, status_buf, stream)) != MPIPE_OK) return rc;
     if ((rope_cos == nullptr) != (rope_sin == nullptr)) return MPIPE_ERR_INVALID_ARG;
     if (rope_cos != nullptr &&
@@ -485,17 +485,17 @@ int32_t mpipe_encoder_layer_fwd(const void* x, void* y, const mpipe_layer_weight
     if ((rc = varlen_attn_fwd(q, k, v, attn, lse, 3 * int64_t(hidden), head_dim, hidden, head_dim, cu_seqlens_dev, n_seg,
                               n_tokens, max_seqlen, fwd_items_dev, n_fwd_items, n_heads, head_dim, softmax_scale, mode,
                               status_buf, stream, true)) != MPIPE_OK) return rc;
-    if ((rc = mpipe_linear_fwd(attn, w->w_o, w->b_o, x, x1, n_tokens, hidden, hidden, hidden, hidden, hidden, hidden, 0,
+    if ((rc = linear_fwd_in_layer(attn, w->w_o, w->b_o, x, x1, n_tokens, hidden, hidden, hidden, hidden, hidden, hidden, 0,
                                status_buf, stream)) != MPIPE_OK) return rc;
     if ((rc = mpipe_layernorm_fwd(x1, w->ln2_gamma, w->ln2_beta, norm, n_tokens, hidden, hidden, hidden, ln_eps, stream)) != MPIPE_OK) return rc;
     if (mode == MPIPE_ENC_TRAINED) {   // the backward needs the pre-activation: the same launch stores it beside GELU(u)
         if ((rc = linear_fwd_gelu_keep_preact(norm, w->w_fc1, w->b_fc1, fc1, ubuf, n_tokens, ffn, hidden, hidden, hidden, ffn, ffn,
                                               status_buf, stream)) != MPIPE_OK) return rc;
-    } else if ((rc = mpipe_linear_fwd(norm, w->w_fc1, w->b_fc1, nullptr, fc1, n_tokens, ffn, hidden, hidden, hidden, 0, ffn,
+    } else if ((rc = linear_fwd_in_layer(norm, w->w_fc1, w->b_fc1, nullptr, fc1, n_tokens, ffn, hidden, hidden, hidden, 0, ffn,
                                       MPIPE_LINEAR_GELU, status_buf, stream)) != MPIPE_OK) {
         return rc;
     }
-    return mpipe_linear_fwd(fc1, w->w_fc2, w->b_fc2, x1, y, n_tokens, hidden, ffn, ffn, ffn, hidden, hidden, 0, status_buf, stream);
+    return linear_fwd_in_layer(fc1, w->w_fc2, w->b_fc2, x1, y, n_tokens, hidden, ffn, ffn, ffn, hidden, hidden, 0, status_buf, stream);
 }
 
 size_t mpipe_encoder_layer_bwd_workspace_bytes(int32_t n_tokens, int32_t hidden, int32_t n_heads, int32_t ffn) {
@@ -546,20 +546,20 @@ int32_t mpipe_encoder_layer_bwd(const void* dy, const void* x, void* dx, const m
 #define MPIPE_TRY(call) do { if ((rc = (call)) != MPIPE_OK) return rc; } while (0)
     // ---- MLP branch: y = x1 + GELU(m W1^T + b1) W2^T + b2, m = LN2(x1) (still in the forward's LN slot)
     MPIPE_TRY(linear_wgrad_bias(dy, act, g->w_fc2, g->b_fc2, n_tokens, hidden, ffn, h, f, f, status_buf, stream));                 // dW2 += dy^T GELU(u), db2
-    MPIPE_TRY(mpipe_linear_dgrad(dy, w->w_fc2, ubuf, nullptr, dubuf, n_tokens, hidden, ffn, h, f, f, 0, f, status_buf, stream));    // du = (dy W2) o GELU'(u)
+    MPIPE_TRY(linear_dgrad_in_layer(dy, w->w_fc2, ubuf, dubuf, n_tokens, hidden, ffn, h, f, f, f, status_buf, stream));    // du = (dy W2) o GELU'(u)
     MPIPE_TRY(linear_wgrad_bias(dubuf, norm, g->w_fc1, g->b_fc1, n_tokens, ffn, hidden, f, h, h, status_buf, stream));            // dW1 += du^T m, db1
-    MPIPE_TRY(mpipe_linear_dgrad(dubuf, w->w_fc1, nullptr, nullptr, tmp, n_tokens, ffn, hidden, f, h, 0, 0, h, status_buf, stream)); // dm = du W1
+    MPIPE_TRY(linear_dgrad_in_layer(dubuf, w->w_fc1, nullptr, tmp, n_tokens, ffn, hidden, f, h, 0, h, status_buf, stream)); // dm = du W1
     MPIPE_TRY(mpipe_layernorm_bwd(x1, tmp, w->ln2_gamma, dy, dx1, g->ln2_gamma, g->ln2_beta, n_tokens, hidden, h, h, h, h, ln_eps, stream)); // dx1 = dy + LN2'(dm)
     // ---- attention branch: x1 = x + o Wo^T + bo, o = attention(rope(a Wqkv^T + bqkv)), a = LN1(x)
     MPIPE_TRY(linear_wgrad_bias(dx1, attn, g->w_o, g->b_o, n_tokens, hidden, hidden, h, h, h, status_buf, stream));                // dWo += dx1^T o, dbo
-    MPIPE_TRY(mpipe_linear_dgrad(dx1, w->w_o, nullptr, nullptr, tmp, n_tokens, hidden, hidden, h, h, 0, 0, h, status_buf, stream)); // do = dx1 Wo
+    MPIPE_TRY(linear_dgrad_in_layer(dx1, w->w_o, nullptr, tmp, n_tokens, hidden, hidden, h, h, 0, h, status_buf, stream)); // do = dx1 Wo
     MPIPE_TRY(varlen_attn_bwd_rope(tmp, qkv, qkv + size_t(hidden) * 2, qkv + size_t(hidden) * 4, attn, lse, dqkv, dqkv + size_t(hidden) * 2,
                                    dqkv + size_t(hidden) * 4, h3, head_dim, h, head_dim, h3, head_dim, cu_seqlens_dev, n_seg, n_tokens,
                                    max_seqlen, bwd_items_dev, n_bwd_items, n_heads, head_dim, softmax_scale, rope_cos, rope_sin, attn_ws,
                                    attn_ws_bytes, status_buf, stream));
     MPIPE_TRY(mpipe_layernorm_fwd(x, w->ln1_gamma, w->ln1_beta, tmp, n_tokens, hidden, h, h, ln_eps, stream));                     // a (recomputed)
     MPIPE_TRY(linear_wgrad_bias(dqkv, tmp, g->w_qkv, g->b_qkv, n_tokens, 3 * hidden, hidden, h3, h, h, status_buf, stream));       // dWqkv += dqkv^T a, dbqkv
-    MPIPE_TRY(mpipe_linear_dgrad(dqkv, w->w_qkv, nullptr, nullptr, tmp, n_tokens, 3 * hidden, hidden, h3, h, 0, 0, h, status_buf, stream)); // da = dqkv Wqkv
+    MPIPE_TRY(linear_dgrad_in_layer(dqkv, w->w_qkv, nullptr, tmp, n_tokens, 3 * hidden, hidden, h3, h, 0, h, status_buf, stream)); // da = dqkv Wqkv
     MPIPE_TRY(mpipe_layernorm_bwd(x, tmp, w->ln1_gamma, dx1, dx, g->ln1_gamma, g->ln1_beta, n_tokens, hidden, h, h, h, h, ln_eps, stream)); // dx = dx1 + LN1'(da)
 #undef MPIPE_TRY
     return MPIPE_OK;

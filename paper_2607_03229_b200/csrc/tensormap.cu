@@ -38,4 +38,16 @@ bool make_tensor_map_thd(CUtensorMap* out, const void* base, int64_t T, int64_t 
     return r == CUDA_SUCCESS;
 }
 
+bool make_tensor_map_chunks(CUtensorMap* out, const void* base, int64_t rows, int64_t chunks, int64_t ld, uint32_t box_rows,
+                            uint32_t box_chunks) {
+    EncodeTiledFn fn = encode_fn();
+    if (fn == nullptr) return false;
+    const cuuint64_t dims[3] = {64, cuuint64_t(rows), cuuint64_t(chunks)};
+    const cuuint64_t strides[2] = {cuuint64_t(ld) * 2, 128};
+    const cuuint32_t box[3] = {64, box_rows, box_chunks}, elem_strides[3] = {1, 1, 1};
+    return fn(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, elem_strides,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 }  // namespace mpipe

@@ -16,4 +16,10 @@ bool make_tensor_map_thd(CUtensorMap* out, const void* base, int64_t T, int64_t 
                          int64_t head_stride, uint32_t box_d, uint32_t box_rows, int swizzle_bytes,
                          int elem_bytes = 2);
 
+// View a bf16 matrix [rows, 64 * chunks] (row stride ld elements) as the 3-D tensor (64, rows, chunks) and describe boxes of
+// 64 x box_rows x box_chunks elements, 128-byte swizzle: one copy brings several 64-element atoms, each [box_rows][128 bytes],
+// one behind the other.  The matrix must have exactly 64 * chunks columns: inside a chunk nothing is out of range.
+bool make_tensor_map_chunks(CUtensorMap* out, const void* base, int64_t rows, int64_t chunks, int64_t ld, uint32_t box_rows,
+                            uint32_t box_chunks);
+
 }  // namespace mpipe

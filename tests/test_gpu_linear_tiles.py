@@ -27,6 +27,7 @@ def _close(got, ref):
                                    (777, 4096, 1024),   # width 256
                                    (300, 520, 2048),    # contraction split over two pairs, ragged last chunk
                                    (777, 1024, 4096),   # the same, four row tiles
+                                   (90, 320, 192), (90, 320, 200),   # two blocks of the contraction per stage, an odd number of them; whole atoms or not
                                    (4000, 1288, 136)])  # several tiles per pair
 def test_linear_and_dgrad_tile_choices(M, N, K):
     a, w = W.normal_bf16(51, 0, (M, K)), W.scaled_normal_bf16(51, 1, (N, K), std=K ** -0.5)
