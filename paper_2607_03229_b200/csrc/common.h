@@ -62,16 +62,23 @@ int32_t linear_fwd_gelu_keep_preact(const void* a, const void* w, const void* bi
                                     int32_t K, int64_t lda, int64_t ldw, int64_t ldact, int64_t ldpre, int32_t* status_buf,
                                     void* stream);
 
+// Up to two matrices that a projection brings into L2 for the kernels behind it.
+struct LayerAhead {
+    const void* ptr[2] = {nullptr, nullptr};
+    uint32_t bytes[2] = {0, 0};
+};
+
 // Defined in gemm.cu, used by the layer: mpipe_linear_fwd / mpipe_linear_dgrad whose weights were complete before the previous kernel
 // of the stream started (true behind any other kernel of the layer): they are loaded while that kernel still runs.
 int32_t linear_fwd_in_layer(const void* a, const void* w, const void* bias, const void* residual, void* c, int32_t M, int32_t N, int32_t K,
-                            int64_t lda, int64_t ldw, int64_t ldr, int64_t ldc, int32_t flags, int32_t* status_buf, void* stream);
+                            int64_t lda, int64_t ldw, int64_t ldr, int64_t ldc, int32_t flags, int32_t* status_buf, void* stream,
+                            const LayerAhead& ahead);
 int32_t linear_dgrad_in_layer(const void* dy, const void* w, const void* gelu_input, void* dx, int32_t M, int32_t N, int32_t K, int64_t lddy,
                               int64_t ldw, int64_t ldu, int64_t lddx, int32_t* status_buf, void* stream);
 
 // Defined in gemm.cu, used by the layer backward: mpipe_linear_wgrad that also adds the column sums of dy to db (fp32 [N]).
 int32_t linear_wgrad_bias(const void* dy, const void* x, float* dw, float* db, int32_t n_tokens, int32_t N, int32_t K, int64_t lddy,
-                          int64_t ldx, int64_t lddw, int32_t* status_buf, void* stream);
+                          int64_t ldx, int64_t lddw, int32_t* status_buf, void* stream, const LayerAhead& ahead);
 
 // Defined in attn_bwd.cu, used by the layer backward: mpipe_varlen_attn_bwd whose dQ and dK leave turned back by the rotary tables
 // (both NULL: as they are).

@@ -69,6 +69,8 @@ struct GemmParams {
     int64_t ldr;
     int32_t side;                    // the side operand of map_s: residual (plain, GELU) or pre-activation (GELU gradient)
     int32_t store_pre;               // GELU only: also store the pre-activation (bf16) through map_u
+    const void* ahead[2];            // matrices that the next kernels of the layer read: brought into L2 meanwhile, or null
+    uint32_t ahead_bytes[2];
     float* colsum;                   // weight gradient: [M] or null, the column sums of the first operand are added to it
     int32_t* status_buf;
 };
@@ -128,6 +130,16 @@ linear_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
     cluster_sync_all();                                       // the peer's barriers exist before anything arrives on them
     tc_fence_after();
     const uint32_t tmem = tmem_base_slot;
+    if (kMode != 1 && warp == 2) {   // every CTA a slice, a lane 4 KB at a time
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            constexpr uint32_t kPiece = 4096;
+            const uint8_t* src = static_cast<const uint8_t*>(p.ahead[i]);
+            const uint32_t bytes = src != nullptr ? p.ahead_bytes[i] : 0u;
+            for (uint32_t off = (blockIdx.x * 32u + lane) * kPiece; off < bytes; off += gridDim.x * 32u * kPiece)
+                prefetch_l2_bulk(src + off, min(kPiece, bytes - off));
+        }
+    }
     if (!(warp == 3 && p.settled_w)) pdl_wait();   // weights inside a layer are loaded while the kernel before still runs
     if (warp == 0) pdl_launch();
     const int kpb = kMode == 2 ? 1 : p.kpb, nk = (p.K + kpb * kGemmBK - 1) / (kpb * kGemmBK);   // stages of the whole contraction
@@ -565,6 +577,7 @@ struct LinearCall {   // one forward projection or input gradient
     int32_t gelu;
     int32_t* status_buf;
     bool settled_w;      // see GemmParams
+    LayerAhead ahead;    // see GemmParams
 };
 
 template <int kMode, int kEpi>
@@ -581,6 +594,10 @@ static int32_t launch_linear_as(const LinearCall& x, cudaStream_t st) {
     p.wide = wide ? 1 : 0;
     p.kpb = wide && p.bn <= 128 ? 2 : 1;
     p.settled_w = x.settled_w ? 1 : 0;
+    for (int i = 0; i < 2; ++i) {
+        p.ahead[i] = x.ahead.ptr[i];
+        p.ahead_bytes[i] = x.ahead.bytes[i];
+    }
     p.stages = gemm_stages(p.bn, p.kpb);
     p.splits = shape.splits;
     p.tiles_m = cdiv(x.M, 2 * kGemmBM);
@@ -644,7 +661,7 @@ static int32_t launch_linear(int b_mode, const LinearCall& x, void* stream) {
 
 // dW[n_rows, n_cols] (fp32) += dY[tokens, n_rows]^T X[tokens, n_cols]; with db also db[n_rows] += column sums of dY
 static int32_t launch_wgrad(const void* dy, const void* x, float* dw, float* db, int32_t tokens, int32_t n_rows, int32_t n_cols, int64_t lddy,
-                            int64_t ldx, int64_t lddw, int32_t* status_buf, void* stream) {
+                            int64_t ldx, int64_t lddw, int32_t* status_buf, void* stream, const LayerAhead& ahead) {
     if (tokens < 0 || n_rows <= 0 || n_cols <= 0) return MPIPE_ERR_INVALID_ARG;
     if (tokens == 0) return MPIPE_OK;
     if (dy == nullptr || x == nullptr || dw == nullptr || lddy < n_rows || ldx < n_cols || lddw < n_cols) return MPIPE_ERR_INVALID_ARG;
@@ -691,6 +708,10 @@ static int32_t launch_wgrad(const void* dy, const void* x, float* dw, float* db,
     p.tiles_m = cdiv(n_rows, 2 * kGemmBM);
     p.tiles_n = cdiv(n_cols, p.bn);
     p.colsum = db;
+    for (int i = 0; i < 2; ++i) {
+        p.ahead[i] = ahead.ptr[i];
+        p.ahead_bytes[i] = ahead.bytes[i];
+    }
     p.status_buf = status_buf;
     const long long items = (long long)p.tiles_m * p.tiles_n * p.splits;
     const int clusters = int(items < pairs ? items : pairs);
@@ -699,8 +720,8 @@ static int32_t launch_wgrad(const void* dy, const void* x, float* dw, float* db,
 
 // Weight and bias gradient of a projection in one launch.
 int32_t linear_wgrad_bias(const void* dy, const void* x, float* dw, float* db, int32_t n_tokens, int32_t N, int32_t K, int64_t lddy,
-                          int64_t ldx, int64_t lddw, int32_t* status_buf, void* stream) {
-    return launch_wgrad(dy, x, dw, db, n_tokens, N, K, lddy, ldx, lddw, status_buf, stream);
+                          int64_t ldx, int64_t lddw, int32_t* status_buf, void* stream, const LayerAhead& ahead) {
+    return launch_wgrad(dy, x, dw, db, n_tokens, N, K, lddy, ldx, lddw, status_buf, stream, ahead);
 }
 
 // fc1 of a TRAINED layer forward: act = GELU(a W^T + bias) and pre = a W^T + bias from ONE accumulator, so that the
@@ -714,9 +735,10 @@ int32_t linear_fwd_gelu_keep_preact(const void* a, const void* w, const void* bi
 
 // mpipe_linear_fwd / mpipe_linear_dgrad inside a layer, where the weights are older than the kernel before.
 int32_t linear_fwd_in_layer(const void* a, const void* w, const void* bias, const void* residual, void* c, int32_t M, int32_t N, int32_t K,
-                            int64_t lda, int64_t ldw, int64_t ldr, int64_t ldc, int32_t flags, int32_t* status_buf, void* stream) {
+                            int64_t lda, int64_t ldw, int64_t ldr, int64_t ldc, int32_t flags, int32_t* status_buf, void* stream,
+                            const LayerAhead& ahead) {
     const LinearCall x = {a, w, bias, residual, nullptr, c, nullptr, M, N, K, lda, ldw, ldr, 0, ldc, 0,
-                          (flags & MPIPE_LINEAR_GELU) ? 1 : 0, status_buf, true};
+                          (flags & MPIPE_LINEAR_GELU) ? 1 : 0, status_buf, true, ahead};
     return launch_linear(0, x, stream);
 }
 int32_t linear_dgrad_in_layer(const void* dy, const void* w, const void* gelu_input, void* dx, int32_t M, int32_t N, int32_t K, int64_t lddy,
@@ -731,7 +753,7 @@ extern "C" {
 
 int32_t mpipe_linear_wgrad(const void* dy, const void* x, float* dw, int32_t n_tokens, int32_t N, int32_t K, int64_t lddy,
                            int64_t ldx, int64_t lddw, int32_t* status_buf, void* stream) {
-    return mpipe::launch_wgrad(dy, x, dw, nullptr, n_tokens, N, K, lddy, ldx, lddw, status_buf, stream);
+    return mpipe::launch_wgrad(dy, x, dw, nullptr, n_tokens, N, K, lddy, ldx, lddw, status_buf, stream, mpipe::LayerAhead());
 }
 
 int32_t mpipe_linear_fwd(const void* a, const void* w, const void* bias, const void* residual, void* c, int32_t M,
