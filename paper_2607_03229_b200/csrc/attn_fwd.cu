@@ -1,7 +1,8 @@
 // mpipe_varlen_attn_fwd: block-diagonal (per-image) softmax attention over a packed token sequence,
 // the attention of the relocated Fwd(enc, r, m) event (Section 4.2).
 //
-// One persistent CTA per SM walks the (work item x head) list.  A work item is up to 256 query rows of
+// Persistent CTAs, one per SM, take (work item, head) units from the longest-first list as they get free (units.cuh; mix of eight
+// 819-token images 47.6 -> 44.8 us, ViT-L microbatch 523 -> 513 against a fixed assignment).  A work item is up to 256 query rows of
 // one segment = two 128-row query tiles that share every K/V tile.  Warp roles:
 //   warp 0      TMA producer: Q tiles once per unit, K and V tiles through a kStages-deep ring
 //   warp 1      tcgen05 issuer: S_w = Q_w K^T into TMEM, O_w += P_w V with P_w read from TMEM
@@ -21,6 +22,7 @@
 #include "common.h"
 #include "sm100_ptx.cuh"
 #include "tensormap.h"
+#include "units.cuh"
 
 namespace mpipe {
 
@@ -88,6 +90,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     __shared__ FwdBarriers bars;
+    __shared__ UnitRing units;
     __shared__ uint32_t tmem_base_slot;
     __shared__ int abort_flag;
 
@@ -97,6 +100,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
 
     if (tid == 0) {
         abort_flag = 0;
+        unit_ring_init(&units, 9);   // the issuer and the softmax warps read it
         mbar_init(&bars.q_full, 1);
         mbar_init(&bars.q_empty, 1);
         for (int s = 0; s < 4; ++s) {
@@ -136,26 +140,21 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
     const int n_units = plan_ok_cta(p.items, p.n_items, 2 * kTileM, p.total_tokens, p.status_buf, &plan_flag) ? p.n_items * p.n_heads * (kSplit ? 2 : 1) : 0;
     if (p.settled) pdl_wait();
     pdl_launch();
-    // Units are sorted by decreasing cost; CTAs walk them in boustrophedon order (0..G-1, then G-1..0, ...) so
-    // that the CTA that got the most expensive unit of one round gets the cheapest of the next.
-    auto unit_of = [&](int round) {
-        const int g = int(gridDim.x), i = int(blockIdx.x);
-        return round * g + ((round & 1) ? g - 1 - i : i);
-    };
+    // Unit -> work item with the head in its `seg` field.  kSplit: the second half of an item with one query tile comes back
+    // without rows; every role passes over it.
     auto item_at = [&](int u) {
         mpipe_work_item_t z = {0, 0, 0, 0, 0, 0};
-        if constexpr (kSplit) {   // the second half of an item with one query tile comes back without rows: every role passes over it
-            if (u < n_units) {
-                z = p.items[u / (2 * p.n_heads)];
-                const int off = (u % 2) * kTileM;
-                z.row_start += off;
-                z.row_len = min(z.row_len - off, kTileM);
-            }
-            return z;
+        if (u < 0 || u >= n_units) return z;
+        const int v = kSplit ? u / 2 : u;
+        z = p.items[v / p.n_heads];
+        z.seg = v % p.n_heads;
+        if (kSplit) {
+            const int off = (u % 2) * kTileM;
+            z.row_start += off;
+            z.row_len = min(z.row_len - off, kTileM);
         }
-        return (u < n_units) ? p.items[u / p.n_heads] : z;
+        return z;
     };
-    auto head_of = [&](int u) { return kSplit ? (u / 2) % p.n_heads : u % p.n_heads; };
 
     if (warp == 0) {
         setmaxnreg_dec<kFwdRegsLight>();
@@ -163,12 +162,21 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
         if (lane == 0) {
             uint32_t kv_it = 0, unit_it = 0;
             bool ok = true;
-            mpipe_work_item_t it_next = item_at(unit_of(0));   // one unit ahead: the global load is off the unit's critical path
-            for (int ur = 0, u = unit_of(0); u < n_units && ok; ++ur, u = unit_of(ur), ++unit_it) {
-                const mpipe_work_item_t it = it_next;
-                it_next = item_at(unit_of(ur + 1));
-                if (kSplit && it.row_len <= 0) { --unit_it; continue; }
-                const int head = head_of(u);
+            UnitSource source{&units, &abort_flag};
+            bool outstanding = false;
+            for (int u = int(blockIdx.x); ok; ++unit_it) {
+                const mpipe_work_item_t it = item_at(u);
+                ok = source.put(it);
+                if (!ok || it.kv_len <= 0) break;
+                source.ask();
+                outstanding = true;
+                if (kSplit && it.row_len <= 0) {
+                    u = source.take(&ok);
+                    outstanding = false;
+                    --unit_it;
+                    continue;
+                }
+                const int head = it.seg;
                 const bool two = it.row_len > kTileM;
                 const int nkv = (it.kv_len + kTileN - 1) / kTileN;
                 ok = mbar_wait(&bars.q_empty, (unit_it & 1) ^ 1, &abort_flag);
@@ -196,7 +204,11 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
                     tma_load_3d(vdst, &map_v, &bars.v_full[s], 0, head, row);
                     if (Cfg::kTail) tma_load_3d(vdst + kTileN * 128, &map_v, &bars.v_full[s], 64, head, row);
                 }
+                if (!ok) break;
+                u = source.take(&ok);
+                outstanding = false;
             }
+            if (!ok) source.cancel_rest(outstanding);
         }
         __syncwarp();
     } else if (warp == 1) {
@@ -244,10 +256,8 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
                     }
                 }
             };
-            mpipe_work_item_t it_next = item_at(unit_of(0));   // one unit ahead: the global load is off the unit's critical path
-            for (int ur = 0, u = unit_of(0); u < n_units && ok; ++ur, u = unit_of(ur), ++unit_it) {
-                const mpipe_work_item_t it = it_next;
-                it_next = item_at(unit_of(ur + 1));
+            mpipe_work_item_t it;
+            for (uint32_t ui = 0; ok && next_unit(&units, ui, &it, lane, &abort_flag); ++ui, ++unit_it) {
                 if (kSplit && it.row_len <= 0) { --unit_it; continue; }
                 const bool two = it.row_len > kTileM;
                 const int nkv = (it.kv_len + kTileN - 1) / kTileN;
@@ -385,11 +395,9 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
         const uint32_t t_p = tmem + lane_base + Cfg::kColP0 + w * Cfg::kColPStride;   // = t_s when P overlays S
         uint32_t cnt = 0, ocnt = 0;
         bool ok = true;
-        mpipe_work_item_t it_next = item_at(unit_of(0));   // one unit ahead: the global load is off the unit's critical path
-        for (int ur = 0, u = unit_of(0); u < n_units && ok; ++ur, u = unit_of(ur)) {
-            const mpipe_work_item_t it = it_next;
-            it_next = item_at(unit_of(ur + 1));
-            const int head = head_of(u);
+        mpipe_work_item_t it;
+        for (uint32_t ui = 0; ok && next_unit(&units, ui, &it, lane, &abort_flag); ++ui) {
+            const int head = it.seg;
             const int rows_here = it.row_len - w * kTileM;  // valid rows of this tile
             if (rows_here <= 0) continue;
             const int nkv = (it.kv_len + kTileN - 1) / kTileN;
@@ -539,9 +547,8 @@ static int32_t launch_fwd(const void* q, const void* k, const void* v, int64_t t
     }
     if (!ensure_dynamic_smem<attn_fwd_kernel<D, kSplit>>(Cfg::kSmemAlloc)) return MPIPE_ERR_CUDA;
     const int n_units = prm.n_items * prm.n_heads * (kSplit ? 2 : 1);
-    const int grid = n_units < sm_count() ? n_units : sm_count();
     profile_start(kProfileFwd, stream);
-    const cudaError_t e = launch_kernel(attn_fwd_kernel<D, kSplit>, unsigned(grid), kFwdThreads, Cfg::kSmemAlloc, stream, 1, mq, mk, mv, mqt, mkt, prm);
+    const cudaError_t e = launch_kernel_as(true, attn_fwd_kernel<D, kSplit>, unsigned(n_units), kFwdThreads, Cfg::kSmemAlloc, stream, 1, mq, mk, mv, mqt, mkt, prm);
     profile_stop(kProfileFwd, stream);
     return e == cudaSuccess && cudaGetLastError() == cudaSuccess ? MPIPE_OK : MPIPE_ERR_CUDA;
 }

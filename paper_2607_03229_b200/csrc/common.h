@@ -39,8 +39,8 @@ inline bool ensure_dynamic_smem(int bytes) {
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_kernel(void (*kernel)(KArgs...), unsigned grid, unsigned block, size_t smem, cudaStream_t st,
-                                 unsigned cluster, Args... args) {
+inline cudaError_t launch_kernel_as(bool early, void (*kernel)(KArgs...), unsigned grid, unsigned block, size_t smem, cudaStream_t st,
+                                    unsigned cluster, Args... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(block);
@@ -48,13 +48,18 @@ inline cudaError_t launch_kernel(void (*kernel)(KArgs...), unsigned grid, unsign
     cfg.stream = st;
     cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = grid <= unsigned(8 * sm_count()) ? 1 : 0;
+    at[0].val.programmaticStreamSerializationAllowed = early ? 1 : 0;
     at[1].id = cudaLaunchAttributeClusterDimension;
     at[1].val.clusterDim.x = cluster;
     at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = cluster > 1 ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_kernel(void (*kernel)(KArgs...), unsigned grid, unsigned block, size_t smem, cudaStream_t st,
+                                 unsigned cluster, Args... args) {
+    return launch_kernel_as(grid <= unsigned(8 * sm_count()), kernel, grid, block, smem, st, cluster, args...);
 }
 
 // Defined in gemm.cu, used by the layer forward: one projection that stores both GELU(u) and u.
