@@ -3,7 +3,7 @@
 //
 // Three launches on the caller's stream:
 //   1. prepass   Delta[h,t] = sum_d dO[t,h,d] O[t,h,d]  and the fp32 dQ accumulator is cleared
-//   2. main      one persistent CTA per SM walks (key tile x head) units; a unit keeps one 128-key
+//   2. main      persistent CTAs, one per SM, take (key tile, head) units as they get free (units.cuh); a unit keeps one 128-key
 //                K/V tile resident and steps through the 128-row query tiles of the same segment
 //   3. convert   dQ = softmax_scale * accumulator -> bf16
 //
@@ -38,6 +38,7 @@
 #include "common.h"
 #include "sm100_ptx.cuh"
 #include "tensormap.h"
+#include "units.cuh"
 
 namespace mpipe {
 
@@ -132,6 +133,8 @@ attn_bwd_kernel(const __grid_constant__ BwdMaps maps, const BwdParams p) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     __shared__ BwdBarriers bars;
+    __shared__ UnitRing units;
+    __shared__ mpipe_work_item_t reducer_item;
     __shared__ uint32_t tmem_base_slot;
     __shared__ int abort_flag;
 
@@ -141,6 +144,7 @@ attn_bwd_kernel(const __grid_constant__ BwdMaps maps, const BwdParams p) {
 
     if (tid == 0) {
         abort_flag = 0;
+        unit_ring_init(&units, 11);             // the issuer, the staging warp, the softmax warps and the reducer warpgroup read it
         for (int i = 0; i < 2; ++i) {
             mbar_init(&bars.kv_full[i], 1);
             mbar_init(&bars.kv_empty[i], 1);
@@ -184,12 +188,6 @@ attn_bwd_kernel(const __grid_constant__ BwdMaps maps, const BwdParams p) {
     const int n_units = plan_ok_cta(p.items, p.n_items, kBT, p.total_tokens, p.status_buf, &plan_flag) ? p.n_items * p.n_heads : 0;
     pdl_wait();
     pdl_launch();
-    // Units are sorted by decreasing cost; CTAs walk them in boustrophedon order (0..G-1, then G-1..0, ...) so
-    // that the CTA that got the most expensive unit of one round gets the cheapest of the next.
-    auto unit_of = [&](int round) {
-        const int g = int(gridDim.x), i = int(blockIdx.x);
-        return round * g + ((round & 1) ? g - 1 - i : i);
-    };
     // Unit u -> (work item, head).  The items of one segment are consecutive in the list (tile 0, 1, ...), and their
     // units occupy the same stretch of the unit sequence whichever way it is ordered inside.  Short segments: tile by
     // tile, heads innermost.  Segments of more than kHeadMajorTiles key tiles: head by head, so that the CTAs running
@@ -200,7 +198,7 @@ attn_bwd_kernel(const __grid_constant__ BwdMaps maps, const BwdParams p) {
     constexpr int kHeadMajorTiles = 32;
     auto item_at = [&](int u) {
         mpipe_work_item_t z = {0, 0, 0, 0, 0, 0};
-        if (u >= n_units) return z;
+        if (u < 0 || u >= n_units) return z;
         const int i0 = u / p.n_heads;
         const mpipe_work_item_t a = p.items[i0];
         const int nt = (a.kv_len + kBT - 1) / kBT;                   // key tiles of this item's segment
@@ -235,10 +233,12 @@ attn_bwd_kernel(const __grid_constant__ BwdMaps maps, const BwdParams p) {
                 for (int bx = 0; bx < Cfg::kBoxes; ++bx)
                     tma_load_3d(dst + bx * Cfg::kBoxBytes, map, bar, bx * Cfg::kBoxElems, head, row);
             };
-            mpipe_work_item_t it_next = item_at(unit_of(0));   // one unit ahead: the global load is off the unit's critical path
-            for (int ur = 0, u = unit_of(0); u < n_units && ok; ++ur, u = unit_of(ur), ++unit_it) {
-                const mpipe_work_item_t it = it_next;
-                it_next = item_at(unit_of(ur + 1));
+            UnitSource source{&units, &abort_flag};
+            bool outstanding = false;
+            for (int u = int(blockIdx.x); ok; ++unit_it) {
+                const mpipe_work_item_t it = item_at(u);
+                ok = source.put(it);
+                if (!ok || it.kv_len <= 0) break;
                 const int head = it.seg;
                 const int nq = steps_of(it);
                 const int kb = unit_it % Cfg::kKVBufs;            // K/V buffer of this unit
@@ -248,7 +248,12 @@ attn_bwd_kernel(const __grid_constant__ BwdMaps maps, const BwdParams p) {
                 mbar_expect_tx(&bars.kv_full[kb], 2 * Cfg::kTile);
                 load_tile(kv + Cfg::kSmemK, &maps.k, &bars.kv_full[kb], head, it.row_start);
                 load_tile(kv + Cfg::kSmemV, &maps.v, &bars.kv_full[kb], head, it.row_start);
+                const int ask_at = nq > 3 ? nq - 3 : 0;   // late enough to go to the CTA that is free first, early enough to be answered
                 for (int j = 0; j < nq; ++j, ++sc) {
+                    if (j == ask_at) {
+                        source.ask();
+                        outstanding = true;
+                    }
                     const int rs = sc % NR;
                     const int row = it.kv_start + q_tile_of(it, j, nq) * kBQ;
                     ok = mbar_wait<kSleepAux>(&bars.qdo_empty[rs], ((sc / NR) & 1) ^ 1, &abort_flag);
@@ -257,7 +262,11 @@ attn_bwd_kernel(const __grid_constant__ BwdMaps maps, const BwdParams p) {
                     load_tile(smem + Cfg::kSmemQ + rs * Cfg::kTile, &maps.q, &bars.qdo_full[rs], head, row);
                     load_tile(smem + Cfg::kSmemDO + rs * Cfg::kTile, &maps.dout, &bars.qdo_full[rs], head, row);
                 }
+                if (!ok) break;
+                u = source.take(&ok);
+                outstanding = false;
             }
+            if (!ok) source.cancel_rest(outstanding);
         }
         __syncwarp();
     } else if (warp == 1) {
@@ -308,10 +317,10 @@ attn_bwd_kernel(const __grid_constant__ BwdMaps maps, const BwdParams p) {
             };
             uint32_t unit_it = 0, sc = 0;   // sc: global step counter at the start of the unit
             bool ok = true;
-            mpipe_work_item_t it_next = item_at(unit_of(0));   // one unit ahead: the global load is off the unit's critical path
-            for (int ur = 0, u = unit_of(0); u < n_units && ok; ++ur, u = unit_of(ur), ++unit_it) {
-                const mpipe_work_item_t it = it_next;
-                it_next = item_at(unit_of(ur + 1));
+            mpipe_work_item_t it, it_next;
+            uint32_t ui = 0;                // next entry of the unit ring
+            bool has_unit = next_unit(&units, ui++, &it, lane, &abort_flag), has_next = false;
+            for (; ok && has_unit; has_unit = has_next, it = it_next, ++unit_it) {
                 const int nq = steps_of(it);
                 const int kb = unit_it % Cfg::kKVBufs;
                 const uint32_t kvb = sbase + kb * (2 * Cfg::kTile);
@@ -321,7 +330,7 @@ attn_bwd_kernel(const __grid_constant__ BwdMaps maps, const BwdParams p) {
                 // first step are issued inside this unit's last step, from the other (prefetched) buffer, so the softmax
                 // warps never see the pipeline drain between units.
                 constexpr bool kStream = (Cfg::kKVBufs == 2);
-                const bool has_next = kStream && unit_of(ur + 1) < n_units;
+                has_next = false;
                 const uint32_t kvb_n = sbase + (kb ^ 1) * (2 * Cfg::kTile);
                 const uint32_t k_lo_n = umma_desc_lo(kvb_n + Cfg::kSmemK, 0), v_lo_n = umma_desc_lo(kvb_n + Cfg::kSmemV, 0);
                 ok = mbar_wait(&bars.kv_full[kb], (unit_it / Cfg::kKVBufs) & 1, &abort_flag);
@@ -338,6 +347,7 @@ attn_bwd_kernel(const __grid_constant__ BwdMaps maps, const BwdParams p) {
                 for (int j = 0; j < nq && ok; ++j) {
                     const uint32_t c = sc + j;
                     const uint32_t ph = c & 1;
+                    if (kStream && j + 1 == nq) has_next = next_unit(&units, ui++, &it_next, lane, &abort_flag);
                     const bool cross = (j + 1 == nq) && has_next;   // step j+1 is the next unit's first
                     const bool more = (j + 1 < nq) || cross;
                     auto issue_next_s = [&]() -> bool {   // S^T(j+1), from the next unit's K tile at a unit's last step
@@ -392,6 +402,7 @@ attn_bwd_kernel(const __grid_constant__ BwdMaps maps, const BwdParams p) {
                 if (leader) umma_commit(&bars.dkv_full);
                 if (leader) umma_commit(&bars.kv_empty[kb]);
                 sc += nq;
+                if (!kStream) has_next = next_unit(&units, ui++, &it_next, lane, &abort_flag);
             }
         }
         __syncwarp();
@@ -413,10 +424,8 @@ attn_bwd_kernel(const __grid_constant__ BwdMaps maps, const BwdParams p) {
             return make_uint4(uint32_t(__bfloat16_as_ushort(h)) | (uint32_t(__bfloat16_as_ushort(m)) << 16),
                               uint32_t(__bfloat16_as_ushort(l)), 0u, 0u);
         };
-        mpipe_work_item_t it_next = item_at(unit_of(0));   // one unit ahead: the global load is off the unit's critical path
-        for (int ur = 0, u = unit_of(0); u < n_units && ok; ++ur, u = unit_of(ur)) {
-            const mpipe_work_item_t it = it_next;
-            it_next = item_at(unit_of(ur + 1));
+        mpipe_work_item_t it;
+        for (uint32_t ui = 0; ok && next_unit(&units, ui, &it, lane, &abort_flag); ++ui) {
             const int head = it.seg;
             const int nq = steps_of(it);
             const int q_end = it.kv_start + it.kv_len;
@@ -464,10 +473,8 @@ attn_bwd_kernel(const __grid_constant__ BwdMaps maps, const BwdParams p) {
         uint8_t* ds_row = smem + Cfg::kSmemDS + g * (kBT * 128) + r * 128;
         uint32_t sc = 0;   // global step counter at the start of the unit
         bool ok = true;
-        mpipe_work_item_t it_next = item_at(unit_of(0));   // one unit ahead: the global load is off the unit's critical path
-        for (int ur = 0, u = unit_of(0); u < n_units && ok; ++ur, u = unit_of(ur)) {
-            const mpipe_work_item_t it = it_next;
-            it_next = item_at(unit_of(ur + 1));
+        mpipe_work_item_t it;
+        for (uint32_t ui = 0; ok && next_unit(&units, ui, &it, lane, &abort_flag); ++ui) {
             const int nq = steps_of(it);
             const bool key_valid = r < it.row_len;
             const bool ragged_keys = it.row_len < kBT;
@@ -570,10 +577,23 @@ attn_bwd_kernel(const __grid_constant__ BwdMaps maps, const BwdParams p) {
         const uint32_t lane_base = uint32_t((warp & 3) * 32) << 16;
         uint32_t pc = 0, gc = 0, unit_it = 0;   // step counter, staging-chunk counter
         bool ok = true;
-        mpipe_work_item_t it_next = item_at(unit_of(0));   // one unit ahead: the global load is off the unit's critical path
-        for (int ur = 0, u = unit_of(0); u < n_units; ++ur, u = unit_of(ur), ++unit_it) {
-            const mpipe_work_item_t it = it_next;
-            it_next = item_at(unit_of(ur + 1));
+        // One thread reads the unit ring for the four warps, which meet at named barriers and have to leave the loop together
+        // (reducer_item is read before, and written again after, the barriers of at least one step).
+        mpipe_work_item_t it;
+        auto fetch_unit = [&](uint32_t i) {
+            if (rt == 0) {
+                mpipe_work_item_t x = {0, 0, 0, 0, 0, 0};
+                if (mbar_wait(&units.full[i % kUnitRing], (i / kUnitRing) & 1, &abort_flag)) {
+                    x = units.item[i % kUnitRing];
+                    mbar_arrive(&units.empty[i % kUnitRing]);
+                }
+                reducer_item = x;
+            }
+            named_barrier_sync(1, 128);
+            it = reducer_item;
+            return it.kv_len > 0;
+        };
+        for (uint32_t ui = 0; fetch_unit(ui); ++ui, ++unit_it) {
             const int head = it.seg;
             const int nq = steps_of(it);
             // No early exit inside this loop: the four warps meet at named barriers, so after a time-out
@@ -798,9 +818,8 @@ static int32_t launch_bwd(const void* dout, const void* q, const void* k, const 
                                   n_heads, delta, dq_acc);
     if (e != cudaSuccess) return MPIPE_ERR_CUDA;
     const int n_units = prm.n_items * prm.n_heads;
-    const int grid = n_units < sm_count() ? n_units : sm_count();
     profile_start(kProfileBwdMain, stream);
-    e = launch_kernel(attn_bwd_kernel<D>, unsigned(grid), kBwdThreads, Cfg::kSmemAlloc, stream, 1, m, prm);
+    e = launch_kernel_as(true, attn_bwd_kernel<D>, unsigned(n_units), kBwdThreads, Cfg::kSmemAlloc, stream, 1, m, prm);
     profile_stop(kProfileBwdMain, stream);
     if (e != cudaSuccess) return MPIPE_ERR_CUDA;
     const bool rope = prm.rope_cos != nullptr;
