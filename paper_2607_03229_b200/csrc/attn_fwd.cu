@@ -46,7 +46,10 @@ struct FwdCfg {
     static constexpr int kSmemQ = 0;
     static constexpr int kSmemK = 2 * kQBytes;
     static constexpr int kSmemV = kSmemK + kStages * kQBytes;
-    static constexpr int kSmemTotal = kSmemV + kStages * kVBytes;
+    static constexpr int kOutCols = (D == 64) ? 64 : 32;              // one [32 rows][kOutCols] box of O per softmax warp
+    static constexpr int kOutBox = 32 * kOutCols * 2;
+    static constexpr int kSmemO = kSmemV + kStages * kVBytes;
+    static constexpr int kSmemTotal = kSmemO + 8 * kOutBox;
     static constexpr int kSmemAlloc = kSmemTotal + 1024;              // slack for manual 1024-byte alignment
     // TMEM: S_w at 128 w, O_w at 256 + 128 w.  head_dim 64 leaves 64 columns behind each O_w: P_w (128 keys as bf16) goes
     // there instead of overlaying S_w, so that S_w(j+1) can be issued as soon as the softmax warps have READ S_w(j)
@@ -80,11 +83,12 @@ struct FwdBarriers {
 
 // kSplit: the two query tiles of an item are units of their own (an instantiation apart: the bookkeeping for it in the other one
 // costs 2 to 7 % on long lists).
-template <int D, bool kSplit>
+// kStaged: O leaves through shared memory (see the epilogue).
+template <int D, bool kSplit, bool kStaged>
 __global__ void __maxnreg__(kFwdRegsLaunch)
 attn_fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                 const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_q_tail,
-                const __grid_constant__ CUtensorMap map_k_tail, const FwdParams p) {
+                const __grid_constant__ CUtensorMap map_k_tail, const __grid_constant__ CUtensorMap map_o, const FwdParams p) {
     using Cfg = FwdCfg<D>;
     constexpr int NS = Cfg::kStages;
     extern __shared__ uint8_t smem_raw[];
@@ -126,6 +130,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
         prefetch_tmap(&map_q);
         prefetch_tmap(&map_k);
         prefetch_tmap(&map_v);
+        prefetch_tmap(&map_o);
     }
     tc_fence_before();
     __syncthreads();
@@ -496,29 +501,79 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
             const float inv_l = 1.0f / l;
             const bool store = r < rows_here;
             const int64_t tok = int64_t(it.row_start) + w * kTileM + r;
+            // Staged: in a unit of two query tiles, where all 32 rows of a warp are rows of the segment, the first 64 columns leave
+            // through the warp's staging box (128- or 64-byte swizzle) by a TMA store: straight from the registers every store
+            // of a warp touches 32 rows (256 wavefronts per warp and unit, 2000 clocks for the eight of a 256-row unit).
+            // head_dim 80 has room for half of the columns: the first half is read back and stored in coalesced pieces, so that
+            // nothing waits for the copy engine inside a unit.  A ragged warp and a unit of one tile, whose four warps get in
+            // nobody's way, store directly.
             __nv_bfloat16* orow = p.o + tok * p.tok_stride_o + int64_t(head) * p.head_stride_o;
+            const int row0 = (warp & 3) * 32;                   // first row of this warp in the tile
+            const bool whole = kStaged && it.row_len > kTileM && rows_here - row0 >= 32;
+            int c_done = 0;                                     // columns that have left
+            if (kStaged && (D == 80 || whole)) {                // (head_dim 80: one path with predicated stores measured faster)
+                constexpr int kOC = Cfg::kOutCols, kCh = kOC / 8;
+                auto slot = [](int row, int c) { return row * (kOC * 2) + ((kOC == 64 ? c ^ (row & 7) : c ^ ((row >> 1) & 3)) << 4); };
+                uint32_t orr[64];
+                tmem_ld32(t_o, *reinterpret_cast<uint32_t(*)[32]>(&orr[0]));
+                tmem_ld32(t_o + 32, *reinterpret_cast<uint32_t(*)[32]>(&orr[32]));
+                uint8_t* box = smem + Cfg::kSmemO + (warp - 4) * Cfg::kOutBox;
+                if (whole && lane == 0) bulk_wait_group_read<0>();   // the previous unit's store has read the box
+                tmem_wait_ld();
+                __syncwarp();
+#pragma unroll
+                for (int c0 = 0; c0 < 64; c0 += kOC) {
+#pragma unroll
+                    for (int g = 0; g < kCh; ++g) {
+                        uint32_t o4[4];
+#pragma unroll
+                        for (int e = 0; e < 4; ++e)
+                            o4[e] = pack_bf16(__uint_as_float(orr[c0 + 8 * g + 2 * e]) * inv_l, __uint_as_float(orr[c0 + 8 * g + 2 * e + 1]) * inv_l);
+                        const uint4 v = make_uint4(o4[0], o4[1], o4[2], o4[3]);
+                        if (D == 64 || whole) *reinterpret_cast<uint4*>(box + slot(lane, g)) = v;
+                        else if (store) *reinterpret_cast<uint4*>(orow + c0 + 8 * g) = v;
+                    }
+                    if (whole && c0 + kOC < 64) {
+                        __syncwarp();
+                        __nv_bfloat16* orow0 = orow - lane * p.tok_stride_o + c0;
+#pragma unroll
+                        for (int i = 0; i < kCh; ++i) {
+                            const int rr = (32 / kCh) * i + lane / kCh, c = lane % kCh;
+                            *reinterpret_cast<uint4*>(orow0 + rr * p.tok_stride_o + c * 8) = *reinterpret_cast<const uint4*>(box + slot(rr, c));
+                        }
+                        __syncwarp();                            // (read before it is written again)
+                    } else if (whole) {
+                        fence_async_smem();
+                        __syncwarp();
+                        if (lane == 0) {
+                            tma_store_3d(&map_o, box, c0, head, it.row_start + w * kTileM + row0);
+                            bulk_commit_group();
+                        }
+                    }
+                }
+                c_done = 64;
+            }
 #pragma unroll
             for (int c0 = 0; c0 < D; c0 += 16) {
+                if (c0 < c_done) continue;
                 uint32_t orr[16];
                 tmem_ld16(t_o + c0, orr);
                 tmem_wait_ld();
-                uint4 v0, v1;
-                v0.x = pack_bf16(__uint_as_float(orr[0]) * inv_l, __uint_as_float(orr[1]) * inv_l);
-                v0.y = pack_bf16(__uint_as_float(orr[2]) * inv_l, __uint_as_float(orr[3]) * inv_l);
-                v0.z = pack_bf16(__uint_as_float(orr[4]) * inv_l, __uint_as_float(orr[5]) * inv_l);
-                v0.w = pack_bf16(__uint_as_float(orr[6]) * inv_l, __uint_as_float(orr[7]) * inv_l);
-                v1.x = pack_bf16(__uint_as_float(orr[8]) * inv_l, __uint_as_float(orr[9]) * inv_l);
-                v1.y = pack_bf16(__uint_as_float(orr[10]) * inv_l, __uint_as_float(orr[11]) * inv_l);
-                v1.z = pack_bf16(__uint_as_float(orr[12]) * inv_l, __uint_as_float(orr[13]) * inv_l);
-                v1.w = pack_bf16(__uint_as_float(orr[14]) * inv_l, __uint_as_float(orr[15]) * inv_l);
+                uint32_t o8[8];
+#pragma unroll
+                for (int e = 0; e < 8; ++e) o8[e] = pack_bf16(__uint_as_float(orr[2 * e]) * inv_l, __uint_as_float(orr[2 * e + 1]) * inv_l);
                 if (store) {
-                    *reinterpret_cast<uint4*>(orow + c0) = v0;
-                    *reinterpret_cast<uint4*>(orow + c0 + 8) = v1;
+                    *reinterpret_cast<uint4*>(orow + c0) = make_uint4(o8[0], o8[1], o8[2], o8[3]);
+                    *reinterpret_cast<uint4*>(orow + c0 + 8) = make_uint4(o8[4], o8[5], o8[6], o8[7]);
                 }
             }
             if (store && p.lse != nullptr)
                 p.lse[int64_t(head) * p.total_tokens + tok] = m_ref * 0.6931471805599453f + logf(l);
             tc_fence_before();
+        }
+        if (kStaged) {
+            if (lane == 0) bulk_wait_group_read<0>();   // shared memory must outlive the copy engine's reads
+            __syncwarp();
         }
     }
 
@@ -528,15 +583,16 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
     if (tid == 0 && abort_flag) report_status(p.status_buf, MPIPE_ERR_TIMEOUT, int32_t(blockIdx.x));
 }
 
-template <int D, bool kSplit>
+template <int D, bool kSplit, bool kStaged>
 static int32_t launch_fwd(const void* q, const void* k, const void* v, int64_t tok_stride, int64_t head_stride,
                           int32_t total_tokens, int32_t n_heads, const FwdParams& prm, cudaStream_t stream) {
     using Cfg = FwdCfg<D>;
-    CUtensorMap mq, mk, mv, mqt, mkt;
+    CUtensorMap mq, mk, mv, mqt, mkt, mo;
     const uint32_t main_box = 64;
     if (!make_tensor_map_thd(&mq, q, total_tokens, n_heads, D, tok_stride, head_stride, main_box, kTileM, 128) ||
         !make_tensor_map_thd(&mk, k, total_tokens, n_heads, D, tok_stride, head_stride, main_box, kTileN, 128) ||
-        !make_tensor_map_thd(&mv, v, total_tokens, n_heads, D, tok_stride, head_stride, main_box, kTileN, 128))
+        !make_tensor_map_thd(&mv, v, total_tokens, n_heads, D, tok_stride, head_stride, main_box, kTileN, 128) ||
+        !make_tensor_map_thd(&mo, prm.o, total_tokens, n_heads, D, prm.tok_stride_o, prm.head_stride_o, Cfg::kOutCols, 32, Cfg::kOutCols * 2))
         return MPIPE_ERR_CUDA;
     mqt = mq;
     mkt = mk;
@@ -545,10 +601,10 @@ static int32_t launch_fwd(const void* q, const void* k, const void* v, int64_t t
             !make_tensor_map_thd(&mkt, k, total_tokens, n_heads, D, tok_stride, head_stride, 16, kTileN, 32))
             return MPIPE_ERR_CUDA;
     }
-    if (!ensure_dynamic_smem<attn_fwd_kernel<D, kSplit>>(Cfg::kSmemAlloc)) return MPIPE_ERR_CUDA;
+    if (!ensure_dynamic_smem<attn_fwd_kernel<D, kSplit, kStaged>>(Cfg::kSmemAlloc)) return MPIPE_ERR_CUDA;
     const int n_units = prm.n_items * prm.n_heads * (kSplit ? 2 : 1);
     profile_start(kProfileFwd, stream);
-    const cudaError_t e = launch_kernel_as(true, attn_fwd_kernel<D, kSplit>, unsigned(n_units), kFwdThreads, Cfg::kSmemAlloc, stream, 1, mq, mk, mv, mqt, mkt, prm);
+    const cudaError_t e = launch_kernel_as(true, attn_fwd_kernel<D, kSplit, kStaged>, unsigned(n_units), kFwdThreads, Cfg::kSmemAlloc, stream, 1, mq, mk, mv, mqt, mkt, mo, prm);
     profile_stop(kProfileFwd, stream);
     return e == cudaSuccess && cudaGetLastError() == cudaSuccess ? MPIPE_OK : MPIPE_ERR_CUDA;
 }
@@ -593,8 +649,12 @@ int32_t varlen_attn_fwd(const void* q, const void* k, const void* v, void* o, fl
     // of 300: 9.3 -> 7.7; with 80 units on 148 SMs a second round of single tiles would cost more than it saves).
     const bool split = 2 * int64_t(n_fwd_items) * n_heads <= sm_count();
     auto launch = [&](auto f) { return f(q, k, v, tok_stride_qkv, head_stride_qkv, total_tokens, n_heads, prm, st); };
-    if (head_dim == 64) return split ? launch(launch_fwd<64, true>) : launch(launch_fwd<64, false>);
-    return split ? launch(launch_fwd<80, true>) : launch(launch_fwd<80, false>);
+    // Staged O pays where units have two query tiles and enough key tiles behind them (us direct -> staged): head_dim 64, ViT-L
+    // microbatch 512 -> 505, but images of 300 235 -> 239 and of 819 44.2 -> 44.6; head_dim 80, 200 images of 64 to 256 tokens
+    // 101.5 -> 94.6, 65 536 long-tailed ones 2940 -> 2850, images of 2048 765 -> 700, but of 100 (one tile each) 187 -> 200.
+    const bool staged = max_seqlen > (head_dim == 64 ? 1024 : 128);
+    if (head_dim == 64) return split ? launch(launch_fwd<64, true, false>) : staged ? launch(launch_fwd<64, false, true>) : launch(launch_fwd<64, false, false>);
+    return split ? launch(launch_fwd<80, true, false>) : staged ? launch(launch_fwd<80, false, true>) : launch(launch_fwd<80, false, false>);
 }
 
 }  // namespace mpipe
