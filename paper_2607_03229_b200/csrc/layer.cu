@@ -18,70 +18,96 @@ constexpr int kLnMaxChunks = 8;   // 16-byte chunks per lane: hidden <= 8 * 32 *
 
 // y[t, :] = (x[t, :] - mean) * rsqrt(var + eps) * gamma + beta, biased variance, fp32 statistics (two passes over
 // registers, so no cancellation).  One warp per row; lane l owns chunks l, l + 32, ...
-template <int kChunks>
-__global__ void __launch_bounds__(256) layernorm_kernel(const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __restrict__ gamma,
+// Bound by HBM when there are many rows and by the latency of its loads when there are few.
+// kWalk: a warp walks down the rows with the next row on its way while it works on the present one, gamma and beta from L1; two waves
+// of as many blocks as fit.  Otherwise a row per warp, gamma and beta asked for together with the row instead of one L2 latency after
+// its sums.  us, a row per warp and late gamma -> walking / a row per warp as it is now: 777 x 1024 2.83 -> - / 2.08,
+// 4000 x 256 2.02 -> 2.33 / 2.11, 3489 x 1024 4.49 -> 4.10 / 4.25, 20 000 x 1024 16.5 -> 15.0 / 17.7,
+// 50 439 x 1024 36.1 -> 34.0 (6.1 TB/s) / 39.2, 65 536 x 1280 59.5 -> 55.8 (6.0 TB/s) / 71.4: the line lies at 2 M elements.
+constexpr int64_t kLnWalkElems = 2 << 20;
+constexpr int ln_walk_blocks(int chunks) { return chunks <= 2 ? 6 : chunks <= 4 ? 3 : 2; }   // of 256 threads on an SM, without spills
+template <int kChunks, bool kWalk>
+__global__ void __launch_bounds__(256, kWalk ? ln_walk_blocks(kChunks) : 1) layernorm_kernel(const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __restrict__ gamma,
                                                         const __nv_bfloat16* __restrict__ beta, __nv_bfloat16* __restrict__ y,
                                                         int32_t T, int32_t hidden, int64_t ldx, int64_t ldy, float eps) {
     pdl_wait();
     pdl_launch();
-    const int row = blockIdx.x * 8 + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
-    if (row >= T) return;
     const int n_chunks = hidden >> 3;
-    const uint4* xr = reinterpret_cast<const uint4*>(x + int64_t(row) * ldx);
-    float v[kChunks][8];
-    float sum = 0.f;
-#pragma unroll
-    for (int i = 0; i < kChunks; ++i) {
-        const int c = lane + 32 * i;
-        if (c < n_chunks) {
-            const uint4 q = xr[c];
-            const uint32_t w[4] = {q.x, q.y, q.z, q.w};
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                v[i][2 * j] = __uint_as_float(w[j] << 16);
-                v[i][2 * j + 1] = __uint_as_float(w[j] & 0xffff0000u);
-                sum += v[i][2 * j] + v[i][2 * j + 1];
-            }
-        }
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-    const float mean = sum / float(hidden);
-    float sq = 0.f;
-#pragma unroll
-    for (int i = 0; i < kChunks; ++i) {
-        if (lane + 32 * i < n_chunks) {
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                const float d = v[i][j] - mean;
-                sq = fmaf(d, d, sq);
-            }
-        }
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
-    const float rstd = rsqrtf(sq / float(hidden) + eps);
-    uint4* yr = reinterpret_cast<uint4*>(y + int64_t(row) * ldy);
     const uint4* g4 = reinterpret_cast<const uint4*>(gamma);
     const uint4* b4 = reinterpret_cast<const uint4*>(beta);
+    int row = blockIdx.x * 8 + (threadIdx.x >> 5);
+    uint4 q[kChunks], g[kWalk ? 1 : kChunks], b[kWalk ? 1 : kChunks];
+    auto load = [&](int r) {
+        if (r >= T) return;
+        const uint4* xr = reinterpret_cast<const uint4*>(x + int64_t(r) * ldx);
 #pragma unroll
-    for (int i = 0; i < kChunks; ++i) {
-        const int c = lane + 32 * i;
-        if (c < n_chunks) {
-            const uint4 g = __ldg(g4 + c), b = __ldg(b4 + c);
-            const uint32_t gw[4] = {g.x, g.y, g.z, g.w}, bw[4] = {b.x, b.y, b.z, b.w};
-            uint32_t o[4];
+        for (int i = 0; i < kChunks; ++i)
+            if (lane + 32 * i < n_chunks) q[i] = xr[lane + 32 * i];
+    };
+    load(row);
+    if (!kWalk) {
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const float lo = (v[i][2 * j] - mean) * rstd * __uint_as_float(gw[j] << 16) + __uint_as_float(bw[j] << 16);
-                const float hi = (v[i][2 * j + 1] - mean) * rstd * __uint_as_float(gw[j] & 0xffff0000u) +
-                                 __uint_as_float(bw[j] & 0xffff0000u);
-                const __nv_bfloat162 pk = __floats2bfloat162_rn(lo, hi);
-                o[j] = *reinterpret_cast<const uint32_t*>(&pk);
+        for (int i = 0; i < kChunks; ++i) {
+            if (lane + 32 * i < n_chunks) {
+                g[i] = __ldg(g4 + lane + 32 * i);
+                b[i] = __ldg(b4 + lane + 32 * i);
             }
-            yr[c] = make_uint4(o[0], o[1], o[2], o[3]);
         }
+    }
+    for (; row < T; row += gridDim.x * 8) {
+        float v[kChunks][8];
+        float sum = 0.f;
+#pragma unroll
+        for (int i = 0; i < kChunks; ++i) {
+            if (lane + 32 * i < n_chunks) {
+                const uint32_t w[4] = {q[i].x, q[i].y, q[i].z, q[i].w};
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    v[i][2 * j] = __uint_as_float(w[j] << 16);
+                    v[i][2 * j + 1] = __uint_as_float(w[j] & 0xffff0000u);
+                    sum += v[i][2 * j] + v[i][2 * j + 1];
+                }
+            }
+        }
+        if (kWalk) load(row + gridDim.x * 8);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        const float mean = sum / float(hidden);
+        float sq = 0.f;
+#pragma unroll
+        for (int i = 0; i < kChunks; ++i) {
+            if (lane + 32 * i < n_chunks) {
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const float d = v[i][j] - mean;
+                    sq = fmaf(d, d, sq);
+                }
+            }
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+        const float rstd = rsqrtf(sq / float(hidden) + eps);
+        uint4* yr = reinterpret_cast<uint4*>(y + int64_t(row) * ldy);
+#pragma unroll
+        for (int i = 0; i < kChunks; ++i) {
+            const int c = lane + 32 * i;
+            if (c < n_chunks) {
+                const uint4 gi = kWalk ? __ldg(g4 + c) : g[kWalk ? 0 : i], bi = kWalk ? __ldg(b4 + c) : b[kWalk ? 0 : i];
+                const uint32_t gw[4] = {gi.x, gi.y, gi.z, gi.w}, bw[4] = {bi.x, bi.y, bi.z, bi.w};
+                uint32_t o[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const float lo = (v[i][2 * j] - mean) * rstd * __uint_as_float(gw[j] << 16) + __uint_as_float(bw[j] << 16);
+                    const float hi = (v[i][2 * j + 1] - mean) * rstd * __uint_as_float(gw[j] & 0xffff0000u) +
+                                     __uint_as_float(bw[j] & 0xffff0000u);
+                    const __nv_bfloat162 pk = __floats2bfloat162_rn(lo, hi);
+                    o[j] = *reinterpret_cast<const uint32_t*>(&pk);
+                }
+                yr[c] = make_uint4(o[0], o[1], o[2], o[3]);
+            }
+        }
+        if (!kWalk) break;
     }
 }
 
@@ -338,6 +364,7 @@ int32_t mpipe_layernorm_fwd(const void* x, const void* gamma, const void* beta, 
     if ((hidden % 8) != 0 || hidden > kLnMaxChunks * 256 || (ldx % 8) != 0 || (ldy % 8) != 0) return MPIPE_ERR_UNSUPPORTED;
     if (!aligned16(x) || !aligned16(y) || !aligned16(gamma) || !aligned16(beta)) return MPIPE_ERR_UNSUPPORTED;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
+    const bool walk = int64_t(n_tokens) * hidden > kLnWalkElems;
     const int grid = cdiv(n_tokens, 8);
     const auto* xp = static_cast<const __nv_bfloat16*>(x);
     const auto* gp = static_cast<const __nv_bfloat16*>(gamma);
@@ -346,7 +373,9 @@ int32_t mpipe_layernorm_fwd(const void* x, const void* gamma, const void* beta, 
     profile_start(kProfileLayerNorm, st);
     const int chunks = cdiv(hidden, 256);   // 16-byte chunks per lane: instantiate what the row length needs, not the maximum
     cudaError_t e;
-#define MPIPE_LN_LAUNCH(C) e = launch_kernel(layernorm_kernel<C>, unsigned(grid), 256, 0, st, 1, xp, gp, bp, yp, n_tokens, hidden, ldx, ldy, eps)
+#define MPIPE_LN_LAUNCH(C)                                                                                                       \
+    e = walk ? launch_kernel_as(true, layernorm_kernel<C, true>, unsigned(2 * ln_walk_blocks(C) * sm_count()), 256, 0, st, 1, xp, gp, bp, yp, n_tokens, hidden, ldx, ldy, eps) \
+             : launch_kernel(layernorm_kernel<C, false>, unsigned(grid), 256, 0, st, 1, xp, gp, bp, yp, n_tokens, hidden, ldx, ldy, eps)
     if (chunks <= 1) MPIPE_LN_LAUNCH(1);
     else if (chunks <= 2) MPIPE_LN_LAUNCH(2);
     else if (chunks <= 3) MPIPE_LN_LAUNCH(3);
