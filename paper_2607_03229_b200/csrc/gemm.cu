@@ -24,7 +24,7 @@
 // partial results meet in shared memory (every pair finishes the chunks it owns from the others' fp32 partials).
 // Measured against the one-CTA 128 x 256 kernel with warpgroup-wide staging that this replaces (us, M = 50 439): fc1 + GELU
 // 1024 -> 4096 398 -> 325, its gradient with GELU' 480 -> 383, attention output + residual 115 -> 90, QKV 241 -> 221 (1430
-// TFLOP/s), weight gradient 1024 x 4096 348 -> 292; M = 777: fc2 27.9 -> 13.4 (split), output projection 14.4 -> 7.8, weight
+// TFLOP/s), weight gradient 1024 x 4096 348 -> 292; M = 777: fc2 27.9 -> 13.4 (split), output projection 14.4 -> 7.2, weight
 // gradient 1024 x 4096 34 -> 12.
 // Every mbarrier wait is bounded (status MPIPE_ERR_TIMEOUT), as in the attention kernels.
 #include <cuda_bf16.h>
@@ -163,6 +163,7 @@ linear_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
     const int bn = p.bn, bn_half = bn >> 1;
     const int a_bytes = kpb * kGemmABytes, stage_bytes = a_bytes + kpb * bn_half * kGemmBK * 2, n_stages = p.stages;
 
+    bool left = false;                                        // this warp has arrived at the cluster's last meeting
     if (warp == 0 || warp == 3) {
         // Two producers, one per operand: a thread gets a TMA instruction out every ~90 clocks and a barrier test through in
         // ~110, so one thread issuing both operands' boxes was the slowest role below BN 256 (455 clocks per stage whatever BN)
@@ -205,6 +206,11 @@ linear_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
                     }
                     if (++s == uint32_t(n_stages)) { s = 0; ph ^= 1; }
                 }
+            }
+            // the pair's last commits have arrived on this CTA's barriers, which must not be gone by then
+            for (int i = 0; is_a && ok && i < n_stages; ++i) {
+                ok = mbar_wait(&bars.empty[s], ph, &abort_flag);
+                if (++s == uint32_t(n_stages)) { s = 0; ph ^= 1; }
             }
         }
         __syncwarp();
@@ -313,6 +319,12 @@ linear_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
         uint32_t acc_empty_addr[2] = {mapa_u32(smem_u32(&bars.acc_empty[0]), lead), mapa_u32(smem_u32(&bars.acc_empty[1]), lead)};
         const int n_chunks = bn >> 6;
         uint32_t tile_it = 0, bc = 0;   // bc: boxes used so far by this warp; box = bc & 1
+        // Arrive at the last meeting of the cluster as soon as this warp will touch neither TMEM nor the other CTA any more, under
+        // the arithmetic and the stores of its last chunk (an arrival behind them kept every CTA about half a microsecond longer).
+        auto leave = [&]() {
+            if (!left) cluster_arrive();
+            left = true;
+        };
         bool ok = true;
         for (int t = cid; t < n_items; t += n_clusters, ++tile_it) {
             if (kb_lo_of(t) >= kb_hi_of(t)) { --tile_it; continue; }
@@ -380,6 +392,7 @@ linear_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
                 __syncwarp();
                 if (lane == 0) mbar_arrive_cluster(acc_empty_addr[acc]);
                 released = true;
+                if (t + n_clusters >= n_items) leave();
             };
 #pragma unroll 1
             for (int i = wg; i < own; i += 2) {
@@ -494,8 +507,11 @@ linear_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
     }
 
     __syncwarp();
-    tc_fence_before();
-    cluster_sync_all();   // neither CTA frees TMEM or leaves while the pair's MMAs or the cluster's stores may still touch it
+    if (!left) {
+        tc_fence_before();
+        cluster_arrive();
+    }
+    cluster_wait();       // neither CTA frees TMEM or leaves while the pair's MMAs or the cluster's stores may still touch it
     if (warp == 2) tmem_dealloc_pair(tmem, 512);
     if (tid == 0 && abort_flag) report_status(p.status_buf, MPIPE_ERR_TIMEOUT, int32_t(blockIdx.x));
 }

@@ -312,6 +312,9 @@ __device__ __forceinline__ uint32_t mapa_u32(uint32_t local, uint32_t rank) {
     return r;
 }
 // All threads of all CTAs of the cluster; shared-memory writes (remote ones too) made before are visible after.
+// (cluster_arrive is per thread: the lanes of a warp may come to it by different ways)
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_sync_all() {
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
