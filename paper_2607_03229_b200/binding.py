@@ -110,7 +110,8 @@ def load() -> ctypes.CDLL:
         host = importlib.util.module_from_spec(spec)
         spec.loader.exec_module(host)
         host.bind(*(ctypes.cast(getattr(lib, "mpipe_" + f), ctypes.c_void_p).value for f in
-                    ("seg_plan", "varlen_attn_fwd", "varlen_attn_bwd", "merge_tokens", "merge_tokens_bwd")))
+                    ("seg_plan", "varlen_attn_fwd", "varlen_attn_bwd", "merge_tokens", "merge_tokens_bwd",
+                     "plan_words_to_device")))
         _host, _tile_rows, _lib = host, (lib.mpipe_fwd_tile_rows(), lib.mpipe_bwd_tile_rows()), lib
     return _lib
 
@@ -184,8 +185,8 @@ class SegPlan:
         return self.cu_seqlens.size - 1
 
     def to_device(self, device="cuda") -> "SegPlan":
-        """Upload cu_seqlens and both item lists with ONE asynchronous copy from a pinned staging buffer
-        (stream-ordered on the current stream; the host does not wait for the device)."""
+        """Upload cu_seqlens and both item lists at once (stream-ordered on the current stream; the host does not wait
+        for the device): as the arguments of a kernel, or from a pinned staging buffer where they are too many."""
         if self._packed is not None:
             buf, off_f, off_b, cu, fwd, bwd = self._packed
             dev = torch.device(device)

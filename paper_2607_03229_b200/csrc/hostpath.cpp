@@ -6,6 +6,7 @@
 #include <Python.h>
 
 #include <ATen/ATen.h>
+#include <c10/core/DeviceGuard.h>
 #include <c10/cuda/CUDAStream.h>
 #include <torch/csrc/autograd/python_variable.h>
 
@@ -14,6 +15,8 @@
 
 #include "../../include/mpipe_enc.h"
 
+extern "C" int32_t mpipe_plan_words_to_device(const void* words, int32_t n, void* dst, void* stream);   // plan.cu
+
 namespace {
 
 decltype(&mpipe_seg_plan) f_seg_plan = nullptr;
@@ -21,6 +24,8 @@ decltype(&mpipe_varlen_attn_fwd) f_attn_fwd = nullptr;
 decltype(&mpipe_varlen_attn_bwd) f_attn_bwd = nullptr;
 decltype(&mpipe_merge_tokens) f_merge = nullptr;
 decltype(&mpipe_merge_tokens_bwd) f_merge_bwd = nullptr;
+decltype(&mpipe_plan_words_to_device) f_plan_words = nullptr;
+constexpr int64_t kPlanWordsMax = 8128;   // what a kernel's arguments hold
 
 struct Failed {};   // a Python exception is set
 struct WithoutGil {   // around calls that may block in the driver: other Python threads go on, as under ctypes
@@ -129,13 +134,14 @@ bool count_is(Py_ssize_t n, Py_ssize_t want) {
 }
 
 PyObject* bind(PyObject*, PyObject* const* a, Py_ssize_t n) {
-    if (!count_is(n, 5)) return nullptr;
+    if (!count_is(n, 6)) return nullptr;
     return guarded([&]() -> PyObject* {
         f_seg_plan = reinterpret_cast<decltype(f_seg_plan)>(pointer(a[0]));
         f_attn_fwd = reinterpret_cast<decltype(f_attn_fwd)>(pointer(a[1]));
         f_attn_bwd = reinterpret_cast<decltype(f_attn_bwd)>(pointer(a[2]));
         f_merge = reinterpret_cast<decltype(f_merge)>(pointer(a[3]));
         f_merge_bwd = reinterpret_cast<decltype(f_merge_bwd)>(pointer(a[4]));
+        f_plan_words = reinterpret_cast<decltype(f_plan_words)>(pointer(a[5]));
         Py_RETURN_NONE;
     });
 }
@@ -181,8 +187,9 @@ PyObject* seg_plan(PyObject*, PyObject* const* a, Py_ssize_t n) {
     });
 }
 
-// upload(buffer, n_seg + 1, fwd offset, n_fwd, bwd offset, n_bwd, device index or -1) -> (pinned staging, cu, fwd items, bwd items): one
-// asynchronous copy on the current stream.
+// upload(buffer, n_seg + 1, fwd offset, n_fwd, bwd offset, n_bwd, device index or -1) -> (pinned staging or None, cu, fwd items, bwd
+// items): asynchronous, on the device's current stream.  A plan of up to kPlanWordsMax words travels as the arguments of a kernel, a
+// larger one is copied from pinned memory.
 PyObject* upload(PyObject*, PyObject* const* a, Py_ssize_t n) {
     if (!count_is(n, 7)) return nullptr;
     return guarded([&]() -> PyObject* {
@@ -192,16 +199,30 @@ PyObject* upload(PyObject*, PyObject* const* a, Py_ssize_t n) {
         REQUIRE(n_cu <= words && off_f + 6 * nf <= words && off_b + 6 * nb <= words, "sections outside the buffer");
         const long dev = integer(a[6]);
         const at::TensorOptions ints = at::TensorOptions().dtype(at::kInt);
-        const at::Tensor host = at::empty({words}, ints.pinned_memory(true));
-        std::memcpy(host.data_ptr(), PyByteArray_AS_STRING(a[0]), size_t(words) * 4);
-        at::Tensor d = at::empty({words}, ints.device(at::Device(at::kCUDA, c10::DeviceIndex(dev))));
-        {
+        at::Tensor host, d = at::empty({words}, ints.device(at::Device(at::kCUDA, c10::DeviceIndex(dev))));
+        if (words <= kPlanWordsMax) {
+            const c10::DeviceGuard on(d.device());
+            void* const to = data(d);
+            void* const stream = c10::cuda::getCurrentCUDAStream(d.device().index()).stream();
+            const char* const from = PyByteArray_AS_STRING(a[0]);
+            int32_t st;
+            {
+                WithoutGil off;
+                st = f_plan_words(from, int32_t(words), to, stream);
+            }
+            if (st != MPIPE_OK) {
+                PyErr_Format(PyExc_RuntimeError, "the upload of the plan failed with status %d", int(st));
+                throw Failed();
+            }
+        } else {
+            host = at::empty({words}, ints.pinned_memory(true));
+            std::memcpy(host.data_ptr(), PyByteArray_AS_STRING(a[0]), size_t(words) * 4);
             WithoutGil off;
             d.copy_(host, /*non_blocking=*/true);
         }
         PyObject* r = PyTuple_New(4);
         if (r == nullptr) throw Failed();
-        PyTuple_SET_ITEM(r, 0, THPVariable_Wrap(host));
+        PyTuple_SET_ITEM(r, 0, host.defined() ? THPVariable_Wrap(host) : Py_NewRef(Py_None));
         PyTuple_SET_ITEM(r, 1, THPVariable_Wrap(d.as_strided({n_cu}, {1}, 0)));
         PyTuple_SET_ITEM(r, 2, THPVariable_Wrap(d.as_strided({nf, 6}, {6, 1}, off_f)));
         PyTuple_SET_ITEM(r, 3, THPVariable_Wrap(d.as_strided({nb, 6}, {6, 1}, off_b)));
