@@ -32,7 +32,7 @@
 //
 // Warp roles (512 threads): 0 TMA producer, 1 tcgen05 issuer, 2 TMEM allocation and LSE/Delta staging, 4-11 softmax
 // (thread = key row; warps 4-7 take query columns 0-63 of the block, warps 8-11 columns 64-127), 12-15 dQ reducer
-// and epilogue.  Every wait is bounded (see sm100_ptx.cuh); expiry sets status_buf and drains the CTA.
+// and dK / dV epilogue.  Every wait is bounded (see sm100_ptx.cuh); expiry sets status_buf and drains the CTA.
 #include <cuda.h>
 #include <math_constants.h>
 #include "common.h"
@@ -52,6 +52,11 @@ static_assert(4 * (kRegsLaunch - kRegsService) + 4 * (kRegsLaunch - kRegsReducer
               "setmaxnreg pool arithmetic");
 constexpr int kBT = 128;  // keys per unit = TMEM lanes
 constexpr int kBQ = 128;  // query rows per step
+// head_dim 80, segments of up to three tiles and more units than SMs: the pooled tile buffers (BwdCfg::kPool).  Every tile then costs the
+// issuer and the producer a hand-shake of its own, 0.1 to 0.3 us a step, which a short unit gets back from loads that no longer wait
+// for its end.  us, two buffers a kind -> pool: 1024 segments of 64 rows 748 -> 625, 256 of 256 610 -> 557, 200 thumbnails of 64 to 256
+// 369 -> 330, 218 of 300 813 -> 801, 163 of 400 944 -> 962, 32 of 2048 2151 -> 2278, one of 200 (a unit per CTA) 17.4 -> 18.4.
+constexpr int kPoolSeqlen = 384;
 constexpr int kQH = 64;   // query columns of a step handled by one softmax warpgroup
 
 // Shared-memory layout of a [128 rows x head_dim] bf16 tile.  head_dim 64: one TMA box, rows of 128 bytes, 128-byte
@@ -59,7 +64,7 @@ constexpr int kQH = 64;   // query columns of a step handled by one softmax warp
 // beyond the tensor and zero-filled by TMA; with a single swizzle mode over the whole row a tile serves as a K-major
 // operand (five 16-element K-steps) and, as an MN-major operand, as ONE N = 80 operand (two and a half 32-element
 // atoms) -- a 64 + 16 split needs two MMA instructions for every product over the head dimension.
-template <int D>
+template <int D, bool kPooled>
 struct BwdCfg {
     static constexpr int kBoxElems = (D == 64) ? 64 : 32;
     static constexpr int kBoxes = (D == 64) ? 1 : 3;
@@ -69,6 +74,21 @@ struct BwdCfg {
     static constexpr uint32_t kSwz = (D == 64) ? kSwizzle128 : kSwizzle64;
     static constexpr uint32_t kSBO = 8 * kRowBytes;               // 8 rows of one box
     static constexpr int kKSteps = D / 16;                        // K-steps of a product over the head dimension
+    // head_dim 64 has room for two buffers of each kind of tile.  At head_dim 80 there are six: they form a pool (kPool), in which a
+    // tile takes whatever buffer is given back next, so that the next unit's K and first Q load during the last step of the
+    // current one, and its V and dO as soon as their predecessors have been read for the last time.  With one buffer for each of K and V
+    // and two for each of Q and dO, a unit of one or two steps waited for its K and V (7000 of its 13 000 clocks) instead.  Which of
+    // the two: see kPoolSeqlen.
+    static constexpr bool kPool = kPooled;
+    static_assert(!kPool || D == 80, "the pool is for a head_dim with six tiles");
+    static constexpr int kSlots = 6;
+    // The last dQ of a unit is drained behind its dV and dK where the next unit's first step has been issued by then and its dV waits
+    // for them (head_dim 64: 1024 segments of 64 rows 504 -> 475 us, 218 of 300 606 -> 590; pooled thumbnails 348 -> 334); where the
+    // next unit starts from an empty pipeline, in front of them (thumbnails 369, behind 391).
+    static constexpr bool kEarlyOut = (D == 64) || kPool;
+    // Units of up to so many steps have their first tiles brought into L2 ahead (head_dim 64: 1024 segments of 64 rows 475 -> 461 us,
+    // 218 of 300 600 -> 580, none at 1024 rows; head_dim 80: more of them cost 163 segments of 512 rows 6 %).
+    static constexpr int kPrefetchSteps = (D == 64) ? 4 : 2;
     static constexpr int kKVBufs = (D == 64) ? 2 : 1;             // 2: the next unit's K/V tiles load during the current unit
     static constexpr int kRing = 2;                               // Q / dO / row-term stages
     // One more 16-element K-step carries the per-query row terms into the two score products (see the staging warp):
@@ -116,8 +136,11 @@ struct BwdParams {
 };
 
 struct BwdBarriers {
-    uint64_t kv_full[2], kv_empty[2], dkv_full, dkv_empty;
-    uint64_t qdo_full[4], qdo_empty[4];
+    uint64_t kv_full[2], kv_empty[2], dkv_full, dkv_empty;   // (kv_full, kv_empty: not kPool)
+    uint64_t qdo_full[4], qdo_empty[4];   // kPool: of the row terms alone
+    // kPool, entry n % 8: the n-th tile loaded is in buffer tile_slot, the n-th buffer given back is back_slot
+    uint64_t tile_full[8], back[8];
+    uint32_t tile_slot[8], back_slot[8];
     uint64_t s_full, s_read, p_full, pv_done, dp_full, ds_full, dq_full, dq_empty;
 };
 
@@ -125,10 +148,10 @@ struct BwdMaps {
     CUtensorMap q, k, v, dout, dq_acc;
 };
 
-template <int D>
+template <int D, bool kPooled>
 __global__ void __maxnreg__(kRegsLaunch)
 attn_bwd_kernel(const __grid_constant__ BwdMaps maps, const BwdParams p) {
-    using Cfg = BwdCfg<D>;
+    using Cfg = BwdCfg<D, kPooled>;
     constexpr int NR = Cfg::kRing;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -152,8 +175,12 @@ attn_bwd_kernel(const __grid_constant__ BwdMaps maps, const BwdParams p) {
         mbar_init(&bars.dkv_full, 1);
         mbar_init(&bars.dkv_empty, 4);
         for (int s = 0; s < 4; ++s) {
-            mbar_init(&bars.qdo_full[s], 2);    // the producer's expect_tx arrival + the staging warp
+            mbar_init(&bars.qdo_full[s], Cfg::kPool ? 1 : 2);   // the producer's expect_tx arrival + the staging warp
             mbar_init(&bars.qdo_empty[s], 1);
+        }
+        for (int i = 0; i < 8; ++i) {
+            mbar_init(&bars.tile_full[i], 1);
+            mbar_init(&bars.back[i], 2);        // the commit behind the last read, and the issuer's arrival behind back_slot
         }
         mbar_init(&bars.s_full, 1);
         mbar_init(&bars.s_read, 8);             // (separate P^T only) S^T is in the softmax warps' registers
@@ -233,6 +260,20 @@ attn_bwd_kernel(const __grid_constant__ BwdMaps maps, const BwdParams p) {
                 for (int bx = 0; bx < Cfg::kBoxes; ++bx)
                     tma_load_3d(dst + bx * Cfg::kBoxBytes, map, bar, bx * Cfg::kBoxElems, head, row);
             };
+            uint32_t n_tiles = 0;
+            auto pool_load = [&](const CUtensorMap* map, int head, int row) {   // kPool: the next tile, into the buffer given back next
+                uint32_t slot = n_tiles;
+                if (n_tiles >= uint32_t(Cfg::kSlots)) {
+                    const uint32_t b = n_tiles - Cfg::kSlots;
+                    if (!mbar_wait(&bars.back[b % 8], (b / 8) & 1, &abort_flag)) return false;
+                    slot = *static_cast<volatile uint32_t*>(&bars.back_slot[b % 8]);
+                }
+                bars.tile_slot[n_tiles % 8] = slot;
+                mbar_expect_tx(&bars.tile_full[n_tiles % 8], Cfg::kTile);
+                load_tile(smem + slot * Cfg::kTile, map, &bars.tile_full[n_tiles % 8], head, row);
+                ++n_tiles;
+                return true;
+            };
             UnitSource source{&units, &abort_flag};
             bool outstanding = false;
             for (int u = int(blockIdx.x); ok; ++unit_it) {
@@ -241,6 +282,36 @@ attn_bwd_kernel(const __grid_constant__ BwdMaps maps, const BwdParams p) {
                 if (!ok || it.kv_len <= 0) break;
                 const int head = it.seg;
                 const int nq = steps_of(it);
+                if (Cfg::kPool) {   // K, Q_0, V, dO_0, Q_1, dO_1, ...: the order in which the issuer comes to need them
+                    const int ask_at = nq > 3 ? nq - 3 : 0;
+                    for (int j = 0; j < nq && ok; ++j) {
+                        if (j == ask_at) {
+                            source.ask();
+                            outstanding = true;
+                        }
+                        const int row = it.kv_start + q_tile_of(it, j, nq) * kBQ;
+                        if (j == 0) ok = pool_load(&maps.k, head, it.row_start);
+                        ok = ok && pool_load(&maps.q, head, row);
+                        if (j == 0) ok = ok && pool_load(&maps.v, head, it.row_start);
+                        ok = ok && pool_load(&maps.dout, head, row);
+                    }
+                    if (!ok) break;
+                    u = source.take(&ok);
+                    outstanding = false;
+                    continue;
+                }
+                // Before its buffers are free, a short unit's first tiles are asked for into L2 (a long unit's Q and dO are there
+                // already, and it computes for so long that its K and V do not matter).
+                if (unit_it > 0 && nq <= Cfg::kPrefetchSteps) {
+                    const int row = it.kv_start + q_tile_of(it, 0, nq) * kBQ;
+#pragma unroll
+                    for (int bx = 0; bx < Cfg::kBoxes; ++bx) {
+                        tma_prefetch_3d(&maps.k, bx * Cfg::kBoxElems, head, it.row_start);
+                        tma_prefetch_3d(&maps.q, bx * Cfg::kBoxElems, head, row);
+                        tma_prefetch_3d(&maps.v, bx * Cfg::kBoxElems, head, it.row_start);
+                        tma_prefetch_3d(&maps.dout, bx * Cfg::kBoxElems, head, row);
+                    }
+                }
                 const int kb = unit_it % Cfg::kKVBufs;            // K/V buffer of this unit
                 uint8_t* kv = smem + kb * (2 * Cfg::kTile);
                 ok = mbar_wait<kSleepAux>(&bars.kv_empty[kb], ((unit_it / Cfg::kKVBufs) & 1) ^ 1, &abort_flag);
@@ -320,7 +391,94 @@ attn_bwd_kernel(const __grid_constant__ BwdMaps maps, const BwdParams p) {
             mpipe_work_item_t it, it_next;
             uint32_t ui = 0;                // next entry of the unit ring
             bool has_unit = next_unit(&units, ui++, &it, lane, &abort_flag), has_next = false;
-            for (; ok && has_unit; has_unit = has_next, it = it_next, ++unit_it) {
+            if (Cfg::kPool) {
+                // The stream of steps runs on across the unit boundary: S^T / dP^T of the next unit's first step are issued inside
+                // this unit's last step, so the softmax warps never see the pipeline drain between units.
+                const uint32_t t_lo0 = umma_desc_lo(sbase, 0), t_mn0 = umma_desc_lo(sbase, Cfg::kBoxBytes);
+                auto at = [&](uint32_t lo0, uint32_t slot) { return lo0 + slot * uint32_t(Cfg::kTile >> 4); };
+                uint32_t n_taken = 0, n_back = 0;
+                auto take = [&](uint32_t* slot) {           // the next tile in the producer's order
+                    const uint32_t e = n_taken % 8;
+                    if (!mbar_wait(&bars.tile_full[e], (n_taken / 8) & 1, &abort_flag)) return false;
+                    *slot = *static_cast<volatile uint32_t*>(&bars.tile_slot[e]);
+                    ++n_taken;
+                    return true;
+                };
+                auto give_back = [&](uint32_t slot) {       // everything issued so far is what still reads the buffer
+                    const uint32_t e = n_back++ % 8;
+                    if (leader) {
+                        bars.back_slot[e] = slot;
+                        mbar_arrive(&bars.back[e]);
+                        umma_commit(&bars.back[e]);
+                    }
+                };
+                uint32_t sk = 0, sv = 0, sq = 0, sdo = 0, sk_n = 0, sv_n = 0, sq_n = 0, sdo_n = 0;
+                auto issue_s = [&](uint32_t c, bool first, uint32_t* k, uint32_t* q) {   // S^T of step c; `first`: of its unit
+                    if (first && !take(k)) return false;
+                    if (!take(q) || !mbar_wait(&bars.qdo_full[c % NR], (c / NR) & 1, &abort_flag)) return false;
+                    tc_fence_after();
+                    issue_kk(Cfg::kColS, at(t_lo0, *k), at(t_lo0, *q), qx_lo0 + extra_off(c));
+                    if (leader) umma_commit(&bars.s_full);
+                    return true;
+                };
+                auto issue_dp = [&](uint32_t c, bool first, bool last, uint32_t* v, uint32_t* d) {   // dP^T of step c; the last of a unit gives V back
+                    if ((first && !take(v)) || !take(d)) return false;
+                    tc_fence_after();
+                    issue_kk(Cfg::kColDP, at(t_lo0, *v), at(t_lo0, *d), dox_lo0 + extra_off(c));
+                    if (leader) umma_commit(&bars.dp_full);
+                    if (leader) umma_commit(&bars.qdo_empty[c % NR]);   // the row terms have been read
+                    if (last) give_back(*v);
+                    return true;
+                };
+                if (has_unit) ok = issue_s(0, true, &sk, &sq) && issue_dp(0, true, steps_of(it) == 1, &sv, &sdo);
+                for (; ok && has_unit; has_unit = has_next, it = it_next, ++unit_it) {
+                    const int nq = steps_of(it);
+                    has_next = false;
+                    for (int j = 0; j < nq; ++j) {
+                        const uint32_t c = sc + j, ph = c & 1;
+                        if (j + 1 == nq) has_next = next_unit(&units, ui++, &it_next, lane, &abort_flag);
+                        const bool cross = j + 1 == nq;      // step j + 1 is the next unit's first
+                        const bool more = !cross || has_next;
+                        const bool last_n = cross ? has_next && steps_of(it_next) == 1 : j + 2 == nq;
+                        ok = mbar_wait(&bars.p_full, ph, &abort_flag);
+                        if (ok && j == 0) ok = mbar_wait(&bars.dkv_empty, (unit_it & 1) ^ 1, &abort_flag);   // the previous epilogue has read both
+                        if (!ok) break;
+                        tc_fence_after();
+                        issue_ts(Cfg::kColDV, Cfg::kColP, Cfg::kPStride, at(t_mn0, sdo), j > 0);             // dV += P^T dO
+                        give_back(sdo);
+                        if (more) {                          // P^T overlays S^T: only now may S^T(j+1) be written
+                            if (!cross) sk_n = sk;
+                            ok = issue_s(c + 1, cross, &sk_n, &sq_n);
+                            if (!ok) break;
+                        }
+                        ok = mbar_wait(&bars.ds_full, ph, &abort_flag);
+                        if (!ok) break;
+                        tc_fence_after();
+                        issue_ts(Cfg::kColDK, Cfg::kColDP, kQH, at(t_mn0, sq), j > 0);                       // dK += dS^T Q
+                        if (cross && leader) umma_commit(&bars.dkv_full);
+                        give_back(sq);
+                        ok = mbar_wait(&bars.dq_empty, ph ^ 1, &abort_flag);   // the reducer has taken dQ(j-1) out of TMEM
+                        if (!ok) break;
+                        tc_fence_after();
+                        if (leader) {                                                                        // dQ(j) = dS K
+                            const uint32_t k_mn = at(t_mn0, sk);
+#pragma unroll
+                            for (int ks = 0; ks < kBT / 16; ++ks)
+                                umma_ss(tmem + Cfg::kColDQ, umma_desc(ds_lo + ks * 128, hi128), umma_desc(k_mn + ks * kMnStep, hi_t), idesc_dq, ks > 0);
+                            umma_commit(&bars.dq_full);
+                        }
+                        if (cross) give_back(sk);
+                        if (more) {                          // after dQ(j): its completion then implies that the dS^T tile has been read
+                            if (!cross) sv_n = sv;
+                            ok = issue_dp(c + 1, cross, last_n, &sv_n, &sdo_n);
+                            if (!ok) break;
+                        }
+                        sk = sk_n; sv = sv_n; sq = sq_n; sdo = sdo_n;
+                    }
+                    sc += nq;
+                }
+            }
+            for (; !Cfg::kPool && ok && has_unit; has_unit = has_next, it = it_next, ++unit_it) {
                 const int nq = steps_of(it);
                 const int kb = unit_it % Cfg::kKVBufs;
                 const uint32_t kvb = sbase + kb * (2 * Cfg::kTile);
@@ -383,6 +541,7 @@ attn_bwd_kernel(const __grid_constant__ BwdMaps maps, const BwdParams p) {
                     if (!ok) break;
                     tc_fence_after();
                     issue_ts(Cfg::kColDK, Cfg::kColDP, kQH, q_mn0 + stage_off(c), j > 0);                              // dK += dS^T Q
+                    if (D == 64 && leader && j + 1 == nq) umma_commit(&bars.dkv_full);
                     if (leader) umma_commit(&bars.qdo_empty[c % NR]);   // also frees the LSE / Delta stage (dS^T(j) has arrived)
                     ok = mbar_wait(&bars.dq_empty, ph ^ 1, &abort_flag);   // the reducer has taken dQ(j-1) out of TMEM
                     if (!ok) break;
@@ -399,7 +558,7 @@ attn_bwd_kernel(const __grid_constant__ BwdMaps maps, const BwdParams p) {
                     }
                 }
                 if (!ok) break;
-                if (leader) umma_commit(&bars.dkv_full);
+                if (D != 64 && leader) umma_commit(&bars.dkv_full);
                 if (leader) umma_commit(&bars.kv_empty[kb]);
                 sc += nq;
                 if (!kStream) has_next = next_unit(&units, ui++, &it_next, lane, &abort_flag);
@@ -596,9 +755,49 @@ attn_bwd_kernel(const __grid_constant__ BwdMaps maps, const BwdParams p) {
         for (uint32_t ui = 0; fetch_unit(ui); ++ui, ++unit_it) {
             const int head = it.seg;
             const int nq = steps_of(it);
+            // dV and dK: before the last dQ is drained or behind it (BwdCfg::kEarlyOut)
+            auto epilogue = [&]() {
+                if (ok) ok = mbar_wait<kSleepAux>(&bars.dkv_full, unit_it & 1, &abort_flag);
+                if (!ok) return;   // (and go on walking the units so that the named barriers stay matched)
+                tc_fence_after();
+                const bool store = r < it.row_len;
+                const int64_t tok = int64_t(it.row_start) + r;
+                __nv_bfloat16* dv_row = p.dv + tok * p.tok_stride_g + int64_t(head) * p.head_stride_g;
+                __nv_bfloat16* dk_row = p.dk + tok * p.tok_stride_g + int64_t(head) * p.head_stride_g;
+#pragma unroll
+                for (int which = 0; which < 2; ++which) {
+                    const uint32_t col = which == 0 ? Cfg::kColDV : Cfg::kColDK;
+                    const float mul = which == 0 ? 1.0f : p.scale;
+                    __nv_bfloat16* row = which == 0 ? dv_row : dk_row;
+#pragma unroll
+                    for (int c0 = 0; c0 < D; c0 += 32) {   // 32 columns per round trip (16 in the D = 80 tail)
+                        uint32_t v[2][16];
+                        const bool two = (c0 + 32 <= D);
+                        tmem_ld16(tmem + lane_base + col + c0, v[0]);
+                        if (two) tmem_ld16(tmem + lane_base + col + c0 + 16, v[1]);
+                        tmem_wait_ld();
+                        if (which == 1 && c0 + 32 >= D) {   // both accumulators have left TMEM: the next unit may overwrite them
+                            tc_fence_before();
+                            __syncwarp();
+                            if (lane == 0) mbar_arrive(&bars.dkv_empty);
+                        }
+#pragma unroll
+                        for (int c8 = 0; c8 < (two ? 4 : 2); ++c8) {
+                            const uint32_t* w = &v[c8 / 2][(c8 & 1) * 8];
+                            uint4 a;
+                            a.x = pack_bf16(__uint_as_float(w[0]) * mul, __uint_as_float(w[1]) * mul);
+                            a.y = pack_bf16(__uint_as_float(w[2]) * mul, __uint_as_float(w[3]) * mul);
+                            a.z = pack_bf16(__uint_as_float(w[4]) * mul, __uint_as_float(w[5]) * mul);
+                            a.w = pack_bf16(__uint_as_float(w[6]) * mul, __uint_as_float(w[7]) * mul);
+                            if (store) *reinterpret_cast<uint4*>(row + c0 + 8 * c8) = a;
+                        }
+                    }
+                }
+            };
             // No early exit inside this loop: the four warps meet at named barriers, so after a time-out
             // they keep walking the (now empty) iterations together instead of leaving one another behind.
             for (int i = 0; i < nq; ++i, ++pc) {
+                if (Cfg::kEarlyOut && i + 1 == nq) epilogue();
                 if (ok) ok = mbar_wait<kSleepAux>(&bars.dq_full, pc & 1, &abort_flag);
                 tc_fence_after();
                 const int q0 = it.kv_start + q_tile_of(it, i, nq) * kBQ;
@@ -632,42 +831,7 @@ attn_bwd_kernel(const __grid_constant__ BwdMaps maps, const BwdParams p) {
                     }
                 }
             }
-            if (ok) ok = mbar_wait<kSleepAux>(&bars.dkv_full, unit_it & 1, &abort_flag);
-            if (!ok) continue;   // keep walking the units so that the named barriers above stay matched
-            tc_fence_after();
-            const bool store = r < it.row_len;
-            const int64_t tok = int64_t(it.row_start) + r;
-            __nv_bfloat16* dv_row = p.dv + tok * p.tok_stride_g + int64_t(head) * p.head_stride_g;
-            __nv_bfloat16* dk_row = p.dk + tok * p.tok_stride_g + int64_t(head) * p.head_stride_g;
-#pragma unroll
-            for (int which = 0; which < 2; ++which) {
-                const uint32_t col = which == 0 ? Cfg::kColDV : Cfg::kColDK;
-                const float mul = which == 0 ? 1.0f : p.scale;
-                __nv_bfloat16* row = which == 0 ? dv_row : dk_row;
-#pragma unroll
-                for (int c0 = 0; c0 < D; c0 += 32) {   // 32 columns per round trip (16 in the D = 80 tail)
-                    uint32_t v[2][16];
-                    const bool two = (c0 + 32 <= D);
-                    tmem_ld16(tmem + lane_base + col + c0, v[0]);
-                    if (two) tmem_ld16(tmem + lane_base + col + c0 + 16, v[1]);
-                    tmem_wait_ld();
-                    if (which == 1 && c0 + 32 >= D) {   // both accumulators have left TMEM: the next unit may overwrite them
-                        tc_fence_before();
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive(&bars.dkv_empty);
-                    }
-#pragma unroll
-                    for (int c8 = 0; c8 < (two ? 4 : 2); ++c8) {
-                        const uint32_t* w = &v[c8 / 2][(c8 & 1) * 8];
-                        uint4 a;
-                        a.x = pack_bf16(__uint_as_float(w[0]) * mul, __uint_as_float(w[1]) * mul);
-                        a.y = pack_bf16(__uint_as_float(w[2]) * mul, __uint_as_float(w[3]) * mul);
-                        a.z = pack_bf16(__uint_as_float(w[4]) * mul, __uint_as_float(w[5]) * mul);
-                        a.w = pack_bf16(__uint_as_float(w[6]) * mul, __uint_as_float(w[7]) * mul);
-                        if (store) *reinterpret_cast<uint4*>(row + c0 + 8 * c8) = a;
-                    }
-                }
-            }
+            if (!Cfg::kEarlyOut) epilogue();
         }
         if (rt == 0) bulk_wait_group<0>();   // all reductions have landed before the CTA exits
     }
@@ -801,11 +965,11 @@ bwd_dq_convert_rope_kernel(const float* __restrict__ acc, __nv_bfloat16* __restr
     *reinterpret_cast<uint4*>(row + kHalf) = make_uint4(ob[0], ob[1], ob[2], ob[3]);
 }
 
-template <int D>
+template <int D, bool kPooled>
 static int32_t launch_bwd(const void* dout, const void* q, const void* k, const void* v, const void* o, void* dq,
                           int64_t ts_qkv, int64_t hs_qkv, int64_t ts_o, int64_t hs_o, int32_t total_tokens,
                           int32_t n_heads, BwdParams prm, float* delta, float* dq_acc, cudaStream_t stream) {
-    using Cfg = BwdCfg<D>;
+    using Cfg = BwdCfg<D, kPooled>;
     BwdMaps m;
     constexpr uint32_t box = Cfg::kBoxElems;
     constexpr int swz = Cfg::kRowBytes;
@@ -815,7 +979,7 @@ static int32_t launch_bwd(const void* dout, const void* q, const void* k, const 
         !make_tensor_map_thd(&m.dout, dout, total_tokens, n_heads, D, ts_o, hs_o, box, kBQ, swz) ||
         !make_tensor_map_thd(&m.dq_acc, dq_acc, total_tokens, n_heads, D, int64_t(n_heads) * D, D, 16, kBQ, 64, 4))
         return MPIPE_ERR_CUDA;
-    if (!ensure_dynamic_smem<attn_bwd_kernel<D>>(Cfg::kSmemAlloc)) return MPIPE_ERR_CUDA;
+    if (!ensure_dynamic_smem<attn_bwd_kernel<D, kPooled>>(Cfg::kSmemAlloc)) return MPIPE_ERR_CUDA;
     const int64_t rows = int64_t(total_tokens) * n_heads;
     constexpr int kPrepassRows = 8 * (32 / (D / 16));   // rows of a block
     const int64_t prepass_blocks = (rows + kPrepassRows - 1) / kPrepassRows;
@@ -826,7 +990,7 @@ static int32_t launch_bwd(const void* dout, const void* q, const void* k, const 
     if (e != cudaSuccess) return MPIPE_ERR_CUDA;
     const int n_units = prm.n_items * prm.n_heads;
     profile_start(kProfileBwdMain, stream);
-    e = launch_kernel_as(true, attn_bwd_kernel<D>, unsigned(n_units), kBwdThreads, Cfg::kSmemAlloc, stream, 1, m, prm);
+    e = launch_kernel_as(true, attn_bwd_kernel<D, kPooled>, unsigned(n_units), kBwdThreads, Cfg::kSmemAlloc, stream, 1, m, prm);
     profile_stop(kProfileBwdMain, stream);
     if (e != cudaSuccess) return MPIPE_ERR_CUDA;
     const bool rope = prm.rope_cos != nullptr;
@@ -932,10 +1096,13 @@ static int32_t run_bwd(const float* rope_cos, const float* rope_sin, const void*
     prm.status_buf = status_buf;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if (head_dim == 64)
-        return launch_bwd<64>(dout, q, k, v, o, dq, tok_stride_qkv, head_stride_qkv, tok_stride_o, head_stride_o,
-                              total_tokens, n_heads, prm, delta, dq_acc, st);
-    return launch_bwd<80>(dout, q, k, v, o, dq, tok_stride_qkv, head_stride_qkv, tok_stride_o, head_stride_o,
-                          total_tokens, n_heads, prm, delta, dq_acc, st);
+        return launch_bwd<64, false>(dout, q, k, v, o, dq, tok_stride_qkv, head_stride_qkv, tok_stride_o, head_stride_o,
+                                     total_tokens, n_heads, prm, delta, dq_acc, st);
+    if (max_seqlen <= kPoolSeqlen && int64_t(n_bwd_items) * n_heads > sm_count())
+        return launch_bwd<80, true>(dout, q, k, v, o, dq, tok_stride_qkv, head_stride_qkv, tok_stride_o, head_stride_o,
+                                    total_tokens, n_heads, prm, delta, dq_acc, st);
+    return launch_bwd<80, false>(dout, q, k, v, o, dq, tok_stride_qkv, head_stride_qkv, tok_stride_o, head_stride_o,
+                                 total_tokens, n_heads, prm, delta, dq_acc, st);
 }
 
 int32_t mpipe_varlen_attn_bwd(const void* dout, const void* q, const void* k, const void* v, const void* o,
