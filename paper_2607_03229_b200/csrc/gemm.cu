@@ -20,11 +20,13 @@
 //               gradient of GELU needs) arrives in the box by TMA before the accumulator is ready, the result replaces it in
 //               place, and one TMA store takes it out.  No barrier between warps: with one staging box per warpgroup and two
 //               named barriers per 32 columns the epilogue of the GELU projections was longer than their main loop.
-// Small problems (fewer tiles than pairs): a cluster of `splits` pairs shares a tile, each taking a part of the contraction; the
-// partial results meet in shared memory (every pair finishes the chunks it owns from the others' fp32 partials).
+// A row of a projection is summed over the contraction in one order whatever the number of rows: an image's tokens come out with the same
+// bits alone and in any microbatch.  So the contraction is never split over pairs, though two pairs to a tile of a few hundred rows are
+// up to 4 us sooner done with an input gradient (300 x 4096 -> 1024 11.2 against 13.8 us; forward of 777 rows 12.5 against 11.7): the
+// halves meet in another order than the one accumulator of a large microbatch adds in.
 // Measured against the one-CTA 128 x 256 kernel with warpgroup-wide staging that this replaces (us, M = 50 439): fc1 + GELU
 // 1024 -> 4096 398 -> 325, its gradient with GELU' 480 -> 383, attention output + residual 115 -> 90, QKV 241 -> 221 (1430
-// TFLOP/s), weight gradient 1024 x 4096 348 -> 292; M = 777: fc2 27.9 -> 13.4 (split), output projection 14.4 -> 7.2, weight
+// TFLOP/s), weight gradient 1024 x 4096 348 -> 292; M = 777: fc2 27.9 -> 11.7, output projection 14.4 -> 7.2, weight
 // gradient 1024 x 4096 34 -> 12.
 // Every mbarrier wait is bounded (status MPIPE_ERR_TIMEOUT), as in the attention kernels.
 #include <cuda_bf16.h>
@@ -47,11 +49,7 @@ constexpr int kGemmRing = 160 * 1024, kGemmMaxStages = 8;     // 5 stages at BN 
 constexpr int kGemmBox = 32 * 128;                            // [32 rows][128 bytes] staging box of one warp
 constexpr int kGemmSmemOut = kGemmRing;                       // 8 warps x 2 boxes
 constexpr int kGemmSmem = kGemmSmemOut + 8 * 2 * kGemmBox + 1024;
-constexpr int kGemmMaxSplits = 2;   // four pairs per tile never beat two (measured)
-// a tile's fp32 partials from the other splits: (splits - 1) senders x (BN / 64 / splits) chunks of [16 column groups][128 rows][16 B]
-constexpr int kGemmPartChunk = 16 * 128 * 16;
 static_assert(kGemmSmem <= 227 * 1024, "shared memory budget");
-static_assert((kGemmMaxSplits - 1) * 2 * kGemmPartChunk <= kGemmSmemOut, "partials reuse the stages");
 
 enum { kEpiPlain = 0, kEpiGelu = 1, kEpiGeluGrad = 2 };
 
@@ -63,7 +61,7 @@ struct GemmParams {
     int32_t wide;                    // map_a / map_w bring all atoms of a stage with one copy (make_tensor_map_chunks)
     int32_t settled_w;               // the second operand was complete before the previous kernel of the stream started
     int32_t tiles_m, tiles_n;
-    int32_t splits;                  // pairs that share a tile's contraction (weight gradient: parts of the token range)
+    int32_t splits;                  // weight gradient: parts of the token range
     const __nv_bfloat16* bias;       // [N] or null
     const __nv_bfloat16* direct_res; // [M, ldr] or null: residual read by the epilogue threads (when the boxes carry something else)
     int64_t ldr;
@@ -96,9 +94,7 @@ linear_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
     __shared__ int abort_flag;
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const uint32_t crank = cluster_ctarank();
-    const int half = int(crank & 1);                          // which 128 rows of A / half of B this CTA holds
-    const uint32_t lead = crank & ~1u;                        // the pair's issuing CTA
+    const int half = int(cluster_ctarank());                  // which 128 rows of A / half of B this CTA holds; 0: the issuing CTA
     if (tid == 0) {
         abort_flag = 0;
         for (int s = 0; s < kGemmMaxStages; ++s) {
@@ -145,14 +141,12 @@ linear_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
     const int kpb = kMode == 2 ? 1 : p.kpb, nk = (p.K + kpb * kGemmBK - 1) / (kpb * kGemmBK);   // stages of the whole contraction
     const int n_out_tiles = p.tiles_m * p.tiles_n;
     const int n_items = n_out_tiles * (kMode == 2 ? p.splits : 1);
-    const int ksplit = kMode == 2 ? 1 : p.splits;             // pairs per cluster
-    const int cid = int(blockIdx.x) / (2 * ksplit), n_clusters = int(gridDim.x) / (2 * ksplit);
-    const int my_split = int(crank >> 1);
+    const int cid = int(blockIdx.x) / 2, n_clusters = int(gridDim.x) / 2;
     // work item -> output tile and range of contraction blocks (weight gradient: the split index is the slow one, so that the
     // pairs of a wave work on the same token range and share its dY and X rows through L2)
     auto tile_of = [&](int t) { return kMode == 2 ? t % n_out_tiles : t; };
-    auto kb_lo_of = [&](int t) { return int((long long)(kMode == 2 ? t / n_out_tiles : my_split) * nk / p.splits); };
-    auto kb_hi_of = [&](int t) { return int((long long)(kMode == 2 ? t / n_out_tiles + 1 : my_split + 1) * nk / p.splits); };
+    auto kb_lo_of = [&](int t) { return kMode == 2 ? int((long long)(t / n_out_tiles) * nk / p.splits) : 0; };
+    auto kb_hi_of = [&](int t) { return kMode == 2 ? int((long long)(t / n_out_tiles + 1) * nk / p.splits) : nk; };
     // weight gradient: the tiles of one row of tiles all load the row's first operand; block kb of it is summed by tile kb mod tiles_n
     // (by one tile alone, that tile's delayed stages were 4 us of a 26 us launch)
     const bool summing = kMode == 2 && p.colsum != nullptr;
@@ -171,7 +165,7 @@ linear_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
         if (lane == 0) {
             const bool is_a = warp == 0;
             const uint32_t tx = 2u * uint32_t(stage_bytes);   // both CTAs' boxes; out-of-range elements are zero-filled and still counted
-            const uint32_t bar0 = mapa_u32(smem_u32(&bars.full[0]), lead);
+            const uint32_t bar0 = mapa_u32(smem_u32(&bars.full[0]), 0);
             uint32_t s = 0, ph = 1;                           // ring position; parity of the "empty" phase awaited
             bool ok = true;
             for (int t = cid; t < n_items && ok; t += n_clusters) {
@@ -219,7 +213,7 @@ linear_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
         const uint32_t sbase = smem_u32(smem);
         constexpr uint32_t hi128 = umma_desc_hi(1024, kSwizzle128);
         const uint32_t idesc = umma_idesc_bf16(2 * kGemmBM, bn, kMode == 2 ? 1 : 0, kMode != 0 ? 1 : 0);
-        const uint16_t pair_mask = uint16_t(3u << lead);
+        constexpr uint16_t pair_mask = 3;
         uint32_t s = 0, ph = 0, tile_it = 0;
         bool ok = true;
         for (int t = cid; t < n_items && ok; t += n_clusters, ++tile_it) {
@@ -316,7 +310,7 @@ linear_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
         const int ew = warp - 4, wg = ew >> 2, quarter = warp & 3;
         const uint32_t lane_base = uint32_t(quarter * 32) << 16;
         uint8_t* boxes = smem + kGemmSmemOut + ew * 2 * kGemmBox;
-        uint32_t acc_empty_addr[2] = {mapa_u32(smem_u32(&bars.acc_empty[0]), lead), mapa_u32(smem_u32(&bars.acc_empty[1]), lead)};
+        uint32_t acc_empty_addr[2] = {mapa_u32(smem_u32(&bars.acc_empty[0]), 0), mapa_u32(smem_u32(&bars.acc_empty[1]), 0)};
         const int n_chunks = bn >> 6;
         uint32_t tile_it = 0, bc = 0;   // bc: boxes used so far by this warp; box = bc & 1
         // Arrive at the last meeting of the cluster as soon as this warp will touch neither TMEM nor the other CTA any more, under
@@ -333,19 +327,17 @@ linear_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
             const int m0 = (tile_of(t) / p.tiles_n) * 2 * kGemmBM + half * kGemmBM + quarter * 32;   // first row of this warp
             const int n0 = (tile_of(t) % p.tiles_n) * bn;
             const bool rows_in = m0 < p.M;
-            // the chunks this warp finishes: wg, wg + 2, ... of the tile; with a split contraction, those its pair owns
-            const int own = n_chunks / ksplit;                                // chunks per pair
-            auto chunk_of = [&](int i) { return ksplit == 1 ? i : my_split * own + i; };
-            auto active = [&](int i) { return rows_in && n0 + 64 * chunk_of(i) < p.N; };
+            // the chunks this warp finishes: wg, wg + 2, ... of the tile
+            auto active = [&](int c) { return rows_in && n0 + 64 * c < p.N; };
             if (kMode != 2 && p.side && ok) {   // the side operand of both chunks, before the accumulator is ready
                 uint32_t b = bc;
-                for (int i = wg; i < own; i += 2) {
-                    if (!active(i)) continue;
+                for (int c = wg; c < n_chunks; c += 2) {
+                    if (!active(c)) continue;
                     if (lane == 0) {
-                        if (i == wg) bulk_wait_group_read<1>();   // the store that used this box two boxes ago has read it
+                        if (c == wg) bulk_wait_group_read<1>();   // the store that used this box two boxes ago has read it
                         else bulk_wait_group_read<0>();
                         mbar_expect_tx(&bars.side_full[ew][b & 1], kGemmBox);
-                        tma_load_3d(boxes + (b & 1) * kGemmBox, &map_s, &bars.side_full[ew][b & 1], n0 + 64 * chunk_of(i), 0, m0);
+                        tma_load_3d(boxes + (b & 1) * kGemmBox, &map_s, &bars.side_full[ew][b & 1], n0 + 64 * c, 0, m0);
                     }
                     ++b;
                 }
@@ -354,9 +346,9 @@ linear_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
             // other, each as long as a value from L2 or HBM takes (epilogue of one 64-column chunk 1.9 -> 1.2 us; 777 x 1024 -> 3072
             // 12.2 -> 11.4 us, -> 1024 7.7 -> 7.4).
             uint4 bias[8];
-            auto load_bias = [&](int i) {
-                if (kMode != 0 || p.bias == nullptr || !active(i)) return;
-                const int n = n0 + 64 * chunk_of(i);
+            auto load_bias = [&](int c) {
+                if (kMode != 0 || p.bias == nullptr || !active(c)) return;
+                const int n = n0 + 64 * c;
 #pragma unroll
                 for (int g = 0; g < 8; ++g)
                     if (n + 8 * g < p.N) bias[g] = __ldg(reinterpret_cast<const uint4*>(p.bias + n + 8 * g));   // (N is a multiple of 8)
@@ -364,28 +356,6 @@ linear_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
             load_bias(wg);
             if (ok) ok = mbar_wait(&bars.acc_full[acc], (tile_it >> 1) & 1, &abort_flag);
             tc_fence_after();
-            if (kMode != 2 && ksplit > 1) {
-                // every pair of the cluster is past its main loop: the stages of all of them can take partials
-                __syncwarp();
-                cluster_sync_all();
-                for (int c = wg; c < n_chunks; c += 2) {
-                    const int owner = c / own;
-                    if (owner == my_split) continue;
-                    const int slot = (my_split < owner ? my_split : my_split - 1) * own + (c - owner * own);
-                    const uint32_t dst = mapa_u32(smem_u32(smem + slot * kGemmPartChunk + (quarter * 32 + lane) * 16), uint32_t(2 * owner + half));
-#pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        uint32_t v[32];
-                        tmem_ld32(tacc + c * 64 + h * 32, v);
-                        tmem_wait_ld();
-#pragma unroll
-                        for (int g = 0; g < 8; ++g)
-                            st_cluster_v4(dst + (h * 8 + g) * 2048, v[4 * g], v[4 * g + 1], v[4 * g + 2], v[4 * g + 3]);
-                    }
-                }
-                __syncwarp();
-                cluster_sync_all();
-            }
             bool released = false;
             auto release = [&]() {   // this warp has read its part of the accumulator
                 tc_fence_before();
@@ -395,10 +365,9 @@ linear_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
                 if (t + n_clusters >= n_items) leave();
             };
 #pragma unroll 1
-            for (int i = wg; i < own; i += 2) {
-                const int c = chunk_of(i);
-                const bool last = i + 2 >= own;
-                if (!active(i) || !ok) continue;
+            for (int c = wg; c < n_chunks; c += 2) {
+                const bool last = c + 2 >= n_chunks;
+                if (!active(c) || !ok) continue;
                 const int n = n0 + 64 * c;
                 uint32_t v[64];
                 tmem_ld32(tacc + c * 64, *reinterpret_cast<uint32_t(*)[32]>(&v[0]));
@@ -423,19 +392,6 @@ linear_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
                         }
                     }
                     continue;
-                }
-                if (ksplit > 1) {   // the other pairs' partials of this chunk
-                    for (int s = 0; s < ksplit - 1; ++s) {
-                        const uint4* part = reinterpret_cast<const uint4*>(smem + (s * own + i) * kGemmPartChunk) + quarter * 32 + lane;
-#pragma unroll
-                        for (int g = 0; g < 16; ++g) {
-                            const uint4 q = part[g * 128];
-                            v[4 * g] = __float_as_uint(__uint_as_float(v[4 * g]) + __uint_as_float(q.x));
-                            v[4 * g + 1] = __float_as_uint(__uint_as_float(v[4 * g + 1]) + __uint_as_float(q.y));
-                            v[4 * g + 2] = __float_as_uint(__uint_as_float(v[4 * g + 2]) + __uint_as_float(q.z));
-                            v[4 * g + 3] = __float_as_uint(__uint_as_float(v[4 * g + 3]) + __uint_as_float(q.w));
-                        }
-                    }
                 }
                 uint8_t* box = boxes + (bc & 1) * kGemmBox;          // result (and side operand, in place)
                 uint8_t* pre_box = boxes + ((bc & 1) ^ 1) * kGemmBox; // pre-activation, when it is stored too
@@ -485,7 +441,7 @@ linear_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
                     }
                     *slot = make_uint4(pack_bf16(f[0].x, f[0].y), pack_bf16(f[1].x, f[1].y), pack_bf16(f[2].x, f[2].y), pack_bf16(f[3].x, f[3].y));
                 }
-                if (!last) load_bias(i + 2);
+                if (!last) load_bias(c + 2);
                 fence_async_smem();
                 __syncwarp();
                 if (lane == 0) {
@@ -500,27 +456,18 @@ linear_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
         if (lane == 0) bulk_wait_group_read<0>();   // shared memory must outlive the copy engine's reads
         __syncwarp();
     }
-    if (kMode != 2 && ksplit > 1 && warp < 4) {   // the two meetings of the split contraction
-        __syncwarp();
-        cluster_sync_all();
-        cluster_sync_all();
-    }
-
     __syncwarp();
     if (!left) {
         tc_fence_before();
         cluster_arrive();
     }
-    cluster_wait();       // neither CTA frees TMEM or leaves while the pair's MMAs or the cluster's stores may still touch it
+    cluster_wait();       // neither CTA frees TMEM or leaves while the pair's MMAs or arrivals may still touch it
     if (warp == 2) tmem_dealloc_pair(tmem, 512);
     if (tid == 0 && abort_flag) report_status(p.status_buf, MPIPE_ERR_TIMEOUT, int32_t(blockIdx.x));
 }
 
-// ---- choice of tile width and contraction split, in SM clocks; the constants are fitted to graph-replayed sweeps of every width
-// and split over M 86..12000 and hidden 320..1280 (the pick is within 5 % of the best measured in all but a few of them).
-struct GemmShape {
-    int bn, splits;
-};
+// ---- choice of tile width, in SM clocks; the constants are fitted to graph-replayed sweeps of every width over M 86..12000 and
+// hidden 320..1280.
 // 64 of the contraction of a 256 x bn tile, by the waves of tiles there are: 2 bn clocks of tensor pipe at bn 256 and 192 plus what
 // the other SMs' operand traffic adds; below, first the issuing thread's instructions, then (with every SM loading) that traffic.
 static double gemm_stage_clk(int bn, long long waves) {
@@ -538,20 +485,20 @@ static int gemm_stages(int bn, int kpb) {
     const int n = kGemmRing / (kpb * (kGemmABytes + 64 * bn));
     return n < kGemmMaxStages ? n : kGemmMaxStages;
 }
-// Clusters of `ctas` CTAs that fit on the current device at once (the GPCs' SM counts limit clusters of more than two).
+// CTA pairs that fit on the current device at once.
 template <auto kernel>
-static int max_clusters(int ctas, int threads = gemm_threads(0)) {
-    static int cached[64][2 * kGemmMaxSplits + 1] = {};
+static int max_pairs(int threads) {
+    static int cached[64] = {};
     int dev = -1;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
-    if (cached[dev][ctas] == 0) {
+    if (cached[dev] == 0) {
         cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(unsigned(ctas));
+        cfg.gridDim = dim3(2);
         cfg.blockDim = dim3(unsigned(threads));
         cfg.dynamicSmemBytes = kGemmSmem;
         cudaLaunchAttribute at[1];
         at[0].id = cudaLaunchAttributeClusterDimension;
-        at[0].val.clusterDim.x = unsigned(ctas);
+        at[0].val.clusterDim.x = 2;
         at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
         cfg.attrs = at;
         cfg.numAttrs = 1;
@@ -560,38 +507,31 @@ static int max_clusters(int ctas, int threads = gemm_threads(0)) {
             (void)cudaGetLastError();
             n = 0;
         }
-        cached[dev][ctas] = n > 0 ? n : -1;
+        cached[dev] = n > 0 ? n : -1;
     }
-    return cached[dev][ctas] > 0 ? cached[dev][ctas] : 0;
+    return cached[dev] > 0 ? cached[dev] : 0;
 }
-template <auto kernel>
-static GemmShape choose_shape(int b_mode, bool gelu, int M, int N, int K) {
+static int choose_width(int mode, bool gelu, int pairs, int M, int N, int K) {
     const int nk = cdiv(K, kGemmBK), tiles_m = cdiv(M, 2 * kGemmBM);
-    const int pairs = max_clusters<kernel>(2) > 0 ? max_clusters<kernel>(2) : 1;
-    GemmShape best = {kGemmMaxBN, 1};
+    int best = kGemmMaxBN;
     double best_clk = 1e30;
     for (int bn = kGemmMaxBN; bn >= 64; bn -= 64) {
-        if (b_mode == 1 && (bn % 128) != 0) continue;      // MN-major B: each CTA holds whole 64-column atoms
-        const long long tiles = (long long)tiles_m * cdiv(N, bn);
-        for (int sp = 1; sp <= kGemmMaxSplits; ++sp) {
-            if (sp > 1 && ((bn / 64) % sp != 0 || nk < 4 * sp || tiles > max_clusters<kernel>(2 * sp))) continue;
-            const long long waves = sp > 1 ? 1 : (tiles + pairs - 1) / pairs;
-            const double clk = waves * cdiv(nk, sp) * gemm_stage_clk(bn, waves) + 1000.0 * (waves - 1) + gemm_fixed_clk(bn, gelu) +
-                               (sp == 1 ? 0.0 : bn == 128 ? 4500.0 : 2300.0);
-            if (clk < best_clk) {
-                best_clk = clk;
-                best = {bn, sp};
-            }
+        if (mode == 1 && (bn % 128) != 0) continue;        // MN-major B: each CTA holds whole 64-column atoms
+        const long long tiles = (long long)tiles_m * cdiv(N, bn), waves = (tiles + pairs - 1) / pairs;
+        const double clk = waves * nk * gemm_stage_clk(bn, waves) + 1000.0 * (waves - 1) + gemm_fixed_clk(bn, gelu);
+        if (clk < best_clk) {
+            best_clk = clk;
+            best = bn;
         }
     }
     return best;
 }
 
 template <auto kernel>
-static int32_t launch_gemm(int threads, int cluster_ctas, int grid, const CUtensorMap& map_a, const CUtensorMap& map_w, const CUtensorMap& map_c,
+static int32_t launch_gemm(int threads, int pairs, const CUtensorMap& map_a, const CUtensorMap& map_w, const CUtensorMap& map_c,
                            const CUtensorMap& map_s, const CUtensorMap& map_u, const GemmParams& p, cudaStream_t st) {
     profile_start(kProfileLinear, st);
-    const cudaError_t e = launch_kernel(kernel, unsigned(grid), unsigned(threads), kGemmSmem, st, unsigned(cluster_ctas), map_a, map_w, map_c,
+    const cudaError_t e = launch_kernel(kernel, unsigned(2 * pairs), unsigned(threads), kGemmSmem, st, 2u, map_a, map_w, map_c,
                                         map_s, map_u, p);
     profile_stop(kProfileLinear, st);
     return e == cudaSuccess && cudaGetLastError() == cudaSuccess ? MPIPE_OK : MPIPE_ERR_CUDA;
@@ -611,10 +551,11 @@ struct LinearCall {   // one forward projection or input gradient
 template <int kMode, int kEpi>
 static int32_t launch_linear_as(const LinearCall& x, cudaStream_t st) {
     if (!ensure_dynamic_smem<linear_kernel<kMode, kEpi>>(kGemmSmem)) return MPIPE_ERR_CUDA;
-    const GemmShape shape = choose_shape<linear_kernel<kMode, kEpi>>(kMode, kEpi != kEpiPlain, x.M, x.n_out, x.n_contract);
+    const int pairs = max_pairs<linear_kernel<kMode, kEpi>>(gemm_threads(kMode));
+    if (pairs <= 0) return MPIPE_ERR_CUDA;
     GemmParams p = {};
     p.M = x.M; p.N = x.n_out; p.K = x.n_contract;
-    p.bn = shape.bn;
+    p.bn = choose_width(kMode, kEpi != kEpiPlain, pairs, x.M, x.n_out, x.n_contract);
     // Operands whose 64-element atoms are all whole take one copy per stage; the narrow tiles, whose loop is bound by the
     // producers' and the issuer's instructions and not by the MMAs, then also take two blocks of the contraction per stage
     // (777 x 1024 x 1024 at bn 64: 360 -> 268 clocks per block, 9.1 -> 7.8 us).
@@ -627,7 +568,7 @@ static int32_t launch_linear_as(const LinearCall& x, cudaStream_t st) {
         p.ahead_bytes[i] = x.ahead.bytes[i];
     }
     p.stages = gemm_stages(p.bn, p.kpb);
-    p.splits = shape.splits;
+    p.splits = 1;
     p.tiles_m = cdiv(x.M, 2 * kGemmBM);
     p.tiles_n = cdiv(x.n_out, p.bn);
     p.bias = static_cast<const __nv_bfloat16*>(x.bias);
@@ -656,12 +597,8 @@ static int32_t launch_linear_as(const LinearCall& x, cudaStream_t st) {
                          : make_tensor_map_thd(&map_w, x.w, x.n_contract, 1, x.n_out, x.ldw, x.ldw, 64, kGemmBK, 128));
     if (!ok) return MPIPE_ERR_CUDA;
     const long long tiles = (long long)p.tiles_m * p.tiles_n;
-    const int cap = max_clusters<linear_kernel<kMode, kEpi>>(2 * p.splits);
-    if (cap <= 0) return MPIPE_ERR_CUDA;
-    if (tiles > 0x7fffffffLL / (2 * kGemmMaxSplits)) return MPIPE_ERR_UNSUPPORTED;
-    // a split contraction takes one cluster per tile (its CTAs meet once at a cluster barrier), everything else is persistent
-    const int clusters = int(p.splits > 1 || tiles < cap ? tiles : cap);
-    return launch_gemm<linear_kernel<kMode, kEpi>>(gemm_threads(kMode), 2 * p.splits, clusters * 2 * p.splits, map_a, map_w, map_c, map_s, map_u, p, st);
+    if (tiles > 0x7fffffffLL / 2) return MPIPE_ERR_UNSUPPORTED;
+    return launch_gemm<linear_kernel<kMode, kEpi>>(gemm_threads(kMode), int(tiles < pairs ? tiles : pairs), map_a, map_w, map_c, map_s, map_u, p, st);
 }
 
 // Shared host side of the two entry points: checks, then the instantiation the epilogue needs.
@@ -699,9 +636,9 @@ static int32_t launch_wgrad(const void* dy, const void* x, float* dw, float* db,
     CUtensorMap map_a, map_w, map_c;
     if (!make_tensor_map_thd(&map_c, dw, n_rows, 1, n_cols, lddw, lddw, 32, 32, 128, 4)) return MPIPE_ERR_CUDA;
     if (!ensure_dynamic_smem<linear_kernel<2, kEpiPlain>>(kGemmSmem)) return MPIPE_ERR_CUDA;
-    const int pairs = max_clusters<linear_kernel<2, kEpiPlain>>(2, gemm_threads(2));
+    const int pairs = max_pairs<linear_kernel<2, kEpiPlain>>(gemm_threads(2));
     if (pairs <= 0) return MPIPE_ERR_CUDA;
-    // Tile width and split of the token range, in SM clocks (fitted like choose_shape's constants).  A pair's fp32 tile leaves at
+    // Tile width and split of the token range, in SM clocks (fitted like choose_width's constants).  A pair's fp32 tile leaves at
     // about 12 bytes per clock and SM (the L2's rate of fp32 reductions with every SM adding) beside the next item's main loop.
     // A long token range runs into the power limit, where the sum of the work counts and not its spread over the pairs: no
     // estimate goes below the work at 68 % of the tensor peak, and among equals the fewest splits (least reduction traffic) win
@@ -742,8 +679,7 @@ static int32_t launch_wgrad(const void* dy, const void* x, float* dw, float* db,
     }
     p.status_buf = status_buf;
     const long long items = (long long)p.tiles_m * p.tiles_n * p.splits;
-    const int clusters = int(items < pairs ? items : pairs);
-    return launch_gemm<linear_kernel<2, kEpiPlain>>(gemm_threads(2), 2, 2 * clusters, map_a, map_w, map_c, map_c, map_c, p, st);
+    return launch_gemm<linear_kernel<2, kEpiPlain>>(gemm_threads(2), int(items < pairs ? items : pairs), map_a, map_w, map_c, map_c, map_c, p, st);
 }
 
 // Weight and bias gradient of a projection in one launch.
