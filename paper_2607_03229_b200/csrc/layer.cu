@@ -479,7 +479,18 @@ size_t mpipe_encoder_layer_workspace_bytes(int32_t n_tokens, int32_t hidden, int
            2 * align256(t * ffn * 2);
 }
 
-// What the kernels behind a projection will read (n elements each).  A small microbatch reads every weight once and meets it cold: 24
+// The four matrices of a layer, looked at before anything is launched: a projection asks for matrices of the kernels behind it by bulk
+// prefetches, which take 16-byte aligned addresses only.  The same answers as the projections themselves give.
+static int32_t layer_matrices_ok(const mpipe_layer_weights_t& w) {
+    const void* const m[4] = {w.w_qkv, w.w_o, w.w_fc1, w.w_fc2};
+    for (const void* p : m)
+        if (p == nullptr) return MPIPE_ERR_INVALID_ARG;
+    for (const void* p : m)
+        if (!mpipe::aligned16(p)) return MPIPE_ERR_UNSUPPORTED;
+    return MPIPE_OK;
+}
+
+// What the kernels behind a projection will read (n elements each; 16-byte aligned, see layer_matrices_ok).  A small microbatch reads every weight once and meets it cold: 24
 // layers of 25 MB, one image of 777 tokens, 1676 -> 1640 us; 1500 tokens, forward of 12 layers 1109 -> 1083.  From some
 // thousand tokens on a weight is read by many tiles and its first read is nothing.
 static mpipe::LayerAhead layer_ahead(int32_t n_tokens, const void* w0, size_t n0, const void* w1 = nullptr, size_t n1 = 0) {
@@ -508,6 +519,7 @@ static int32_t layer_fwd(const mpipe_layer_weights_t* next, const void* x, void*
     const int32_t head_dim = hidden / n_heads;
     if (workspace == nullptr || workspace_bytes < mpipe_encoder_layer_workspace_bytes(n_tokens, hidden, ffn)) return MPIPE_ERR_WORKSPACE;
     if ((reinterpret_cast<uintptr_t>(workspace) & 255u) != 0) return MPIPE_ERR_UNSUPPORTED;
+    if (const int32_t bad = layer_matrices_ok(*w)) return bad;
     const size_t t = size_t(n_tokens);
     uint8_t* ws = static_cast<uint8_t*>(workspace);
     uint8_t* norm = ws;               ws += align256(t * hidden * 2);
@@ -580,6 +592,7 @@ int32_t mpipe_encoder_layer_bwd(const void* dy, const void* x, void* dx, const m
     if (workspace == nullptr || workspace_bytes < mpipe_encoder_layer_bwd_workspace_bytes(n_tokens, hidden, n_heads, ffn))
         return MPIPE_ERR_WORKSPACE;
     if (((reinterpret_cast<uintptr_t>(workspace) | reinterpret_cast<uintptr_t>(fwd_workspace)) & 255u) != 0) return MPIPE_ERR_UNSUPPORTED;
+    if (const int32_t bad = layer_matrices_ok(*w)) return bad;
     const int32_t head_dim = hidden / n_heads;
     const size_t t = size_t(n_tokens);
     const int64_t h = hidden, h3 = 3 * int64_t(hidden), f = ffn;
@@ -648,6 +661,8 @@ int32_t mpipe_encoder_fwd(const void* x, void* y, const mpipe_layer_weights_t* l
     if (x == nullptr || y == nullptr || (mode == MPIPE_ENC_TRAINED && lse == nullptr)) return MPIPE_ERR_INVALID_ARG;
     if (workspace == nullptr || workspace_bytes < mpipe_encoder_workspace_bytes(n_layers, n_tokens, hidden, ffn, mode)) return MPIPE_ERR_WORKSPACE;
     if ((reinterpret_cast<uintptr_t>(workspace) & 255u) != 0) return MPIPE_ERR_UNSUPPORTED;
+    for (int l = 0; l < n_layers; ++l)   // (a layer's last projection asks for the next layer's first matrix)
+        if (const int32_t bad = layer_matrices_ok(layers[l])) return bad;
     const size_t per_layer = mpipe_encoder_layer_workspace_bytes(n_tokens, hidden, ffn);
     const size_t act = align256(size_t(n_tokens) * hidden * 2);
     uint8_t* ws = static_cast<uint8_t*>(workspace);

@@ -1,0 +1,64 @@
+"""What a layer or a layer stack refuses, it refuses before anything is launched: on a machine without a device a launch would be
+MPIPE_ERR_CUDA.  The addresses are never read."""
+import ctypes
+
+import pytest
+import torch
+
+from paper_2607_03229_b200 import binding as B
+from paper_2607_03229_b200 import build as build_mod
+
+# (with a device a missing check would launch kernels on made-up addresses)
+pytestmark = pytest.mark.skipif(torch.cuda.is_available(), reason="only where nothing can be launched")
+
+T, HIDDEN, H, FFN, SCALE, EPS = 300, 256, 4, 1024, 0.125, 1e-6
+WS = 1 << 40
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    build_mod.build()
+
+
+def _struct(cls, n, l, **changed):
+    s = (cls * n)()
+    for i in range(n):
+        for j, (name, _) in enumerate(cls._fields_):
+            setattr(s[i], name, 0x10000000 * (1 + i) + 0x100000 * j)
+    for name, value in changed.items():
+        setattr(s[l], name, value)
+    return s
+
+
+def _calls(weights, n, grads=None, rope=(None, None), mode=B.TRAINED):
+    """The status of every entry point that runs these layers (the single-layer ones: the last layer alone)."""
+    lib, last = B.load(), ctypes.addressof(weights) + (n - 1) * ctypes.sizeof(B.LayerWeights)
+    g = _struct(B.LayerGrads, n, 0) if grads is None else grads
+    last_g = ctypes.addressof(g) + (n - 1) * ctypes.sizeof(B.LayerGrads)
+    a, plan = 0x70000000, (0x71000000, 1, T, 0x71100000, 3)
+    fwd = (SCALE, EPS, *rope, mode, 0x72000000, 0x73000000, WS, None, None)
+    bwd = (SCALE, EPS, *rope, mode, 0x72000000, 0x73000000, 0x74000000, WS, None, None)
+    return {"layer_fwd": lib.mpipe_encoder_layer_fwd(a, a, last, # (with a device a missing check would launch kernels on made-up addresses)
+pytestmark = pytest.mark.skipif(torch.cuda.is_available(), reason="only where nothing can be launched")
+
+T, HIDDEN, H, FFN, *plan, *fwd),
+            "fwd": lib.mpipe_encoder_fwd(a, a, ctypes.addressof(weights), n, # (with a device a missing check would launch kernels on made-up addresses)
+pytestmark = pytest.mark.skipif(torch.cuda.is_available(), reason="only where nothing can be launched")
+
+T, HIDDEN, H, FFN, *plan, *fwd),
+            "layer_bwd": lib.mpipe_encoder_layer_bwd(a, a, a, last, last_g, # (with a device a missing check would launch kernels on made-up addresses)
+pytestmark = pytest.mark.skipif(torch.cuda.is_available(), reason="only where nothing can be launched")
+
+T, HIDDEN, H, FFN, *plan, *bwd),
+            "bwd": lib.mpipe_encoder_bwd(a, a, a, ctypes.addressof(weights), ctypes.addressof(g), n, # (with a device a missing check would launch kernels on made-up addresses)
+pytestmark = pytest.mark.skipif(torch.cuda.is_available(), reason="only where nothing can be launched")
+
+T, HIDDEN, H, FFN, *plan, *bwd)}
+
+
+@pytest.mark.parametrize("name", ["w_qkv", "w_o", "w_fc1", "w_fc2"])
+@pytest.mark.parametrize("value,status", [(0x20000002, B.ERR_UNSUPPORTED), (0x20000008, B.ERR_UNSUPPORTED), (None, B.ERR_INVALID_ARG)])
+def test_matrices_that_cannot_be_prefetched(name, value, status):
+    assert set(_calls(_struct(B.LayerWeights, 1, 0, **{name: value}), 1).values()) == {status}
+    got = _calls(_struct(B.LayerWeights, 3, 2, **{name: value}), 3)
+    assert set(got.values()) == {status}
