@@ -593,6 +593,7 @@ int32_t mpipe_encoder_layer_bwd(const void* dy, const void* x, void* dx, const m
         return MPIPE_ERR_WORKSPACE;
     if (((reinterpret_cast<uintptr_t>(workspace) | reinterpret_cast<uintptr_t>(fwd_workspace)) & 255u) != 0) return MPIPE_ERR_UNSUPPORTED;
     if (const int32_t bad = layer_matrices_ok(*w)) return bad;
+    if (!aligned16(rope_cos) || !aligned16(rope_sin)) return MPIPE_ERR_UNSUPPORTED;   // (read 16 bytes at a time where dQ and dK are turned back)
     const int32_t head_dim = hidden / n_heads;
     const size_t t = size_t(n_tokens);
     const int64_t h = hidden, h3 = 3 * int64_t(hidden), f = ffn;

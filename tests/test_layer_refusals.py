@@ -62,3 +62,9 @@ def test_matrices_that_cannot_be_prefetched(name, value, status):
     assert set(_calls(_struct(B.LayerWeights, 1, 0, **{name: value}), 1).values()) == {status}
     got = _calls(_struct(B.LayerWeights, 3, 2, **{name: value}), 3)
     assert set(got.values()) == {status}
+
+
+@pytest.mark.parametrize("rope", [(0x80000004, 0x81000000), (0x80000000, 0x81000008)])
+def test_backward_with_misaligned_tables(rope):
+    got = _calls(_struct(B.LayerWeights, 1, 0), 1, rope=rope)
+    assert got["layer_bwd"] == got["bwd"] == B.ERR_UNSUPPORTED
