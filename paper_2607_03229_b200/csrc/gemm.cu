@@ -685,6 +685,7 @@ static int32_t launch_wgrad(const void* dy, const void* x, float* dw, float* db,
 // Weight and bias gradient of a projection in one launch.
 int32_t linear_wgrad_bias(const void* dy, const void* x, float* dw, float* db, int32_t n_tokens, int32_t N, int32_t K, int64_t lddy,
                           int64_t ldx, int64_t lddw, int32_t* status_buf, void* stream, const LayerAhead& ahead) {
+    if (db == nullptr && n_tokens > 0) return MPIPE_ERR_INVALID_ARG;
     return launch_wgrad(dy, x, dw, db, n_tokens, N, K, lddy, ldx, lddw, status_buf, stream, ahead);
 }
 

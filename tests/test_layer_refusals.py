@@ -68,3 +68,8 @@ def test_matrices_that_cannot_be_prefetched(name, value, status):
 def test_backward_with_misaligned_tables(rope):
     got = _calls(_struct(B.LayerWeights, 1, 0), 1, rope=rope)
     assert got["layer_bwd"] == got["bwd"] == B.ERR_UNSUPPORTED
+
+
+def test_backward_without_a_bias_gradient():
+    got = _calls(_struct(B.LayerWeights, 1, 0), 1, grads=_struct(B.LayerGrads, 1, 0, b_fc2=None))
+    assert got["layer_bwd"] == got["bwd"] == B.ERR_INVALID_ARG
