@@ -38,22 +38,10 @@ def _calls(weights, n, grads=None, rope=(None, None), mode=B.TRAINED):
     a, plan = 0x70000000, (0x71000000, 1, T, 0x71100000, 3)
     fwd = (SCALE, EPS, *rope, mode, 0x72000000, 0x73000000, WS, None, None)
     bwd = (SCALE, EPS, *rope, mode, 0x72000000, 0x73000000, 0x74000000, WS, None, None)
-    return {"layer_fwd": lib.mpipe_encoder_layer_fwd(a, a, last, # (with a device a missing check would launch kernels on made-up addresses)
-pytestmark = pytest.mark.skipif(torch.cuda.is_available(), reason="only where nothing can be launched")
-
-T, HIDDEN, H, FFN, *plan, *fwd),
-            "fwd": lib.mpipe_encoder_fwd(a, a, ctypes.addressof(weights), n, # (with a device a missing check would launch kernels on made-up addresses)
-pytestmark = pytest.mark.skipif(torch.cuda.is_available(), reason="only where nothing can be launched")
-
-T, HIDDEN, H, FFN, *plan, *fwd),
-            "layer_bwd": lib.mpipe_encoder_layer_bwd(a, a, a, last, last_g, # (with a device a missing check would launch kernels on made-up addresses)
-pytestmark = pytest.mark.skipif(torch.cuda.is_available(), reason="only where nothing can be launched")
-
-T, HIDDEN, H, FFN, *plan, *bwd),
-            "bwd": lib.mpipe_encoder_bwd(a, a, a, ctypes.addressof(weights), ctypes.addressof(g), n, # (with a device a missing check would launch kernels on made-up addresses)
-pytestmark = pytest.mark.skipif(torch.cuda.is_available(), reason="only where nothing can be launched")
-
-T, HIDDEN, H, FFN, *plan, *bwd)}
+    return {"layer_fwd": lib.mpipe_encoder_layer_fwd(a, a, last, T, HIDDEN, H, FFN, *plan, *fwd),
+            "fwd": lib.mpipe_encoder_fwd(a, a, ctypes.addressof(weights), n, T, HIDDEN, H, FFN, *plan, *fwd),
+            "layer_bwd": lib.mpipe_encoder_layer_bwd(a, a, a, last, last_g, T, HIDDEN, H, FFN, *plan, *bwd),
+            "bwd": lib.mpipe_encoder_bwd(a, a, a, ctypes.addressof(weights), ctypes.addressof(g), n, T, HIDDEN, H, FFN, *plan, *bwd)}
 
 
 @pytest.mark.parametrize("name", ["w_qkv", "w_o", "w_fc1", "w_fc2"])
