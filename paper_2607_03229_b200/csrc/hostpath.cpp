@@ -156,22 +156,24 @@ PyObject* seg_plan(PyObject*, PyObject* const* a, Py_ssize_t n) {
         const Py_ssize_t n_seg = PyList_GET_SIZE(a[0]);
         const int32_t mode = int32_t(integer(a[1])), fr = int32_t(integer(a[2])), br = int32_t(integer(a[3]));
         std::vector<int32_t> counts(static_cast<size_t>(n_seg) + 1);
-        int64_t want_f = 0, want_b = 0;
+        int64_t want_f = 0, want_b = 0, sum = 0;
+        bool sound = n_seg < 0x7fffffff;   // a list the planner may accept: no negative count, a total of 31 bits
         for (Py_ssize_t i = 0; i < n_seg; ++i) {
             PyObject* o = PyList_GET_ITEM(a[0], i);
             int overflow = 0;
             const long v = PyLong_CheckExact(o) ? PyLong_AsLongAndOverflow(o, &overflow) : 0;
             if (!PyLong_CheckExact(o) || overflow != 0 || v != long(int32_t(v))) Py_RETURN_NONE;
             counts[size_t(i)] = int32_t(v);
-            if (v > 0 && fr > 0 && br > 0) {
+            sound = sound && v >= 0 && (sum += v) < (int64_t(1) << 31);
+            if (sound && fr > 0 && br > 0) {
                 want_f += (v + fr - 1) / fr;
                 want_b += (v + br - 1) / br;
             }
         }
+        if (!sound || (mode != MPIPE_ENC_FROZEN && mode != MPIPE_ENC_TRAINED)) want_f = want_b = 0;   // the planner writes no item then
         if (mode != MPIPE_ENC_TRAINED) want_b = 0;
         auto up4 = [](int64_t w) { return (w + 3) / 4 * 4; };
         const int64_t off_f = up4(n_seg + 1), off_b = off_f + up4(6 * want_f), words = off_b + up4(6 * want_b);
-        if (want_f > 0x7fffffff / 6 || want_b > 0x7fffffff / 6) Py_RETURN_NONE;
         PyObject* buf = PyByteArray_FromStringAndSize(nullptr, Py_ssize_t(words * 4));
         if (buf == nullptr) throw Failed();
         int32_t* w = reinterpret_cast<int32_t*>(PyByteArray_AS_STRING(buf));

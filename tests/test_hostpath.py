@@ -1,5 +1,7 @@
 """The native marshalling of the per-microbatch calls: every accepted form of the patch counts gives the same plan, and what does
 not fit together is refused before anything is called."""
+import resource
+
 import numpy as np
 import pytest
 import torch
@@ -30,6 +32,23 @@ def test_counts_beyond_32_bits_are_refused():
         B.seg_plan([1 << 40], B.TRAINED)
     with pytest.raises(B.MpipeError):
         B.seg_plan([(1 << 31) - 1, 1], B.TRAINED)
+
+
+@pytest.mark.parametrize("counts,mode", [([(1 << 31) - 1] * 4, B.TRAINED), ([(1 << 31) - 1] * 50, B.TRAINED), ([(1 << 31) - 1] * 400, B.FROZEN),
+                                         ([(1 << 31) - 1, -1], B.TRAINED), ([-5], B.FROZEN), ([1 << 30], 7)])
+def test_counts_that_make_no_plan_are_refused_before_anything_is_sized(counts, mode):
+    limits = resource.getrlimit(resource.RLIMIT_AS)
+    B.load()
+    with open("/proc/self/statm") as f:
+        now = int(f.read().split()[0]) * resource.getpagesize()
+    resource.setrlimit(resource.RLIMIT_AS, (now + (64 << 20), limits[1]))   # the items of such counts would be 0.2 to 200 GB
+    try:
+        for form in (counts, tuple(counts)):
+            with pytest.raises(B.MpipeError) as e:
+                B.seg_plan(form, mode)
+            assert e.value.status == B.ERR_INVALID_ARG
+    finally:
+        resource.setrlimit(resource.RLIMIT_AS, limits)
 
 
 def test_mismatched_tensors_are_refused():
