@@ -53,28 +53,38 @@ def build(force: bool = False, verbose: bool = False) -> str:
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
     objs = []
     procs = []
-    os.makedirs(os.path.join(HERE, "build"), exist_ok=True)
-    for src in sources():
-        obj = os.path.join(HERE, "build", os.path.basename(src)[:-3] + ".o")
-        cmd = [nvcc] + [f for f in NVCC_FLAGS if f != "--shared"] + ["-c", src, "-o", obj]
-        if verbose:
-            cmd.insert(1, "-Xptxas=-v")
-        procs.append((src, subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)))
-        objs.append(obj)
-    host_tmp = HOST_LIB + f".{os.getpid()}.tmp"
-    procs.append((HOST_SRC, subprocess.Popen(host_command(host_tmp), stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)))
-    failed = False
-    for src, p in procs:
-        out, _ = p.communicate()
-        if out.strip() and (verbose or p.returncode != 0):
-            print(out, file=sys.stderr)
-        failed |= p.returncode != 0
-    if failed:
-        raise RuntimeError("nvcc failed")
-    tmp = LIB + f".{os.getpid()}.tmp"
-    subprocess.run([nvcc] + NVCC_FLAGS + objs + ["-o", tmp], check=True)
-    os.replace(host_tmp, HOST_LIB)
-    os.replace(tmp, LIB)
+    work = os.path.join(HERE, "build")
+    os.makedirs(work, exist_ok=True)
+    # both libraries are linked beside the objects, each process under its own name, and moved to their place when everything is there
+    tmp, host_tmp = (os.path.join(work, f"{os.getpid()}.{os.path.basename(f)}") for f in (LIB, HOST_LIB))
+    try:
+        for src in sources():
+            obj = os.path.join(work, os.path.basename(src)[:-3] + ".o")
+            cmd = [nvcc] + [f for f in NVCC_FLAGS if f != "--shared"] + ["-c", src, "-o", obj]
+            if verbose:
+                cmd.insert(1, "-Xptxas=-v")
+            procs.append((src, subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)))
+            objs.append(obj)
+        procs.append((HOST_SRC, subprocess.Popen(host_command(host_tmp), stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)))
+        failed = False
+        for src, p in procs:
+            out, _ = p.communicate()
+            if out.strip() and (verbose or p.returncode != 0):
+                print(out, file=sys.stderr)
+            failed |= p.returncode != 0
+        if failed:
+            raise RuntimeError("nvcc failed")
+        subprocess.run([nvcc] + NVCC_FLAGS + objs + ["-o", tmp], check=True)
+        os.replace(host_tmp, HOST_LIB)
+        os.replace(tmp, LIB)
+    finally:   # (after a failure or an interruption)
+        for _, p in procs:
+            if p.poll() is None:
+                p.kill()
+                p.wait()
+        for f in (tmp, host_tmp):
+            if os.path.exists(f):
+                os.remove(f)
     return LIB
 
 
