@@ -180,6 +180,9 @@ class SegPlan:
     _host_staging: Optional[torch.Tensor] = None
     _packed: Optional[tuple] = None   # (bytearray, forward offset, backward offset, the three arrays as views of it)
 
+    def __getstate__(self):   # a copied or saved plan's arrays are no views of the buffer any more
+        return {**self.__dict__, "_packed": None}
+
     @property
     def n_seg(self) -> int:
         return self.cu_seqlens.size - 1

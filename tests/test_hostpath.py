@@ -1,5 +1,7 @@
 """The native marshalling of the per-microbatch calls: every accepted form of the patch counts gives the same plan, and what does
 not fit together is refused before anything is called."""
+import copy
+import pickle
 import resource
 
 import numpy as np
@@ -49,6 +51,30 @@ def test_counts_that_make_no_plan_are_refused_before_anything_is_sized(counts, m
             assert e.value.status == B.ERR_INVALID_ARG
     finally:
         resource.setrlimit(resource.RLIMIT_AS, limits)
+
+
+@pytest.mark.parametrize("make", [lambda p: p, copy.copy, copy.deepcopy, lambda p: pickle.loads(pickle.dumps(p))])
+def test_what_is_uploaded_is_what_the_plan_holds(make, monkeypatch):
+    """A plan, a copy and one that was saved and loaded: an item changed in place is changed in the upload too."""
+    plan = make(B.seg_plan([300, 0, 17], B.TRAINED))
+    plan.fwd_items["row_len"][0] = 5
+    plan.cu_seqlens[1] = 299
+    sent = []
+
+    class Host:
+        def upload(self, buf, n_cu, off_f, n_f, off_b, n_b, device):
+            w = np.frombuffer(buf, dtype=np.int32)
+            sent.extend([w[:n_cu], w[off_f:off_f + 6 * n_f].view(B.ITEM_DTYPE), w[off_b:off_b + 6 * n_b].view(B.ITEM_DTYPE)])
+            return None, None, None, None
+
+    monkeypatch.setattr(B, "_host", Host())
+    monkeypatch.setattr(torch.Tensor, "pin_memory", lambda t: t)
+    monkeypatch.setattr(torch.Tensor, "to", lambda t, *a, **k: t)
+    plan.to_device("cuda")
+    if not sent:   # the general route
+        sent = [plan.cu_seqlens_dev.numpy(), plan.fwd_items_dev.numpy().view(B.ITEM_DTYPE).reshape(-1), plan.bwd_items_dev.numpy().view(B.ITEM_DTYPE).reshape(-1)]
+    for got, want in zip(sent, (plan.cu_seqlens, plan.fwd_items, plan.bwd_items)):
+        assert np.array_equal(got, want)
 
 
 def test_mismatched_tensors_are_refused():
