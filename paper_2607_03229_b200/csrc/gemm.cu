@@ -136,7 +136,7 @@ linear_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
                 prefetch_l2_bulk(src + off, min(kPiece, bytes - off));
         }
     }
-    if (!(warp == 3 && p.settled_w)) pdl_wait();   // weights inside a layer are loaded while the kernel before still runs
+    if (!(warp == 3 && p.settled_w)) pdl_wait();   // weights inside a layer are loaded while the kernel before still runs, a ring of them
     if (warp == 0) pdl_launch();
     const int kpb = kMode == 2 ? 1 : p.kpb, nk = (p.K + kpb * kGemmBK - 1) / (kpb * kGemmBK);   // stages of the whole contraction
     const int n_out_tiles = p.tiles_m * p.tiles_n;
@@ -173,6 +173,8 @@ linear_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
                 const int n0 = (tile_of(t) % p.tiles_n) * bn + half * bn_half;
                 const int kb_hi = kb_hi_of(t);
                 for (int kb = kb_lo_of(t); kb < kb_hi; ++kb) {
+                    // early weights: the ring is full, and stages come back when the kernel before this one has ended and not a second later
+                    if (!is_a && p.settled_w && ph == 0) pdl_wait();
                     ok = mbar_wait(&bars.empty[s], ph, &abort_flag);
                     if (!ok) break;
                     uint8_t* st = smem + s * stage_bytes;
