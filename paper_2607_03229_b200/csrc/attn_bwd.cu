@@ -275,7 +275,6 @@ attn_bwd_kernel(const __grid_constant__ BwdMaps maps, const BwdParams p) {
                 return true;
             };
             UnitSource source{&units, &abort_flag};
-            bool outstanding = false;
             for (int u = int(blockIdx.x); ok; ++unit_it) {
                 const mpipe_work_item_t it = item_at(u);
                 ok = source.put(it);
@@ -285,10 +284,7 @@ attn_bwd_kernel(const __grid_constant__ BwdMaps maps, const BwdParams p) {
                 if (Cfg::kPool) {   // K, Q_0, V, dO_0, Q_1, dO_1, ...: the order in which the issuer comes to need them
                     const int ask_at = nq > 3 ? nq - 3 : 0;
                     for (int j = 0; j < nq && ok; ++j) {
-                        if (j == ask_at) {
-                            source.ask();
-                            outstanding = true;
-                        }
+                        if (j == ask_at) source.ask();
                         const int row = it.kv_start + q_tile_of(it, j, nq) * kBQ;
                         if (j == 0) ok = pool_load(&maps.k, head, it.row_start);
                         ok = ok && pool_load(&maps.q, head, row);
@@ -297,7 +293,6 @@ attn_bwd_kernel(const __grid_constant__ BwdMaps maps, const BwdParams p) {
                     }
                     if (!ok) break;
                     u = source.take(&ok);
-                    outstanding = false;
                     continue;
                 }
                 // Before its buffers are free, a short unit's first tiles are asked for into L2 (a long unit's Q and dO are there
@@ -321,10 +316,7 @@ attn_bwd_kernel(const __grid_constant__ BwdMaps maps, const BwdParams p) {
                 load_tile(kv + Cfg::kSmemV, &maps.v, &bars.kv_full[kb], head, it.row_start);
                 const int ask_at = nq > 3 ? nq - 3 : 0;   // late enough to go to the CTA that is free first, early enough to be answered
                 for (int j = 0; j < nq; ++j, ++sc) {
-                    if (j == ask_at) {
-                        source.ask();
-                        outstanding = true;
-                    }
+                    if (j == ask_at) source.ask();
                     const int rs = sc % NR;
                     const int row = it.kv_start + q_tile_of(it, j, nq) * kBQ;
                     ok = mbar_wait<kSleepAux>(&bars.qdo_empty[rs], ((sc / NR) & 1) ^ 1, &abort_flag);
@@ -335,9 +327,8 @@ attn_bwd_kernel(const __grid_constant__ BwdMaps maps, const BwdParams p) {
                 }
                 if (!ok) break;
                 u = source.take(&ok);
-                outstanding = false;
             }
-            if (!ok) source.cancel_rest(outstanding);
+            if (!ok) source.cancel_rest();
         }
         __syncwarp();
     } else if (warp == 1) {

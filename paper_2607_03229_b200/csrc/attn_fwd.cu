@@ -168,16 +168,13 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
             uint32_t kv_it = 0, unit_it = 0;
             bool ok = true;
             UnitSource source{&units, &abort_flag};
-            bool outstanding = false;
             for (int u = int(blockIdx.x); ok; ++unit_it) {
                 const mpipe_work_item_t it = item_at(u);
                 ok = source.put(it);
                 if (!ok || it.kv_len <= 0) break;
                 source.ask();
-                outstanding = true;
                 if (kSplit && it.row_len <= 0) {
                     u = source.take(&ok);
-                    outstanding = false;
                     --unit_it;
                     continue;
                 }
@@ -211,9 +208,8 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
                 }
                 if (!ok) break;
                 u = source.take(&ok);
-                outstanding = false;
             }
-            if (!ok) source.cancel_rest(outstanding);
+            if (!ok) source.cancel_rest();
         }
         __syncwarp();
     } else if (warp == 1) {

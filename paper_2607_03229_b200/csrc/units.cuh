@@ -28,16 +28,21 @@ struct UnitSource {
     UnitRing* ring;
     volatile int* abort_flag;
     uint32_t taken = 0, asked = 0;
+    bool outstanding = false;              // a request whose answer has not been seen
+    bool ended = false;                    // an answer without a block has come: no more may be asked for
     __device__ __forceinline__ void ask() {
         mbar_expect_tx(&ring->answered, 16);
         clc_try_cancel(&ring->answer, &ring->answered);
         ++asked;
+        outstanding = true;
     }
     // The unit of the outstanding request, -1 at the end of the list (or after a time-out, *ok = false).
     __device__ __forceinline__ int take(bool* ok) {
         *ok = mbar_wait(&ring->answered, (asked - 1) & 1, abort_flag);
         if (!*ok) return -1;
+        outstanding = false;
         const int u = clc_block_of(&ring->answer);
+        ended = u < 0;
         fence_async_smem();                // the answer has been read before the next one is asked for
         return u;
     }
@@ -49,14 +54,15 @@ struct UnitSource {
         ++taken;
         return true;
     }
-    // After a time-out: nothing of this grid shall start any more, or every further block would run into its own time-out.
-    __device__ __forceinline__ void cancel_rest(bool outstanding) {
+    // After a time-out: nothing of this grid shall start any more, or every further block would run into its own time-out.  An answer
+    // still on its way is waited for first: the barrier counts one at a time.
+    __device__ __forceinline__ void cancel_rest() {
         int dummy = 0;
-        for (;;) {
+        while (!ended) {
             if (!outstanding) ask();
-            outstanding = false;
             if (!mbar_wait_budget(&ring->answered, (asked - 1) & 1, &dummy, 10000000ll)) return;
-            if (clc_block_of(&ring->answer) < 0) return;
+            outstanding = false;
+            ended = clc_block_of(&ring->answer) < 0;
             fence_async_smem();
         }
     }
