@@ -886,13 +886,13 @@ bwd_prepass_kernel(const __nv_bfloat16* __restrict__ dout, const __nv_bfloat16* 
 template <int D>
 __global__ void __launch_bounds__(256)
 bwd_dq_convert_kernel(const float* __restrict__ acc, __nv_bfloat16* __restrict__ dq, int64_t tok_stride_g,
-                      int64_t head_stride_g, uint32_t n_chunks, uint32_t n_heads, float scale) {
+                      int64_t head_stride_g, int64_t n_chunks, uint32_t n_heads, float scale) {
     pdl_wait();
     pdl_launch();
-    const uint32_t idx = blockIdx.x * 256u + threadIdx.x;
+    const int64_t idx = int64_t(blockIdx.x) * 256 + threadIdx.x;
     if (idx >= n_chunks) return;
-    const uint32_t th = idx / (D / 8), c = idx % (D / 8), t = th / n_heads, h = th % n_heads;
-    const float4* src = reinterpret_cast<const float4*>(acc) + size_t(idx) * 2;
+    const uint32_t th = uint32_t(idx / (D / 8)), c = uint32_t(idx % (D / 8)), t = th / n_heads, h = th % n_heads;   // (th: launch_bwd)
+    const float4* src = reinterpret_cast<const float4*>(acc) + idx * 2;
     const float4 x = __ldg(src), y = __ldg(src + 1);
     uint4 out;
     out.x = pack_bf16(x.x * scale, x.y * scale);
@@ -910,15 +910,15 @@ template <int D>
 __global__ void __launch_bounds__(256)
 bwd_dq_convert_rope_kernel(const float* __restrict__ acc, __nv_bfloat16* __restrict__ dq, __nv_bfloat16* __restrict__ dk,
                            int64_t tok_stride_g, int64_t head_stride_g, const float* __restrict__ cos_t,
-                           const float* __restrict__ sin_t, uint32_t n_chunks, uint32_t n_heads, float scale) {
+                           const float* __restrict__ sin_t, int64_t n_chunks, uint32_t n_heads, float scale) {
     pdl_wait();
     pdl_launch();
     constexpr int kHalf = D / 2, kPer = kHalf / 8;
-    uint32_t idx = blockIdx.x * 256u + threadIdx.x;
+    int64_t idx = int64_t(blockIdx.x) * 256 + threadIdx.x;
     if (idx >= 2 * n_chunks) return;
     const bool is_k = idx >= n_chunks;
     if (is_k) idx -= n_chunks;
-    const uint32_t th = idx / kPer, c = idx % kPer, t = th / n_heads, h = th % n_heads;
+    const uint32_t th = uint32_t(idx / kPer), c = uint32_t(idx % kPer), t = th / n_heads, h = th % n_heads;
     __nv_bfloat16* row = (is_k ? dk : dq) + t * tok_stride_g + h * head_stride_g + c * 8;
     float2 a[4], b[4];
     if (is_k) {
@@ -960,6 +960,8 @@ template <int D, bool kPooled>
 static int32_t launch_bwd(const void* dout, const void* q, const void* k, const void* v, const void* o, void* dq,
                           int64_t ts_qkv, int64_t hs_qkv, int64_t ts_o, int64_t hs_o, int32_t total_tokens,
                           int32_t n_heads, BwdParams prm, float* delta, float* dq_acc, cudaStream_t stream) {
+    const int64_t rows = int64_t(total_tokens) * n_heads;
+    if (rows > 0xffffffffLL) return MPIPE_ERR_UNSUPPORTED;     // the conversion's row index; an accumulator of a terabyte
     using Cfg = BwdCfg<D, kPooled>;
     BwdMaps m;
     constexpr uint32_t box = Cfg::kBoxElems;
@@ -971,7 +973,8 @@ static int32_t launch_bwd(const void* dout, const void* q, const void* k, const 
         !make_tensor_map_thd(&m.dq_acc, dq_acc, total_tokens, n_heads, D, int64_t(n_heads) * D, D, 16, kBQ, 64, 4))
         return MPIPE_ERR_CUDA;
     if (!ensure_dynamic_smem<attn_bwd_kernel<D, kPooled>>(Cfg::kSmemAlloc)) return MPIPE_ERR_CUDA;
-    const int64_t rows = int64_t(total_tokens) * n_heads;
+    const bool rope = prm.rope_cos != nullptr;
+    const int64_t chunks = rows * (rope ? D / 16 : D / 8);
     constexpr int kPrepassRows = 8 * (32 / (D / 16));   // rows of a block
     const int64_t prepass_blocks = (rows + kPrepassRows - 1) / kPrepassRows;
     const int64_t prepass_cap = int64_t(sm_count()) * 64;
@@ -984,16 +987,13 @@ static int32_t launch_bwd(const void* dout, const void* q, const void* k, const 
     e = launch_kernel_as(true, attn_bwd_kernel<D, kPooled>, unsigned(n_units), kBwdThreads, Cfg::kSmemAlloc, stream, 1, m, prm);
     profile_stop(kProfileBwdMain, stream);
     if (e != cudaSuccess) return MPIPE_ERR_CUDA;
-    const bool rope = prm.rope_cos != nullptr;
-    const int64_t chunks = rows * (rope ? D / 16 : D / 8);
-    if (chunks > 0x7fffffffLL) return MPIPE_ERR_UNSUPPORTED;   // (a Q of 32 GB)
     if (rope)
         e = launch_kernel(bwd_dq_convert_rope_kernel<D>, unsigned((2 * chunks + 255) / 256), 256, 0, stream, 1, static_cast<const float*>(dq_acc),
                           static_cast<__nv_bfloat16*>(dq), prm.dk, prm.tok_stride_g, prm.head_stride_g, prm.rope_cos, prm.rope_sin,
-                          uint32_t(chunks), uint32_t(n_heads), prm.scale);
+                          chunks, uint32_t(n_heads), prm.scale);
     else
         e = launch_kernel(bwd_dq_convert_kernel<D>, unsigned((chunks + 255) / 256), 256, 0, stream, 1, static_cast<const float*>(dq_acc),
-                          static_cast<__nv_bfloat16*>(dq), prm.tok_stride_g, prm.head_stride_g, uint32_t(chunks), uint32_t(n_heads), prm.scale);
+                          static_cast<__nv_bfloat16*>(dq), prm.tok_stride_g, prm.head_stride_g, chunks, uint32_t(n_heads), prm.scale);
     return e == cudaSuccess && cudaGetLastError() == cudaSuccess ? MPIPE_OK : MPIPE_ERR_CUDA;
 }
 

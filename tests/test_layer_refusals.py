@@ -1,4 +1,4 @@
-"""What a layer or a layer stack refuses, it refuses before anything is launched: on a machine without a device a launch would be
+"""What a layer, a layer stack or the attention backward refuses, it refuses before anything is launched: on a machine without a device a launch would be
 MPIPE_ERR_CUDA.  The addresses are never read."""
 import ctypes
 
@@ -61,3 +61,11 @@ def test_backward_with_misaligned_tables(rope):
 def test_backward_without_a_bias_gradient():
     got = _calls(_struct(B.LayerWeights, 1, 0), 1, grads=_struct(B.LayerGrads, 1, 0, b_fc2=None))
     assert got["layer_bwd"] == got["bwd"] == B.ERR_INVALID_ARG
+
+
+@pytest.mark.parametrize("tokens,heads,status", [(1 << 30, 8, B.ERR_UNSUPPORTED),      # 2^33 rows of heads: more than the last pass counts
+                                                 (1 << 28, 8, B.ERR_CUDA)])            # 2^31 of them, 2^34 pieces: goes on to the device
+def test_attention_backward_is_refused_before_its_first_launch(tokens, heads, status):
+    a, ts = 0x70000000, heads * 64
+    got = B.load().mpipe_varlen_attn_bwd(*[a] * 9, *[ts, 64] * 3, a, 1, tokens, tokens, a, 1, heads, 64, SCALE, B.TRAINED, a, 1 << 50, None, None)
+    assert got == status
