@@ -14,8 +14,7 @@
 #include <vector>
 
 #include "../../include/mpipe_enc.h"
-
-extern "C" int32_t mpipe_plan_words_to_device(const void* words, int32_t n, void* dst, void* stream);   // plan.cu
+#include "plan_words.h"
 
 namespace {
 
@@ -25,7 +24,6 @@ decltype(&mpipe_varlen_attn_bwd) f_attn_bwd = nullptr;
 decltype(&mpipe_merge_tokens) f_merge = nullptr;
 decltype(&mpipe_merge_tokens_bwd) f_merge_bwd = nullptr;
 decltype(&mpipe_plan_words_to_device) f_plan_words = nullptr;
-constexpr int64_t kPlanWordsMax = 8128;   // what a kernel's arguments hold
 
 struct Failed {};   // a Python exception is set
 struct WithoutGil {   // around calls that may block in the driver: other Python threads go on, as under ctypes
@@ -202,7 +200,7 @@ PyObject* upload(PyObject*, PyObject* const* a, Py_ssize_t n) {
         const long dev = integer(a[6]);
         const at::TensorOptions ints = at::TensorOptions().dtype(at::kInt);
         at::Tensor host, d = at::empty({words}, ints.device(at::Device(at::kCUDA, c10::DeviceIndex(dev))));
-        if (words <= kPlanWordsMax) {
+        if (words <= mpipe::kPlanWordsMax) {
             const c10::DeviceGuard on(d.device());
             void* const to = data(d);
             void* const stream = c10::cuda::getCurrentCUDAStream(d.device().index()).stream();

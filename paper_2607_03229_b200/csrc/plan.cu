@@ -4,6 +4,7 @@
 #include <numeric>
 #include <vector>
 #include "common.h"
+#include "plan_words.h"
 #include "sm100_ptx.cuh"
 
 namespace mpipe {
@@ -84,18 +85,16 @@ static int32_t emit_items(const int32_t* counts, const int32_t* cu, const std::v
 
 extern "C" {
 
-// Internal: n <= 8128 words of a plan to device memory, in stream order (the arguments of a kernel end at 32 764 bytes).
 int32_t mpipe_plan_words_to_device(const void* words, int32_t n, void* dst, void* stream) {
     using namespace mpipe;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    if (n < 0 || n > 8128 || (n > 0 && (words == nullptr || dst == nullptr))) return MPIPE_ERR_INVALID_ARG;
+    if (n < 0 || n > kPlanWordsMax || (n > 0 && (words == nullptr || dst == nullptr))) return MPIPE_ERR_INVALID_ARG;
     if (n == 0) return MPIPE_OK;
     if (n <= 256) return launch_plan_words<256>(words, n, dst, st);      // (what a launch costs grows with the arguments' size)
     if (n <= 1024) return launch_plan_words<1024>(words, n, dst, st);
     if (n <= 3072) return launch_plan_words<3072>(words, n, dst, st);
-    return launch_plan_words<8128>(words, n, dst, st);
+    return launch_plan_words<kPlanWordsMax>(words, n, dst, st);
 }
-
 
 int32_t mpipe_seg_plan(const int32_t* patch_counts, int32_t n_seg, int32_t fwd_tile_rows, int32_t bwd_tile_rows,
                        int32_t mode, int32_t* cu_seqlens, int32_t* total_tokens, int32_t* max_seqlen,
