@@ -17,13 +17,14 @@ from typing import List, Optional
 import numpy as np
 import torch
 
-_HERE = os.path.dirname(os.path.abspath(__file__))
-LIB_PATH = os.path.join(_HERE, "libmpipe_enc.so")
+from . import build as _build
+
+LIB_PATH = _build.LIB
 
 OK, ERR_INVALID_ARG, ERR_UNSUPPORTED, ERR_WORKSPACE, ERR_CUDA, ERR_TIMEOUT, ERR_INDEX = range(7)
 FROZEN, TRAINED = 0, 1
 
-HOSTPATH = os.path.join(_HERE, "_hostpath.so")
+HOSTPATH = _build.HOST_LIB
 _lib = None
 _host = None            # the native marshalling module
 _tile_rows = (0, 0)     # the library's native tile heights
@@ -102,6 +103,9 @@ def load() -> ctypes.CDLL:
             if not os.path.exists(path):
                 raise RuntimeError(f"{path} is missing: build it with `python -m paper_2607_03229_b200.build` "
                                    "(there is no fallback path)")
+        if not _build.host_is_current():
+            raise RuntimeError(f"{HOSTPATH} was built for another torch or Python than {_build.built_for()}: "
+                               "rebuild it with `python -m paper_2607_03229_b200.build`")
         lib = ctypes.CDLL(LIB_PATH)
         for name, (res, args) in _SIGNATURES.items():
             fn = getattr(lib, name)

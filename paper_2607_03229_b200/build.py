@@ -28,8 +28,20 @@ def _deps():
         [os.path.join(HERE, "..", "include", "mpipe_enc.h")]
 
 
+def built_for() -> str:
+    """What the marshalling module is compiled against and works with only: torch's and Python's C++ interfaces."""
+    import torch
+    return f"marshalling for torch {torch.__version__}, {sys.implementation.cache_tag}"
+
+
+def host_is_current() -> bool:
+    """Whether the marshalling module there is was built for this torch and this Python (it carries their names)."""
+    with open(HOST_LIB, "rb") as f:
+        return built_for().encode() in f.read()
+
+
 def is_stale() -> bool:
-    if not os.path.exists(LIB) or not os.path.exists(HOST_LIB):
+    if not os.path.exists(LIB) or not os.path.exists(HOST_LIB) or not host_is_current():
         return True
     t = min(os.path.getmtime(LIB), os.path.getmtime(HOST_LIB))
     return any(os.path.getmtime(f) > t for f in _deps())
@@ -42,7 +54,7 @@ def host_command(out: str):
     inc = [sysconfig.get_paths()["include"], os.path.join(tdir, "include"), os.path.join(tdir, "include", "torch", "csrc", "api", "include"),
            "/usr/local/cuda/include"]
     return ([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
-             f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}"] + ["-I" + d for d in inc] +
+             f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", f'-DMPIPE_BUILT_FOR="{built_for()}"'] + ["-I" + d for d in inc] +
             [HOST_SRC, "-o", out, "-L" + os.path.join(tdir, "lib"), "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch", "-ltorch_python"])
 
 

@@ -359,4 +359,8 @@ PyModuleDef module = {PyModuleDef_HEAD_INIT, "_hostpath", nullptr, -1, methods, 
 
 }  // namespace
 
-PyMODINIT_FUNC PyInit__hostpath(void) { return PyModule_Create(&module); }
+PyMODINIT_FUNC PyInit__hostpath(void) {
+    PyObject* m = PyModule_Create(&module);
+    if (m != nullptr) PyModule_AddStringConstant(m, "built_for", MPIPE_BUILT_FOR);   // (build.py looks for it before the module is loaded)
+    return m;
+}

@@ -1,10 +1,11 @@
-"""A build that fails leaves nothing behind, and no built file is in the history."""
+"""A build that fails leaves nothing behind, no built file is in the history, and what was built for another torch is not used."""
 import os
 import shutil
 import subprocess
 
 import pytest
 
+from paper_2607_03229_b200 import binding as B
 from paper_2607_03229_b200 import build as build_mod
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
@@ -34,3 +35,13 @@ def test_no_built_file_is_tracked():
     names = got.stdout.split()
     assert got.returncode == 0 and names
     assert [n for n in names if ".so" in os.path.basename(n) or n.endswith((".o", ".a", ".tmp", ".cubin"))] == []
+
+
+def test_a_module_of_another_torch_is_rebuilt_and_not_loaded(monkeypatch):
+    build_mod.build()
+    assert build_mod.host_is_current() and not build_mod.is_stale()
+    monkeypatch.setattr(build_mod, "built_for", lambda: "marshalling for torch 0.0.0, cpython-27")
+    assert build_mod.is_stale()
+    monkeypatch.setattr(B, "_lib", None)
+    with pytest.raises(RuntimeError, match="another torch"):
+        B.load()
