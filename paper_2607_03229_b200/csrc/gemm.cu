@@ -35,6 +35,7 @@
 
 #include "common.h"
 #include "gelu.cuh"
+#include "per_device.h"
 #include "sm100_ptx.cuh"
 #include "tensormap.h"
 
@@ -490,10 +491,10 @@ static int gemm_stages(int bn, int kpb) {
 // CTA pairs that fit on the current device at once.
 template <auto kernel>
 static int max_pairs(int threads) {
-    static int cached[64] = {};
+    static PerDevice pairs;
     int dev = -1;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
-    if (cached[dev] == 0) {
+    if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+    return pairs.get(dev, [&]() {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(2);
         cfg.blockDim = dim3(unsigned(threads));
@@ -505,13 +506,10 @@ static int max_pairs(int threads) {
         cfg.attrs = at;
         cfg.numAttrs = 1;
         int n = 0;
-        if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
-            (void)cudaGetLastError();
-            n = 0;
-        }
-        cached[dev] = n > 0 ? n : -1;
-    }
-    return cached[dev] > 0 ? cached[dev] : 0;
+        if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) == cudaSuccess) return n;
+        (void)cudaGetLastError();
+        return 0;
+    });
 }
 static int choose_width(int mode, bool gelu, int pairs, int M, int N, int K) {
     const int nk = cdiv(K, kGemmBK), tiles_m = cdiv(M, 2 * kGemmBM);
