@@ -18,35 +18,51 @@ constexpr int kLnMaxChunks = 8;   // 16-byte chunks per lane: hidden <= 8 * 32 *
 
 // y[t, :] = (x[t, :] - mean) * rsqrt(var + eps) * gamma + beta, biased variance, fp32 statistics (two passes over
 // registers, so no cancellation).  One warp per row; lane l owns chunks l, l + 32, ...
-// Bound by HBM when there are many rows and by the latency of its loads when there are few.
-// kWalk: a warp walks down the rows with the next row on its way while it works on the present one, gamma and beta from L1; two waves
-// of as many blocks as fit.  Otherwise a row per warp, gamma and beta asked for together with the row instead of one L2 latency after
-// its sums.  us, a row per warp and late gamma -> walking / a row per warp as it is now: 777 x 1024 2.83 -> - / 2.08,
-// 4000 x 256 2.02 -> 2.33 / 2.11, 3489 x 1024 4.49 -> 4.10 / 4.25, 20 000 x 1024 16.5 -> 15.0 / 17.7,
-// 50 439 x 1024 36.1 -> 34.0 (6.1 TB/s) / 39.2, 65 536 x 1280 59.5 -> 55.8 (6.0 TB/s) / 71.4: the line lies at 2 M elements.
-constexpr int64_t kLnWalkElems = 2 << 20;
+// Bound by HBM when there are many rows and by the latency of its loads when there are few.  Three ways through the rows:
+//   kLnEarly  a warp per row, gamma and beta asked for together with the row: the fewest latencies and the most registers
+//   kLnLate   a warp per row, gamma and beta (from L1) behind the row's sums, as many blocks on an SM as registers allow
+//   kLnWalk   a warp walks down the rows with the next one on its way while it works on the present one: two waves of blocks
+// What decides is how many rows an SM holds at once (ln_way; us with the input in L2, early / late / walk):
+//   512 columns, 2000 rows 2.1 / 2.2 / 2.4, 5000 3.2 / 2.9 / 3.6, 12 000 from HBM 7.4 / 7.2 / 6.8
+//   1024, 2000 rows 2.7 / 3.2 / 3.2, 3489 4.0 / 4.4 / 3.3 (every warp of the walk has a row), 5000 5.3 / 4.5 / 5.5, 20 000 16.8 / 12.7 / 11.7,
+//         50 439 49.4 / 35.1 / 34.5 (6.0 TB/s)
+//   1280, 2000 rows 3.0 / 3.6 / 3.5, 3489 4.7 / 4.3 / 6.0, 8000 8.4 / 6.8 / 8.7, 50 439 55.6 / 41.4 (6.2 TB/s) / 44.4
+//   2048, 777 rows 2.9 / 4.5 / 4.4, 2000 5.2 / 5.4 / 4.7, 3489 7.7 / 5.5 / 8.2, 50 439 119 / 67 / 70
+enum { kLnEarly, kLnLate, kLnWalk };
 constexpr int ln_walk_blocks(int chunks) { return chunks <= 2 ? 6 : chunks <= 4 ? 3 : 2; }   // of 256 threads on an SM, without spills
-template <int kChunks, bool kWalk>
-__global__ void __launch_bounds__(256, kWalk ? ln_walk_blocks(kChunks) : 1) layernorm_kernel(const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __restrict__ gamma,
-                                                        const __nv_bfloat16* __restrict__ beta, __nv_bfloat16* __restrict__ y,
-                                                        int32_t T, int32_t hidden, int64_t ldx, int64_t ldy, float eps) {
+constexpr int ln_min_blocks(int chunks, int way) {
+    return way == kLnWalk ? ln_walk_blocks(chunks) : way == kLnEarly || chunks <= 2 ? 1 : chunks <= 4 ? 5 : chunks <= 6 ? 4 : 3;
+}
+static int ln_way(int chunks, int rows, int hidden) {
+    const int wave = 8 * sm_count();   // rows of one block on every SM
+    if (rows <= wave * (chunks == 1 || chunks == 3 ? 3 : chunks <= 6 ? 2 : 1)) return kLnEarly;
+    if (chunks >= 3 && rows <= wave * ln_walk_blocks(chunks)) return kLnWalk;
+    if (rows <= 8 * wave || chunks == 5 || chunks == 6) return kLnLate;
+    return chunks == 2 && int64_t(rows) * hidden <= 16 << 20 ? kLnLate : kLnWalk;   // (what is in L2: 20 000 x 512 7.2 / 7.9, not 50 439: 20.4 / 19.2)
+}
+template <int kChunks, int kWay>
+__global__ void __launch_bounds__(256, ln_min_blocks(kChunks, kWay))
+layernorm_kernel(const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __restrict__ gamma, const __nv_bfloat16* __restrict__ beta,
+                 __nv_bfloat16* __restrict__ y, int32_t T, int32_t hidden, int64_t ldx, int64_t ldy, float eps) {
+    constexpr bool kEarly = kWay == kLnEarly, kWalk = kWay == kLnWalk;
     pdl_wait();
     pdl_launch();
     const int lane = threadIdx.x & 31;
     const int n_chunks = hidden >> 3;
     const uint4* g4 = reinterpret_cast<const uint4*>(gamma);
     const uint4* b4 = reinterpret_cast<const uint4*>(beta);
-    int row = blockIdx.x * 8 + (threadIdx.x >> 5);
-    uint4 q[kChunks], g[kWalk ? 1 : kChunks], b[kWalk ? 1 : kChunks];
-    auto load = [&](int r) {
-        if (r >= T) return;
+    const uint32_t n_rows = uint32_t(T), step = gridDim.x * 8;   // (unsigned: a row and a step beyond the last one still fit)
+    uint32_t row = blockIdx.x * 8 + (threadIdx.x >> 5);
+    uint4 q[kChunks], g[kEarly ? kChunks : 1], b[kEarly ? kChunks : 1];
+    auto load = [&](uint32_t r) {
+        if (r >= n_rows) return;
         const uint4* xr = reinterpret_cast<const uint4*>(x + int64_t(r) * ldx);
 #pragma unroll
         for (int i = 0; i < kChunks; ++i)
             if (lane + 32 * i < n_chunks) q[i] = xr[lane + 32 * i];
     };
     load(row);
-    if (!kWalk) {
+    if (kEarly) {
 #pragma unroll
         for (int i = 0; i < kChunks; ++i) {
             if (lane + 32 * i < n_chunks) {
@@ -55,7 +71,7 @@ __global__ void __launch_bounds__(256, kWalk ? ln_walk_blocks(kChunks) : 1) laye
             }
         }
     }
-    for (; row < T; row += gridDim.x * 8) {
+    for (; row < n_rows; row += step) {
         float v[kChunks][8];
         float sum = 0.f;
 #pragma unroll
@@ -70,7 +86,7 @@ __global__ void __launch_bounds__(256, kWalk ? ln_walk_blocks(kChunks) : 1) laye
                 }
             }
         }
-        if (kWalk) load(row + gridDim.x * 8);
+        if (kWalk) load(row + step);
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
         const float mean = sum / float(hidden);
@@ -93,7 +109,7 @@ __global__ void __launch_bounds__(256, kWalk ? ln_walk_blocks(kChunks) : 1) laye
         for (int i = 0; i < kChunks; ++i) {
             const int c = lane + 32 * i;
             if (c < n_chunks) {
-                const uint4 gi = kWalk ? __ldg(g4 + c) : g[kWalk ? 0 : i], bi = kWalk ? __ldg(b4 + c) : b[kWalk ? 0 : i];
+                const uint4 gi = kEarly ? g[kEarly ? i : 0] : __ldg(g4 + c), bi = kEarly ? b[kEarly ? i : 0] : __ldg(b4 + c);
                 const uint32_t gw[4] = {gi.x, gi.y, gi.z, gi.w}, bw[4] = {bi.x, bi.y, bi.z, bi.w};
                 uint32_t o[4];
 #pragma unroll
@@ -364,8 +380,7 @@ int32_t mpipe_layernorm_fwd(const void* x, const void* gamma, const void* beta, 
     if ((hidden % 8) != 0 || hidden > kLnMaxChunks * 256 || (ldx % 8) != 0 || (ldy % 8) != 0) return MPIPE_ERR_UNSUPPORTED;
     if (!aligned16(x) || !aligned16(y) || !aligned16(gamma) || !aligned16(beta)) return MPIPE_ERR_UNSUPPORTED;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    const bool walk = int64_t(n_tokens) * hidden > kLnWalkElems;
-    const int grid = cdiv(n_tokens, 8);
+    const unsigned grid = unsigned(cdiv(n_tokens, 8));
     const auto* xp = static_cast<const __nv_bfloat16*>(x);
     const auto* gp = static_cast<const __nv_bfloat16*>(gamma);
     const auto* bp = static_cast<const __nv_bfloat16*>(beta);
@@ -374,15 +389,19 @@ int32_t mpipe_layernorm_fwd(const void* x, const void* gamma, const void* beta, 
     const int chunks = cdiv(hidden, 256);   // 16-byte chunks per lane: instantiate what the row length needs, not the maximum
     cudaError_t e;
 #define MPIPE_LN_LAUNCH(C)                                                                                                       \
-    e = walk ? launch_kernel_as(true, layernorm_kernel<C, true>, unsigned(2 * ln_walk_blocks(C) * sm_count()), 256, 0, st, 1, xp, gp, bp, yp, n_tokens, hidden, ldx, ldy, eps) \
-             : launch_kernel(layernorm_kernel<C, false>, unsigned(grid), 256, 0, st, 1, xp, gp, bp, yp, n_tokens, hidden, ldx, ldy, eps)
-    if (chunks <= 1) MPIPE_LN_LAUNCH(1);
-    else if (chunks <= 2) MPIPE_LN_LAUNCH(2);
-    else if (chunks <= 3) MPIPE_LN_LAUNCH(3);
-    else if (chunks <= 4) MPIPE_LN_LAUNCH(4);
-    else if (chunks <= 5) MPIPE_LN_LAUNCH(5);
-    else if (chunks <= 6) MPIPE_LN_LAUNCH(6);
-    else MPIPE_LN_LAUNCH(kLnMaxChunks);
+    switch (ln_way(C, n_tokens, hidden)) {                                                                                            \
+        case kLnEarly: e = launch_kernel(layernorm_kernel<C, kLnEarly>, grid, 256, 0, st, 1, xp, gp, bp, yp, n_tokens, hidden, ldx, ldy, eps); break; \
+        case kLnLate: e = launch_kernel(layernorm_kernel<C, kLnLate>, grid, 256, 0, st, 1, xp, gp, bp, yp, n_tokens, hidden, ldx, ldy, eps); break;   \
+        default: e = launch_kernel_as(true, layernorm_kernel<C, kLnWalk>, std::min(grid, unsigned(2 * ln_walk_blocks(C) * sm_count())), 256, 0, st, 1, \
+                                      xp, gp, bp, yp, n_tokens, hidden, ldx, ldy, eps);                                          \
+    }
+    if (chunks <= 1) { MPIPE_LN_LAUNCH(1) }
+    else if (chunks <= 2) { MPIPE_LN_LAUNCH(2) }
+    else if (chunks <= 3) { MPIPE_LN_LAUNCH(3) }
+    else if (chunks <= 4) { MPIPE_LN_LAUNCH(4) }
+    else if (chunks <= 5) { MPIPE_LN_LAUNCH(5) }
+    else if (chunks <= 6) { MPIPE_LN_LAUNCH(6) }
+    else { MPIPE_LN_LAUNCH(kLnMaxChunks) }
 #undef MPIPE_LN_LAUNCH
     profile_stop(kProfileLayerNorm, st);
     return e == cudaSuccess && cudaGetLastError() == cudaSuccess ? MPIPE_OK : MPIPE_ERR_CUDA;

@@ -1,4 +1,4 @@
-"""Layer norm forward on both sides of the line between a row per warp and warps that walk down the rows (2 M elements), with
+"""Layer norm forward on both sides of the lines between its three ways through the rows (multiples of the rows that 148 SMs hold), with
 row lengths that do not fill the last 32-chunk group and row counts that leave some warps a row less."""
 import pytest
 import torch
@@ -7,7 +7,9 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("hidden,rows", [(8, 1), (264, 7945), (264, 7944), (1024, 2048), (1024, 2049), (1024, 9001), (1280, 1639),
-                                         (1280, 13337), (2048, 1025), (2048, 5003), (512, 20011)])
+                                         (1280, 13337), (2048, 1025), (2048, 5003), (512, 20011),
+                                         (8, 3553), (200, 9473), (512, 2369), (640, 3552), (640, 3553), (768, 9473), (1024, 2369), (1024, 3553),
+                                         (1000, 9473), (1280, 2369), (1536, 20011), (2048, 1185), (1800, 2369), (2048, 9473)])
 def test_layernorm_rows(hidden, rows):
     from paper_2607_03229_b200 import binding as B
 
