@@ -19,6 +19,9 @@
 // and MPIPE_ERR_TIMEOUT is reported through status_buf.
 #include <cuda.h>
 #include <math_constants.h>
+
+#include <type_traits>
+
 #include "common.h"
 #include "sm100_ptx.cuh"
 #include "tensormap.h"
@@ -84,7 +87,8 @@ struct FwdBarriers {
 // kSplit: the two query tiles of an item are units of their own (an instantiation apart: the bookkeeping for it in the other one
 // costs 2 to 7 % on long lists).
 // kStaged: O leaves through shared memory (see the epilogue).
-template <int D, bool kSplit, bool kStaged>
+// kLate: when a unit asks for the next one (see the launch).
+template <int D, bool kSplit, bool kStaged, bool kLate>
 __global__ void __maxnreg__(kFwdRegsLaunch)
 attn_fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                 const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_q_tail,
@@ -172,7 +176,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
                 const mpipe_work_item_t it = item_at(u);
                 ok = source.put(it);
                 if (!ok || it.kv_len <= 0) break;
-                source.ask();
+                if (!kLate) source.ask();
                 if (kSplit && it.row_len <= 0) {
                     u = source.take(&ok);
                     --unit_it;
@@ -207,6 +211,14 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
                     if (Cfg::kTail) tma_load_3d(vdst + kTileN * 128, &map_v, &bars.v_full[s], 64, head, row);
                 }
                 if (!ok) break;
+                if (kLate) {   // the scores of the last key tile but one are there (of the last: head_dim 64, two or three of them)
+                    if (nkv > 1) {
+                        const uint32_t at = kv_it - (D == 64 && nkv <= 3 ? 1 : 2);
+                        ok = mbar_wait(&bars.k_empty[at % NS], (at / NS) & 1, &abort_flag);
+                        if (!ok) break;
+                    }
+                    source.ask();
+                }
                 u = source.take(&ok);
             }
             if (!ok) source.cancel_rest();
@@ -579,7 +591,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
     if (tid == 0 && abort_flag) report_status(p.status_buf, MPIPE_ERR_TIMEOUT, int32_t(blockIdx.x));
 }
 
-template <int D, bool kSplit, bool kStaged>
+template <int D, bool kSplit, bool kStaged, bool kLate>
 static int32_t launch_fwd(const void* q, const void* k, const void* v, int64_t tok_stride, int64_t head_stride,
                           int32_t total_tokens, int32_t n_heads, const FwdParams& prm, cudaStream_t stream) {
     using Cfg = FwdCfg<D>;
@@ -597,10 +609,11 @@ static int32_t launch_fwd(const void* q, const void* k, const void* v, int64_t t
             !make_tensor_map_thd(&mkt, k, total_tokens, n_heads, D, tok_stride, head_stride, 16, kTileN, 32))
             return MPIPE_ERR_CUDA;
     }
-    if (!ensure_dynamic_smem<attn_fwd_kernel<D, kSplit, kStaged>>(Cfg::kSmemAlloc)) return MPIPE_ERR_CUDA;
+    if (!ensure_dynamic_smem<attn_fwd_kernel<D, kSplit, kStaged, kLate>>(Cfg::kSmemAlloc)) return MPIPE_ERR_CUDA;
     const int n_units = prm.n_items * prm.n_heads * (kSplit ? 2 : 1);
     profile_start(kProfileFwd, stream);
-    const cudaError_t e = launch_kernel_as(true, attn_fwd_kernel<D, kSplit, kStaged>, unsigned(n_units), kFwdThreads, Cfg::kSmemAlloc, stream, 1, mq, mk, mv, mqt, mkt, mo, prm);
+    const cudaError_t e = launch_kernel_as(true, attn_fwd_kernel<D, kSplit, kStaged, kLate>, unsigned(n_units), kFwdThreads, Cfg::kSmemAlloc, stream, 1,
+                                           mq, mk, mv, mqt, mkt, mo, prm);
     profile_stop(kProfileFwd, stream);
     return e == cudaSuccess && cudaGetLastError() == cudaSuccess ? MPIPE_OK : MPIPE_ERR_CUDA;
 }
@@ -649,8 +662,21 @@ int32_t varlen_attn_fwd(const void* q, const void* k, const void* v, void* o, fl
     // microbatch 512 -> 505, but images of 300 235 -> 239 and of 819 44.2 -> 44.6; head_dim 80, 200 images of 64 to 256 tokens
     // 101.5 -> 94.6, 65 536 long-tailed ones 2940 -> 2850, images of 2048 765 -> 700, but of 100 (one tile each) 187 -> 200.
     const bool staged = max_seqlen > (head_dim == 64 ? 1024 : 128);
-    if (head_dim == 64) return split ? launch(launch_fwd<64, true, false>) : staged ? launch(launch_fwd<64, false, true>) : launch(launch_fwd<64, false, false>);
-    return split ? launch(launch_fwd<80, true, false>) : staged ? launch(launch_fwd<80, false, true>) : launch(launch_fwd<80, false, false>);
+    // Who gets the next unit.  Asked for at the start of a unit, the units of the second wave go to the CTAs whose first ones are the
+    // longest, as all start at once; asked for towards the end (kLate), to those that are done first.  That is worth it where a
+    // list of several lengths goes around a few times only: 29 images of 35 to 154, 8 heads, 9.9 -> 8.1 us (head_dim 80 10.8 -> 8.7), 25
+    // of 300 20.1 -> 19.1, 74 of 300 at head_dim 80 52.3 -> 51.2, 64 of 512 53.6 -> 53.2.  The answer is then waited for by units of
+    // one key tile (2062 of 16 tokens 458 -> 468, head_dim 80 490 -> 522) and by the end of a list without a second wave (one
+    // image of 4096, 4 heads, 36.0 -> 36.9), and over many waves the lengths even out (40 of 819, 16 heads, 182.7 -> 184.5).
+    const int64_t units = int64_t(n_fwd_items) * n_heads;
+    const bool late = max_seqlen > kTileN && units > sm_count() && units <= 8 * int64_t(sm_count());
+    auto pick = [&](auto dim) {
+        constexpr int D = decltype(dim)::value;
+        if (split) return launch(launch_fwd<D, true, false, false>);
+        if (staged) return late ? launch(launch_fwd<D, false, true, true>) : launch(launch_fwd<D, false, true, false>);
+        return late ? launch(launch_fwd<D, false, false, true>) : launch(launch_fwd<D, false, false, false>);
+    };
+    return head_dim == 64 ? pick(std::integral_constant<int, 64>()) : pick(std::integral_constant<int, 80>());
 }
 
 }  // namespace mpipe
