@@ -568,7 +568,7 @@ def layer_flops(w, ffn):
 
 def layer_arm(args):
     """The whole packed encoder layer forward (frozen mode: the layer a frozen encoder executes per microbatch) through
-    mpipe_encoder_layer_fwd.  Same line format; `roofline` covers linear_fwd_kernel over the layer's four projections."""
+    mpipe_encoder_layer_fwd.  Same line format; `roofline` covers linear_kernel over the layer's four projections."""
     import torch
     from paper_2607_03229_b200 import binding as B
     from paper_2607_03229_b200 import dist as D
@@ -725,7 +725,7 @@ def layer_arm(args):
                           "layernorm_gbs": 4.0 * T * hidden / (kern_ms["layernorm"] * 1e-3) / 1e9,
                           "frac_of_bf16_peak": {"measured_sustained": value / world / peak_tf, "measured_burst": value / world / peaks["bf16_tflops"],
                                                 "nominal_2250": value / world / NOMINAL_BF16_TFLOPS}},
-            "roofline": {"kernel": "linear_fwd_kernel (4 launches per step)", "bound": "tensor", "achieved": lin_tf, "peak": peak_tf,
+            "roofline": {"kernel": "linear_kernel (4 launches per step)", "bound": "tensor", "achieved": lin_tf, "peak": peak_tf,
                          "unit": "TFLOP/s", "frac": lin_tf / peak_tf, "peak_kind": f"{peak_kind}, sustained bf16 GEMM", "traffic": None},
             "e2e": {"value": flops_all / (ms_e2e_mx * 1e-3) / 1e12, "unit": UNIT, "ms_per_step": ms_e2e_mx, "steps": Ke,
                     "h2d_bytes_per_step": int(hx.numel() * 2) * (2 if trained else 1),
