@@ -246,6 +246,7 @@ int32_t mpipe_validate_positions(const int32_t* positions, int32_t n, int32_t n_
  *                        aligned), fp32 accumulation on the tensor cores, act = GELU (u Phi(u), erf form) when
  *                        flags has MPIPE_LINEAR_GELU, identity otherwise; bias and residual may be NULL.
  *                        N and K multiples of 8 (MPIPE_ERR_UNSUPPORTED otherwise); M == 0 launches nothing.
+ *                        A row of C has the same bits whatever M is: every tile sums the contraction in one order.
  *   mpipe_layernorm_fwd  y[t, :] = (x[t, :] - mean_t) * rsqrt(var_t + eps) * gamma + beta, biased variance, fp32
  *                        statistics; bf16 in and out, hidden a multiple of 8 and <= 2048.
  *   mpipe_rope_apply     rotary position encoding, rotate-half form, in place on q and k of a packed projection:
@@ -267,7 +268,9 @@ int32_t mpipe_validate_positions(const int32_t* positions, int32_t n, int32_t n_
  *        caller-owned; after a TRAINED call it holds what mpipe_encoder_layer_bwd reads (see there), otherwise its contents are
  *        undefined afterwards.  In both modes the activation is applied to the fp32 accumulator of the fc1 projection;
  *        the TRAINED forward stores the pre-activation (bf16) from the same accumulator in the same launch, so y is
- *        bit-identical in the two modes (Corollary 1: freezing changes nothing in the forward).  Seven launches (eight
+ *        bit-identical in the two modes (Corollary 1: freezing changes nothing in the forward), and an image's rows of y are
+ *        the same bits alone and packed with others.  A weight matrix that is NULL (MPIPE_ERR_INVALID_ARG) or not 16-byte
+ *        aligned (MPIPE_ERR_UNSUPPORTED) is refused before anything is launched.  Seven launches (eight
  *        with rope) on `stream`, no allocation, no sync.
  *        head_dim = hidden / n_heads must be one the attention kernels support (64, 80).
  * Device-side findings (a bounded wait that ran out) are reported through status_buf as for the attention calls.
@@ -327,7 +330,7 @@ int32_t mpipe_colsum_accumulate(const void* a, float* out, int32_t n_tokens, int
  * rope tables), untouched since: it holds the LN2 output, the rotated q | k | v, the attention output, x1, GELU(u) and
  * (TRAINED forward only) the MLP pre-activation u; nothing in it is changed here.  lse is that call's LSE.  The LN1 output
  * is recomputed instead of being stored by the forward.  workspace: device, 256-byte aligned,
- * >= mpipe_encoder_layer_bwd_workspace_bytes.  Fifteen launches on `stream`, nothing allocated.  bwd_items_dev /
+ * >= mpipe_encoder_layer_bwd_workspace_bytes.  Fourteen launches on `stream`, nothing allocated.  bwd_items_dev /
  * n_bwd_items are the plan's backward list.  Sums over tokens use fp32 atomics and TMA reductions: parameter gradients
  * are reproducible to rounding order only.
  */

@@ -654,8 +654,8 @@ int32_t varlen_attn_fwd(const void* q, const void* k, const void* v, void* o, fl
     prm.status_buf = status_buf;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     // Two query tiles per CTA share every K/V tile and run side by side, which is 1.4 x the work per clock of one; where so few
-    // units would leave half of the SMs idle, one tile each is sooner done (one image of 777 tokens, 16 heads of 64: 14.9 -> 12.4 us,
-    // of 300: 9.3 -> 7.7; with 80 units on 148 SMs a second round of single tiles would cost more than it saves).
+    // units would leave half of the SMs idle, one tile each is sooner done (one image of 777 tokens, 16 heads of 64: 13.8 -> 11.8 us,
+    // of 300: 8.9 -> 7.5; with 80 units on 148 SMs a second round of single tiles would cost more than it saves).
     const bool split = 2 * int64_t(n_fwd_items) * n_heads <= sm_count();
     auto launch = [&](auto f) { return f(q, k, v, tok_stride_qkv, head_stride_qkv, total_tokens, n_heads, prm, st); };
     // Staged O pays where units have two query tiles and enough key tiles behind them (us direct -> staged): head_dim 64, ViT-L

@@ -11,7 +11,7 @@
 // pair 64.  Persistent: pair i takes tiles i, i + pairs, ... (n fastest, so that a wave shares the weight tiles in L2 and walks
 // down the token rows together).  Warp roles of each CTA (384 threads):
 //   warps 0, 3  TMA producers of the CTA's half, A box [128 rows][64 k] and B box [BN / 2 rows][64 k] (MN-major: boxes of 64
-//               columns) per stage, 128-byte swizzle, 5 to 8 stages; the bytes of both CTAs are counted on the even CTA's barrier
+//               columns) per stage, 128-byte swizzle, 3 to 8 stages of 20 to 48 KB; the bytes of both CTAs are counted on the even CTA's barrier
 //   warp 1      (even CTA) tcgen05 issuer: 4 x (M 256, N BN, K 16) per stage into one of TWO accumulators of up to 256 columns, so
 //               that the epilogue of tile i overlaps the main loop of tile i + 1
 //   warp 2      TMEM allocation
@@ -25,8 +25,8 @@
 // up to 4 us sooner done with an input gradient (300 x 4096 -> 1024 11.2 against 13.8 us; forward of 777 rows 12.5 against 11.7): the
 // halves meet in another order than the one accumulator of a large microbatch adds in.
 // Measured against the one-CTA 128 x 256 kernel with warpgroup-wide staging that this replaces (us, M = 50 439): fc1 + GELU
-// 1024 -> 4096 398 -> 325, its gradient with GELU' 480 -> 383, attention output + residual 115 -> 90, QKV 241 -> 221 (1430
-// TFLOP/s), weight gradient 1024 x 4096 348 -> 292; M = 777: fc2 27.9 -> 11.7, output projection 14.4 -> 7.2, weight
+// 1024 -> 4096 394 -> 322, its gradient with GELU' 480 -> 374, attention output + residual 120 -> 87, QKV 232 -> 214 (1480
+// TFLOP/s), weight gradient 1024 x 4096 345 -> 288, one launch at a time; M = 777: fc2 27.9 -> 11.7, output projection 14.4 -> 7.2, weight
 // gradient 1024 x 4096 34 -> 12.
 // Every mbarrier wait is bounded (status MPIPE_ERR_TIMEOUT), as in the attention kernels.
 #include <cuda_bf16.h>
@@ -46,7 +46,7 @@ constexpr int kGemmMaxBN = 256;
 // the weight gradient has four more warps, which add up the columns of its first operand (the bias gradient) from the stages
 __host__ __device__ constexpr int gemm_threads(int mode) { return mode == 2 ? 512 : 384; }
 constexpr int kGemmABytes = kGemmBM * kGemmBK * 2;            // 16 KB
-constexpr int kGemmRing = 160 * 1024, kGemmMaxStages = 8;     // 5 stages at BN 256 and 192, 6 at 128, 8 at 64
+constexpr int kGemmRing = 160 * 1024, kGemmMaxStages = 8;     // 5 stages at BN 256 and 192, 6 at 128, 8 at 64 (of two blocks of the contraction: 3 and 4)
 constexpr int kGemmBox = 32 * 128;                            // [32 rows][128 bytes] staging box of one warp
 constexpr int kGemmSmemOut = kGemmRing;                       // 8 warps x 2 boxes
 constexpr int kGemmSmem = kGemmSmemOut + 8 * 2 * kGemmBox + 1024;
@@ -642,7 +642,7 @@ static int32_t launch_wgrad(const void* dy, const void* x, float* dw, float* db,
     // about 12 bytes per clock and SM (the L2's rate of fp32 reductions with every SM adding) beside the next item's main loop.
     // A long token range runs into the power limit, where the sum of the work counts and not its spread over the pairs: no
     // estimate goes below the work at 68 % of the tensor peak, and among equals the fewest splits (least reduction traffic) win
-    // (1024 x 4096 over 50 439 tokens: 322 us unsplit on 64 of the 74 pairs, 355 to 415 us for any split).
+    // (1024 x 4096 over 50 439 tokens, back to back under that limit: 322 us unsplit on 64 of the 74 pairs, 355 to 415 us for any split).
     GemmParams p = {};
     const int nk = cdiv(tokens, kGemmBK);
     double best_clk = 1e30;

@@ -510,7 +510,7 @@ static int32_t layer_matrices_ok(const mpipe_layer_weights_t& w) {
 }
 
 // What the kernels behind a projection will read (n elements each; 16-byte aligned, see layer_matrices_ok).  A small microbatch reads every weight once and meets it cold: 24
-// layers of 25 MB, one image of 777 tokens, 1676 -> 1640 us; 1500 tokens, forward of 12 layers 1109 -> 1083.  From some
+// layers of 25 MB, one image of 777 tokens, 1420 -> 1389 us, of 300 at hidden 1280 1379 -> 1284; 1500 tokens, 12 layers 964 -> 940.  From some
 // thousand tokens on a weight is read by many tiles and its first read is nothing.
 static mpipe::LayerAhead layer_ahead(int32_t n_tokens, const void* w0, size_t n0, const void* w1 = nullptr, size_t n1 = 0) {
     mpipe::LayerAhead a;

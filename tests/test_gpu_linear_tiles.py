@@ -1,6 +1,5 @@
-"""The projection kernel at the sizes where its tile width, its contraction split and its ragged edges change, against the fp64
-oracle: every width (64, 128, 192, 256), a contraction split over two CTA pairs, rows on both sides of a 256-row tile, and the
-epilogues that carry two operands at once."""
+"""The projection kernel at the sizes where its tile width and its ragged edges change, against the fp64 oracle: every width (64, 128,
+192, 256), rows on both sides of a 256-row tile, and the epilogues that carry two operands at once."""
 import numpy as np
 import pytest
 import torch
@@ -25,8 +24,8 @@ def _close(got, ref):
                                    (255, 1032, 72), (257, 1032, 72),   # one 256-row tile and two
                                    (777, 3072, 1024),   # width 192
                                    (777, 4096, 1024),   # width 256
-                                   (300, 520, 2048),    # contraction split over two pairs, ragged last chunk
-                                   (777, 1024, 4096),   # the same, four row tiles
+                                   (300, 520, 2048),    # two tiles of rows, ragged last chunk
+                                   (777, 1024, 4096),   # four row tiles, a long contraction
                                    (90, 320, 192), (90, 320, 200),   # two blocks of the contraction per stage, an odd number of them; whole atoms or not
                                    (4000, 1288, 136)])  # several tiles per pair
 def test_linear_and_dgrad_tile_choices(M, N, K):
