@@ -6,6 +6,7 @@
 //   2. main      persistent CTAs, one per SM, take (key tile, head) units as they get free (units.cuh); a unit keeps one 128-key
 //                K/V tile resident and steps through the 128-row query tiles of the same segment
 //   3. convert   dQ = softmax_scale * accumulator -> bf16
+// Lists of short segments go without the accumulator and the third launch: there a CTA takes all key tiles of a segment (kOwn, own_segments).
 //
 // Main kernel, per step = one [128 keys x 128 queries] block (everything transposed so that the key index is the
 // TMEM lane):
@@ -52,11 +53,29 @@ static_assert(4 * (kRegsLaunch - kRegsService) + 4 * (kRegsLaunch - kRegsReducer
               "setmaxnreg pool arithmetic");
 constexpr int kBT = 128;  // keys per unit = TMEM lanes
 constexpr int kBQ = 128;  // query rows per step
-// head_dim 80, segments of up to three tiles and more units than SMs: the pooled tile buffers (BwdCfg::kPool).  Every tile then costs the
+// head_dim 80, segments of up to three tiles and more units than SMs, or a CTA per segment: the pooled tile buffers (BwdCfg::kPool).  Every tile then costs the
 // issuer and the producer a hand-shake of its own, 0.1 to 0.3 us a step, which a short unit gets back from loads that no longer wait
 // for its end.  us, two buffers a kind -> pool: 1024 segments of 64 rows 748 -> 625, 256 of 256 610 -> 557, 200 thumbnails of 64 to 256
 // 369 -> 330, 218 of 300 813 -> 801, 163 of 400 944 -> 962, 32 of 2048 2151 -> 2278, one of 200 (a unit per CTA) 17.4 -> 18.4.
 constexpr int kPoolSeqlen = 384;
+// Lists of short segments: one CTA takes all key tiles of a (segment, head), one after the other, instead of one CTA per key tile.  dQ then
+// needs no sum across CTAs: no accumulator to clear (prepass) and to convert (third launch), no reductions through the copy engine, and
+// the same bits on every run.  A query tile's partial dQ waits in the workspace between key tiles, in L2, each thread's row for that
+// thread.  us, a CTA per key tile -> per segment (16 heads of 64 | 80): 4 segments of 64 14.1 -> 10.0 | 15.4 -> 10.8, 512 of 64 229 -> 206 |
+// 338 -> 302, 256 of 128 184 -> 130 | 239 -> 175, 6 of 192 19.3 -> 17.2 | 25.1 -> 22.7, 128 of 256 226 -> 190 | 310 -> 262, 85 of 384
+// 263 -> 237 | 349 -> 351, 200 thumbnails of 64 to 256 243 -> 196 | 316 -> 265.  From four tiles on it is level or slower (64 of 512
+// 324 -> 298 | 454 -> 443, but 32 of 512 164 -> 168 | 228 -> 240, 32 of 1024 544 -> 634 | 720 -> 1057: every step stores and reloads 128 rows), and so it
+// is where whole segments spread worse over the SMs than key tiles do (3 of 192 13.5 -> 15.3 | 17.5 -> 20.5, 12 of 384 45 -> 51 | 66 -> 78):
+// estimated in rounds of one key tile per SM, it may take a tenth more of them.
+constexpr int kOwnTiles = 3;
+static bool own_segments(int64_t n_seg, int64_t n_items, int32_t max_seqlen, int64_t heads, int64_t sms) {
+    const int64_t tiles = (int64_t(max_seqlen) + kBT - 1) / kBT, segs = n_seg < n_items ? n_seg : n_items;
+    if (tiles > kOwnTiles) return false;
+    const int64_t by_tile = (n_items * heads + sms - 1) / sms;
+    // all of the longest: whole waves of them; mixed lengths, longest first, even out to about one key tile
+    const int64_t by_segment = n_items == segs * tiles ? (segs * heads + sms - 1) / sms * tiles : by_tile + 1;
+    return 10 * by_segment <= 11 * by_tile;
+}
 constexpr int kQH = 64;   // query columns of a step handled by one softmax warpgroup
 
 // Shared-memory layout of a [128 rows x head_dim] bf16 tile.  head_dim 64: one TMA box, rows of 128 bytes, 128-byte
@@ -128,7 +147,8 @@ struct BwdParams {
     int32_t n_items, n_heads, total_tokens;
     const float* lse;    // [H, T]
     const float* delta;  // [H, T]
-    __nv_bfloat16 *dk, *dv;
+    __nv_bfloat16 *dq, *dk, *dv;   // dq, dq_acc: read where a CTA owns its segments; elsewhere dQ goes through BwdMaps::dq_acc
+    float* dq_acc;
     int64_t tok_stride_g, head_stride_g;
     float scale, scale_log2;
     const float *rope_cos, *rope_sin;   // host only: tables of the rotation that dQ and dK are turned back by, or null
@@ -148,7 +168,17 @@ struct BwdMaps {
     CUtensorMap q, k, v, dout, dq_acc;
 };
 
-template <int D, bool kPooled>
+// A rejected plan leaves dQ all zeros.  (A function apart: its divisions, inlined, cost the kernel's roles registers.)
+template <int D>
+static __device__ __noinline__ void zero_dq(__nv_bfloat16* dq, int64_t tok_stride, int64_t head_stride, int32_t total_tokens, int32_t n_heads) {
+    const int64_t n = int64_t(total_tokens) * n_heads * (D / 8);
+    for (int64_t i = int64_t(blockIdx.x) * kBwdThreads + threadIdx.x; i < n; i += int64_t(gridDim.x) * kBwdThreads) {
+        const int64_t th = i / (D / 8), t = th / n_heads;
+        *reinterpret_cast<uint4*>(dq + t * tok_stride + (th - t * n_heads) * head_stride + (i - th * (D / 8)) * 8) = make_uint4(0u, 0u, 0u, 0u);
+    }
+}
+
+template <int D, bool kPooled, bool kOwn>
 __global__ void __maxnreg__(kRegsLaunch)
 attn_bwd_kernel(const __grid_constant__ BwdMaps maps, const BwdParams p) {
     using Cfg = BwdCfg<D, kPooled>;
@@ -167,7 +197,7 @@ attn_bwd_kernel(const __grid_constant__ BwdMaps maps, const BwdParams p) {
 
     if (tid == 0) {
         abort_flag = 0;
-        unit_ring_init(&units, 11);             // the issuer, the staging warp, the softmax warps and the reducer warpgroup read it
+        unit_ring_init(&units, kOwn ? 14 : 11); // the issuer, the staging warp, the softmax warps and the reducer warps (one thread for all four) read it
         for (int i = 0; i < 2; ++i) {
             mbar_init(&bars.kv_full[i], 1);
             mbar_init(&bars.kv_empty[i], 1);
@@ -215,6 +245,7 @@ attn_bwd_kernel(const __grid_constant__ BwdMaps maps, const BwdParams p) {
     const int n_units = plan_ok_cta(p.items, p.n_items, kBT, p.total_tokens, p.status_buf, &plan_flag) ? p.n_items * p.n_heads : 0;
     pdl_wait();
     pdl_launch();
+    if (kOwn && plan_flag >= 0) zero_dq<D>(p.dq, p.tok_stride_g, p.head_stride_g, p.total_tokens, p.n_heads);
     // Unit u -> (work item, head).  The items of one segment are consecutive in the list (tile 0, 1, ...), and their
     // units occupy the same stretch of the unit sequence whichever way it is ordered inside.  Short segments: tile by
     // tile, heads innermost.  Segments of more than kHeadMajorTiles key tiles: head by head, so that the CTAs running
@@ -229,7 +260,7 @@ attn_bwd_kernel(const __grid_constant__ BwdMaps maps, const BwdParams p) {
         const int i0 = u / p.n_heads;
         const mpipe_work_item_t a = p.items[i0];
         const int nt = (a.kv_len + kBT - 1) / kBT;                   // key tiles of this item's segment
-        if (nt <= kHeadMajorTiles) {
+        if (kOwn || nt <= kHeadMajorTiles) {
             z = a;
             z.seg = u % p.n_heads;
             return z;
@@ -247,7 +278,7 @@ attn_bwd_kernel(const __grid_constant__ BwdMaps maps, const BwdParams p) {
     // The j-th step of a unit works on query tile (j + key tile index) mod steps: the CTAs that hold the key tiles of
     // one (segment, head) run at the same time, and started on the same query tile they would all add to the same rows
     // of the dQ accumulator at once (fp32 adds to one address serialise in L2) and ask for the same Q / dO tile.
-    auto q_tile_of = [](const mpipe_work_item_t& it, int j, int nq) { return (j + (it.tile >= 0 ? it.tile : 0)) % nq; };
+    auto q_tile_of = [](const mpipe_work_item_t& it, int j, int nq) { return kOwn ? j : (j + (it.tile >= 0 ? it.tile : 0)) % nq; };
 
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer
@@ -275,25 +306,21 @@ attn_bwd_kernel(const __grid_constant__ BwdMaps maps, const BwdParams p) {
                 return true;
             };
             UnitSource source{&units, &abort_flag};
-            for (int u = int(blockIdx.x); ok; ++unit_it) {
-                const mpipe_work_item_t it = item_at(u);
-                ok = source.put(it);
-                if (!ok || it.kv_len <= 0) break;
+            // The key tile `it` of a unit; after_last: the unit ends with it, and the next one is asked for.
+            auto load_unit = [&](const mpipe_work_item_t& it, bool after_last) {
                 const int head = it.seg;
                 const int nq = steps_of(it);
+                const int ask_at = !after_last ? -1 : nq > 3 ? nq - 3 : 0;   // late enough to go to the CTA that is free first, early enough to be answered
                 if (Cfg::kPool) {   // K, Q_0, V, dO_0, Q_1, dO_1, ...: the order in which the issuer comes to need them
-                    const int ask_at = nq > 3 ? nq - 3 : 0;
-                    for (int j = 0; j < nq && ok; ++j) {
+                    for (int j = 0; j < nq; ++j) {
                         if (j == ask_at) source.ask();
                         const int row = it.kv_start + q_tile_of(it, j, nq) * kBQ;
-                        if (j == 0) ok = pool_load(&maps.k, head, it.row_start);
-                        ok = ok && pool_load(&maps.q, head, row);
-                        if (j == 0) ok = ok && pool_load(&maps.v, head, it.row_start);
-                        ok = ok && pool_load(&maps.dout, head, row);
+                        if (j == 0 && !pool_load(&maps.k, head, it.row_start)) return false;
+                        if (!pool_load(&maps.q, head, row)) return false;
+                        if (j == 0 && !pool_load(&maps.v, head, it.row_start)) return false;
+                        if (!pool_load(&maps.dout, head, row)) return false;
                     }
-                    if (!ok) break;
-                    u = source.take(&ok);
-                    continue;
+                    return true;
                 }
                 // Before its buffers are free, a short unit's first tiles are asked for into L2 (a long unit's Q and dO are there
                 // already, and it computes for so long that its K and V do not matter).
@@ -309,23 +336,41 @@ attn_bwd_kernel(const __grid_constant__ BwdMaps maps, const BwdParams p) {
                 }
                 const int kb = unit_it % Cfg::kKVBufs;            // K/V buffer of this unit
                 uint8_t* kv = smem + kb * (2 * Cfg::kTile);
-                ok = mbar_wait<kSleepAux>(&bars.kv_empty[kb], ((unit_it / Cfg::kKVBufs) & 1) ^ 1, &abort_flag);
-                if (!ok) break;
+                if (!mbar_wait<kSleepAux>(&bars.kv_empty[kb], ((unit_it / Cfg::kKVBufs) & 1) ^ 1, &abort_flag)) return false;
                 mbar_expect_tx(&bars.kv_full[kb], 2 * Cfg::kTile);
                 load_tile(kv + Cfg::kSmemK, &maps.k, &bars.kv_full[kb], head, it.row_start);
                 load_tile(kv + Cfg::kSmemV, &maps.v, &bars.kv_full[kb], head, it.row_start);
-                const int ask_at = nq > 3 ? nq - 3 : 0;   // late enough to go to the CTA that is free first, early enough to be answered
                 for (int j = 0; j < nq; ++j, ++sc) {
                     if (j == ask_at) source.ask();
                     const int rs = sc % NR;
                     const int row = it.kv_start + q_tile_of(it, j, nq) * kBQ;
-                    ok = mbar_wait<kSleepAux>(&bars.qdo_empty[rs], ((sc / NR) & 1) ^ 1, &abort_flag);
-                    if (!ok) break;
+                    if (!mbar_wait<kSleepAux>(&bars.qdo_empty[rs], ((sc / NR) & 1) ^ 1, &abort_flag)) return false;
                     mbar_expect_tx(&bars.qdo_full[rs], 2 * Cfg::kTile);
                     load_tile(smem + Cfg::kSmemQ + rs * Cfg::kTile, &maps.q, &bars.qdo_full[rs], head, row);
                     load_tile(smem + Cfg::kSmemDO + rs * Cfg::kTile, &maps.dout, &bars.qdo_full[rs], head, row);
                 }
-                if (!ok) break;
+                return true;
+            };
+            for (int u = int(blockIdx.x); ok;) {
+                mpipe_work_item_t it = item_at(u);
+                if (kOwn && it.row_start != it.kv_start) {        // a later key tile: the CTA with its segment's first one does it
+                    source.ask();
+                    u = source.take(&ok);
+                    continue;
+                }
+                const int nt = kOwn ? steps_of(it) : 1;
+                for (int t = 0; t < nt || it.kv_len <= 0; ++t, ++unit_it) {
+                    if (kOwn) {
+                        it.tile = t;
+                        it.row_start = it.kv_start + t * kBT;
+                        it.row_len = min(kBT, it.kv_len - t * kBT);
+                    }
+                    ok = source.put(it);
+                    if (!ok || it.kv_len <= 0) break;
+                    ok = load_unit(it, t + 1 == nt);
+                    if (!ok) break;
+                }
+                if (!ok || it.kv_len <= 0) break;
                 u = source.take(&ok);
             }
             if (!ok) source.cancel_rest();
@@ -731,6 +776,7 @@ attn_bwd_kernel(const __grid_constant__ BwdMaps maps, const BwdParams p) {
         // (reducer_item is read before, and written again after, the barriers of at least one step).
         mpipe_work_item_t it;
         auto fetch_unit = [&](uint32_t i) {
+            if (kOwn) return next_unit(&units, i, &it, lane, &abort_flag);
             if (rt == 0) {
                 mpipe_work_item_t x = {0, 0, 0, 0, 0, 0};
                 if (mbar_wait(&units.full[i % kUnitRing], (i / kUnitRing) & 1, &abort_flag)) {
@@ -789,6 +835,60 @@ attn_bwd_kernel(const __grid_constant__ BwdMaps maps, const BwdParams p) {
             // they keep walking the (now empty) iterations together instead of leaving one another behind.
             for (int i = 0; i < nq; ++i, ++pc) {
                 if (Cfg::kEarlyOut && i + 1 == nq) epilogue();
+                if (kOwn) {
+                    // dQ of a query tile waits in the workspace for the next key tile, each thread's row for that thread (element group g
+                    // of row r at [g][r]: whole lines), and leaves as bf16 with the last one.
+                    const int rows = min(kBQ, it.kv_len - i * kBQ);
+                    const bool first = it.row_start == it.kv_start, last = it.row_start + it.row_len == it.kv_start + it.kv_len;
+                    const bool in = r < rows;
+                    float4* part = reinterpret_cast<float4*>(p.dq_acc + (int64_t(it.kv_start) * p.n_heads + int64_t(head) * it.kv_len + i * kBQ) * D) + r;
+                    __nv_bfloat16* row = p.dq + (int64_t(it.kv_start) + i * kBQ + r) * p.tok_stride_g + int64_t(head) * p.head_stride_g;
+                    float4 x[2][4];   // asked for 16 columns ahead
+                    auto ask = [&](int ch) {
+#pragma unroll
+                        for (int g = 0; g < 4; ++g) x[ch & 1][g] = !first && in ? __ldcg(part + (4 * ch + g) * rows) : make_float4(0.f, 0.f, 0.f, 0.f);
+                    };
+                    ask(0);
+                    if (ok) ok = mbar_wait<kSleepAux>(&bars.dq_full, pc & 1, &abort_flag);
+                    if (!ok) break;
+                    tc_fence_after();
+#pragma unroll
+                    for (int ch = 0; ch < D / 16; ++ch) {
+                        uint32_t v[16];
+                        if (ch + 1 < D / 16) ask(ch + 1);
+                        tmem_ld16(tmem + lane_base + Cfg::kColDQ + 16 * ch, v);
+                        tmem_wait_ld();
+                        if (ch == D / 16 - 1) {   // the whole row has left TMEM: the next step's dQ may be issued
+                            tc_fence_before();
+                            __syncwarp();
+                            if (lane == 0) mbar_arrive(&bars.dq_empty);
+                        }
+                        float4 y[4];
+#pragma unroll
+                        for (int g = 0; g < 4; ++g) {
+                            const float2 a = add2(make_float2(x[ch & 1][g].x, x[ch & 1][g].y), make_float2(__uint_as_float(v[4 * g]), __uint_as_float(v[4 * g + 1])));
+                            const float2 b = add2(make_float2(x[ch & 1][g].z, x[ch & 1][g].w), make_float2(__uint_as_float(v[4 * g + 2]), __uint_as_float(v[4 * g + 3])));
+                            y[g] = make_float4(a.x, a.y, b.x, b.y);
+                        }
+                        if (!last) {
+#pragma unroll
+                            for (int g = 0; g < 4; ++g)
+                                if (in) __stcg(part + (4 * ch + g) * rows, y[g]);
+                        } else {
+#pragma unroll
+                            for (int c8 = 0; c8 < 2; ++c8) {
+                                const float4 a = y[2 * c8], b = y[2 * c8 + 1];
+                                uint4 o;
+                                o.x = pack_bf16(a.x * p.scale, a.y * p.scale);
+                                o.y = pack_bf16(a.z * p.scale, a.w * p.scale);
+                                o.z = pack_bf16(b.x * p.scale, b.y * p.scale);
+                                o.w = pack_bf16(b.z * p.scale, b.w * p.scale);
+                                if (in) *reinterpret_cast<uint4*>(row + 16 * ch + 8 * c8) = o;
+                            }
+                        }
+                    }
+                    continue;
+                }
                 if (ok) ok = mbar_wait<kSleepAux>(&bars.dq_full, pc & 1, &abort_flag);
                 tc_fence_after();
                 const int q0 = it.kv_start + q_tile_of(it, i, nq) * kBQ;
@@ -824,7 +924,7 @@ attn_bwd_kernel(const __grid_constant__ BwdMaps maps, const BwdParams p) {
             }
             if (!Cfg::kEarlyOut) epilogue();
         }
-        if (rt == 0) bulk_wait_group<0>();   // all reductions have landed before the CTA exits
+        if (!kOwn && rt == 0) bulk_wait_group<0>();   // all reductions have landed before the CTA exits
     }
 
     tc_fence_before();
@@ -833,7 +933,7 @@ attn_bwd_kernel(const __grid_constant__ BwdMaps maps, const BwdParams p) {
     if (tid == 0 && abort_flag) report_status(p.status_buf, MPIPE_ERR_TIMEOUT, int32_t(blockIdx.x));
 }
 
-// Delta[h,t] = sum_d dO[t,h,d] * O[t,h,d], and the fp32 dQ accumulator is cleared.  HBM-bound helper, 8 bytes per element:
+// Delta[h,t] = sum_d dO[t,h,d] * O[t,h,d], and the fp32 dQ accumulator (where there is one) is cleared.  HBM-bound helper, 8 bytes per element:
 // D / 16 lanes share one (t,h) row, each with 32 bytes of dO and of O (head_dim 64: 4 lanes, 8 rows per warp; 80: 5 lanes, 6 rows and
 // two idle lanes), partial dot products are combined with shuffles; the accumulator is cleared with flat 16-byte stores.
 // (With 16 lanes per row, ten of them busy, head_dim 80 ran at 4.7 TB/s: 72.5 us for 33 012 tokens of 16 heads.)
@@ -869,7 +969,7 @@ bwd_prepass_kernel(const __nv_bfloat16* __restrict__ dout, const __nv_bfloat16* 
         // clear the accumulator rows of this block: kRowsPerBlock * D floats, contiguous
         const int64_t z0 = row0 * D, z1 = (row0 + kRowsPerBlock < n_rows ? row0 + kRowsPerBlock : n_rows) * D;
         float4* z = reinterpret_cast<float4*>(dq_acc);
-        for (int64_t i = z0 / 4 + threadIdx.x; i < z1 / 4; i += 256) z[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int64_t i = z0 / 4 + threadIdx.x; dq_acc != nullptr && i < z1 / 4; i += 256) z[i] = make_float4(0.f, 0.f, 0.f, 0.f);
         // sum over the row's lanes into its first one: lane + 4 (of 5), then + 2, then + 1
         if (kLanes == 5) {
             const float last = __shfl_down_sync(0xffffffffu, acc, 4);
@@ -956,7 +1056,7 @@ bwd_dq_convert_rope_kernel(const float* __restrict__ acc, __nv_bfloat16* __restr
     *reinterpret_cast<uint4*>(row + kHalf) = make_uint4(ob[0], ob[1], ob[2], ob[3]);
 }
 
-template <int D, bool kPooled>
+template <int D, bool kPooled, bool kOwn>
 static int32_t launch_bwd(const void* dout, const void* q, const void* k, const void* v, const void* o, void* dq,
                           int64_t ts_qkv, int64_t hs_qkv, int64_t ts_o, int64_t hs_o, int32_t total_tokens,
                           int32_t n_heads, BwdParams prm, float* delta, float* dq_acc, cudaStream_t stream) {
@@ -972,7 +1072,7 @@ static int32_t launch_bwd(const void* dout, const void* q, const void* k, const 
         !make_tensor_map_thd(&m.dout, dout, total_tokens, n_heads, D, ts_o, hs_o, box, kBQ, swz) ||
         !make_tensor_map_thd(&m.dq_acc, dq_acc, total_tokens, n_heads, D, int64_t(n_heads) * D, D, 16, kBQ, 64, 4))
         return MPIPE_ERR_CUDA;
-    if (!ensure_dynamic_smem<attn_bwd_kernel<D, kPooled>>(Cfg::kSmemAlloc)) return MPIPE_ERR_CUDA;
+    if (!ensure_dynamic_smem<attn_bwd_kernel<D, kPooled, kOwn>>(Cfg::kSmemAlloc)) return MPIPE_ERR_CUDA;
     const bool rope = prm.rope_cos != nullptr;
     const int64_t chunks = rows * (rope ? D / 16 : D / 8);
     constexpr int kPrepassRows = 8 * (32 / (D / 16));   // rows of a block
@@ -980,13 +1080,14 @@ static int32_t launch_bwd(const void* dout, const void* q, const void* k, const 
     const int64_t prepass_cap = int64_t(sm_count()) * 64;
     cudaError_t e = launch_kernel(bwd_prepass_kernel<D>, unsigned(prepass_blocks < prepass_cap ? prepass_blocks : prepass_cap), 256, 0, stream, 1,
                                   static_cast<const __nv_bfloat16*>(dout), static_cast<const __nv_bfloat16*>(o), ts_o, hs_o, total_tokens,
-                                  n_heads, delta, dq_acc);
+                                  n_heads, delta, kOwn ? static_cast<float*>(nullptr) : dq_acc);
     if (e != cudaSuccess) return MPIPE_ERR_CUDA;
     const int n_units = prm.n_items * prm.n_heads;
     profile_start(kProfileBwdMain, stream);
-    e = launch_kernel_as(true, attn_bwd_kernel<D, kPooled>, unsigned(n_units), kBwdThreads, Cfg::kSmemAlloc, stream, 1, m, prm);
+    e = launch_kernel_as(true, attn_bwd_kernel<D, kPooled, kOwn>, unsigned(n_units), kBwdThreads, Cfg::kSmemAlloc, stream, 1, m, prm);
     profile_stop(kProfileBwdMain, stream);
     if (e != cudaSuccess) return MPIPE_ERR_CUDA;
+    if (kOwn) return cudaGetLastError() == cudaSuccess ? MPIPE_OK : MPIPE_ERR_CUDA;
     if (rope)
         e = launch_kernel(bwd_dq_convert_rope_kernel<D>, unsigned((2 * chunks + 255) / 256), 256, 0, stream, 1, static_cast<const float*>(dq_acc),
                           static_cast<__nv_bfloat16*>(dq), prm.dk, prm.tok_stride_g, prm.head_stride_g, prm.rope_cos, prm.rope_sin,
@@ -997,6 +1098,14 @@ static int32_t launch_bwd(const void* dout, const void* q, const void* k, const 
     return e == cudaSuccess && cudaGetLastError() == cudaSuccess ? MPIPE_OK : MPIPE_ERR_CUDA;
 }
 
+// Bytes from the first to behind the last element of a [tokens, heads, head_dim] tensor.
+static size_t extent_bytes(int64_t tokens, int64_t heads, int64_t head_dim, int64_t tok_stride, int64_t head_stride, size_t elem) {
+    return size_t((tokens - 1) * tok_stride + (heads - 1) * head_stride + head_dim) * elem;
+}
+static bool overlap(const void* a, size_t a_bytes, const void* b, size_t b_bytes) {
+    const uintptr_t x = reinterpret_cast<uintptr_t>(a), y = reinterpret_cast<uintptr_t>(b);
+    return x < y + b_bytes && y < x + a_bytes;
+}
 static size_t round256(size_t x) { return (x + 255) & ~size_t(255); }
 
 }  // namespace mpipe
@@ -1076,6 +1185,8 @@ static int32_t run_bwd(const float* rope_cos, const float* rope_sin, const void*
     prm.total_tokens = total_tokens;
     prm.lse = lse;
     prm.delta = delta;
+    prm.dq = static_cast<__nv_bfloat16*>(dq);
+    prm.dq_acc = dq_acc;
     prm.dk = static_cast<__nv_bfloat16*>(dk);
     prm.dv = static_cast<__nv_bfloat16*>(dv);
     prm.tok_stride_g = tok_stride_grad;
@@ -1086,14 +1197,22 @@ static int32_t run_bwd(const float* rope_cos, const float* rope_sin, const void*
     prm.rope_sin = rope_sin;
     prm.status_buf = status_buf;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    if (head_dim == 64)
-        return launch_bwd<64, false>(dout, q, k, v, o, dq, tok_stride_qkv, head_stride_qkv, tok_stride_o, head_stride_o,
-                                     total_tokens, n_heads, prm, delta, dq_acc, st);
-    if (max_seqlen <= kPoolSeqlen && int64_t(n_bwd_items) * n_heads > sm_count())
-        return launch_bwd<80, true>(dout, q, k, v, o, dq, tok_stride_qkv, head_stride_qkv, tok_stride_o, head_stride_o,
-                                    total_tokens, n_heads, prm, delta, dq_acc, st);
-    return launch_bwd<80, false>(dout, q, k, v, o, dq, tok_stride_qkv, head_stride_qkv, tok_stride_o, head_stride_o,
-                                 total_tokens, n_heads, prm, delta, dq_acc, st);
+    const int64_t units = int64_t(n_bwd_items) * n_heads;
+    // A CTA to a segment: not where dQ shares memory with something the kernel reads (an input may be replaced by its gradient
+    // where dQ is converted behind it) or is turned by the rotary encoding on its way.
+    const size_t dq_bytes = extent_bytes(total_tokens, n_heads, head_dim, tok_stride_grad, head_stride_grad, 2);
+    const size_t in_bytes = extent_bytes(total_tokens, n_heads, head_dim, tok_stride_qkv, head_stride_qkv, 2);
+    const size_t o_bytes = extent_bytes(total_tokens, n_heads, head_dim, tok_stride_o, head_stride_o, 2);
+    const bool own = rope_cos == nullptr && own_segments(n_seg, n_bwd_items, max_seqlen, n_heads, sm_count()) &&
+                     !overlap(dq, dq_bytes, q, in_bytes) && !overlap(dq, dq_bytes, k, in_bytes) && !overlap(dq, dq_bytes, v, in_bytes) &&
+                     !overlap(dq, dq_bytes, dout, o_bytes) && !overlap(dq, dq_bytes, o, o_bytes) &&
+                     !overlap(dq, dq_bytes, lse, size_t(total_tokens) * n_heads * 4);
+    auto launch = [&](auto run) {
+        return run(dout, q, k, v, o, dq, tok_stride_qkv, head_stride_qkv, tok_stride_o, head_stride_o, total_tokens, n_heads, prm, delta, dq_acc, st);
+    };
+    if (head_dim == 64) return own ? launch(launch_bwd<64, false, true>) : launch(launch_bwd<64, false, false>);
+    if (own) return launch(launch_bwd<80, true, true>);
+    return max_seqlen <= kPoolSeqlen && units > sm_count() ? launch(launch_bwd<80, true, false>) : launch(launch_bwd<80, false, false>);
 }
 
 int32_t mpipe_varlen_attn_bwd(const void* dout, const void* q, const void* k, const void* v, const void* o,

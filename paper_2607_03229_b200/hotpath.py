@@ -88,7 +88,8 @@ def run_step(w: Workload, buf: StepBuffers, plan: Optional[B.SegPlan] = None, st
 
 
 def kernels_per_step(w: Workload) -> int:
-    """Kernels of this library launched by one run_step (forward 1, backward 3, merge 1; the plan's upload is not counted)."""
+    """Kernels of this library launched by one run_step (forward 1, backward 3, or 2 where no segment is longer than a key tile, merge 1;
+    the plan's upload is not counted)."""
     if w.total_tokens == 0:
         return 0
-    return 1 + (3 if w.trained else 0) + (1 if w.merge_hidden is not None else 0)
+    return 1 + ((2 if max(w.patch_counts) <= B.bwd_tile_rows() else 3) if w.trained else 0) + (1 if w.merge_hidden is not None else 0)

@@ -1,0 +1,49 @@
+"""Attention backward of lists of short segments, where one CTA takes all key tiles of a segment and dQ never passes through the zeroed
+accumulator: segment lengths around the edges of a tile, key tiles of other heights than the native one, gradients in a strided tensor,
+and dQ in the memory of an input (which takes the general kernels), against the oracle."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2607_03229_b200 import binding as B, workloads as W
+from _util import GRAD_REL_L2, rel_l2, status_buf, to_dev, to_f64
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("D", [64, 80])
+@pytest.mark.parametrize("counts,rows", [([1], None), ([128, 127], None), ([129, 128, 1], None), ([255, 257, 3, 256], None),
+                                         ([384, 300], None), ([300, 64, 129], 64), ([300, 130], 100)])
+@pytest.mark.parametrize("into", ["own", "strided", "q", "dout"])
+def test_short_segments_at_tile_edges(counts, rows, D, into):
+    H, t = 3, sum(counts)
+    copies = torch.cuda.get_device_properties(0).multi_processor_count   # whole waves of segments: the rule takes every list here
+    T = copies * t
+    q, k, v, do = (W.normal_bf16(77, i, (t, H, D)) for i in range(4))
+    scale = float(np.float32(D ** -0.5))
+    plan = B.seg_plan(counts * copies, B.TRAINED, bwd_rows=rows).to_device()
+    cu = np.concatenate([[0], np.cumsum(counts)]).astype(np.int32)
+    qd, kd, vd, dod = (to_dev(x).repeat(copies, 1, 1) for x in (q, k, v, do))
+    o, lse, st = torch.empty_like(qd), torch.empty((H, T), device="cuda"), status_buf()
+    B.varlen_attn_fwd(qd, kd, vd, o, lse, plan, scale, st)
+    if into == "strided":
+        packed = torch.full((T, 3, H + 1, D + 8), 7.0, dtype=torch.bfloat16, device="cuda")
+        dq, dk, dv = (packed[:, i, :H, :D] for i in range(3))
+    else:
+        dq, dk, dv = (torch.full_like(qd, 7.0) for _ in range(3))
+        dq = {"own": dq, "q": qd, "dout": dod}[into]
+    ws = torch.full((B.attn_workspace_bytes(T, H, D, B.TRAINED),), 0x7f, dtype=torch.uint8, device="cuda")
+    B.varlen_attn_bwd(dod, qd, kd, vd, o, lse, dq, dk, dv, plan, scale, ws, st)
+    torch.cuda.synchronize()
+    assert st.cpu().tolist()[0] == 0
+    for i, (got, ref) in enumerate(zip((dq, dk, dv), oracle.attn_bwd(do, q, k, v, cu, scale))):
+        first = got[:t].contiguous()
+        if i > 0 or into in ("own", "strided"):                   # one order of additions: every copy has the same bits
+            assert torch.equal(got.reshape(copies, t, H, D), first.expand(copies, t, H, D))
+        if np.linalg.norm(ref) == 0:   # one token has no gradient; what is left is |dO| |O| |K| / sqrt(D) times the 2^-9 of O's rounding
+            assert np.abs(to_f64(first)).max() <= 2.0 ** -9 * D * 4 * 4 * scale
+        else:
+            assert rel_l2(to_f64(first), ref) <= GRAD_REL_L2
+    if into == "strided":
+        assert torch.all(packed[:, :, H:] == 7.0) and torch.all(packed[..., D:] == 7.0)
