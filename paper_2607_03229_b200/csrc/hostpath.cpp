@@ -115,6 +115,14 @@ Plan plan_of(PyObject* const* a, int64_t T, const char* what, bool used) {
     return p;
 }
 
+// A part of an integer tensor, which no gradient flows through: as_strided without the dispatcher.
+at::Tensor section(const at::Tensor& t, at::IntArrayRef sizes, at::IntArrayRef strides, int64_t offset) {
+    at::Tensor s = at::detail::make_tensor<c10::TensorImpl>(c10::TensorImpl::VIEW, c10::Storage(t.storage()), t.key_set(), t.dtype());
+    s.unsafeGetTensorImpl()->set_storage_offset(offset);
+    s.unsafeGetTensorImpl()->set_sizes_and_strides(sizes, strides);
+    return s;
+}
+
 template <typename F>
 PyObject* guarded(F&& f) {
     try {
@@ -223,9 +231,9 @@ PyObject* upload(PyObject*, PyObject* const* a, Py_ssize_t n) {
         PyObject* r = PyTuple_New(4);
         if (r == nullptr) throw Failed();
         PyTuple_SET_ITEM(r, 0, host.defined() ? THPVariable_Wrap(host) : Py_NewRef(Py_None));
-        PyTuple_SET_ITEM(r, 1, THPVariable_Wrap(d.as_strided({n_cu}, {1}, 0)));
-        PyTuple_SET_ITEM(r, 2, THPVariable_Wrap(d.as_strided({nf, 6}, {6, 1}, off_f)));
-        PyTuple_SET_ITEM(r, 3, THPVariable_Wrap(d.as_strided({nb, 6}, {6, 1}, off_b)));
+        PyTuple_SET_ITEM(r, 1, THPVariable_Wrap(section(d, {n_cu}, {1}, 0)));
+        PyTuple_SET_ITEM(r, 2, THPVariable_Wrap(section(d, {nf, 6}, {6, 1}, off_f)));
+        PyTuple_SET_ITEM(r, 3, THPVariable_Wrap(section(d, {nb, 6}, {6, 1}, off_b)));
         return r;
     });
 }
