@@ -843,47 +843,49 @@ attn_bwd_kernel(const __grid_constant__ BwdMaps maps, const BwdParams p) {
                     const bool in = r < rows;
                     float4* part = reinterpret_cast<float4*>(p.dq_acc + (int64_t(it.kv_start) * p.n_heads + int64_t(head) * it.kv_len + i * kBQ) * D) + r;
                     __nv_bfloat16* row = p.dq + (int64_t(it.kv_start) + i * kBQ + r) * p.tok_stride_g + int64_t(head) * p.head_stride_g;
-                    float4 x[2][4];   // asked for 16 columns ahead
-                    auto ask = [&](int ch) {
+                    float4 x[8];      // of 32 columns, asked for before they are needed
+                    auto ask = [&](int c0) {
 #pragma unroll
-                        for (int g = 0; g < 4; ++g) x[ch & 1][g] = !first && in ? __ldcg(part + (4 * ch + g) * rows) : make_float4(0.f, 0.f, 0.f, 0.f);
+                        for (int g = 0; g < (c0 + 32 <= D ? 8 : 4); ++g) x[g] = !first && in ? __ldcg(part + (c0 / 4 + g) * rows) : make_float4(0.f, 0.f, 0.f, 0.f);
                     };
                     ask(0);
                     if (ok) ok = mbar_wait<kSleepAux>(&bars.dq_full, pc & 1, &abort_flag);
                     if (!ok) break;
                     tc_fence_after();
 #pragma unroll
-                    for (int ch = 0; ch < D / 16; ++ch) {
-                        uint32_t v[16];
-                        if (ch + 1 < D / 16) ask(ch + 1);
-                        tmem_ld16(tmem + lane_base + Cfg::kColDQ + 16 * ch, v);
+                    for (int c0 = 0; c0 < D; c0 += 32) {   // 32 columns per round trip (16 in the D = 80 tail)
+                        const int n4 = c0 + 32 <= D ? 8 : 4;
+                        uint32_t v[2][16];
+                        tmem_ld16(tmem + lane_base + Cfg::kColDQ + c0, v[0]);
+                        if (n4 == 8) tmem_ld16(tmem + lane_base + Cfg::kColDQ + c0 + 16, v[1]);
                         tmem_wait_ld();
-                        if (ch == D / 16 - 1) {   // the whole row has left TMEM: the next step's dQ may be issued
+                        if (c0 + 32 >= D) {   // the whole row has left TMEM: the next step's dQ may be issued
                             tc_fence_before();
                             __syncwarp();
                             if (lane == 0) mbar_arrive(&bars.dq_empty);
                         }
-                        float4 y[4];
+                        float4 y[8];
 #pragma unroll
-                        for (int g = 0; g < 4; ++g) {
-                            const float2 a = add2(make_float2(x[ch & 1][g].x, x[ch & 1][g].y), make_float2(__uint_as_float(v[4 * g]), __uint_as_float(v[4 * g + 1])));
-                            const float2 b = add2(make_float2(x[ch & 1][g].z, x[ch & 1][g].w), make_float2(__uint_as_float(v[4 * g + 2]), __uint_as_float(v[4 * g + 3])));
+                        for (int g = 0; g < n4; ++g) {
+                            const uint32_t* w = &v[g / 4][(g & 3) * 4];
+                            const float2 a = add2(make_float2(x[g].x, x[g].y), make_float2(__uint_as_float(w[0]), __uint_as_float(w[1])));
+                            const float2 b = add2(make_float2(x[g].z, x[g].w), make_float2(__uint_as_float(w[2]), __uint_as_float(w[3])));
                             y[g] = make_float4(a.x, a.y, b.x, b.y);
                         }
+                        if (c0 + 32 < D) ask(c0 + 32);
                         if (!last) {
 #pragma unroll
-                            for (int g = 0; g < 4; ++g)
-                                if (in) __stcg(part + (4 * ch + g) * rows, y[g]);
+                            for (int g = 0; g < n4; ++g)
+                                if (in) __stcg(part + (c0 / 4 + g) * rows, y[g]);
                         } else {
 #pragma unroll
-                            for (int c8 = 0; c8 < 2; ++c8) {
-                                const float4 a = y[2 * c8], b = y[2 * c8 + 1];
+                            for (int g = 0; g < n4; g += 2) {
                                 uint4 o;
-                                o.x = pack_bf16(a.x * p.scale, a.y * p.scale);
-                                o.y = pack_bf16(a.z * p.scale, a.w * p.scale);
-                                o.z = pack_bf16(b.x * p.scale, b.y * p.scale);
-                                o.w = pack_bf16(b.z * p.scale, b.w * p.scale);
-                                if (in) *reinterpret_cast<uint4*>(row + 16 * ch + 8 * c8) = o;
+                                o.x = pack_bf16(y[g].x * p.scale, y[g].y * p.scale);
+                                o.y = pack_bf16(y[g].z * p.scale, y[g].w * p.scale);
+                                o.z = pack_bf16(y[g + 1].x * p.scale, y[g + 1].y * p.scale);
+                                o.w = pack_bf16(y[g + 1].z * p.scale, y[g + 1].w * p.scale);
+                                if (in) *reinterpret_cast<uint4*>(row + c0 + 4 * g) = o;
                             }
                         }
                     }
