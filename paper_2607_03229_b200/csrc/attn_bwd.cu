@@ -53,7 +53,7 @@ static_assert(4 * (kRegsLaunch - kRegsService) + 4 * (kRegsLaunch - kRegsReducer
               "setmaxnreg pool arithmetic");
 constexpr int kBT = 128;  // keys per unit = TMEM lanes
 constexpr int kBQ = 128;  // query rows per step
-// head_dim 80, segments of up to three tiles and more units than SMs, or a CTA per segment: the pooled tile buffers (BwdCfg::kPool).  Every tile then costs the
+// head_dim 80, segments of up to three tiles and more units than SMs, or a CTA to a segment: the pooled tile buffers (BwdCfg::kPool).  Every tile then costs the
 // issuer and the producer a hand-shake of its own, 0.1 to 0.3 us a step, which a short unit gets back from loads that no longer wait
 // for its end.  us, two buffers a kind -> pool: 1024 segments of 64 rows 748 -> 625, 256 of 256 610 -> 557, 200 thumbnails of 64 to 256
 // 369 -> 330, 218 of 300 813 -> 801, 163 of 400 944 -> 962, 32 of 2048 2151 -> 2278, one of 200 (a unit per CTA) 17.4 -> 18.4.
@@ -61,20 +61,20 @@ constexpr int kPoolSeqlen = 384;
 // Lists of short segments: one CTA takes all key tiles of a (segment, head), one after the other, instead of one CTA per key tile.  dQ then
 // needs no sum across CTAs: no accumulator to clear (prepass) and to convert (third launch), no reductions through the copy engine, and
 // the same bits on every run.  A query tile's partial dQ waits in the workspace between key tiles, in L2, each thread's row for that
-// thread.  us, a CTA per key tile -> per segment (16 heads of 64 | 80): 4 segments of 64 14.1 -> 10.0 | 15.4 -> 10.8, 512 of 64 229 -> 206 |
-// 338 -> 302, 256 of 128 184 -> 130 | 239 -> 175, 6 of 192 19.3 -> 17.2 | 25.1 -> 22.7, 128 of 256 226 -> 190 | 310 -> 262, 85 of 384
-// 263 -> 237 | 349 -> 351, 200 thumbnails of 64 to 256 243 -> 196 | 316 -> 265.  From four tiles on it is level or slower (64 of 512
-// 324 -> 298 | 454 -> 443, but 32 of 512 164 -> 168 | 228 -> 240, 32 of 1024 544 -> 634 | 720 -> 1057: every step stores and reloads 128 rows), and so it
-// is where whole segments spread worse over the SMs than key tiles do (3 of 192 13.5 -> 15.3 | 17.5 -> 20.5, 12 of 384 45 -> 51 | 66 -> 78):
-// estimated in rounds of one key tile per SM, it may take a tenth more of them.
-constexpr int kOwnTiles = 3;
-static bool own_segments(int64_t n_seg, int64_t n_items, int32_t max_seqlen, int64_t heads, int64_t sms) {
+// thread.  us, a CTA per key tile -> per segment (16 heads of 64 | 80): 4 segments of 64 14.1 -> 10.0 | 15.4 -> 10.8, 512 of 64 232 -> 200 |
+// 315 -> 269, 256 of 128 184 -> 130 | 239 -> 175, 6 of 192 19.3 -> 17.2 | 25.1 -> 22.7, 50 of 192 80 -> 72 | 108 -> 101, 85 of 384 263 -> 230 |
+// 351 -> 329, 64 of 512 299 -> 278 | 405 -> 414, 37 of 512 176 -> 164 | 267 -> 261, 8 of 640 72 -> 61 | 90 -> 98, 8 of 819 116 -> 114 | 160 -> 184,
+// 37 of 1024 548 -> 593 | 761 -> 1062 (every step but a segment's last ones stores 128 rows of dQ and reloads them).  Hence the numbers of tiles.
+// Whole segments spread worse over the SMs than key tiles do (3 of 192 13.5 -> 15.3 | 17.5 -> 20.5, 12 of 384 45 -> 51 | 66 -> 78, 32 of 512
+// 164 -> 168 | 228 -> 240), so they are counted in rounds, a key tile to an SM: up to three tiles a tenth more of them is made up for, above
+// none.  Equal lengths go in whole waves.  Mixed ones, longest first, even out to about a tile if the others keep the SMs
+// busy for as long as the longest, tiles^2 steps (up to three tiles the tenth implies it).
+static bool own_segments(int64_t n_seg, int64_t n_items, int32_t max_seqlen, int64_t heads, int32_t head_dim, int64_t sms) {
     const int64_t tiles = (int64_t(max_seqlen) + kBT - 1) / kBT, segs = n_seg < n_items ? n_seg : n_items;
-    if (tiles > kOwnTiles) return false;
+    if (tiles > (head_dim == 64 ? 7 : 4)) return false;
     const int64_t by_tile = (n_items * heads + sms - 1) / sms;
-    // all of the longest: whole waves of them; mixed lengths, longest first, even out to about one key tile
-    const int64_t by_segment = n_items == segs * tiles ? (segs * heads + sms - 1) / sms * tiles : by_tile + 1;
-    return 10 * by_segment <= 11 * by_tile;
+    if (n_items == segs * tiles) return 10 * ((segs * heads + sms - 1) / sms * tiles) <= (tiles <= 3 ? 11 : 10) * by_tile;
+    return 10 * (by_tile + 1) <= 11 * by_tile && by_tile >= tiles * tiles;
 }
 constexpr int kQH = 64;   // query columns of a step handled by one softmax warpgroup
 
@@ -1205,7 +1205,7 @@ static int32_t run_bwd(const float* rope_cos, const float* rope_sin, const void*
     const size_t dq_bytes = extent_bytes(total_tokens, n_heads, head_dim, tok_stride_grad, head_stride_grad, 2);
     const size_t in_bytes = extent_bytes(total_tokens, n_heads, head_dim, tok_stride_qkv, head_stride_qkv, 2);
     const size_t o_bytes = extent_bytes(total_tokens, n_heads, head_dim, tok_stride_o, head_stride_o, 2);
-    const bool own = rope_cos == nullptr && own_segments(n_seg, n_bwd_items, max_seqlen, n_heads, sm_count()) &&
+    const bool own = rope_cos == nullptr && own_segments(n_seg, n_bwd_items, max_seqlen, n_heads, head_dim, sm_count()) &&
                      !overlap(dq, dq_bytes, q, in_bytes) && !overlap(dq, dq_bytes, k, in_bytes) && !overlap(dq, dq_bytes, v, in_bytes) &&
                      !overlap(dq, dq_bytes, dout, o_bytes) && !overlap(dq, dq_bytes, o, o_bytes) &&
                      !overlap(dq, dq_bytes, lse, size_t(total_tokens) * n_heads * 4);

@@ -14,7 +14,7 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("D", [64, 80])
 @pytest.mark.parametrize("counts,rows", [([1], None), ([128, 127], None), ([129, 128, 1], None), ([255, 257, 3, 256], None),
-                                         ([384, 300], None), ([300, 64, 129], 64), ([300, 130], 100)])
+                                         ([384, 384], None), ([512], None), ([896], None), ([300, 64, 129], 64), ([300, 130], 100)])
 @pytest.mark.parametrize("into", ["own", "strided", "q", "dout"])
 def test_short_segments_at_tile_edges(counts, rows, D, into):
     H, t = 3, sum(counts)
