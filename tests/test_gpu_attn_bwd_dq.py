@@ -39,7 +39,8 @@ def test_short_segments_at_tile_edges(counts, rows, D, into):
     assert st.cpu().tolist()[0] == 0
     for i, (got, ref) in enumerate(zip((dq, dk, dv), oracle.attn_bwd(do, q, k, v, cu, scale))):
         first = got[:t].contiguous()
-        if i > 0 or into in ("own", "strided"):                   # one order of additions: every copy has the same bits
+        # one order of additions, every copy has the same bits (dQ: where a CTA takes the segment, up to seven tiles, or four)
+        if i > 0 or (into in ("own", "strided") and max(counts) <= (896 if D == 64 else 512)):
             assert torch.equal(got.reshape(copies, t, H, D), first.expand(copies, t, H, D))
         if np.linalg.norm(ref) == 0:   # one token has no gradient; what is left is |dO| |O| |K| / sqrt(D) times the 2^-9 of O's rounding
             assert np.abs(to_f64(first)).max() <= 2.0 ** -9 * D * 4 * 4 * scale
